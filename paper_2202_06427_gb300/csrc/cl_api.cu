@@ -5,6 +5,7 @@
 #include <cstdlib>
 #include <cstring>
 #include <new>
+#include <type_traits>
 
 #include "cl_internal.cuh"
 
@@ -45,6 +46,10 @@ struct cl_list {
   clk::SweepArgs* half;
   clk::SweepArgs* full;
   clk::HoodArgs* hood;  // 3D neighbourhood sweep arguments
+  // workspace of the two-set calls, kept between them (see QueryWs)
+  char* qws;
+  size_t qws_bytes;
+  int qws_busy;
   size_t bytes;
 };
 
@@ -97,6 +102,7 @@ void free_all(cl_list* c) {
   cudaFree(c->pl_tiles);
   cudaFree(c->pl_meta);
   cudaFree(c->pl_long);
+  cudaFree(c->qws);
   delete c->half;
   delete c->full;
   delete c->hood;
@@ -507,24 +513,107 @@ int check_query(const cl_list* c, const double* posb, long long nb) {
   return CL_OK;
 }
 
-// Per-call workspace of the two-set queries (allocated and freed here).
+// Workspace of one two-set call: pieces of one device block. The list keeps
+// the block for its next call, up to kQueryKeep bytes (six cudaMalloc and
+// cudaFree a call cost more host time than the sweeps of a small set); a call
+// that finds it in use by another thread allocates its own. Every call is over
+// on its stream before it gives the block back.
+constexpr size_t kQueryKeep = (size_t)256 << 20;
+
 struct QueryWs {
+  clk::QueryBufs bin{};
   int* count = nullptr;
-  long long* start = nullptr;  // 64-bit offsets of the cross list
+  long long* start = nullptr;  // nb + 1 offsets (64-bit), then the error latch
   long long* tiles = nullptr;
   int* meta = nullptr;
   int* err = nullptr;
   int* longs = nullptr;
-  unsigned long long* total = nullptr;
+  int* knn_a = nullptr;
+  float* knn_d = nullptr;
+  float* part_d = nullptr;
+  long long* part_id = nullptr;
+
+  QueryWs(cl_list* list, cudaStream_t stream) : c(list), s(stream) {}
   ~QueryWs() {
-    cudaFree(longs);
-    cudaFree(count);
-    cudaFree(start);
-    cudaFree(tiles);
-    cudaFree(meta);
-    cudaFree(err);
-    cudaFree(total);
+    if (!base) return;
+    cudaStreamSynchronize(s);
+    if (!kept) {
+      cudaFree(base);
+      return;
+    }
+    if (c->qws_bytes > kQueryKeep) {
+      cudaFree(c->qws);
+      c->qws = nullptr;
+      c->qws_bytes = 0;
+    }
+    __atomic_store_n(&c->qws_busy, 0, __ATOMIC_RELEASE);
   }
+  // list: the arrays of the cross list; k > 0: those of the global k closest.
+  int open(long long nb, bool list, int k) {
+    size_t need = carve(nullptr, nb, list, k);
+    if (__atomic_exchange_n(&c->qws_busy, 1, __ATOMIC_ACQUIRE) == 0) {
+      kept = true;
+      if (c->qws_bytes < need) {
+        cudaFree(c->qws);
+        c->qws_bytes = 0;
+        if (cudaMalloc((void**)&c->qws, need) != cudaSuccess) {
+          cudaGetLastError();
+          c->qws = nullptr;
+          __atomic_store_n(&c->qws_busy, 0, __ATOMIC_RELEASE);
+          return CL_ERR_OOM;
+        }
+        c->qws_bytes = need;
+      }
+      base = c->qws;
+    } else if (cudaMalloc((void**)&base, need) != cudaSuccess) {
+      cudaGetLastError();
+      base = nullptr;
+      return CL_ERR_OOM;
+    }
+    carve(base, nb, list, k);
+    return cudaMemsetAsync(err, 0, sizeof(long long), s) == cudaSuccess ? CL_OK : CL_ERR_CUDA;
+  }
+
+ private:
+  size_t carve(char* at, long long nb, bool list, int k) {
+    size_t used = 0;
+    auto take = [&](auto** p, size_t count) {
+      *p = at ? reinterpret_cast<std::remove_reference_t<decltype(*p)>>(at + used) : nullptr;
+      used += (count * sizeof(**p) + 255) & ~(size_t)255;
+    };
+    const size_t n = nb > 0 ? (size_t)nb : 1;
+    const long long nc = c->geo.ncells;
+    take(&bin.q, n);
+    take(&bin.cell, n);
+    if (clk::queries_sorted(nb, nc)) {
+      take(&bin.raw, n);
+      take(&bin.slot, n);
+      take(&bin.counts, (size_t)nc);
+      take(&bin.start, (size_t)nc + 1);
+      take(&bin.tiles, (size_t)clk::scan_tiles_for(nc) + 1);
+      take(&bin.meta, 4);
+    }
+    if (list) {
+      take(&count, n);
+      take(&tiles, (size_t)clk::scan_tiles_for((long long)n));
+      take(&meta, 4);
+      take(&longs, n);
+    }
+    take(&start, list ? n + 2 : 1);
+    err = reinterpret_cast<int*>(start + (list ? n + 1 : 0));
+    if (k > 0) {
+      const size_t parts = (size_t)clk::topk_parts((long long)n, k);
+      take(&knn_a, n * k);
+      take(&knn_d, n * k);
+      take(&part_d, parts * k);
+      take(&part_id, parts * k);
+    }
+    return used;
+  }
+  cl_list* c;
+  cudaStream_t s;
+  char* base = nullptr;
+  bool kept = false;
 };
 
 int read_err(const int* err_dev, cudaStream_t s) {
@@ -544,12 +633,10 @@ int cl_cross_count(const cl_list* cc, const double* posb_dev, long long nb, unsi
   cl_list* c = const_cast<cl_list*>(cc);
   cudaStream_t s = (cudaStream_t)stream;
   if (cudaMemsetAsync(count_dev, 0, sizeof(unsigned long long), s) != cudaSuccess) return CL_ERR_CUDA;
-  size_t b = 0;
-  QueryWs w;
-  if ((e = dev_alloc(&w.err, 1, &b))) return e;
-  if (cudaMemsetAsync(w.err, 0, sizeof(int), s) != cudaSuccess) return CL_ERR_CUDA;
-  if ((e = clk::launch_cross(0, *c->full, c->geo, posb_dev, nb, 0, nullptr, count_dev, nullptr, nullptr, nullptr,
-                             nullptr, nullptr, nullptr, w.err, s)))
+  QueryWs w(c, s);
+  clk::Queries q;
+  if ((e = w.open(nb, false, 0)) || (e = clk::launch_query_bin(*c->full, c->geo, posb_dev, nb, w.bin, w.err, &q, s)) ||
+      (e = clk::launch_cross_count(*c->full, c->d_off_full, q, nullptr, count_dev, s)))
     return e;
   return read_err(w.err, s);
 }
@@ -564,31 +651,25 @@ int cl_cross_pairlist(const cl_list* cc, const double* posb_dev, long long nb, l
   cudaStream_t s = (cudaStream_t)stream;
   *npairs = 0;
   if (nb == 0) return CL_OK;
-  size_t b = 0;
-  QueryWs w;
-  if ((e = dev_alloc(&w.count, (size_t)nb, &b)) || (e = dev_alloc(&w.start, (size_t)nb + 1, &b)) ||
-      (e = dev_alloc(&w.tiles, (size_t)clk::scan_tiles_for(nb), &b)) || (e = dev_alloc(&w.meta, 4, &b)) ||
-      (e = dev_alloc(&w.err, 1, &b)) || (e = dev_alloc(&w.longs, (size_t)nb, &b)))
+  QueryWs w(c, s);
+  clk::Queries q;
+  if ((e = w.open(nb, true, 0)) || (e = clk::launch_query_bin(*c->full, c->geo, posb_dev, nb, w.bin, w.err, &q, s)) ||
+      (e = clk::launch_cross_count(*c->full, c->d_off_full, q, w.count, nullptr, s)) ||
+      (e = clk::launch_scan64(w.count, nb, w.tiles, w.start, w.meta, s)))
     return e;
-  if (cudaMemsetAsync(w.err, 0, sizeof(int), s) != cudaSuccess) return CL_ERR_CUDA;
-  if ((e = clk::launch_cross(0, *c->full, c->geo, posb_dev, nb, 0, w.count, nullptr, nullptr, nullptr, nullptr,
-                             nullptr, nullptr, nullptr, w.err, s)))
-    return e;
-  if ((e = clk::launch_scan64(w.count, nb, w.tiles, w.start, w.meta, s))) return e;
-  long long total = 0;
-  int meta[4] = {0, 0, 0, 0};
-  if (cudaMemcpyAsync(&total, w.start + nb, sizeof(long long), cudaMemcpyDeviceToHost, s) != cudaSuccess ||
-      cudaMemcpyAsync(meta, w.meta, sizeof(meta), cudaMemcpyDeviceToHost, s) != cudaSuccess)
+  long long back[2] = {0, 0};  // the total and, after it, the error latch
+  if (cudaMemcpyAsync(back, w.start + nb, sizeof(back), cudaMemcpyDeviceToHost, s) != cudaSuccess ||
+      cudaStreamSynchronize(s) != cudaSuccess)
     return CL_ERR_CUDA;
-  if ((e = read_err(w.err, s))) return e;
+  if (back[1]) return CL_ERR_NONFINITE;
+  const long long total = back[0];
   *npairs = total;
   if ((e = cl_pairlist_fits(total, capacity))) return e;
   if (total == 0) return CL_OK;
   if (!pa_dev || !pb_dev || !pd_dev) return CL_ERR_INVALID_ARG;
-  if ((e = clk::launch_cross(1, *c->full, c->geo, posb_dev, nb, 0, nullptr, nullptr, w.start, pa_dev, pb_dev, pd_dev,
-                             nullptr, nullptr, w.err, s)))
+  if ((e = clk::launch_cross_fill(*c->full, c->d_off_full, q, w.count, w.start, pa_dev, pb_dev, pd_dev, w.longs,
+                                  w.meta + 3, s)))
     return e;
-  if ((e = clk::launch_pairs_sort((int)nb, w.count, w.start, pa_dev, pd_dev, w.longs, w.meta + 3, s))) return e;
   return cudaStreamSynchronize(s) == cudaSuccess ? CL_OK : CL_ERR_CUDA;
 }
 
@@ -599,12 +680,10 @@ int cl_cross_knn(const cl_list* cc, const double* posb_dev, long long nb, int k,
   cl_list* c = const_cast<cl_list*>(cc);
   cudaStream_t s = (cudaStream_t)stream;
   if (nb == 0) return CL_OK;
-  size_t b = 0;
-  QueryWs w;
-  if ((e = dev_alloc(&w.err, 1, &b))) return e;
-  if (cudaMemsetAsync(w.err, 0, sizeof(int), s) != cudaSuccess) return CL_ERR_CUDA;
-  if ((e = clk::launch_cross(2, *c->full, c->geo, posb_dev, nb, k, nullptr, nullptr, nullptr, nullptr, nullptr,
-                             nullptr, knn_a_dev, knn_d_dev, w.err, s)))
+  QueryWs w(c, s);
+  clk::Queries q;
+  if ((e = w.open(nb, false, 0)) || (e = clk::launch_query_bin(*c->full, c->geo, posb_dev, nb, w.bin, w.err, &q, s)) ||
+      (e = clk::launch_cross_knn(*c->full, c->d_off_full, q, k, knn_a_dev, knn_d_dev, s)))
     return e;
   return read_err(w.err, s);
 }
@@ -616,29 +695,20 @@ int cl_cross_topk(const cl_list* cc, const double* posb_dev, long long nb, int k
   cl_list* c = const_cast<cl_list*>(cc);
   cudaStream_t s = (cudaStream_t)stream;
   *nfound = 0;
-  size_t b = 0;
-  QueryWs w;
-  int* la = nullptr;
-  float* ld = nullptr;
-  const size_t m = (size_t)(nb > 0 ? nb : 1) * k;
-  if ((e = dev_alloc(&w.err, 2, &b)) || (e = dev_alloc(&la, m, &b)) || (e = dev_alloc(&ld, m, &b))) {
-    cudaFree(la);
-    cudaFree(ld);
+  QueryWs w(c, s);
+  clk::Queries q;
+  // err[0]: the error latch, err[1]: the number found
+  if ((e = w.open(nb, false, k)) || (e = clk::launch_query_bin(*c->full, c->geo, posb_dev, nb, w.bin, w.err, &q, s)) ||
+      (e = clk::launch_cross_knn(*c->full, c->d_off_full, q, k, w.knn_a, w.knn_d, s)) ||
+      (e = clk::launch_topk_merge(w.knn_a, w.knn_d, nb, k, w.part_d, w.part_id, a_dev, b_dev, d_dev, w.err + 1, s)))
     return e;
-  }
-  if (cudaMemsetAsync(w.err, 0, 2 * sizeof(int), s) != cudaSuccess) e = CL_ERR_CUDA;
-  if (!e && nb > 0)
-    e = clk::launch_cross(2, *c->full, c->geo, posb_dev, nb, k, nullptr, nullptr, nullptr, nullptr, nullptr,
-                          nullptr, la, ld, w.err, s);
-  if (!e) e = clk::launch_topk_merge(la, ld, nb, k, a_dev, b_dev, d_dev, w.err + 1, s);
-  int found = 0;
-  if (!e && cudaMemcpyAsync(&found, w.err + 1, sizeof(int), cudaMemcpyDeviceToHost, s) != cudaSuccess)
-    e = CL_ERR_CUDA;
-  if (!e) e = read_err(w.err, s);
-  cudaFree(la);
-  cudaFree(ld);
-  if (!e) *nfound = found;
-  return e;
+  int back[2] = {0, 0};
+  if (cudaMemcpyAsync(back, w.err, sizeof(back), cudaMemcpyDeviceToHost, s) != cudaSuccess ||
+      cudaStreamSynchronize(s) != cudaSuccess)
+    return CL_ERR_CUDA;
+  if (back[0]) return CL_ERR_NONFINITE;
+  *nfound = back[1];
+  return CL_OK;
 }
 
 int cl_query(const cl_list* c, int what, long long* value, void* stream) {

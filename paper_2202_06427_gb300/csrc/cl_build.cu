@@ -407,10 +407,25 @@ int launch_octsort(const int* cells, const int* ncells_listed, const int* cell_s
 
 int scan_tiles_for(long long ncells) { return (int)((ncells + kScanTile - 1) / kScanTile); }
 
+int launch_scan_cells(const int* counts, long long ncells, int* tile_sum, int* meta, int* cell_start, cudaStream_t s) {
+  const int ntiles = scan_tiles_for(ncells);
+  k_scan_reduce<int><<<ntiles, kScanThreads, 0, s>>>(counts, ncells, tile_sum, meta);
+  k_scan_final<int><<<ntiles, kScanThreads, 0, s>>>(counts, ncells, tile_sum, cell_start);
+  return cudaGetLastError() == cudaSuccess ? CL_OK : CL_ERR_CUDA;
+}
+
+int launch_cell_order(int n, int nx, int ny, long long ncells, const int* slot, const float4* xl,
+                      const int* cell_start, float4* xs, unsigned* cellc, cudaStream_t s) {
+  const int blocks = (int)(((long long)n + 256 * kBinPer - 1) / (256 * kBinPer));
+  k_scatter<<<blocks, 256, 0, s>>>(n, nx, ny, slot, xl, cell_start, xs);
+  const long long cb = std::min<long long>((ncells + 255) / 256, 152 * 8);
+  k_cellc<<<(int)cb, 256, 0, s>>>(ncells, nx, ny, cell_start, cellc);
+  return cudaGetLastError() == cudaSuccess ? CL_OK : CL_ERR_CUDA;
+}
+
 // Enqueue the whole binning pipeline on `s`. Returns CL_OK or CL_ERR_CUDA.
 int launch_build(const Geo& g, const BuildBufs& b, cudaStream_t s) {
   const long long nc = g.ncells;
-  const int ntiles = scan_tiles_for(nc);
   if (cudaMemsetAsync(b.counts, 0, sizeof(int) * nc, s) != cudaSuccess) return CL_ERR_CUDA;
   if (cudaMemsetAsync(b.meta + 1, 0, sizeof(int) * 2, s) != cudaSuccess) return CL_ERR_CUDA;
   BinArgs a;
@@ -442,14 +457,9 @@ int launch_build(const Geo& g, const BuildBufs& b, cudaStream_t s) {
       else k_bin<2, false><<<blocks, 256, 0, s>>>(a);
     }
   }
-  k_scan_reduce<int><<<ntiles, kScanThreads, 0, s>>>(b.counts, nc, b.tile_sum, b.meta);
-  k_scan_final<int><<<ntiles, kScanThreads, 0, s>>>(b.counts, nc, b.tile_sum, b.cell_start);
-  if (b.n > 0) {
-    k_scatter<<<blocks, 256, 0, s>>>(b.n, g.n[0], g.n[1], b.slot, b.xl, b.cell_start, b.xs);
-    const long long cb = std::min<long long>((nc + 255) / 256, 152 * 8);
-    k_cellc<<<(int)cb, 256, 0, s>>>(nc, g.n[0], g.n[1], b.cell_start, b.cellc);
-  }
-  return cudaGetLastError() == cudaSuccess ? CL_OK : CL_ERR_CUDA;
+  int e = launch_scan_cells(b.counts, nc, b.tile_sum, b.meta, b.cell_start, s);
+  if (!e && b.n > 0) e = launch_cell_order(b.n, g.n[0], g.n[1], nc, b.slot, b.xl, b.cell_start, b.xs, b.cellc, s);
+  return e;
 }
 
 }  // namespace clk

@@ -1,260 +1,633 @@
 // cl_cross.cu -- pairs between two sets of particles (Sec. 3.2, Code 8: a cell
 // list of x and a second set y; Sec. 4.1: neighbour lists between two sets).
 // The cell list is the one of set A (cl_build); every particle b of set B is
-// binned on A's grid like k_bin does (FP64 wrap and cell, FP32 coordinate
-// relative to the cell centre) and sweeps the FULL stencil of its cell, the
-// displacement to a being (xs_a + S_o) - x_b as in the one-set sweep. Every
-// (a, b) pair-image within the cutoff is visited once; there is no a < b rule.
+// binned on A's grid (FP64 wrap and cell, FP32 coordinate relative to the cell
+// centre) and sweeps the FULL stencil of its cell, the displacement to a being
+// (xs_a + S_o) - x_b as in the one-set sweep. Every (a, b) pair-image within
+// the cutoff is visited once; there is no a < b rule.
 //
-//   k_cross<COUNT>   per-b counts (and their sum)
-//   k_cross<FILL>    writes (a, b, r) into b's segment of the list
+//   k_query_bin      cell and local coordinate of each query point
+//   (cell order)     the queries counting-sorted by cell, when they are many
+//   k_cross_count    per-b counts (and their sum), one warp per query
+//   k_cross_fill     (a, b, r) of b's segment of the list, sorted by a
 //   k_cross_knn      per b the k nearest a within the cutoff (k <= 32)
-//   k_topk_merge     the k smallest over all per-b lists (one CTA)
+//   k_topk_part, k_topk_last  the k smallest over all per-b lists
+//
+// A warp takes one query: its lanes test the stencil's cells 32 at a time
+// (the cell's bounding box against the cutoff, as in sweep_particle2), the
+// kept ones are compacted in shared memory, and groups of G lanes run over
+// them, G chosen by the mean occupancy so that a group's passes are mostly
+// full. One thread per query in input order, the form before this one, was
+// bound by its serial chain of uncoalesced loads and wrote each segment with
+// one lane's stores.
+#include <algorithm>
 #include <cfloat>
+#include <climits>
+#include <cmath>
 
+#include "cl_sort.cuh"
 #include "cl_sweep.cuh"
 
 namespace clk {
 namespace {
 
 constexpr int kKnnMax = CL_KNN_MAX;
+constexpr int kCrossWarps = 8;
+constexpr int kFillWarps = 4;  // 8.4 KB of segment per warp: five CTAs of four warps fit an SM, two of eight
 
 struct QueryArgs {
   const double* pos;  // (nb, dim) FP64
   long long nb;
-  int dim, ortho;
+  int nx, ny, nz;
   double m[9];        // t = x M (cell units)
   float g[9];         // cell edge vectors (rows)
 };
 
-// Cell and centred FP32 coordinate of query point b; false when not finite.
-__device__ __forceinline__ bool bin_query(const SweepArgs& A, const QueryArgs& Q, long long b, int& cx, int& cy,
-                                          int& cz, float& px, float& py, float& pz) {
-  double x[3] = {0.0, 0.0, 0.0};
-  bool finite = true;
-  for (int k = 0; k < Q.dim; ++k) {
-    x[k] = Q.pos[b * Q.dim + k];
-    finite = finite && isfinite(x[k]);
-  }
-  if (!finite) return false;
-  const int nk[3] = {A.nx, A.ny, A.nz};
-  int c[3] = {0, 0, 0};
-  float u[3] = {0.f, 0.f, 0.f};
-  for (int k = 0; k < Q.dim; ++k) {
-    double t;
-    if (Q.ortho) {
-      t = x[k] * Q.m[k * 3 + k];
-    } else {
-      t = 0.0;
-      for (int q = 0; q < Q.dim; ++q) t = fma(x[q], Q.m[q * 3 + k], t);
-    }
-    const double f = floor(t);
-    long long ci = (long long)f % nk[k];
-    if (ci < 0) ci += nk[k];
-    c[k] = (int)ci;
-    u[k] = (float)(t - f) - 0.5f;
-  }
-  px = py = pz = 0.f;
-  for (int k = 0; k < Q.dim; ++k) {
-    px = fmaf(u[k], Q.g[k * 3 + 0], px);
-    py = fmaf(u[k], Q.g[k * 3 + 1], py);
-    pz = fmaf(u[k], Q.g[k * 3 + 2], pz);
-  }
-  cx = c[0];
-  cy = c[1];
-  cz = c[2];
-  return true;
-}
-
-// Visits every a within the cutoff of query b: f(a_original, r^2).
-template <class Fn>
-__device__ __forceinline__ void query_sweep(const SweepArgs& A, int cx, int cy, int cz, float px, float py, float pz,
-                                           Fn&& f) {
-  for (int k = 0; k < A.noff; ++k) {
-    const Off& o = A.off[k];
-    const int c = stencil_cell(A, k, cx, cy, cz);
-    const float sx = o.sx - px, sy = o.sy - py, sz = o.sz - pz;
-    const int j1 = A.cell_start[c + 1];
-    for (int j = A.cell_start[c]; j < j1; ++j) {
-      const float4 q = __ldg(&A.xs[j]);
-      const float dx = q.x + sx, dy = q.y + sy, dz = q.z + sz;
-      const float d2 = fmaf(dx, dx, fmaf(dy, dy, dz * dz));
-      if (d2 < A.rc2) f(__float_as_int(q.w), d2);
-    }
-  }
-}
-
-__global__ void __launch_bounds__(256) k_cross_count(const __grid_constant__ SweepArgs A,
-                                                     const __grid_constant__ QueryArgs Q, int* __restrict__ count,
-                                                     unsigned long long* __restrict__ total, int* __restrict__ err) {
-  const long long b = blockIdx.x * (long long)blockDim.x + threadIdx.x;
-  unsigned n = 0;
-  if (b < Q.nb) {
-    int cx, cy, cz;
-    float px, py, pz;
-    if (bin_query(A, Q, b, cx, cy, cz, px, py, pz)) {
-      query_sweep(A, cx, cy, cz, px, py, pz, [&](int, float) { ++n; });
-    } else {
-      atomicOr(err, kErrNonFinite);
-    }
-    if (count) count[b] = (int)n;
-  }
-#pragma unroll
-  for (int o = 16; o; o >>= 1) n += __shfl_xor_sync(0xffffffffu, n, o);
-  if ((threadIdx.x & 31) == 0 && n && total) atomicAdd(total, (unsigned long long)n);
-}
-
-__global__ void __launch_bounds__(256) k_cross_fill(const __grid_constant__ SweepArgs A,
-                                                    const __grid_constant__ QueryArgs Q, const long long* __restrict__ start,
-                                                    int* __restrict__ pa, int* __restrict__ pb,
-                                                    float* __restrict__ pd) {
+// Packed cell and centred FP32 coordinate of every query point; a point that
+// is not finite is parked in cell 0 at its sentinel position, where every
+// distance test against it fails. With counts the point also takes its slot
+// in its cell (q then holds the packed cell in w, for the reordering).
+template <int DIM, bool ORTHO>
+__global__ void __launch_bounds__(256) k_query_bin(const __grid_constant__ QueryArgs Q, float4* __restrict__ q,
+                                                   unsigned* __restrict__ cell, int* __restrict__ counts,
+                                                   int* __restrict__ slot, int* __restrict__ err) {
   const long long b = blockIdx.x * (long long)blockDim.x + threadIdx.x;
   if (b >= Q.nb) return;
-  int cx, cy, cz;
-  float px, py, pz;
-  if (!bin_query(A, Q, b, cx, cy, cz, px, py, pz)) return;
-  long long pos = start[b];
-  query_sweep(A, cx, cy, cz, px, py, pz, [&](int a, float d2) {
-    pa[pos] = a;
-    pb[pos] = (int)b;
-    pd[pos] = sqrtf(d2);
-    ++pos;
-  });
+  double x[DIM];
+  bool finite = true;
+#pragma unroll
+  for (int k = 0; k < DIM; ++k) {
+    x[k] = Q.pos[b * DIM + k];
+    finite = finite && isfinite(x[k]);
+  }
+  const int nk[3] = {Q.nx, Q.ny, Q.nz};
+  int c[3] = {0, 0, 0};
+  float4 o = make_float4(0.f, 0.f, 0.f, 0.f);
+  if (finite) {
+    float u[DIM];
+#pragma unroll
+    for (int k = 0; k < DIM; ++k) {
+      double t;
+      if (ORTHO) {
+        t = x[k] * Q.m[k * 3 + k];
+      } else {
+        t = 0.0;
+#pragma unroll
+        for (int p = 0; p < DIM; ++p) t = fma(x[p], Q.m[p * 3 + k], t);
+      }
+      const double f = floor(t);
+      long long ci = (long long)f;
+      if (ci < 0 || ci >= nk[k]) {
+        ci %= nk[k];
+        if (ci < 0) ci += nk[k];
+      }
+      c[k] = (int)ci;
+      u[k] = (float)(t - f) - 0.5f;
+    }
+#pragma unroll
+    for (int k = 0; k < DIM; ++k) {
+      o.x = fmaf(u[k], Q.g[k * 3 + 0], o.x);
+      o.y = fmaf(u[k], Q.g[k * 3 + 1], o.y);
+      o.z = fmaf(u[k], Q.g[k * 3 + 2], o.z);
+    }
+  } else {
+    o = sentinel_pos((int)b);
+    atomicOr(err, kErrNonFinite);
+  }
+  const unsigned pc = (unsigned)c[0] | ((unsigned)c[1] << 10) | ((unsigned)c[2] << 20);
+  if (counts) {
+    o.w = __uint_as_float(pc);
+    slot[b] = atomicAdd(&counts[c[0] + Q.nx * (c[1] + Q.ny * c[2])], 1);
+  } else {
+    o.w = __int_as_float((int)b);
+    cell[b] = pc;
+  }
+  q[b] = o;
+}
+
+struct CrossArgs {
+  const float4* xs;
+  const int* cell_start;
+  const Off* off;  // device memory
+  int noff;
+  int nx, ny, nz;
+  float rc2;
+  float ex, ey, ez;  // padded half-widths of a cell's bounding box; cull: use them
+  bool cull;
+};
+
+// A warp's stencil cells under way: shift minus the query (w: squared distance
+// of the query to the cell's bounding box) and range of sorted particles.
+struct WarpCells {
+  float4 s[32];
+  int2 j[32];
+};
+
+// Stencil to shared memory: (S_x, S_y, S_z, dx | dy << 10 | dz << 20).
+// NEAR: in order of |S|, so that the nearest cells come first.
+template <bool NEAR>
+__device__ __forceinline__ void load_stencil(const CrossArgs& A, float4* stab, float* key) {
+  for (int k = threadIdx.x; k < A.noff; k += blockDim.x) {
+    const Off o = A.off[k];
+    const float4 e = make_float4(o.sx, o.sy, o.sz,
+                                 __uint_as_float((unsigned)o.dx | ((unsigned)o.dy << 10) | ((unsigned)o.dz << 20)));
+    if (NEAR) key[k] = fmaf(o.sx, o.sx, fmaf(o.sy, o.sy, o.sz * o.sz));
+    else stab[k] = e;
+  }
+  if (NEAR) {
+    __syncthreads();
+    for (int k = threadIdx.x; k < A.noff; k += blockDim.x) {
+      const float v = key[k];
+      int r = 0;  // entries before k in the order (|S|^2, k)
+      for (int t = 0; t < A.noff; ++t) r += (key[t] < v || (key[t] == v && t < k)) ? 1 : 0;
+      const Off o = A.off[k];
+      stab[r] = make_float4(o.sx, o.sy, o.sz,
+                            __uint_as_float((unsigned)o.dx | ((unsigned)o.dy << 10) | ((unsigned)o.dz << 20)));
+    }
+  }
+  __syncthreads();
+}
+
+// Entries k0 + lane of the stencil about the query's cell: the non-empty cells
+// within sqrt(lim) of the query (all of them without culling) go to W; returns
+// their number.
+__device__ __forceinline__ int query_cells(const CrossArgs& A, const float4* stab, WarpCells& W, int k0, int lane,
+                                           unsigned cc, const float4& p, float lim) {
+  const int k = k0 + lane;
+  bool keep = false;
+  float4 e = make_float4(0.f, 0.f, 0.f, 0.f);
+  int2 r = make_int2(0, 0);
+  if (k < A.noff) {
+    e = stab[k];
+    const unsigned d = __float_as_uint(e.w);
+    const float bx = fmaxf(fabsf(p.x - e.x) - A.ex, 0.f), by = fmaxf(fabsf(p.y - e.y) - A.ey, 0.f),
+                bz = fmaxf(fabsf(p.z - e.z) - A.ez, 0.f);
+    e.w = fmaf(bx, bx, fmaf(by, by, bz * bz));
+    if (!A.cull) e.w = 0.f;
+    if (e.w < lim) {
+      int x2 = (int)(cc & 1023u) + (int)(d & 1023u);
+      x2 -= (x2 >= A.nx) ? A.nx : 0;
+      int y2 = (int)((cc >> 10) & 1023u) + (int)((d >> 10) & 1023u);
+      y2 -= (y2 >= A.ny) ? A.ny : 0;
+      int z2 = (int)(cc >> 20) + (int)(d >> 20);
+      z2 -= (z2 >= A.nz) ? A.nz : 0;
+      const int c = x2 + A.nx * (y2 + A.ny * z2);
+      r.x = __ldg(A.cell_start + c);
+      r.y = __ldg(A.cell_start + c + 1);
+      keep = r.y > r.x;
+    }
+  }
+  const unsigned m = __ballot_sync(0xffffffffu, keep);
+  __syncwarp();
+  if (keep) {
+    const int at = __popc(m & ((1u << lane) - 1u));
+    W.s[at] = make_float4(e.x - p.x, e.y - p.y, e.z - p.z, e.w);
+    W.j[at] = r;
+  }
+  __syncwarp();
+  return __popc(m);
+}
+
+__device__ __forceinline__ float query_d2(const float4& q, const float4& s) {
+  const float dx = q.x + s.x, dy = q.y + s.y, dz = q.z + s.z;
+  return fmaf(dx, dx, fmaf(dy, dy, dz * dz));
+}
+
+template <int G>
+__global__ void __launch_bounds__(32 * kCrossWarps) k_cross_count(const __grid_constant__ CrossArgs A,
+                                                                  const Queries Q, int* __restrict__ count,
+                                                                  unsigned long long* __restrict__ total) {
+  extern __shared__ float4 stab[];
+  __shared__ WarpCells cells[kCrossWarps];
+  load_stencil<false>(A, stab, nullptr);
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  WarpCells& W = cells[warp];
+  unsigned long long sum = 0;
+  for (long long b = blockIdx.x * (long long)kCrossWarps + warp; b < Q.nb; b += (long long)gridDim.x * kCrossWarps) {
+    const float4 p = Q.q[b];
+    const unsigned cc = Q.cell[b];
+    unsigned n = 0;
+    for (int k0 = 0; k0 < A.noff; k0 += 32) {
+      const int nk = query_cells(A, stab, W, k0, lane, cc, p, A.rc2);
+      for (int i = lane / G; i < nk; i += 32 / G) {
+        const float4 s = W.s[i];
+        const int2 r = W.j[i];
+#pragma unroll 2
+        for (int j = r.x + lane % G; j < r.y; j += G) n += query_d2(__ldg(&A.xs[j]), s) < A.rc2 ? 1u : 0u;
+      }
+    }
+    n = __reduce_add_sync(0xffffffffu, n);
+    if (count && lane == 0) count[__float_as_int(p.w)] = (int)n;
+    sum += n;
+  }
+  if (total && lane == 0 && sum) atomicAdd(total, sum);
+}
+
+// The kept pairs of a query are compacted into the warp's shared-memory
+// segment and sorted by a. WIDE false (set A has fewer than 2^22 particles):
+// the key is a << 10 | slot, one word, and the distances stay in place; WIDE:
+// (a, distance) pairs. A segment longer than kMaxSegment is written unsorted
+// and listed in longs.
+template <int G, bool WIDE>
+__global__ void __launch_bounds__(32 * kFillWarps, 5) k_cross_fill(const __grid_constant__ CrossArgs A,
+                                                                    const Queries Q, const int* __restrict__ count,
+                                                                    const long long* __restrict__ start,
+                                                                    int* __restrict__ pa, int* __restrict__ pb,
+                                                                    float* __restrict__ pd, int* __restrict__ longs,
+                                                                    int* __restrict__ nlong) {
+  extern __shared__ float4 stab[];
+  __shared__ WarpCells cells[kFillWarps];
+  float* seg = reinterpret_cast<float*>(stab + A.noff);
+  load_stencil<false>(A, stab, nullptr);
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const unsigned lt = (1u << lane) - 1u;
+  WarpCells& W = cells[warp];
+  float* V = seg + (size_t)warp * 2 * kSegPad;
+  unsigned* K = reinterpret_cast<unsigned*>(V + kSegPad);
+  for (long long t = blockIdx.x * (long long)kFillWarps + warp; t < Q.nb; t += (long long)gridDim.x * kFillWarps) {
+    const float4 p = Q.q[t];
+    const unsigned cc = Q.cell[t];
+    const int b = __float_as_int(p.w);
+    const int cnt = __ldg(count + b);
+    if (cnt == 0) continue;
+    const long long base = __ldg(start + b);
+    const bool big = cnt > kMaxSegment;
+    int L = 0;
+    for (int k0 = 0; k0 < A.noff; k0 += 32) {
+      const int nk = query_cells(A, stab, W, k0, lane, cc, p, A.rc2);
+      for (int i0 = 0; i0 < nk; i0 += 32 / G) {
+        const int i = i0 + lane / G;
+        float4 s = make_float4(0.f, 0.f, 0.f, 0.f);
+        int j = 0, j1 = 0;
+        if (i < nk) {
+          s = W.s[i];
+          const int2 r = W.j[i];
+          j = r.x + lane % G;
+          j1 = r.y;
+        }
+        while (__any_sync(0xffffffffu, j < j1)) {
+          int a[2];
+          float d2[2];
+#pragma unroll
+          for (int u = 0; u < 2; ++u) {
+            a[u] = 0;
+            d2[u] = FLT_MAX;
+            if (j + u * G < j1) {
+              const float4 q = __ldg(&A.xs[j + u * G]);
+              a[u] = __float_as_int(q.w);
+              d2[u] = query_d2(q, s);
+            }
+          }
+          j += 2 * G;
+#pragma unroll
+          for (int u = 0; u < 2; ++u) {
+            const bool hit = d2[u] < A.rc2;
+            const unsigned m = __ballot_sync(0xffffffffu, hit);
+            const int e = L + __popc(m & lt);
+            if (hit && e < cnt) {
+              if (big) {
+                pa[base + e] = a[u];
+                pb[base + e] = b;
+                pd[base + e] = sqrtf(d2[u]);
+              } else {
+                K[seg_at(e)] = WIDE ? (unsigned)a[u] : ((unsigned)a[u] << 10) | (unsigned)e;
+                V[seg_at(e)] = d2[u];
+              }
+            }
+            L += __popc(m);
+          }
+        }
+      }
+    }
+    __syncwarp();
+    if (big) {
+      if (lane == 0) longs[atomicAdd(nlong, 1)] = b;
+      continue;
+    }
+    const int nw = min(L, cnt);
+    if (WIDE) sort_segment(reinterpret_cast<int*>(K), V, nw, lane);
+    else sort_keys(K, nw, lane);
+    for (int i = lane; i < nw; i += 32) {
+      const unsigned key = K[seg_at(i)];
+      pa[base + i] = WIDE ? (int)key : (int)(key >> 10);
+      pb[base + i] = b;
+      pd[base + i] = sqrtf(V[WIDE ? seg_at(i) : seg_at((int)(key & 1023u))]);
+    }
+    __syncwarp();
+  }
+}
+
+// A warp's running best k of (distance, id), ascending, entry l in lane l
+// (l < k): offers the lanes' candidates (ok ones) and keeps the k smallest.
+template <class ID>
+__device__ __forceinline__ void best_offer(float& bd, ID& bi, float& kd, ID& ki, int k, bool ok, float d, ID id) {
+  const int lane = threadIdx.x & 31;
+  unsigned m = __ballot_sync(0xffffffffu, ok && (d < kd || (d == kd && id < ki)));
+  while (m) {
+    const int src = __ffs(m) - 1;
+    m &= m - 1;
+    const float cd = __shfl_sync(0xffffffffu, d, src);
+    const ID ci = __shfl_sync(0xffffffffu, id, src);
+    if (!(cd < kd || (cd == kd && ci < ki))) continue;  // uniform: a better one came in since
+    const bool before = lane < k && (bd < cd || (bd == cd && bi <= ci));
+    const int at = __popc(__ballot_sync(0xffffffffu, before));
+    const float ud = __shfl_up_sync(0xffffffffu, bd, 1);
+    const ID ui = __shfl_up_sync(0xffffffffu, bi, 1);
+    if (lane > at) {
+      bd = ud;
+      bi = ui;
+    } else if (lane == at) {
+      bd = cd;
+      bi = ci;
+    }
+    kd = __shfl_sync(0xffffffffu, bd, k - 1);
+    ki = __shfl_sync(0xffffffffu, bi, k - 1);
+  }
 }
 
 // Per query b: the k nearest a within the cutoff, ascending by distance (ties:
-// smaller a first); empty slots hold a = -1, r = +inf.
-__global__ void __launch_bounds__(128) k_cross_knn(const __grid_constant__ SweepArgs A,
-                                                   const __grid_constant__ QueryArgs Q, int k, int* __restrict__ out_a,
-                                                   float* __restrict__ out_d, int* __restrict__ err) {
-  const long long b = blockIdx.x * (long long)blockDim.x + threadIdx.x;
-  if (b >= Q.nb) return;
-  float bd[kKnnMax];
-  int ba[kKnnMax];
-  for (int q = 0; q < k; ++q) {
-    bd[q] = FLT_MAX;
-    ba[q] = -1;
-  }
-  int cx, cy, cz;
-  float px, py, pz;
-  if (bin_query(A, Q, b, cx, cy, cz, px, py, pz)) {
-    query_sweep(A, cx, cy, cz, px, py, pz, [&](int a, float d2) {
-      if (d2 > bd[k - 1] || (d2 == bd[k - 1] && (ba[k - 1] >= 0 && a > ba[k - 1]))) return;
-      int q = k - 1;  // insertion: shift the larger entries up
-      while (q > 0 && (bd[q - 1] > d2 || (bd[q - 1] == d2 && ba[q - 1] > a))) {
-        bd[q] = bd[q - 1];
-        ba[q] = ba[q - 1];
-        --q;
+// smaller a first); empty slots hold a = -1, r = +inf. The stencil's cells are
+// visited nearest first and a cell beyond the k-th distance found so far is
+// skipped, so a query tests the particles of about the ball of its k-th
+// neighbour and not of the cutoff's.
+template <int G>
+__global__ void __launch_bounds__(32 * kCrossWarps) k_cross_knn(const __grid_constant__ CrossArgs A, const Queries Q,
+                                                                int k, int* __restrict__ out_a,
+                                                                float* __restrict__ out_d) {
+  extern __shared__ float4 stab[];
+  __shared__ WarpCells cells[kCrossWarps];
+  load_stencil<true>(A, stab, reinterpret_cast<float*>(stab + A.noff));
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  WarpCells& W = cells[warp];
+  for (long long t = blockIdx.x * (long long)kCrossWarps + warp; t < Q.nb; t += (long long)gridDim.x * kCrossWarps) {
+    const float4 p = Q.q[t];
+    const unsigned cc = Q.cell[t];
+    float bd = FLT_MAX, kd = FLT_MAX;
+    int ba = INT_MAX, ka = INT_MAX;
+    for (int k0 = 0; k0 < A.noff; k0 += 32) {
+      const int nk = query_cells(A, stab, W, k0, lane, cc, p, fminf(A.rc2, kd));
+      for (int i0 = 0; i0 < nk; i0 += 32 / G) {
+        const int i = i0 + lane / G;
+        float4 s = make_float4(0.f, 0.f, 0.f, 0.f);
+        int j = 0, j1 = 0;
+        if (i < nk) {
+          s = W.s[i];
+          const int2 r = W.j[i];
+          j = r.x + lane % G;
+          j1 = s.w < kd ? r.y : 0;
+        }
+        while (__any_sync(0xffffffffu, j < j1)) {
+          int a = 0;
+          float d2 = FLT_MAX;
+          if (j < j1) {
+            const float4 q = __ldg(&A.xs[j]);
+            a = __float_as_int(q.w);
+            d2 = query_d2(q, s);
+          }
+          j += G;
+          best_offer(bd, ba, kd, ka, k, d2 < A.rc2, d2, a);
+        }
       }
-      bd[q] = d2;
-      ba[q] = a;
-    });
-  } else {
-    atomicOr(err, kErrNonFinite);
-  }
-  for (int q = 0; q < k; ++q) {
-    out_a[b * k + q] = ba[q];
-    out_d[b * k + q] = ba[q] >= 0 ? sqrtf(bd[q]) : INFINITY;
+    }
+    if (lane < k) {
+      const long long o = (long long)__float_as_int(p.w) * k + lane;
+      const bool have = bd < FLT_MAX;
+      out_a[o] = have ? ba : -1;
+      out_d[o] = have ? sqrtf(bd) : INFINITY;
+    }
   }
 }
 
-// The k smallest (r, a, b) over nb per-query lists of k (one CTA of 1024
-// threads): chunks of 1024 candidates are sorted in shared memory by a bitonic
-// network and merged into the running best k.
-__global__ void __launch_bounds__(1024) k_topk_merge(const int* __restrict__ la, const float* __restrict__ ld,
-                                                     long long nb, int k, int* __restrict__ oa, int* __restrict__ ob,
-                                                     float* __restrict__ od, int* __restrict__ found) {
-  __shared__ float cd[1024];
-  __shared__ long long cid[1024];
-  __shared__ float bd[kKnnMax];
-  __shared__ long long bid[kKnnMax];
-  __shared__ float md[2 * kKnnMax];
-  __shared__ long long mid[2 * kKnnMax];
-  const int t = threadIdx.x;
-  if (t < k) {
-    bd[t] = INFINITY;
-    bid[t] = -1;
+// The k smallest (r, id), id = b * k + q, over nb per-query lists of k: each
+// warp keeps the best of its share, the last kernel the best of theirs. (One
+// CTA sorting 1,024 candidates at a time took 5.0 ms for 60,000 lists of 5.)
+constexpr int kTopkWarps = 8;
+
+__global__ void __launch_bounds__(32 * kTopkWarps) k_topk_part(const int* __restrict__ la, const float* __restrict__ ld,
+                                                               long long total, long long share, int k,
+                                                               float* __restrict__ part_d,
+                                                               long long* __restrict__ part_id) {
+  const int lane = threadIdx.x & 31;
+  const long long w = blockIdx.x * (long long)kTopkWarps + (threadIdx.x >> 5);
+  const long long e1 = min(total, (w + 1) * share);
+  float bd = INFINITY, kd = INFINITY;
+  long long bi = LLONG_MAX, ki = LLONG_MAX;
+  for (long long e0 = w * share; e0 < e1; e0 += 32) {
+    const long long e = e0 + lane;
+    const bool ok = e < e1 && la[e] >= 0;
+    best_offer(bd, bi, kd, ki, k, ok, ok ? ld[e] : INFINITY, e);
   }
-  const long long total = nb * k;
-  for (long long base = 0; base < total; base += 1024) {
-    const long long e = base + t;
-    // candidate id e = b * k + q; empty slots sort last
-    cd[t] = (e < total && la[e] >= 0) ? ld[e] : INFINITY;
-    cid[t] = (e < total && la[e] >= 0) ? e : LLONG_MAX;
-    __syncthreads();
-    for (int size = 2; size <= 1024; size <<= 1)
-      for (int stride = size >> 1; stride > 0; stride >>= 1) {
-        const int p = t ^ stride;
-        if (p > t) {
-          const bool up = (t & size) == 0;
-          const bool gt = cd[t] > cd[p] || (cd[t] == cd[p] && cid[t] > cid[p]);
-          if (gt == up) {
-            const float td = cd[t];
-            cd[t] = cd[p];
-            cd[p] = td;
-            const long long ti = cid[t];
-            cid[t] = cid[p];
-            cid[p] = ti;
-          }
-        }
-        __syncthreads();
-      }
-    if (t == 0) {  // merge the k best of the chunk with the running best
-      int i = 0, j = 0;
-      for (int q = 0; q < k; ++q) {
-        const bool take_b = bd[i] < cd[j] || (bd[i] == cd[j] && bid[i] <= cid[j]);
-        if (take_b) {
-          md[q] = bd[i];
-          mid[q] = bid[i];
-          ++i;
-        } else {
-          md[q] = cd[j];
-          mid[q] = cid[j];
-          ++j;
-        }
-      }
-      for (int q = 0; q < k; ++q) {
-        bd[q] = md[q];
-        bid[q] = mid[q];
-      }
-    }
-    __syncthreads();
+  if (lane < k) {
+    part_d[w * k + lane] = bd;
+    part_id[w * k + lane] = bi;
   }
-  if (t < k) {
-    const bool ok = bid[t] >= 0 && bid[t] != LLONG_MAX && bd[t] < INFINITY;
-    oa[t] = ok ? la[bid[t]] : -1;
-    ob[t] = ok ? (int)(bid[t] / k) : -1;
-    od[t] = ok ? bd[t] : INFINITY;
-    if (ok) atomicAdd(found, 1);
+}
+
+__global__ void __launch_bounds__(1024) k_topk_last(const int* __restrict__ la, const float* __restrict__ part_d,
+                                                    const long long* __restrict__ part_id, long long m, int k,
+                                                    int* __restrict__ oa, int* __restrict__ ob, float* __restrict__ od,
+                                                    int* __restrict__ found) {
+  __shared__ float sd[32 * kKnnMax];
+  __shared__ long long sid[32 * kKnnMax];
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  float bd = INFINITY, kd = INFINITY;
+  long long bi = LLONG_MAX, ki = LLONG_MAX;
+  for (long long e0 = warp * 32LL; e0 < m; e0 += 1024) {
+    const long long e = e0 + lane;
+    const long long id = e < m ? part_id[e] : LLONG_MAX;
+    best_offer(bd, bi, kd, ki, k, id != LLONG_MAX, e < m ? part_d[e] : INFINITY, id);
   }
+  if (lane < k) {
+    sd[warp * k + lane] = bd;
+    sid[warp * k + lane] = bi;
+  }
+  __syncthreads();
+  if (warp) return;
+  bd = kd = INFINITY;
+  bi = ki = LLONG_MAX;
+  for (int e = lane; e < 32 * k; e += 32) best_offer(bd, bi, kd, ki, k, sid[e] != LLONG_MAX, sd[e], sid[e]);
+  const bool ok = lane < k && bi != LLONG_MAX;
+  if (lane < k) {
+    oa[lane] = ok ? la[bi] : -1;
+    ob[lane] = ok ? (int)(bi / k) : -1;
+    od[lane] = ok ? bd : INFINITY;
+  }
+  const unsigned have = __ballot_sync(0xffffffffu, ok);
+  if (lane == 0) *found = __popc(have);
+}
+
+CrossArgs cross_args(const SweepArgs& A, const Off* off) {
+  CrossArgs C;
+  C.xs = A.xs;
+  C.cell_start = A.cell_start;
+  C.off = off;
+  C.noff = A.noff;
+  C.nx = A.nx;
+  C.ny = A.ny;
+  C.nz = A.nz;
+  C.rc2 = A.rc2;
+  C.ex = A.ex;
+  C.ey = A.ey;
+  C.ez = A.ez;
+  // The padding of the box test covers the FP32 rounding of the coordinates
+  // while cells are not thousands of cutoffs wide (capped grids).
+  const float rc = sqrtf(A.rc2);
+  C.cull = A.ex > 0.f && A.ex < 512.f * rc && A.ey < 512.f * rc && A.ez < 512.f * rc;
+  return C;
+}
+
+// Lanes per cell: a group's last pass over a cell is partly empty, so small
+// cells want small groups.
+int group_lanes(const SweepArgs& A) {
+  const double occ = (double)A.n / ((double)A.nx * A.ny * A.nz);
+  return occ < 3.0 ? 2 : (occ < 8.0 ? 4 : 8);
+}
+
+template <class K>
+int cross_grid(K kernel, int warps, size_t smem, long long nb) {
+  int dev = 0, sms = 0, per = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess ||
+      cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
+    return 0;
+  if (smem > 32 * 1024 &&
+      cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess)
+    return 0;
+  if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, kernel, 32 * warps, smem) != cudaSuccess || per < 1)
+    return 0;
+  const long long want = (nb + warps - 1) / warps;
+  return (int)(want < (long long)sms * per ? want : (long long)sms * per);
+}
+
+template <int G>
+int run_count(const CrossArgs& C, const Queries& Q, int* count, unsigned long long* total, cudaStream_t s) {
+  const size_t smem = (size_t)C.noff * sizeof(float4);
+  const int grid = cross_grid(k_cross_count<G>, kCrossWarps, smem, Q.nb);
+  if (grid < 1) return CL_ERR_CUDA;
+  k_cross_count<G><<<grid, 32 * kCrossWarps, smem, s>>>(C, Q, count, total);
+  return cudaGetLastError() == cudaSuccess ? CL_OK : CL_ERR_CUDA;
+}
+
+template <int G, bool WIDE>
+int run_fill(const CrossArgs& C, const Queries& Q, const int* count, const long long* start, int* pa, int* pb,
+             float* pd, int* longs, int* nlong, cudaStream_t s) {
+  const size_t smem = (size_t)C.noff * sizeof(float4) + (size_t)kFillWarps * 2 * kSegPad * sizeof(float);
+  const int grid = cross_grid(k_cross_fill<G, WIDE>, kFillWarps, smem, Q.nb);
+  if (grid < 1) return CL_ERR_CUDA;
+  k_cross_fill<G, WIDE><<<grid, 32 * kFillWarps, smem, s>>>(C, Q, count, start, pa, pb, pd, longs, nlong);
+  return cudaGetLastError() == cudaSuccess ? CL_OK : CL_ERR_CUDA;
+}
+
+template <int G>
+int run_knn(const CrossArgs& C, const Queries& Q, int k, int* out_a, float* out_d, cudaStream_t s) {
+  const size_t smem = (size_t)C.noff * (sizeof(float4) + sizeof(float));
+  const int grid = cross_grid(k_cross_knn<G>, kCrossWarps, smem, Q.nb);
+  if (grid < 1) return CL_ERR_CUDA;
+  k_cross_knn<G><<<grid, 32 * kCrossWarps, smem, s>>>(C, Q, k, out_a, out_d);
+  return cudaGetLastError() == cudaSuccess ? CL_OK : CL_ERR_CUDA;
 }
 
 }  // namespace
 
-int launch_cross(int what, const SweepArgs& A, const Geo& g, const double* posb, long long nb, int k, int* count,
-                 unsigned long long* total, const long long* start, int* pa, int* pb, float* pd, int* knn_a, float* knn_d,
-                 int* err, cudaStream_t s) {
+// Queries are sorted by cell when they are at least a quarter as many as the
+// cells: neighbouring warps then read the same cells of set A from L1, against
+// five more launches and a pass over the cell counts.
+bool queries_sorted(long long nb, long long ncells) { return nb >= 2048 && nb * 4 >= ncells; }
+
+int launch_query_bin(const SweepArgs& A, const Geo& g, const double* posb, long long nb, const QueryBufs& b, int* err,
+                     Queries* out, cudaStream_t s) {
+  out->q = b.q;
+  out->cell = b.cell;
+  out->nb = nb;
+  if (nb <= 0) return CL_OK;
   QueryArgs Q;
   Q.pos = posb;
   Q.nb = nb;
-  Q.dim = g.dim;
-  Q.ortho = g.ortho;
+  Q.nx = A.nx;
+  Q.ny = A.ny;
+  Q.nz = A.nz;
   for (int q = 0; q < 9; ++q) {
     Q.m[q] = g.m[q];
     Q.g[q] = g.g[q];
   }
-  if (nb <= 0) return CL_OK;
-  const long long blocks = (nb + 255) / 256;
-  if (what == 0) k_cross_count<<<(unsigned)blocks, 256, 0, s>>>(A, Q, count, total, err);
-  else if (what == 1) k_cross_fill<<<(unsigned)blocks, 256, 0, s>>>(A, Q, start, pa, pb, pd);
-  else k_cross_knn<<<(unsigned)((nb + 127) / 128), 128, 0, s>>>(A, Q, k, knn_a, knn_d, err);
-  return cudaGetLastError() == cudaSuccess ? CL_OK : CL_ERR_CUDA;
+  const bool sorted = queries_sorted(nb, g.ncells);
+  int* counts = sorted ? b.counts : nullptr;
+  if (sorted && (cudaMemsetAsync(b.counts, 0, sizeof(int) * g.ncells, s) != cudaSuccess ||
+                 cudaMemsetAsync(b.meta, 0, sizeof(int) * 4, s) != cudaSuccess))
+    return CL_ERR_CUDA;
+  const unsigned blocks = (unsigned)((nb + 255) / 256);
+  float4* q = sorted ? b.raw : b.q;
+  if (g.dim == 3) {
+    if (g.ortho) k_query_bin<3, true><<<blocks, 256, 0, s>>>(Q, q, b.cell, counts, b.slot, err);
+    else k_query_bin<3, false><<<blocks, 256, 0, s>>>(Q, q, b.cell, counts, b.slot, err);
+  } else {
+    if (g.ortho) k_query_bin<2, true><<<blocks, 256, 0, s>>>(Q, q, b.cell, counts, b.slot, err);
+    else k_query_bin<2, false><<<blocks, 256, 0, s>>>(Q, q, b.cell, counts, b.slot, err);
+  }
+  if (cudaGetLastError() != cudaSuccess) return CL_ERR_CUDA;
+  if (!sorted) return CL_OK;
+  const int e = launch_scan_cells(b.counts, g.ncells, b.tiles, b.meta, b.start, s);
+  return e ? e : launch_cell_order((int)nb, A.nx, A.ny, g.ncells, b.slot, b.raw, b.start, b.q, b.cell, s);
 }
 
-int launch_topk_merge(const int* la, const float* ld, long long nb, int k, int* oa, int* ob, float* od, int* found,
-                      cudaStream_t s) {
-  if (cudaMemsetAsync(found, 0, sizeof(int), s) != cudaSuccess) return CL_ERR_CUDA;
-  k_topk_merge<<<1, 1024, 0, s>>>(la, ld, nb, k, oa, ob, od, found);
+int launch_cross_count(const SweepArgs& A, const Off* off, const Queries& Q, int* count, unsigned long long* total,
+                       cudaStream_t s) {
+  if (Q.nb <= 0) return CL_OK;
+  const CrossArgs C = cross_args(A, off);
+  switch (group_lanes(A)) {
+    case 2: return run_count<2>(C, Q, count, total, s);
+    case 4: return run_count<4>(C, Q, count, total, s);
+    default: return run_count<8>(C, Q, count, total, s);
+  }
+}
+
+int launch_cross_fill(const SweepArgs& A, const Off* off, const Queries& Q, const int* count, const long long* start,
+                      int* pa, int* pb, float* pd, int* longs, int* nlong, cudaStream_t s) {
+  if (Q.nb <= 0) return CL_OK;
+  if (cudaMemsetAsync(nlong, 0, sizeof(int), s) != cudaSuccess) return CL_ERR_CUDA;
+  const CrossArgs C = cross_args(A, off);
+  int e;
+  if (A.n >= (1 << 22)) {
+    e = run_fill<8, true>(C, Q, count, start, pa, pb, pd, longs, nlong, s);
+  } else {
+    switch (group_lanes(A)) {
+      case 2: e = run_fill<2, false>(C, Q, count, start, pa, pb, pd, longs, nlong, s); break;
+      case 4: e = run_fill<4, false>(C, Q, count, start, pa, pb, pd, longs, nlong, s); break;
+      default: e = run_fill<8, false>(C, Q, count, start, pa, pb, pd, longs, nlong, s); break;
+    }
+  }
+  return e ? e : launch_sort_long(longs, nlong, count, start, pa, pd, s);
+}
+
+int launch_cross_knn(const SweepArgs& A, const Off* off, const Queries& Q, int k, int* out_a, float* out_d,
+                     cudaStream_t s) {
+  if (Q.nb <= 0) return CL_OK;
+  const CrossArgs C = cross_args(A, off);
+  switch (group_lanes(A)) {
+    case 2: return run_knn<2>(C, Q, k, out_a, out_d, s);
+    case 4: return run_knn<4>(C, Q, k, out_a, out_d, s);
+    default: return run_knn<8>(C, Q, k, out_a, out_d, s);
+  }
+}
+
+// A warp's share is at least 2,048 candidates, and at most 1,024 warps share
+// the lists, so that the last kernel reads at most 1,024 k entries.
+static long long topk_share(long long nb, int k) {
+  const long long total = nb * k;
+  const long long share = (total + 1023) / 1024;
+  return (std::max<long long>(share, 2048) + 31) / 32 * 32;
+}
+
+long long topk_parts(long long nb, int k) {
+  const long long share = topk_share(nb, k), w = (nb * k + share - 1) / share;
+  return (std::max<long long>(w, 1) + kTopkWarps - 1) / kTopkWarps * kTopkWarps;
+}
+
+int launch_topk_merge(const int* la, const float* ld, long long nb, int k, float* part_d, long long* part_id, int* oa,
+                      int* ob, float* od, int* found, cudaStream_t s) {
+  const long long parts = topk_parts(nb, k);
+  k_topk_part<<<(unsigned)(parts / kTopkWarps), 32 * kTopkWarps, 0, s>>>(la, ld, nb * k, topk_share(nb, k), k, part_d,
+                                                                         part_id);
+  k_topk_last<<<1, 1024, 0, s>>>(la, part_d, part_id, parts * k, k, oa, ob, od, found);
   return cudaGetLastError() == cudaSuccess ? CL_OK : CL_ERR_CUDA;
 }
 

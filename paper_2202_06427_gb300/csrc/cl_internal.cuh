@@ -133,6 +133,13 @@ int launch_build(const Geo& g, const BuildBufs& b, cudaStream_t s);
 // device) with kOctMin..kOctCap particles by octant; slots follow.
 int launch_octsort(const int* cells, const int* ncells_listed, const int* cell_start, float4* xs, int* slot,
                    cudaStream_t s);
+// Prefix sum of the per-cell counts into cell_start; meta[1], meta[2] (zeroed
+// by the caller): non-empty cells, largest count.
+int launch_scan_cells(const int* counts, long long ncells, int* tile_sum, int* meta, int* cell_start, cudaStream_t s);
+// Moves xl[i] (w = packed cell) to its place in cell order (w = i) and writes
+// the packed cells along the sorted array.
+int launch_cell_order(int n, int nx, int ny, long long ncells, const int* slot, const float4* xl,
+                      const int* cell_start, float4* xs, unsigned* cellc, cudaStream_t s);
 int launch_scan64(const int* counts, long long n, long long* tile_sum, long long* start, int* meta, cudaStream_t s);
 
 // Sweeps and reductions (cl_sweep.cu).
@@ -227,14 +234,42 @@ int launch_hood_scalar(const SweepArgs& A, const HoodArgs& H, int* work, int kin
                        double* partials, long long partials_cap, double* sums, double* scalar_out, int nbins,
                        float rmax, unsigned long long* hist, cudaStream_t s, int* lists_half = nullptr);
 
-// Two sets (cl_cross.cu): what 0 counts per query (count may be null) and their
-// total, 1 fills the pairs of each query's segment (start), 2 the per-query k
-// nearest. err: device error latch.
-int launch_cross(int what, const SweepArgs& A, const Geo& g, const double* posb, long long nb, int k, int* count,
-                 unsigned long long* total, const long long* start, int* pa, int* pb, float* pd, int* knn_a, float* knn_d,
-                 int* err, cudaStream_t s);
-int launch_topk_merge(const int* la, const float* ld, long long nb, int k, int* oa, int* ob, float* od, int* found,
-                      cudaStream_t s);
+// Two sets (cl_cross.cu). The query points of set B, binned on set A's grid.
+struct Queries {
+  const float4* q;        // coordinate relative to the cell centre, w = query index (int bits)
+  const unsigned* cell;   // packed cell
+  long long nb;
+};
+// Workspace of the query binning: the prepared arrays and, when the queries
+// are sorted by cell (queries_sorted), the counting sort's.
+struct QueryBufs {
+  float4* q;        // nb
+  unsigned* cell;   // nb
+  float4* raw;      // nb, sorted only
+  int* slot;        // nb, sorted only
+  int* counts;      // ncells, sorted only
+  int* start;       // ncells + 1, sorted only
+  int* tiles;       // scan_tiles_for(ncells), sorted only
+  int* meta;        // 4, sorted only
+};
+bool queries_sorted(long long nb, long long ncells);
+int launch_query_bin(const SweepArgs& A, const Geo& g, const double* posb, long long nb, const QueryBufs& b, int* err,
+                     Queries* out, cudaStream_t s);
+// The sweeps (off: the full stencil in device memory). Count: per query (count
+// may be null) and their sum (total may be null). Fill: segments of the list at
+// start, each sorted by a; those longer than kMaxSegment are listed in longs
+// for launch_sort_long. knn: per query the k nearest.
+int launch_cross_count(const SweepArgs& A, const Off* off, const Queries& Q, int* count, unsigned long long* total,
+                       cudaStream_t s);
+int launch_cross_fill(const SweepArgs& A, const Off* off, const Queries& Q, const int* count, const long long* start,
+                      int* pa, int* pb, float* pd, int* longs, int* nlong, cudaStream_t s);
+int launch_cross_knn(const SweepArgs& A, const Off* off, const Queries& Q, int k, int* out_a, float* out_d,
+                     cudaStream_t s);
+// The k closest of nb per-query lists of k (each ascending, -1 past its end);
+// part_d, part_id: topk_parts(nb, k) * k entries of workspace.
+long long topk_parts(long long nb, int k);
+int launch_topk_merge(const int* la, const float* ld, long long nb, int k, float* part_d, long long* part_id, int* oa,
+                      int* ob, float* od, int* found, cudaStream_t s);
 
 // Neighbour list (cl_pairs.cu). count[n] (int: one particle's pairs), start[n+1]
 // (64-bit scan of count: the list may pass 2^31 pairs), tiles, meta:
@@ -246,10 +281,10 @@ constexpr int kMaxSegment = 1024;  // segments up to this length are sorted by o
 // cap: staged entries per cell (32..3072), the same for the count and fill passes.
 int launch_pairs_count(const SweepArgs& A, int dim, float ball2, int cap, unsigned char* flag, int* fcells,
                        int* nfcells, int* count, cudaStream_t s);
-// Sorts each segment [start[a], start[a] + count[a]) of pj (carrying pd) by pj;
-// longs (n ints) and nlong (1 int) are workspace.
-int launch_pairs_sort(int n, const int* count, const long long* start, int* pj, float* pd, int* longs, int* nlong,
-                      cudaStream_t s);
+// Sorts each listed segment [start[a], start[a] + count[a]), a = longs[q], q <
+// *nlong, of pj (carrying pd) by pj.
+int launch_sort_long(const int* longs, const int* nlong, const int* count, const long long* start, int* pj, float* pd,
+                     cudaStream_t s);
 // Fill pass: the same two sweeps, each segment sorted by j and written.
 // longs (n ints) and nlong (1 int): workspace for segments longer than kMaxSegment.
 int launch_pairs_fill(const SweepArgs& A, int dim, float ball2, int cap, const unsigned char* flag, const int* fcells,

@@ -20,9 +20,6 @@
 //                  (fill) per particle straight from the sorted arrays; a
 //                  segment longer than kMaxSegment is written unsorted and
 //                  listed for k_pairs_sort_long
-//   k_pairs_sort   one warp per segment, in place, for the two-set list (its
-//                  segments are filled by a per-query sweep); longer segments
-//                  are listed for k_pairs_sort_long
 //   k_pairs_sort_long  one CTA per listed segment, in place in global memory
 //
 // Each particle's count and fill run the same arithmetic in the same kernel
@@ -32,6 +29,7 @@
 // (rc <= w_min / 2), which the host checks before launching.
 #include <climits>
 
+#include "cl_sort.cuh"
 #include "cl_sweep.cuh"
 
 namespace clk {
@@ -62,67 +60,6 @@ __global__ void __launch_bounds__(256) k_pairs_count(const __grid_constant__ Swe
       sweep_particle<DIM>(A, red, acc, p, pi);
       count[acc.a] = acc.n;
     }
-  }
-}
-
-constexpr int kSortWarps = 4;
-
-// One warp per segment (grid-stride): bitonic sort of up to kMaxSegment keys
-// (j, distinct within a segment) with their distances, in shared memory.
-// Longer segments are appended to longs[] (counter *nlong) for
-// k_pairs_sort_long.
-__global__ void __launch_bounds__(32 * kSortWarps) k_pairs_sort(int n, const int* __restrict__ count,
-                                                               const long long* __restrict__ start, int* __restrict__ pj,
-                                                               float* __restrict__ pd, int* __restrict__ longs,
-                                                               int* __restrict__ nlong) {
-  __shared__ int sk[kSortWarps][kMaxSegment];
-  __shared__ float sv[kSortWarps][kMaxSegment];
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  int* K = sk[warp];
-  float* V = sv[warp];
-  for (int a = blockIdx.x * kSortWarps + warp; a < n; a += gridDim.x * kSortWarps) {
-    const int L = count[a];
-    if (L <= 1) continue;
-    if (L > kMaxSegment) {
-      if (lane == 0) longs[atomicAdd(nlong, 1)] = a;
-      continue;
-    }
-    const long long base = start[a];
-    int P = 32;
-    while (P < L) P <<= 1;
-    for (int k = lane; k < P; k += 32) {
-      if (k < L) {
-        K[k] = pj[base + k];
-        V[k] = pd[base + k];
-      } else {
-        K[k] = INT_MAX;
-        V[k] = 0.f;
-      }
-    }
-    __syncwarp();
-    for (int size = 2; size <= P; size <<= 1) {
-      for (int stride = size >> 1; stride > 0; stride >>= 1) {
-        for (int t = lane; t < (P >> 1); t += 32) {
-          const int lo = 2 * stride * (t / stride) + (t % stride);
-          const int hi = lo + stride;
-          const bool up = (lo & size) == 0;
-          const int ka = K[lo], kb = K[hi];
-          if ((ka > kb) == up) {
-            K[lo] = kb;
-            K[hi] = ka;
-            const float va = V[lo];
-            V[lo] = V[hi];
-            V[hi] = va;
-          }
-        }
-        __syncwarp();
-      }
-    }
-    for (int k = lane; k < L; k += 32) {
-      pj[base + k] = K[k];
-      pd[base + k] = V[k];
-    }
-    __syncwarp();
   }
 }
 
@@ -184,106 +121,6 @@ __global__ void __launch_bounds__(1024) k_pairs_sort_long(const int* __restrict_
 // kMaxSegment long (the host checks the counts first).
 constexpr int kFillWarps = 4;
 constexpr int kStageMax = 3072;  // largest staged neighbourhood of one cell (the launch picks its capacity)
-constexpr int kSegPad = kMaxSegment + kMaxSegment / 32;
-
-// Segment buffer index with one pad word per 32: conflict-free both for lane i
-// at i (coalesced order) and for lane l at l * E + e (blocked order, E <= 32).
-__device__ __forceinline__ int seg_at(int i) { return i + (i >> 5); }
-
-// Bitonic sort, ascending by key, of 32 E elements held E per lane in blocked
-// order (element lane * E + e). Pairs closer than E apart are in one lane's
-// registers; farther ones are exchanged with a shuffle.
-template <int E>
-__device__ __forceinline__ void sort_blocked(int (&k)[E], float (&v)[E], int lane) {
-#pragma unroll
-  for (int size = 2; size <= 32 * E; size <<= 1) {
-#pragma unroll
-    for (int stride = size >> 1; stride > 0; stride >>= 1) {
-      if (stride >= E) {
-        const int ls = stride / E;
-        const bool lower = (lane & ls) == 0;
-#pragma unroll
-        for (int e = 0; e < E; ++e) {
-          const bool up = ((lane * E + e) & size) == 0;
-          const int ok = __shfl_xor_sync(0xffffffffu, k[e], ls);
-          const float ov = __shfl_xor_sync(0xffffffffu, v[e], ls);
-          const bool take = (lower == up) ? (ok < k[e]) : (ok > k[e]);
-          k[e] = take ? ok : k[e];
-          v[e] = take ? ov : v[e];
-        }
-      } else {
-#pragma unroll
-        for (int e = 0; e < E; ++e) {
-          if ((e & stride) == 0) {
-            const int f = e | stride;
-            const bool up = ((lane * E + e) & size) == 0;
-            const bool sw = up ? (k[e] > k[f]) : (k[e] < k[f]);
-            const int tk = k[e];
-            const float tv = v[e];
-            k[e] = sw ? k[f] : k[e];
-            v[e] = sw ? v[f] : v[e];
-            k[f] = sw ? tk : k[f];
-            v[f] = sw ? tv : v[f];
-          }
-        }
-      }
-    }
-  }
-}
-
-template <int E>
-__device__ __forceinline__ void sort_segment_regs(int* K, float* V, int L, int lane) {
-  int k[E];
-  float v[E];
-#pragma unroll
-  for (int e = 0; e < E; ++e) {
-    const int i = lane * E + e;
-    k[e] = i < L ? K[seg_at(i)] : INT_MAX;
-    v[e] = i < L ? V[seg_at(i)] : 0.f;
-  }
-  sort_blocked<E>(k, v, lane);
-  __syncwarp();
-#pragma unroll
-  for (int e = 0; e < E; ++e) {
-    const int i = lane * E + e;
-    if (i < L) {
-      K[seg_at(i)] = k[e];
-      V[seg_at(i)] = v[e];
-    }
-  }
-  __syncwarp();
-}
-
-// Segments longer than 16 per lane: the same network in shared memory.
-__device__ void sort_segment_smem(int* K, float* V, int L, int lane) {
-  int P = 32;
-  while (P < L) P <<= 1;
-  for (int i = L + lane; i < P; i += 32) {
-    K[seg_at(i)] = INT_MAX;
-    V[seg_at(i)] = 0.f;
-  }
-  __syncwarp();
-  for (int size = 2; size <= P; size <<= 1) {
-    for (int stride = size >> 1; stride > 0; stride >>= 1) {
-      for (int t = lane; t < (P >> 1); t += 32) {
-        const int lo = 2 * stride * (t / stride) + (t % stride);
-        const int hi = lo + stride;
-        const bool up = (lo & size) == 0;
-        const int ka = K[seg_at(lo)], kb = K[seg_at(hi)];
-        if ((ka > kb) == up) {
-          K[seg_at(lo)] = kb;
-          K[seg_at(hi)] = ka;
-          const float va = V[seg_at(lo)];
-          V[seg_at(lo)] = V[seg_at(hi)];
-          V[seg_at(hi)] = va;
-        }
-      }
-      __syncwarp();
-    }
-  }
-}
-
-
 // Stencil entries k0 + lane of cell (cx, cy, cz): the lane's range [j0, j0 +
 // len) of sorted particles, its shift (stencil shift + (bx, by, bz)) and, over
 // the warp, the exclusive offsets of the ranges laid end to end and their total.
@@ -355,20 +192,7 @@ __device__ __forceinline__ void stencil_to_smem(const SweepArgs& A, float4* stab
 // Sorts the warp's segment of nw kept pairs by j and writes it at base.
 __device__ __forceinline__ void segment_out(int* K, float* V, int nw, int a, long long base, int lane, int* pi_out,
                                             int* pj_out, float* pd_out) {
-  if (nw <= 1) {
-  } else if (nw <= 32) {
-    sort_segment_regs<1>(K, V, nw, lane);
-  } else if (nw <= 64) {
-    sort_segment_regs<2>(K, V, nw, lane);
-  } else if (nw <= 128) {
-    sort_segment_regs<4>(K, V, nw, lane);
-  } else if (nw <= 256) {
-    sort_segment_regs<8>(K, V, nw, lane);
-  } else if (nw <= 512) {
-    sort_segment_regs<16>(K, V, nw, lane);
-  } else {
-    sort_segment_smem(K, V, nw, lane);
-  }
+  sort_segment(K, V, nw, lane);
   for (int i = lane; i < nw; i += 32) {
     pi_out[base + i] = a;
     pj_out[base + i] = K[seg_at(i)];
@@ -808,7 +632,7 @@ int launch_pairs_count(const SweepArgs& A, int dim, float ball2, int cap, unsign
   return cudaGetLastError() == cudaSuccess ? CL_OK : CL_ERR_CUDA;
 }
 
-static int launch_sort_long(const int* longs, const int* nlong, const int* count, const long long* start, int* pj,
+int launch_sort_long(const int* longs, const int* nlong, const int* count, const long long* start, int* pj,
                             float* pd, cudaStream_t s) {
   k_pairs_sort_long<<<152, 1024, 0, s>>>(longs, nlong, count, start, pj, pd);
   return cudaGetLastError() == cudaSuccess ? CL_OK : CL_ERR_CUDA;
@@ -831,17 +655,6 @@ int launch_pairs_fill(const SweepArgs& A, int dim, float ball2, int cap, const u
   else
     k_pairs_fill_sorted<2><<<152 * 6, 32 * kFillWarps, dyn, s>>>(A, fcells, nfcells, count, start, pi, pj, pd, longs,
                                                                 nlong);
-  if (cudaGetLastError() != cudaSuccess) return CL_ERR_CUDA;
-  return launch_sort_long(longs, nlong, count, start, pj, pd, s);
-}
-
-int launch_pairs_sort(int n, const int* count, const long long* start, int* pj, float* pd, int* longs, int* nlong,
-                      cudaStream_t s) {
-  if (n <= 0) return CL_OK;
-  if (cudaMemsetAsync(nlong, 0, sizeof(int), s) != cudaSuccess) return CL_ERR_CUDA;
-  int blocks = (n + kSortWarps - 1) / kSortWarps;
-  if (blocks > 152 * 32) blocks = 152 * 32;
-  k_pairs_sort<<<blocks, 32 * kSortWarps, 0, s>>>(n, count, start, pj, pd, longs, nlong);
   if (cudaGetLastError() != cudaSuccess) return CL_ERR_CUDA;
   return launch_sort_long(longs, nlong, count, start, pj, pd, s);
 }
