@@ -111,15 +111,16 @@ typedef struct {
  * coordinates into cell order, and list the work tiles of the sweep.
  * pos_dev: (n, dim) FP64 device array (0 <= n < 2^31). The pointer is kept by
  * the handle (cl_backward reads the raw positions again) and must stay valid
- * until the next cl_update or cl_free. Allocates device memory (synchronous
- * cudaMalloc); the kernels run on `stream`. On success *out receives a new
+ * until the next cl_update or cl_free. Allocates device memory from the
+ * library's pool, stream-ordered on `stream`, where the kernels run too. On success *out receives a new
  * handle. Errors: INVALID_ARG, INVALID_BOX, CUTOFF_TOO_LARGE, UNSUPPORTED,
  * OOM, CUDA. */
 int cl_build(const double* pos_dev, long long n, const cl_box* box, void* stream, cl_list** out);
 
 /* Rebuild the cell list for new positions of the same n particles (Sec. 4.2:
  * the lists are updated between steps), reusing the workspace. box may be
- * NULL (unchanged) or a new box; a new box that changes the grid reallocates.
+ * NULL (unchanged) or a box; one that needs more cells than any before it
+ * reallocates.
  * Same errors as cl_build. */
 int cl_update(cl_list* cl, const double* pos_dev, const cl_box* box, void* stream);
 
@@ -190,7 +191,7 @@ int cl_query(const cl_list* cl, int what, long long* value, void* stream);
  * The pair-images are every (a, b, t) with |y_b - x_a + t.H| < cutoff (no
  * a < b rule); a and b are 0-based indices into A and B. Each b is binned on
  * A's grid in FP64 and sweeps the full stencil of its cell. These calls
- * synchronize `stream` and allocate their workspace (cudaMalloc/cudaFree).
+ * synchronize `stream` and take their workspace from the library's pool.
  * Errors: INVALID_ARG, NONFINITE (a position of B), OOM, CUDA, and as noted.
  *
  * cl_cross_count: count_dev[0] = number of cross pair-images (u64).

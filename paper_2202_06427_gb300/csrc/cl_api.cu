@@ -4,17 +4,22 @@
 #include <cmath>
 #include <cstdlib>
 #include <cstring>
+#include <memory>
 #include <new>
-#include <type_traits>
 
 #include "cl_internal.cuh"
 
 struct cl_list {
   clk::Geo geo;
+  cl_box box;  // the box geo was prepared from
+  int device;
   int n;
   const double* pos;
-  long long ncells_alloc;
-  // device workspace
+  long long ncells_alloc;  // cells the per-cell arrays have room for
+  // device workspace: blocks of the library's pool, and the arrays in them
+  void* block;        // per particle and fixed
+  void* cell_block;   // per cell
+  void* pair_block;   // neighbour list, on its first call
   int* slot;
   float4* xl;
   float4* xs;
@@ -46,79 +51,85 @@ struct cl_list {
   clk::SweepArgs* half;
   clk::SweepArgs* full;
   clk::HoodArgs* hood;  // 3D neighbourhood sweep arguments
-  // workspace of the two-set calls, kept between them (see QueryWs)
-  char* qws;
-  size_t qws_bytes;
-  int qws_busy;
   size_t bytes;
 };
 
 namespace {
 
-template <class T>
-int dev_alloc(T** p, size_t count, size_t* bytes) {
-  *p = nullptr;
-  if (count == 0) count = 1;
-  if (cudaMalloc((void**)p, sizeof(T) * count) != cudaSuccess) {
-    cudaGetLastError();
-    *p = nullptr;
-    return CL_ERR_OOM;
-  }
-  *bytes += sizeof(T) * count;
-  return CL_OK;
+// The list's per-particle and fixed-size arrays in one block: with base null
+// their size. Those from `zero_from` on (zero_bytes) start as zeros.
+size_t carve_list(cl_list* c, char* base, int dim, char** zero_from, size_t* zero_bytes) {
+  clk::Carver v{base};
+  const size_t n = (size_t)c->n;
+  v.take(&c->slot, n);
+  v.take(&c->xl, n);
+  v.take(&c->xs, n);
+  v.take(&c->cellc, n);
+  v.take(&c->partials, (size_t)clk::sweep_partials_needed(c->n));
+  v.take(&c->work, 8);  // [0] work counter, [2..3] candidate counter, [5] the dense
+                        // cells' work counter, [6] list length, [7] dense cells
+  v.take(&c->u64, 8);
+  v.take(&c->d_off_half, 2 * (size_t)clk::kMaxOff);  // both stencils, one after the other
+  const size_t at = v.used;
+  v.take(&c->meta, 4);
+  v.take(&c->sums, 32);  // [31]: the final reduction's completion counter, zero between launches
+  if (dim == 3) v.take(&c->hforce, n);
+  *zero_from = base + at;
+  *zero_bytes = v.used - at;
+  return v.used;
 }
 
-void free_cells(cl_list* c) {
-  cudaFree(c->counts);
-  cudaFree(c->cell_start);
-  cudaFree(c->tile_sum);
-  cudaFree(c->hflag);
-  cudaFree(c->hlist);
-  c->hlist = nullptr;
-  cudaFree(c->hdense);
-  c->hdense = nullptr;
-  c->counts = nullptr;
-  c->cell_start = nullptr;
-  c->tile_sum = nullptr;
-  c->hflag = nullptr;
+struct Cells {
+  int *counts, *cell_start, *tile_sum, *hlist, *hdense;
+  unsigned char* hflag;
+};
+
+size_t carve_cells(Cells* p, char* base, long long ncells) {
+  clk::Carver v{base};
+  v.take(&p->counts, (size_t)ncells);
+  v.take(&p->cell_start, (size_t)ncells + 1);
+  v.take(&p->tile_sum, (size_t)clk::scan_tiles_for(ncells));
+  v.take(&p->hlist, (size_t)ncells);
+  v.take(&p->hdense, (size_t)ncells);
+  v.take(&p->hflag, (size_t)ncells);
+  return v.used;
 }
 
+// Gives the list's memory back; no work on it may be in flight.
 void free_all(cl_list* c) {
-  free_cells(c);
-  cudaFree(c->slot);
-  cudaFree(c->xl);
-  cudaFree(c->xs);
-  cudaFree(c->cellc);
-  cudaFree(c->meta);
-  cudaFree(c->partials);
-  cudaFree(c->sums);
-  cudaFree(c->work);
-  cudaFree(c->hforce);
-  cudaFree(c->u64);
-  cudaFree(c->d_off_half);
-  cudaFree(c->d_off_full);
-  cudaFree(c->pl_count);
-  cudaFree(c->pl_start);
-  cudaFree(c->pl_tiles);
-  cudaFree(c->pl_meta);
-  cudaFree(c->pl_long);
-  cudaFree(c->qws);
+  clk::mem_free(c->block, nullptr);
+  clk::mem_free(c->cell_block, nullptr);
+  clk::mem_free(c->pair_block, nullptr);
   delete c->half;
   delete c->full;
   delete c->hood;
 }
 
-int alloc_cells(cl_list* c, long long ncells) {
-  size_t b = 0;
-  int e;
-  if ((e = dev_alloc(&c->counts, (size_t)ncells, &b))) return e;
-  if ((e = dev_alloc(&c->cell_start, (size_t)ncells + 1, &b))) return e;
-  if ((e = dev_alloc(&c->tile_sum, (size_t)clk::scan_tiles_for(ncells), &b))) return e;
-  if ((e = dev_alloc(&c->hflag, (size_t)ncells, &b))) return e;
-  if ((e = dev_alloc(&c->hlist, (size_t)ncells, &b))) return e;
-  if ((e = dev_alloc(&c->hdense, (size_t)ncells, &b))) return e;
+// Room for ncells cells. A larger grid than before gets a new block first, so
+// that a failure leaves the list as it was; the old one may still be in use on
+// another stream, so it is given back after a device synchronisation.
+int alloc_cells(cl_list* c, long long ncells, cudaStream_t s) {
+  Cells p;
+  const size_t bytes = carve_cells(&p, nullptr, ncells);
+  void* block = nullptr;
+  int e = clk::mem_alloc(&block, bytes, s);
+  if (e) return e;
+  carve_cells(&p, (char*)block, ncells);
+  if (c->cell_block) {
+    Cells old;
+    c->bytes -= carve_cells(&old, nullptr, c->ncells_alloc);
+    cudaDeviceSynchronize();
+    clk::mem_free(c->cell_block, s);
+  }
+  c->cell_block = block;
+  c->counts = p.counts;
+  c->cell_start = p.cell_start;
+  c->tile_sum = p.tile_sum;
+  c->hlist = p.hlist;
+  c->hdense = p.hdense;
+  c->hflag = p.hflag;
   c->ncells_alloc = ncells;
-  c->bytes += b;
+  c->bytes += bytes;
   return CL_OK;
 }
 
@@ -153,59 +164,45 @@ void fill_sweep_args(cl_list* c, clk::SweepArgs* A) {
   A->ez = e[2];
 }
 
-int set_geometry(cl_list* c, const cl_box* box) {
+bool same_box(const cl_box& a, const cl_box& b) {
+  if (a.dim != b.dim || a.lcell != b.lcell || !(a.cutoff == b.cutoff)) return false;
+  for (int k = 0; k < a.dim * a.dim; ++k)
+    if (!(a.h[k] == b.h[k])) return false;
+  return true;
+}
+
+int set_geometry(cl_list* c, const cl_box* box, cudaStream_t s) {
   clk::Geo g;
   int e = clk::prepare_geometry(box, &g);
   if (e) return e;
-  clk::Off* th = new (std::nothrow) clk::Off[2 * clk::kMaxOff];
-  int* opk = new (std::nothrow) int[2 * clk::kMaxOff];
-  clk::HoodArgs* hood = new (std::nothrow) clk::HoodArgs;
-  if (!th || !opk || !hood) {
-    delete[] th;
-    delete[] opk;
-    delete hood;
-    return CL_ERR_OOM;
-  }
-  clk::Off* tf = th + clk::kMaxOff;
-  int nh = clk::build_stencil(g, 1, th, clk::kMaxOff, opk + clk::kMaxOff);
-  int nf = nh < 0 ? nh : clk::build_stencil(g, 0, tf, clk::kMaxOff, opk);
-  if (nh < 0 || nf < 0) {
-    delete[] th;
-    delete[] opk;
-    delete hood;
-    return nh < 0 ? nh : nf;
-  }
-  std::memset(hood, 0, sizeof(*hood));
-  if (g.dim == 3) clk::fill_hood_args(g, opk, nf, opk + clk::kMaxOff, nh, hood);
-  delete[] opk;
-  if (g.ncells != c->ncells_alloc) {
-    free_cells(c);
-    if ((e = alloc_cells(c, g.ncells))) {
-      delete[] th;
-      delete hood;
-      return e;
-    }
-  }
-  std::memcpy(c->half->off, th, sizeof(clk::Off) * nh);
-  std::memcpy(c->full->off, tf, sizeof(clk::Off) * nf);
-  if (cudaMemcpy(c->d_off_half, th, sizeof(clk::Off) * nh, cudaMemcpyHostToDevice) != cudaSuccess ||
-      cudaMemcpy(c->d_off_full, tf, sizeof(clk::Off) * nf, cudaMemcpyHostToDevice) != cudaSuccess) {
-    delete[] th;
-    delete hood;
-    return CL_ERR_CUDA;
-  }
-  *c->hood = *hood;
+  struct Host {
+    clk::Off off[2 * clk::kMaxOff];
+    int opk_half[clk::kMaxOff], opk_full[clk::kMaxOff];
+  };
+  std::unique_ptr<Host> t(new (std::nothrow) Host);
+  if (!t) return CL_ERR_OOM;
+  int nh = 0, nf = 0;
+  if ((e = clk::build_stencils(g, clk::kMaxOff, t->off, t->opk_half, &nh, t->off + clk::kMaxOff, t->opk_full, &nf)))
+    return e;
+  if (g.ncells > c->ncells_alloc && (e = alloc_cells(c, g.ncells, s))) return e;
+  std::memmove(t->off + nh, t->off + clk::kMaxOff, sizeof(clk::Off) * nf);  // one after the other: one copy
+  if (cudaMemcpyAsync(c->d_off_half, t->off, sizeof(clk::Off) * (nh + nf), cudaMemcpyHostToDevice, s) != cudaSuccess)
+    return CL_ERR_CUDA;  // pageable source: staged before the call returns
+  c->d_off_full = c->d_off_half + nh;
+  std::memcpy(c->half->off, t->off, sizeof(clk::Off) * nh);
+  std::memcpy(c->full->off, t->off + nh, sizeof(clk::Off) * nf);
+  std::memset(c->hood, 0, sizeof(*c->hood));
+  if (g.dim == 3) clk::fill_hood_args(g, t->opk_full, nf, t->opk_half, nh, c->hood);
   c->hood->flag = c->hflag;
   c->hood->list = c->hlist;
   c->hood->dense = c->hdense;
   c->hood->hforce = c->hforce;
   c->hood->xl = c->xl;
   c->hood->slot = c->slot;
-  delete hood;
   c->half->noff = nh;
   c->full->noff = nf;
-  delete[] th;
   c->geo = g;
+  c->box = *box;
   fill_sweep_args(c, c->half);
   fill_sweep_args(c, c->full);
   return CL_OK;
@@ -267,22 +264,21 @@ int map_pairlist(cl_list* c, cl_result* r, cudaStream_t s) {
   for (int k = 0; k < c->geo.dim; ++k)
     if (!(2.0 * c->geo.rc <= c->geo.w[k])) return CL_ERR_CUTOFF_TOO_LARGE;  // unique images only
   int e;
-  if (!c->pl_count) {
-    size_t b = 0;
+  if (!c->pair_block) {
     const size_t n = (size_t)c->n;
-    if ((e = dev_alloc(&c->pl_count, n, &b)) || (e = dev_alloc(&c->pl_start, n + 1, &b)) ||
-        (e = dev_alloc(&c->pl_tiles, (size_t)clk::scan_tiles_for(c->n), &b)) || (e = dev_alloc(&c->pl_meta, 8, &b)) ||
-        (e = dev_alloc(&c->pl_long, n, &b))) {
-      cudaFree(c->pl_count);
-      cudaFree(c->pl_start);
-      cudaFree(c->pl_tiles);
-      cudaFree(c->pl_meta);
-      cudaFree(c->pl_long);
-      c->pl_count = c->pl_meta = c->pl_long = nullptr;
-      c->pl_start = c->pl_tiles = nullptr;
-      return e;
-    }
-    c->bytes += b;
+    auto carve = [&](char* base) {
+      clk::Carver v{base};
+      v.take(&c->pl_count, n);
+      v.take(&c->pl_start, n + 1);
+      v.take(&c->pl_tiles, (size_t)clk::scan_tiles_for(c->n));
+      v.take(&c->pl_meta, 8);
+      v.take(&c->pl_long, n);
+      return v.used;
+    };
+    const size_t bytes = carve(nullptr);
+    if ((e = clk::mem_alloc(&c->pair_block, bytes, s))) return e;
+    carve((char*)c->pair_block);
+    c->bytes += bytes;
   }
   const int dim = c->geo.dim;
   const float ball2 = pairs_ball2(c->geo);
@@ -374,31 +370,20 @@ int cl_build(const double* pos_dev, long long n, const cl_box* box, void* stream
   c->n = (int)n;
   c->pos = pos_dev;
   c->ncells_alloc = -1;
-  int e = CL_OK;
-  size_t b = 0;
-  const size_t nn = (size_t)n;
-  if (!e) e = dev_alloc(&c->slot, nn, &b);
-  if (!e) e = dev_alloc(&c->xl, nn, &b);
-  if (!e) e = dev_alloc(&c->xs, nn, &b);
-  if (!e) e = dev_alloc(&c->cellc, nn, &b);
-  if (!e) e = dev_alloc(&c->meta, 4, &b);
-  if (!e) e = dev_alloc(&c->partials, (size_t)clk::sweep_partials_needed(c->n), &b);
-  if (!e) e = dev_alloc(&c->sums, 32, &b);
-  if (!e) e = dev_alloc(&c->work, 8, &b);  // [0] work counter, [2..3] candidate counter, [5] the dense
-                                           // cells' work counter, [6] list length, [7] dense cells
-  if (!e && box->dim == 3) e = dev_alloc(&c->hforce, nn, &b);
-  if (!e && box->dim == 3 && nn > 0 && cudaMemset(c->hforce, 0, sizeof(float4) * nn) != cudaSuccess) e = CL_ERR_CUDA;
-  if (!e) e = dev_alloc(&c->u64, 8, &b);
-  if (!e) e = dev_alloc(&c->d_off_half, (size_t)clk::kMaxOff, &b);
-  if (!e) e = dev_alloc(&c->d_off_full, (size_t)clk::kMaxOff, &b);
-  c->bytes = b;
-  if (!e) e = set_geometry(c, box);
   cudaStream_t s = (cudaStream_t)stream;
-  if (!e && cudaMemsetAsync(c->meta, 0, sizeof(int) * 4, s) != cudaSuccess) e = CL_ERR_CUDA;
-  // sums[31]: the final reduction's completion counter, zero between launches
-  if (!e && cudaMemsetAsync(c->sums, 0, sizeof(double) * 32, s) != cudaSuccess) e = CL_ERR_CUDA;
+  int e = cudaGetDevice(&c->device) == cudaSuccess ? CL_OK : CL_ERR_CUDA;
+  char* zero = nullptr;
+  size_t zero_bytes = 0;
+  c->bytes = carve_list(c, nullptr, box->dim, &zero, &zero_bytes);
+  if (!e) e = clk::mem_alloc(&c->block, c->bytes, s);
+  if (!e) {
+    carve_list(c, (char*)c->block, box->dim, &zero, &zero_bytes);
+    if (cudaMemsetAsync(zero, 0, zero_bytes, s) != cudaSuccess) e = CL_ERR_CUDA;
+  }
+  if (!e) e = set_geometry(c, box, s);
   if (!e) e = run_build(c, s);
   if (e) {
+    cudaStreamSynchronize(s);
     free_all(c);
     delete c;
     return e;
@@ -409,8 +394,10 @@ int cl_build(const double* pos_dev, long long n, const cl_box* box, void* stream
 
 int cl_update(cl_list* c, const double* pos_dev, const cl_box* box, void* stream) {
   if (!c || (c->n > 0 && !pos_dev)) return CL_ERR_INVALID_ARG;
-  if (box) {
-    int e = set_geometry(c, box);
+  // an unchanged box keeps its grid, stencils and buffers (a differentiable
+  // step passes its box every time)
+  if (box && !same_box(*box, c->box)) {
+    int e = set_geometry(c, box, (cudaStream_t)stream);
     if (e) return e;
   }
   c->pos = pos_dev;
@@ -513,13 +500,7 @@ int check_query(const cl_list* c, const double* posb, long long nb) {
   return CL_OK;
 }
 
-// Workspace of one two-set call: pieces of one device block. The list keeps
-// the block for its next call, up to kQueryKeep bytes (six cudaMalloc and
-// cudaFree a call cost more host time than the sweeps of a small set); a call
-// that finds it in use by another thread allocates its own. Every call is over
-// on its stream before it gives the block back.
-constexpr size_t kQueryKeep = (size_t)256 << 20;
-
+// Workspace of one two-set call: pieces of one block of the library's pool.
 struct QueryWs {
   clk::QueryBufs bin{};
   int* count = nullptr;
@@ -534,86 +515,49 @@ struct QueryWs {
   long long* part_id = nullptr;
 
   QueryWs(cl_list* list, cudaStream_t stream) : c(list), s(stream) {}
-  ~QueryWs() {
-    if (!base) return;
-    cudaStreamSynchronize(s);
-    if (!kept) {
-      cudaFree(base);
-      return;
-    }
-    if (c->qws_bytes > kQueryKeep) {
-      cudaFree(c->qws);
-      c->qws = nullptr;
-      c->qws_bytes = 0;
-    }
-    __atomic_store_n(&c->qws_busy, 0, __ATOMIC_RELEASE);
-  }
+  ~QueryWs() { clk::mem_free(base, s); }
   // list: the arrays of the cross list; k > 0: those of the global k closest.
   int open(long long nb, bool list, int k) {
-    size_t need = carve(nullptr, nb, list, k);
-    if (__atomic_exchange_n(&c->qws_busy, 1, __ATOMIC_ACQUIRE) == 0) {
-      kept = true;
-      if (c->qws_bytes < need) {
-        cudaFree(c->qws);
-        c->qws_bytes = 0;
-        if (cudaMalloc((void**)&c->qws, need) != cudaSuccess) {
-          cudaGetLastError();
-          c->qws = nullptr;
-          __atomic_store_n(&c->qws_busy, 0, __ATOMIC_RELEASE);
-          return CL_ERR_OOM;
-        }
-        c->qws_bytes = need;
-      }
-      base = c->qws;
-    } else if (cudaMalloc((void**)&base, need) != cudaSuccess) {
-      cudaGetLastError();
-      base = nullptr;
-      return CL_ERR_OOM;
-    }
-    carve(base, nb, list, k);
+    if (int e = clk::mem_alloc(&base, carve(nullptr, nb, list, k), s)) return e;
+    carve((char*)base, nb, list, k);
     return cudaMemsetAsync(err, 0, sizeof(long long), s) == cudaSuccess ? CL_OK : CL_ERR_CUDA;
   }
 
  private:
   size_t carve(char* at, long long nb, bool list, int k) {
-    size_t used = 0;
-    auto take = [&](auto** p, size_t count) {
-      *p = at ? reinterpret_cast<std::remove_reference_t<decltype(*p)>>(at + used) : nullptr;
-      used += (count * sizeof(**p) + 255) & ~(size_t)255;
-    };
+    clk::Carver v{at};
     const size_t n = nb > 0 ? (size_t)nb : 1;
     const long long nc = c->geo.ncells;
-    take(&bin.q, n);
-    take(&bin.cell, n);
+    v.take(&bin.q, n);
+    v.take(&bin.cell, n);
     if (clk::queries_sorted(nb, nc)) {
-      take(&bin.raw, n);
-      take(&bin.slot, n);
-      take(&bin.counts, (size_t)nc);
-      take(&bin.start, (size_t)nc + 1);
-      take(&bin.tiles, (size_t)clk::scan_tiles_for(nc) + 1);
-      take(&bin.meta, 4);
+      v.take(&bin.raw, n);
+      v.take(&bin.slot, n);
+      v.take(&bin.counts, (size_t)nc);
+      v.take(&bin.start, (size_t)nc + 1);
+      v.take(&bin.tiles, (size_t)clk::scan_tiles_for(nc));
+      v.take(&bin.meta, 4);
     }
     if (list) {
-      take(&count, n);
-      take(&tiles, (size_t)clk::scan_tiles_for((long long)n));
-      take(&meta, 4);
-      take(&longs, n);
+      v.take(&count, n);
+      v.take(&tiles, (size_t)clk::scan_tiles_for((long long)n));
+      v.take(&meta, 4);
+      v.take(&longs, n);
     }
-    take(&start, list ? n + 2 : 1);
+    v.take(&start, list ? n + 2 : 1);
     err = reinterpret_cast<int*>(start + (list ? n + 1 : 0));
     if (k > 0) {
       const size_t parts = (size_t)clk::topk_parts((long long)n, k);
-      take(&knn_a, n * k);
-      take(&knn_d, n * k);
-      take(&part_d, parts * k);
-      take(&part_id, parts * k);
+      v.take(&knn_a, n * k);
+      v.take(&knn_d, n * k);
+      v.take(&part_d, parts * k);
+      v.take(&part_id, parts * k);
     }
-    return used;
+    return v.used;
   }
   cl_list* c;
   cudaStream_t s;
-  char* base = nullptr;
-  bool kept = false;
+  void* base = nullptr;
 };
 
 int read_err(const int* err_dev, cudaStream_t s) {
@@ -790,8 +734,12 @@ int cl_status(cl_list* c, void* stream) {
 
 void cl_free(cl_list* c) {
   if (!c) return;
+  int dev = -1;
+  const bool other = cudaGetDevice(&dev) == cudaSuccess && dev != c->device;
+  if (other) cudaSetDevice(c->device);
   cudaDeviceSynchronize();
   free_all(c);
+  if (other) cudaSetDevice(dev);
   delete c;
 }
 

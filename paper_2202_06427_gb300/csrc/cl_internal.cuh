@@ -103,9 +103,11 @@ struct SweepArgs {
 // Host helpers implemented in cl_geom.cu.
 int prepare_geometry(const cl_box* box, Geo* geo);
 // Builds the half-shell (half = 1) or full stencil; returns the entry count or a
-// negative error. opk (optional) receives each entry's unwrapped offset packed
+// negative error.
+int build_stencil(const Geo& geo, int half, Off* out, int cap);
+// Both at once; opk_* (optional) receive each entry's unwrapped offset packed
 // as bytes: (ox & 255) | (oy & 255) << 8 | (oz & 255) << 16.
-int build_stencil(const Geo& geo, int half, Off* out, int cap, int* opk = nullptr);
+int build_stencils(const Geo& geo, int cap, Off* half, int* opk_half, int* nhalf, Off* full, int* opk_full, int* nfull);
 // Half-widths of one cell's Cartesian bounding box (sum over the cell edge
 // vectors of |G_k,a| / 2 per axis a), each padded by 1e-3 rc.
 void cell_halfwidths(const Geo& geo, float* e);
@@ -114,6 +116,22 @@ void cell_halfwidths(const Geo& geo, float* e);
 
 namespace clk {
 
+// Stream-ordered device memory of the library (cl_mem.cu): a pool per device
+// that keeps at most kPoolKeep bytes of freed memory for later calls.
+int mem_alloc(void** p, size_t bytes, cudaStream_t s);
+void mem_free(void* p, cudaStream_t s);
+// Pieces of one block, 256-byte aligned: with base null only their total is
+// counted.
+struct Carver {
+  char* base;
+  size_t used = 0;
+  template <class T>
+  void take(T** p, size_t count) {
+    *p = base ? reinterpret_cast<T*>(base + used) : nullptr;
+    used += ((count ? count : 1) * sizeof(T) + 255) & ~(size_t)255;
+  }
+};
+
 // Buffers of one binning pipeline (cl_build.cu).
 struct BuildBufs {
   const double* pos;
@@ -121,6 +139,7 @@ struct BuildBufs {
   int* slot;    // per original particle: position inside its cell
   float4* xl;   // per original particle: centred local coordinate, w = packed cell (cx | cy << 10 | cz << 20)
   int* counts;
+  bool counts_zeroed = false;  // the caller has zeroed counts
   int* cell_start;
   int* tile_sum;
   int* meta;  // [0] error latch, [1] non-empty cells, [2] max occupancy

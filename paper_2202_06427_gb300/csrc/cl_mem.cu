@@ -1,0 +1,60 @@
+// cl_mem.cu -- device memory of the library: one stream-ordered memory pool
+// per device, shared by every handle and thread (the CUDA pool is safe for
+// both). A list's arrays are two blocks of it and the two-set calls' workspace
+// one, where each array was a cudaMalloc of its own (about twenty per list,
+// 0.5 ms of host time per build and free at 200,000 particles). Freed memory
+// beyond kPoolKeep goes back to the device at the next synchronisation.
+#include <mutex>
+
+#include "cl_internal.cuh"
+
+namespace clk {
+
+namespace {
+
+constexpr unsigned long long kPoolKeep = 256ull << 20;
+
+std::mutex pool_mu;
+cudaMemPool_t pools[kCacheDevices];
+
+int device_pool(cudaMemPool_t* out) {
+  int dev = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= kCacheDevices) return CL_ERR_CUDA;
+  std::lock_guard<std::mutex> g(pool_mu);
+  if (!pools[dev]) {
+    cudaMemPoolProps props = {};
+    props.allocType = cudaMemAllocationTypePinned;
+    props.location.type = cudaMemLocationTypeDevice;
+    props.location.id = dev;
+    cudaMemPool_t p = nullptr;
+    unsigned long long keep = kPoolKeep;
+    if (cudaMemPoolCreate(&p, &props) != cudaSuccess) return CL_ERR_CUDA;
+    if (cudaMemPoolSetAttribute(p, cudaMemPoolAttrReleaseThreshold, &keep) != cudaSuccess) {
+      cudaMemPoolDestroy(p);
+      return CL_ERR_CUDA;
+    }
+    pools[dev] = p;
+  }
+  *out = pools[dev];
+  return CL_OK;
+}
+
+}  // namespace
+
+int mem_alloc(void** p, size_t bytes, cudaStream_t s) {
+  *p = nullptr;
+  cudaMemPool_t pool;
+  int e = device_pool(&pool);
+  if (!e && cudaMallocFromPoolAsync(p, bytes ? bytes : 1, pool, s) != cudaSuccess) e = CL_ERR_OOM;
+  if (e) {
+    cudaGetLastError();
+    *p = nullptr;
+  }
+  return e;
+}
+
+void mem_free(void* p, cudaStream_t s) {
+  if (p) cudaFreeAsync(p, s);
+}
+
+}  // namespace clk

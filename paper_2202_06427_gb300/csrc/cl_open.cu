@@ -60,11 +60,9 @@ int open_box(const double* const* sets, const long long* ns, int nsets, int dim,
              cudaStream_t s, cl_box* box) {
   if (dim != 2 && dim != 3) return CL_ERR_INVALID_ARG;
   if (!(cutoff > 0) || !std::isfinite(cutoff)) return CL_ERR_INVALID_ARG;
-  unsigned long long* mm = nullptr;
-  if (cudaMalloc((void**)&mm, sizeof(unsigned long long) * 6 + sizeof(int)) != cudaSuccess) {
-    cudaGetLastError();
-    return CL_ERR_OOM;
-  }
+  void* block = nullptr;
+  if (const int e = mem_alloc(&block, sizeof(unsigned long long) * 6 + sizeof(int), s)) return e;
+  unsigned long long* mm = (unsigned long long*)block;
   int* bad = reinterpret_cast<int*>(mm + 6);
   unsigned long long init[6];
   for (int k = 0; k < 3; ++k) {
@@ -90,7 +88,7 @@ int open_box(const double* const* sets, const long long* ns, int nsets, int dim,
              cudaMemcpyAsync(&nonfinite, bad, sizeof(int), cudaMemcpyDeviceToHost, s) != cudaSuccess ||
              cudaStreamSynchronize(s) != cudaSuccess))
     e = CL_ERR_CUDA;
-  cudaFree(mm);
+  mem_free(block, s);
   if (e) return e;
   if (nonfinite) return CL_ERR_NONFINITE;
   std::memset(box, 0, sizeof(*box));
