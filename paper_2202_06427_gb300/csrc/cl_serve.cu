@@ -9,8 +9,8 @@
 // request) sums the per-tile FP64 partials in a fixed order.
 //
 // Host side: a scheduling thread admits requests by device-arena space,
-// builds their cell lists on build streams, launches batches on the main
-// stream (at most two in flight) and completes requests when their batch's
+// builds their cell lists on build streams, launches batches (at most two in
+// flight, each on a stream of its own) and completes requests when their batch's
 // event has fired.
 #include <algorithm>
 #include <atomic>
@@ -276,6 +276,7 @@ struct Req {
   double* d_virial = nullptr;
   int latched = 0;  // host copy of the error latch
   int nitems = 0;
+  double tile_cost = 0;  // candidates of one particle, weighted by the task
   cudaEvent_t built = nullptr;
 };
 
@@ -285,6 +286,7 @@ struct Batch {
   clk::ReqDesc* d_desc = nullptr;
   int* d_counter = nullptr;
   int* h_latch = nullptr;          // pinned, one per request of the batch
+  cudaStream_t stream = nullptr;   // of its own: one batch's result copies and last tiles overlap the next one's sweep
   cudaEvent_t done = nullptr;
   bool busy = false;
   int err = CL_OK;                 // CL_ERR_CUDA when a copy or launch of the batch failed
@@ -295,7 +297,6 @@ struct Batch {
 struct cl_server {
   int device = 0;
   int max_inflight = 0;
-  cudaStream_t main = nullptr;
   cudaStream_t build[kBuildStreams] = {};
   int next_build = 0;
   char* arena_base = nullptr;
@@ -333,7 +334,7 @@ size_t request_bytes(const Req& q) {
   const size_t tiles = (size_t)clk::scan_tiles_for((long long)C);
   const size_t items = n > 0 ? (n + clk::kServeThreads - 1) / clk::kServeThreads : 1;
   size_t b = up(n * d * 8) + 2 * up(n * 16) + 2 * up(n * 4) + up(C * 4) + up((C + 1) * 4) + up(tiles * 4 + 4) +
-             up(16) + up(q.off.size() * sizeof(clk::Off)) + up(items * 7 * 8) + up(8) + up(72);
+             up(16) + up(q.off.size() * sizeof(clk::Off)) + up(items * 7 * 8) + up(8 + 72);
   if (q.r.task == CL_TASK_FORCES) b += up(n * d * 4);
   if (q.r.task == CL_TASK_HIST) b += up((size_t)q.r.nbins * 8);
   return b;
@@ -384,16 +385,18 @@ bool cl_server::admit_one(Req* q) {
   B.xs = reinterpret_cast<float4*>(take(n * 16));
   B.slot = reinterpret_cast<int*>(take(n * 4));
   B.cellc = reinterpret_cast<unsigned*>(take(n * 4));
-  B.counts = reinterpret_cast<int*>(take(C * 4));
   B.cell_start = reinterpret_cast<int*>(take((C + 1) * 4));
   B.tile_sum = reinterpret_cast<int*>(take((size_t)clk::scan_tiles_for((long long)C) * 4 + 4));
-  B.meta = reinterpret_cast<int*>(take(16));
   q->d_off = reinterpret_cast<clk::Off*>(take(q->off.size() * sizeof(clk::Off)));
   q->nitems = n > 0 ? (int)((n + clk::kServeThreads - 1) / clk::kServeThreads) : 0;
   q->d_partials = reinterpret_cast<double*>(take((size_t)std::max(q->nitems, 1) * 7 * 8));
-  q->d_energy = reinterpret_cast<double*>(take(8));
-  q->d_virial = reinterpret_cast<double*>(take(72));
   if (q->r.task == CL_TASK_FORCES) q->d_forces = reinterpret_cast<float*>(take(n * d * 4));
+  char* const zeros = p;  // the arrays that start as zeros, one after the other: one memset
+  B.counts = reinterpret_cast<int*>(take(C * 4));
+  B.counts_zeroed = true;
+  B.meta = reinterpret_cast<int*>(take(16));
+  q->d_energy = reinterpret_cast<double*>(take(8 + 72));
+  q->d_virial = q->d_energy + 1;
   if (q->r.task == CL_TASK_HIST) q->d_hist = reinterpret_cast<unsigned long long*>(take((size_t)q->r.nbins * 8));
   cudaStream_t s = build[next_build];
   next_build = (next_build + 1) % kBuildStreams;
@@ -403,9 +406,7 @@ bool cl_server::admit_one(Req* q) {
   if (!e && cudaMemcpyAsync(q->d_off, q->off.data(), q->off.size() * sizeof(clk::Off), cudaMemcpyHostToDevice, s) !=
                 cudaSuccess)
     e = CL_ERR_CUDA;
-  if (!e && cudaMemsetAsync(B.meta, 0, 16, s) != cudaSuccess) e = CL_ERR_CUDA;
-  if (!e && q->d_hist && cudaMemsetAsync(q->d_hist, 0, (size_t)q->r.nbins * 8, s) != cudaSuccess) e = CL_ERR_CUDA;
-  if (!e && cudaMemsetAsync(q->d_energy, 0, 8 + 72, s) != cudaSuccess) e = CL_ERR_CUDA;
+  if (!e && cudaMemsetAsync(zeros, 0, (size_t)(p - zeros), s) != cudaSuccess) e = CL_ERR_CUDA;
   if (!e) e = clk::launch_build(q->geo, B, s);
   if (!e && cudaEventRecord(q->built, s) != cudaSuccess) e = CL_ERR_CUDA;
   {
@@ -434,6 +435,9 @@ void cl_server::launch_batch(Batch& b) {
   };
   int items = 0, maxbins = 0;
   const double tl = now();
+  // The requests' tiles are taken in order, so the costliest tiles go first:
+  // the batch then ends on cheap tiles instead of waiting for a few long ones.
+  std::stable_sort(b.reqs.begin(), b.reqs.end(), [](const Req* x, const Req* y) { return x->tile_cost > y->tile_cost; });
   for (size_t k = 0; k < b.reqs.size(); ++k) {
     Req* q = b.reqs[k];
     q->t[2] = tl;
@@ -473,40 +477,40 @@ void cl_server::launch_batch(Batch& b) {
     D.virial = q->d_virial;
     items += q->nitems;
     if (q->r.task == CL_TASK_HIST) maxbins = std::max(maxbins, q->r.nbins);
-    ok(cudaStreamWaitEvent(main, q->built, 0));
+    ok(cudaStreamWaitEvent(b.stream, q->built, 0));
   }
   const int nreq = (int)b.reqs.size();
-  ok(cudaMemcpyAsync(b.d_desc, b.h_desc, sizeof(clk::ReqDesc) * nreq, cudaMemcpyHostToDevice, main));
-  ok(cudaMemsetAsync(b.d_counter, 0, sizeof(int), main));
+  ok(cudaMemcpyAsync(b.d_desc, b.h_desc, sizeof(clk::ReqDesc) * nreq, cudaMemcpyHostToDevice, b.stream));
+  ok(cudaMemsetAsync(b.d_counter, 0, sizeof(int), b.stream));
   if (items > 0 && !b.err) {
     int grid = std::min(items, sm_count * ctas_per_sm);
-    clk::k_serve_sweep<<<grid, clk::kServeThreads, sizeof(unsigned) * maxbins, main>>>(b.d_desc, nreq, items,
+    clk::k_serve_sweep<<<grid, clk::kServeThreads, sizeof(unsigned) * maxbins, b.stream>>>(b.d_desc, nreq, items,
                                                                                        b.d_counter);
     ok(cudaGetLastError());
   }
   if (!b.err) {
-    clk::k_serve_finalize<<<nreq, 256, 0, main>>>(b.d_desc);
+    clk::k_serve_finalize<<<nreq, 256, 0, b.stream>>>(b.d_desc);
     ok(cudaGetLastError());
   }
   for (int k = 0; k < nreq && !b.err; ++k) {
     Req* q = b.reqs[k];
     const size_t n = (size_t)q->r.n, d = (size_t)q->geo.dim;
     if (q->r.task != CL_TASK_HIST && q->r.energy_host)
-      ok(cudaMemcpyAsync(q->r.energy_host, q->d_energy, 8, cudaMemcpyDeviceToHost, main));
+      ok(cudaMemcpyAsync(q->r.energy_host, q->d_energy, 8, cudaMemcpyDeviceToHost, b.stream));
     if (q->r.task == CL_TASK_FORCES) {
       if (q->r.forces_host && n)
-        ok(cudaMemcpyAsync(q->r.forces_host, q->d_forces, n * d * 4, cudaMemcpyDeviceToHost, main));
+        ok(cudaMemcpyAsync(q->r.forces_host, q->d_forces, n * d * 4, cudaMemcpyDeviceToHost, b.stream));
       if (q->r.virial_host)
-        ok(cudaMemcpyAsync(q->r.virial_host, q->d_virial, d * d * 8, cudaMemcpyDeviceToHost, main));
+        ok(cudaMemcpyAsync(q->r.virial_host, q->d_virial, d * d * 8, cudaMemcpyDeviceToHost, b.stream));
     }
     if (q->r.task == CL_TASK_HIST && q->r.hist_host)
-      ok(cudaMemcpyAsync(q->r.hist_host, q->d_hist, (size_t)q->r.nbins * 8, cudaMemcpyDeviceToHost, main));
-    ok(cudaMemcpyAsync(b.h_latch + k, q->bufs.meta, sizeof(int), cudaMemcpyDeviceToHost, main));
+      ok(cudaMemcpyAsync(q->r.hist_host, q->d_hist, (size_t)q->r.nbins * 8, cudaMemcpyDeviceToHost, b.stream));
+    ok(cudaMemcpyAsync(b.h_latch + k, q->bufs.meta, sizeof(int), cudaMemcpyDeviceToHost, b.stream));
   }
-  if (cudaEventRecord(b.done, main) != cudaSuccess) {
+  if (cudaEventRecord(b.done, b.stream) != cudaSuccess) {
     // no event to poll: wait for what was queued, then finish the batch now
     b.err = CL_ERR_CUDA;
-    cudaStreamSynchronize(main);
+    cudaStreamSynchronize(b.stream);
     b.busy = true;
     complete(b);
   } else {
@@ -597,7 +601,6 @@ int cl_serve_create(long long arena_bytes, int max_inflight, int device, cl_serv
   }
   if (!e && cudaMalloc((void**)&s->arena_base, (size_t)arena_bytes) != cudaSuccess) e = CL_ERR_OOM;
   if (!e) s->arena.init((size_t)arena_bytes);
-  if (!e && cudaStreamCreateWithFlags(&s->main, cudaStreamNonBlocking) != cudaSuccess) e = CL_ERR_CUDA;
   for (int k = 0; k < kBuildStreams && !e; ++k)
     if (cudaStreamCreateWithFlags(&s->build[k], cudaStreamNonBlocking) != cudaSuccess) e = CL_ERR_CUDA;
   for (Batch& b : s->batches) {
@@ -606,6 +609,7 @@ int cl_serve_create(long long arena_bytes, int max_inflight, int device, cl_serv
         cudaMalloc((void**)&b.d_desc, sizeof(clk::ReqDesc) * max_inflight) != cudaSuccess ||
         cudaMalloc((void**)&b.d_counter, sizeof(int)) != cudaSuccess ||
         cudaMallocHost((void**)&b.h_latch, sizeof(int) * max_inflight) != cudaSuccess ||
+        cudaStreamCreateWithFlags(&b.stream, cudaStreamNonBlocking) != cudaSuccess ||
         cudaEventCreateWithFlags(&b.done, cudaEventDisableTiming) != cudaSuccess)
       e = CL_ERR_OOM;
   }
@@ -634,6 +638,9 @@ int cl_serve_submit(cl_server* s, const cl_request* req, long long* ticket) {
     int noff = clk::build_stencil(q->geo, req->task == CL_TASK_FORCES ? 0 : 1, q->off.data(), clk::kMaxOff);
     if (noff < 0) e = noff;
     else q->off.resize(noff);
+    // pair terms per particle: candidates, and about twice the work for forces
+    q->tile_cost = (double)q->off.size() * (double)req->n / (double)q->geo.ncells *
+                   (req->task == CL_TASK_ENERGY ? 1.0 : 1.5);
   }
   if (!e && cudaEventCreateWithFlags(&q->built, cudaEventDisableTiming) != cudaSuccess) e = CL_ERR_CUDA;
   if (e) {
@@ -714,14 +721,16 @@ void cl_serve_free(cl_server* s) {
     s->th.join();
   }
   cudaSetDevice(s->device);
-  if (s->main) cudaStreamSynchronize(s->main);
   for (int k = 0; k < kBuildStreams; ++k)
     if (s->build[k]) {
       cudaStreamSynchronize(s->build[k]);
       cudaStreamDestroy(s->build[k]);
     }
-  if (s->main) cudaStreamDestroy(s->main);
   for (Batch& b : s->batches) {
+    if (b.stream) {
+      cudaStreamSynchronize(b.stream);
+      cudaStreamDestroy(b.stream);
+    }
     cudaFreeHost(b.h_desc);
     cudaFree(b.d_desc);
     cudaFree(b.d_counter);
