@@ -609,12 +609,12 @@ int launch_cross_knn(const SweepArgs& A, const Off* off, const Queries& Q, int k
   }
 }
 
-// A warp's share is at least 2,048 candidates, and at most 1,024 warps share
-// the lists, so that the last kernel reads at most 1,024 k entries.
+// A warp's share is at least 256 candidates (its first ones all enter its list,
+// one at a time), and at most 1,216 warps, one wave, share the lists.
 static long long topk_share(long long nb, int k) {
   const long long total = nb * k;
-  const long long share = (total + 1023) / 1024;
-  return (std::max<long long>(share, 2048) + 31) / 32 * 32;
+  const long long share = (total + 1215) / 1216;
+  return (std::max<long long>(share, 256) + 31) / 32 * 32;
 }
 
 long long topk_parts(long long nb, int k) {

@@ -150,7 +150,7 @@ __device__ __forceinline__ void sort_keys_blocked(unsigned (&k)[E], int lane) {
         if ((e & stride) == 0) key_cas(k[e], k[e | stride]);
     }
   }
-#pragma unroll
+#pragma unroll 1  // rolled: unrolled, the 512- and 1,024-key networks overflow the instruction cache
   for (int lanes = 2; lanes <= 32; lanes <<= 1) {
     const bool low = (lane & (lanes >> 1)) == 0;
 #pragma unroll
@@ -161,7 +161,7 @@ __device__ __forceinline__ void sort_keys_blocked(unsigned (&k)[E], int lane) {
       k[e] = low ? min(k[e], a) : max(k[e], a);
       if (f != e) k[f] = low ? min(k[f], b) : max(k[f], b);
     }
-#pragma unroll
+#pragma unroll 1
     for (int ls = lanes >> 2; ls > 0; ls >>= 1) {
       const bool lo = (lane & ls) == 0;
 #pragma unroll
