@@ -321,7 +321,7 @@ typedef struct {
  * the full stencil all of them. All pointers are device memory owned by the
  * handle, valid until the next cl_update or cl_free. The order of the
  * particles within a cell is not fixed: the 3D sweeps may reorder the
- * particles of cells of more than 128 particles by octant (xs and cellc stay
+ * particles of cells of 65 or more particles by octant (xs and cellc stay
  * consistent; cell_start does not change). */
 typedef struct {
   int dim;

@@ -66,8 +66,7 @@ size_t carve_list(cl_list* c, char* base, int dim, char** zero_from, size_t* zer
   v.take(&c->xs, n);
   v.take(&c->cellc, n);
   v.take(&c->partials, (size_t)clk::sweep_partials_needed(c->n));
-  v.take(&c->work, 8);  // [0] work counter, [2..3] candidate counter, [5] the dense
-                        // cells' work counter, [6] list length, [7] dense cells
+  v.take(&c->work, clk::kWorkWords);  // see HoodArgs
   v.take(&c->u64, 8);
   v.take(&c->d_off_half, 2 * (size_t)clk::kMaxOff);  // both stencils, one after the other
   const size_t at = v.used;

@@ -355,42 +355,48 @@ __global__ void __launch_bounds__(1024) k_scan_one(const int* __restrict__ count
   if (blockIdx.x == gridDim.x - 1 && threadIdx.x == 1023) cell_start[ncells] = run;
 }
 
+// Order key of a particle within its cell: the octant of its local coordinate
+// (signs of x, y, z), then the octant within it, in Gray-code order so that
+// neighbours in the order are neighbours in space.
+__device__ __forceinline__ int oct_key(const float4& v, float qx, float qy, float qz) {
+  const int g = (fabsf(v.x) > qx ? 1 : 0) | (fabsf(v.y) > qy ? 2 : 0) | (fabsf(v.z) > qz ? 4 : 0);
+  return ((v.x > 0.f ? 1 : 0) | (v.y > 0.f ? 2 : 0) | (v.z > 0.f ? 4 : 0)) * 8 + (g ^ (g >> 1) ^ (g >> 2));
+}
+
 // Orders the particles of each listed cell of kOctMin..kOctCap particles by
-// the octant of their local coordinate (key = (x > 0) | (y > 0) << 1 |
-// (z > 0) << 2): a counting sort through shared memory, writing the cell's
-// range of xs back in key order and each moved particle's slot. The order of
+// oct_key: a counting sort through shared memory, writing the cell's range of
+// xs back in key order and each moved particle's slot. The order of
 // particles within a cell is free (every sweep indexes them through xs.w and
 // slot), so the cell list stays valid. One CTA per cell, persistent over the
 // list; other listed cells are skipped.
 __global__ void __launch_bounds__(256) k_octsort(const int* __restrict__ big, const int* __restrict__ nbig,
-                                                const int* __restrict__ cell_start, float4* __restrict__ xs,
-                                                int* __restrict__ slot) {
+                                                const int* __restrict__ cell_start, float qx, float qy, float qz,
+                                                float4* __restrict__ xs, int* __restrict__ slot) {
   __shared__ float4 buf[kOctCap];
-  __shared__ int cnt[8], at[8];
+  __shared__ int at[64];
   const int nb = *nbig;
   for (int q = blockIdx.x; q < nb; q += gridDim.x) {
     const int c = big[q];
     const int hs = cell_start[c], nh = cell_start[c + 1] - hs;
     if (nh < kOctMin || nh > kOctCap) continue;  // uniform over the CTA
-    if (threadIdx.x < 8) cnt[threadIdx.x] = 0;
+    if (threadIdx.x < 64) at[threadIdx.x] = 0;
     __syncthreads();
     for (int t = threadIdx.x; t < nh; t += blockDim.x) {
       const float4 v = xs[hs + t];
       buf[t] = v;
-      atomicAdd(&cnt[(v.x > 0.f ? 1 : 0) | (v.y > 0.f ? 2 : 0) | (v.z > 0.f ? 4 : 0)], 1);
+      atomicAdd(&at[oct_key(v, qx, qy, qz)], 1);
     }
     __syncthreads();
-    if (threadIdx.x == 0) {
-      int run = 0;
-      for (int k = 0; k < 8; ++k) {
-        at[k] = run;
-        run += cnt[k];
-      }
+    if (threadIdx.x < 32) {  // counts to starts, two keys per lane
+      const int a = at[2 * threadIdx.x], b = at[2 * threadIdx.x + 1];
+      const int before = warp_incl_scan(a + b) - (a + b);
+      at[2 * threadIdx.x] = before;
+      at[2 * threadIdx.x + 1] = before + a;
     }
     __syncthreads();
     for (int t = threadIdx.x; t < nh; t += blockDim.x) {
       const float4 v = buf[t];
-      const int p = atomicAdd(&at[(v.x > 0.f ? 1 : 0) | (v.y > 0.f ? 2 : 0) | (v.z > 0.f ? 4 : 0)], 1);
+      const int p = atomicAdd(&at[oct_key(v, qx, qy, qz)], 1);
       xs[hs + p] = v;
       slot[__float_as_int(v.w)] = p;
     }
@@ -461,9 +467,9 @@ __global__ void __launch_bounds__(256) k_cellc(long long ncells, int nx, int ny,
 
 
 
-int launch_octsort(const int* cells, const int* ncells_listed, const int* cell_start, float4* xs, int* slot,
-                   cudaStream_t s) {
-  k_octsort<<<152 * 4, 256, 0, s>>>(cells, ncells_listed, cell_start, xs, slot);
+int launch_octsort(const int* cells, const int* ncells_listed, const int* cell_start, float hx, float hy, float hz,
+                   float4* xs, int* slot, cudaStream_t s) {
+  k_octsort<<<152 * 4, 256, 0, s>>>(cells, ncells_listed, cell_start, 0.5f * hx, 0.5f * hy, 0.5f * hz, xs, slot);
   return cudaGetLastError() == cudaSuccess ? CL_OK : CL_ERR_CUDA;
 }
 

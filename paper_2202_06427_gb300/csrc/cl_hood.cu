@@ -708,13 +708,6 @@ __device__ unsigned long long particle_sweep(const SweepArgs& A, const HoodArgs&
   return ncand;
 }
 
-// Work lists: cells with kMinHome..kHome particles (and a stencil that fits
-// the table) go to the neighbourhood sweep (list, work[6] of them); cells with
-// more than kHome particles are flagged 2 and listed for the dense-cell sweep
-// (dense, *ndense of them); the other non-empty cells (fewer particles, or a
-// stencil larger than the table) are flagged 1 for the per-particle companion.
-// A cell whose staged neighbourhood overflows is moved to the dense list by
-// the sweep itself.
 // Particles in the neighbour cells (cx + ox, cy + oy, cz + oz), ox0 <= ox <= ox1
 // (wrapped): one contiguous range unless the run crosses the box edge in x.
 __device__ __forceinline__ int run_count(const int* __restrict__ cell_start, int nx, int ny, int nz, int cx, int cy,
@@ -741,8 +734,10 @@ __device__ __forceinline__ int run_count(const int* __restrict__ cell_start, int
 // A cell whose staged neighbourhood overflows is moved to the dense list by
 // the sweep itself. With half != 0 (the half-shell sweep takes the launch)
 // every non-empty cell is listed: on list when it holds at most kHome
-// particles and its half stencil's cells (opk_half, noff_half entries) at most
-// kHCap, on dense (the windowed cells) otherwise.
+// particles and its half stencil's cells at most H.rawcap, on dense (the
+// windowed cells) otherwise. kListLanes lanes share a cell's rows: one thread
+// per cell took 13 us on a grid of 343 cells and 18 on one of 42,875.
+constexpr int kListLanes = 8;
 __global__ void __launch_bounds__(256) k_hood_list(const int* __restrict__ cell_start, int ncells, int noff,
                                                    int* __restrict__ work, int* __restrict__ list,
                                                    unsigned char* __restrict__ flag, int* __restrict__ dense,
@@ -750,23 +745,22 @@ __global__ void __launch_bounds__(256) k_hood_list(const int* __restrict__ cell_
                                                    int noff_half, int nx, int ny, int nz) {
   const int half = H.half;
   const int* opk_half = H.opk[1];
-  const int h = blockIdx.x * blockDim.x + threadIdx.x;
+  const int h = (blockIdx.x * blockDim.x + threadIdx.x) / kListLanes, sub = threadIdx.x % kListLanes;
   const unsigned lt = (1u << (threadIdx.x & 31)) - 1u;
   bool take = false, big = false;
+  int cnt = 0;
   if (h < ncells) {
     const int nh = cell_start[h + 1] - cell_start[h];
     take = (half ? nh >= 1 : nh >= kMinHome) && nh <= kHome && noff <= kTab;
     big = half ? (nh > 0 && !take) : nh > kHome;
-    flag[h] = (nh > 0 && !take) ? (big ? 2 : 1) : 0;
     if (half && take) {
       const int cx = h % nx, cy = (h / nx) % ny, cz = h / (nx * ny);
-      int cnt = 0;
-      if (H.nrows_half > 0) {  // the rows from the host: independent loads
+      if (H.nrows_half > 0) {  // the rows from the host, shared among the cell's lanes: independent loads
 #pragma unroll 4
-        for (int r = 0; r < H.nrows_half; ++r)
+        for (int r = sub; r < H.nrows_half; r += kListLanes)
           cnt += run_count(cell_start, nx, ny, nz, cx, cy, cz, H.rows_half[r][0], H.rows_half[r][1],
                            H.rows_half[r][2], H.rows_half[r][3]);
-      } else {
+      } else if (sub == 0) {
         int r0 = 0, px = 0, py = 0, pz = 0;
         for (int k = 1; k <= noff_half; ++k) {
           int ox = 0, oy = 0, oz = 0;
@@ -781,12 +775,28 @@ __global__ void __launch_bounds__(256) k_hood_list(const int* __restrict__ cell_
           pz = oz;
         }
       }
-      if (cnt > kHCap) {
-        take = false;
-        big = true;
-      }
     }
   }
+#pragma unroll
+  for (int o = kListLanes / 2; o; o >>= 1) cnt += __shfl_xor_sync(0xffffffffu, cnt, o);
+  if (take && cnt > H.rawcap) {
+    take = false;
+    big = half != 0;
+  }
+  take = take && sub == 0;
+  big = big && sub == 0;
+  // small cells go to the end of list
+  const bool small = take && half && h < ncells && cnt + (cell_start[h + 1] - cell_start[h]) <= H.smallcap;
+  const unsigned ms = __ballot_sync(0xffffffffu, small);
+  int sbase = 0;
+  if ((threadIdx.x & 31) == 0 && ms) sbase = atomicAdd(work + 8, __popc(ms));
+  sbase = __shfl_sync(0xffffffffu, sbase, 0);
+  if (small) {
+    list[ncells - 1 - (sbase + __popc(ms & lt))] = h;
+    flag[h] = 0;
+    take = false;
+  }
+  if (h < ncells && sub == 0 && !small) flag[h] = take || cell_start[h + 1] == cell_start[h] ? 0 : (big ? 2 : 1);
   const unsigned m = __ballot_sync(0xffffffffu, take), mb = __ballot_sync(0xffffffffu, big);
   int base = 0, bbase = 0;
   if ((threadIdx.x & 31) == 0) {
@@ -1151,17 +1161,18 @@ __global__ void __launch_bounds__(kThreads, 5) k_hood(const __grid_constant__ Sw
   for (;;) {
     __syncthreads();
     if (tid == 0) {
-      S.item = next1 < nlist ? H.list[next1] : -1;
+      S.item = next1 < nlist ? H.list[next1] : -2;
       S.nf = 0;
       S.nb = 0;
     }
     __syncthreads();
     const int h = S.item;
-    if (h < 0) break;
+    if (h == -2) break;
     if (tid == 0) {
       next1 = next2;
       next2 = atomicAdd(H.work, 1);
     }
+    if (h < 0) continue;  // on the dense list (moved there by the half-shell sweep)
     const int hs = A.cell_start[h];
     const int nh = A.cell_start[h + 1] - hs;
     const int cx = h % A.nx, cy = (h / A.nx) % A.ny, cz = h / (A.nx * A.ny);
@@ -1395,11 +1406,32 @@ __global__ void __launch_bounds__(kThreads, 5) k_hood(const __grid_constant__ Sw
 // swept, so the path covers the whole grid whenever both stencils fit the
 // table.
 
+constexpr int kEnt = 4;             // staged entries per lane in a chunk of the half-shell sweep
+constexpr int kChunk = 32 * kEnt;   // entries per chunk
+constexpr int kBatch = 32;          // home particles of a batch, swept by one warp
+static_assert(kWarps * kBatch == kHome, "the batches' force sums share the fast path's");
+// Small cells: the cell and its half neighbourhood in one warp's share of the
+// entry buffer, its row segments in the warp's share of the segment table.
+constexpr int kSmallCap = (kHCap + 32) / kWarps & ~31;
+constexpr int kSmallSegs = 32;
+static_assert(kWarps * kSmallCap <= kHCap && kWarps * kSmallSegs <= kTab, "the warps' shares fit");
+
+// What a batch's sweep reads of the launch arguments, in shared memory.
+struct HalfCtx {
+  const float4* xs;
+  float4* hforce;
+  float rc2, irc, irc2, rc, eps;
+  float hrow[9];
+};
+
 struct HalfSmem {
+  HalfCtx ctx;
   float4 ent[kHCap + 32];  // (x, y, z in the home frame, sorted position as int bits); 32 trash entries
   unsigned short img[kHCap];  // lattice image of the T != 0 entries, (tx, ty, tz) as 5-bit signed fields
-  unsigned short ilist[kHCap];  // windowed cells: the staged entries within a batch's ball
-  float4 home[kHome + 4];  // home particles (-x, -y, -z, sorted position), padded by far entries
+  unsigned short wlist[kWarps][kChunk + 32];  // windowed cells: a warp's staged entries within its batch's ball
+  // home particles (-x, -y, -z, sorted position), padded by far entries: the
+  // cell's (fast path), or kBatch + 4 per warp (windowed cells)
+  float4 home[kWarps * (kBatch + 4)];
   float4 own[kHome];       // the same with (x, y, z): the own cell's entries
   float hg[kHome][3];      // per home particle: sum of fsn r over its entries
   float4 otab[kTab];       // half stencil: (shift x, y, z, unwrapped offset as int bits)
@@ -1407,7 +1439,8 @@ struct HalfSmem {
   unsigned short rowk[kTab + 1];
   int nrows, nseg, ctot;
   int oct[9];              // windowed cells: octant ranges of the cell's particles
-  float bmin[kWarps][6];   // batch_ball: per-warp minima
+  int nbatch;              // windowed cells: batches of the cell
+  int kind;                // fast path: this item's place on the list
   float wmax[kWarps];
   int nf, nb, item, next, nl;
   unsigned long long ncand;
@@ -1544,34 +1577,34 @@ __device__ __forceinline__ void half_stage(const SweepArgs& A, HalfSmem& S, int 
   }
 }
 
-constexpr int kEnt = 4;             // staged entries per lane in a chunk of the half-shell sweep
-constexpr int kChunk = 32 * kEnt;   // entries per chunk
-
 // The staged entries of a cell taken as one sequence: the T = 0 entries
 // [0, nf), then the T != 0 entries (stored at the back of the buffer), then
 // the home particles themselves (own cell). Position j of the sequence: its
 // entry, and (own cell) its home index, else a large value.
 struct SeqInfo {
   int nf, nb, nh;
-  int obase;  // own pass of a windowed cell: position j is own particle j + obase of the batch
-  int wf;     // list pass of a windowed cell: the window's T = 0 entries (the others are T != 0)
+  int obase, oown;  // own part of a windowed cell: position j is entry j + obase, home index j + oown
+  int wf;           // list part: entries from here on have a lattice image in S.img, the ones before T = 0
+  const unsigned short* list;
 };
-// Kinds of sequence: the staged entries then the home particles (fast path),
-// a windowed cell's own particles (own pass), the entries of S.ilist (list
-// pass: a window's entries within a batch's ball; nf = list length).
+// Kinds of sequence: the staged entries then the home particles (fast path);
+// a windowed cell's batch against its own particles (own part: masked by
+// index) and against listed entries of the window (list part: those within
+// the batch's ball; nf = list length).
 constexpr int kSeqPlain = 0, kSeqOwn = 1, kSeqList = 2;
 
 template <int SEQ>
 __device__ __forceinline__ float4 seq_entry(const HalfSmem& S, const SeqInfo& q, int j, int& own, bool far_up) {
   own = 0x7fffffff;
   if (SEQ == kSeqList) {
-    if (j < q.nf) return S.ent[S.ilist[j]];
+    if (j < q.nf) return S.ent[q.list[j]];
     return far_up ? make_float4(kFar, kFar, kFar, 0.f) : make_float4(-kFar, -kFar, -kFar, 0.f);
   }
-  if (j < q.nf) {
-    if (SEQ == kSeqOwn) own = j + q.obase;
-    return S.ent[j];
+  if (SEQ == kSeqOwn && j < q.nf) {
+    own = j + q.oown;
+    return S.ent[j + q.obase];
   }
+  if (j < q.nf) return S.ent[j];
   if (j < q.nf + q.nb) return S.ent[kHCap - q.nb + (j - q.nf)];
   if (j < q.nf + q.nb + q.nh) {
     own = j - q.nf - q.nb;
@@ -1586,17 +1619,16 @@ __device__ __forceinline__ float4 seq_entry(const HalfSmem& S, const SeqInfo& q,
 // when the entry comes after the home particle. The lane's entries' forces
 // (sum of fsn r, r = entry - home) accumulate in jx, jy, jz (pair k: positions
 // u = 2k, 2k + 1); each home particle's sum of fsn r over the chunk is
-// warp-summed per step into S.hg. SEQ: the kind of sequence (seq_entry); in
-// the own pass of a windowed cell every entry is an own-cell particle (index
-// j + obase within the batch).
+// warp-summed per step into hg (shared by the CTA's warps on the fast path,
+// the warp's own otherwise). SEQ: the kind of sequence (seq_entry).
 // Scalar modes (MODE 2 energy, 4 count, 5 sum 1/r, 6 histogram) evaluate the
 // same candidates with the reduction of scalar_pair and no forces: the count
 // in cnt, the energy or sum 1/r in e, the bins in R.hist.
 // KB: the chunk's blocks of 64 positions that hold sequence positions (a last
 // chunk of at most 64 skips the second block's arithmetic).
 template <bool MASK, int SEQ = kSeqPlain, int MODE = 3, int KB = kEnt / 2>
-__device__ __forceinline__ void half_chunk(HalfSmem& S, const SeqInfo& sq, int base, int nh, float rc2, float irc,
-                                           float irc2, float2 (&jx)[kEnt / 2], float2 (&jy)[kEnt / 2],
+__device__ __forceinline__ void half_chunk(const HalfSmem& S, const float4* home, float (*hg)[3], const SeqInfo& sq,
+                                           int base, int nh, float rc2, float irc, float irc2, float2 (&jx)[kEnt / 2], float2 (&jy)[kEnt / 2],
                                            float2 (&jz)[kEnt / 2], float2& e, unsigned& cnt, const ScalarRed& R) {
   constexpr bool SCALAR = MODE == 2 || MODE >= 4;
   const int lane = threadIdx.x & 31;
@@ -1614,7 +1646,7 @@ __device__ __forceinline__ void half_chunk(HalfSmem& S, const SeqInfo& sq, int b
   }
   if (SCALAR) {
     for (int h = 0; h < nh; ++h) {
-      const float4 hp = S.home[h];  // broadcast; negated coordinates
+      const float4 hp = home[h];  // broadcast; negated coordinates
 #pragma unroll
       for (int k = 0; k < KB; ++k) {
         const bool m0 = !MASK || own[2 * k] > h, m1 = !MASK || own[2 * k + 1] > h;
@@ -1623,11 +1655,18 @@ __device__ __forceinline__ void half_chunk(HalfSmem& S, const SeqInfo& sq, int b
     }
     return;
   }
+  // Four home particles per step. Lane l takes them in the order u ^ lx, lx =
+  // l >> 3: the first two levels of the warp sum then exchange fixed halves of
+  // a lane's values (which lane keeps which is in the order, not selected),
+  // and lane l ends with the sums of home particle h0 + lx over its eight
+  // lanes' group (36 instructions a step against 62 with selects).
+  const int lx = lane >> 3;
   for (int h0 = 0; h0 < nh; h0 += 4) {
-    float v[16];
+    float v[12];
 #pragma unroll
     for (int u = 0; u < 4; ++u) {
-      const float4 hp = S.home[h0 + u];  // broadcast; negated coordinates, padded past nh by far entries
+      const int hu = h0 + (u ^ lx);
+      const float4 hp = home[hu];  // four addresses a warp; negated coordinates, padded past nh by far entries
       float2 gx = f2(0.f), gy = f2(0.f), gz = f2(0.f);
 #pragma unroll
       for (int k = 0; k < KB; ++k) {
@@ -1638,8 +1677,8 @@ __device__ __forceinline__ void half_chunk(HalfSmem& S, const SeqInfo& sq, int b
         d2 = __ffma2_rn(dx, dx, d2);
         float2 y = make_float2(rsqrtf(d2.x), rsqrtf(d2.y));
         if (MASK) {
-          y.x = (own[2 * k] > h0 + u && d2.x < rc2) ? y.x : 0.f;
-          y.y = (own[2 * k + 1] > h0 + u && d2.y < rc2) ? y.y : 0.f;
+          y.x = (own[2 * k] > hu && d2.x < rc2) ? y.x : 0.f;
+          y.y = (own[2 * k + 1] > hu && d2.y < rc2) ? y.y : 0.f;
         }
         float2 fsn = __fmul2_rn(__ffma2_rn(y, y, f2(-irc2)), y);
         fsn.x = fmaxf(fsn.x, 0.f);
@@ -1659,10 +1698,22 @@ __device__ __forceinline__ void half_chunk(HalfSmem& S, const SeqInfo& sq, int b
       v[3 * u + 1] = gy.x + gy.y;
       v[3 * u + 2] = gz.x + gz.y;
     }
-    v[12] = v[13] = v[14] = v[15] = 0.f;
-    warp_reduce_multi<16>(v);  // lane l: value l >> 1
-    const int k = lane >> 1;
-    if ((lane & 1) == 0 && k < 12 && h0 + k / 3 < nh) atomicAdd(&S.hg[h0 + k / 3][k % 3], v[0]);
+    // over lane bit 4 (values 6.. are the partner's first six), bit 3, then
+    // the eight lanes of the group
+#pragma unroll
+    for (int i = 0; i < 6; ++i) v[i] += __shfl_xor_sync(0xffffffffu, v[6 + i], 16);
+#pragma unroll
+    for (int i = 0; i < 3; ++i) v[i] += __shfl_xor_sync(0xffffffffu, v[3 + i], 8);
+#pragma unroll
+    for (int o = 4; o; o >>= 1)
+#pragma unroll
+      for (int i = 0; i < 3; ++i) v[i] += __shfl_xor_sync(0xffffffffu, v[i], o);
+    const int k = lane & 7;
+    if (k < 3 && h0 + lx < nh) {
+      const float f = k == 0 ? v[0] : (k == 1 ? v[1] : v[2]);
+      if (SEQ == kSeqPlain) atomicAdd(&hg[h0 + lx][k], f);
+      else hg[h0 + lx][k] += f;
+    }
   }
 }
 
@@ -1670,26 +1721,29 @@ __device__ __forceinline__ void half_chunk(HalfSmem& S, const SeqInfo& sq, int b
 // atomic) and, for an entry across the boundary, the symmetric part of
 // (T.H) (x) f to the lane's virial sums.
 template <int SEQ = kSeqPlain>
-__device__ __forceinline__ void half_flush(const HoodArgs& H, const HalfSmem& S, const SeqInfo& q, int j, float fx,
-                                           float fy, float fz, float* wv) {
+__device__ __forceinline__ void half_flush(float4* hforce, const float* hrow, const HalfSmem& S, const SeqInfo& q,
+                                           int j, float fx, float fy, float fz, float* wv) {
   if (j >= q.nf + q.nb + q.nh || (fx == 0.f && fy == 0.f && fz == 0.f)) return;
   bool back;
   int idx;
   if (SEQ == kSeqList) {
-    idx = S.ilist[j];
+    idx = q.list[j];
     back = idx >= q.wf;
+  } else if (SEQ == kSeqOwn) {
+    idx = j + q.obase;
+    back = false;
   } else {
     back = j >= q.nf && j < q.nf + q.nb;
     idx = j < q.nf ? j : (back ? kHCap - q.nb + (j - q.nf) : -1);
   }
   const int p = __float_as_int(idx >= 0 ? S.ent[idx].w : S.own[j - q.nf - q.nb].w);
-  atomicAdd(&H.hforce[p], make_float4(fx, fy, fz, 0.f));
+  atomicAdd(&hforce[p], make_float4(fx, fy, fz, 0.f));
   if (back) {
     const int im = S.img[idx];
     const float tx = (float)((im << 27) >> 27), ty = (float)((im << 22) >> 27), tz = (float)((im << 17) >> 27);
     float t[3];
 #pragma unroll
-    for (int a = 0; a < 3; ++a) t[a] = tx * H.hrow[a] + ty * H.hrow[3 + a] + tz * H.hrow[6 + a];
+    for (int a = 0; a < 3; ++a) t[a] = tx * hrow[a] + ty * hrow[3 + a] + tz * hrow[6 + a];
     const float f[3] = {fx, fy, fz};
     wv[0] += t[0] * f[0];
     wv[1] += 0.5f * (t[0] * f[1] + t[1] * f[0]);
@@ -1814,248 +1868,397 @@ __device__ void half_stage_window(const SweepArgs& A, HalfSmem& S, int w0, int w
   }
 }
 
-// One batch of at most kHome home particles (sorted positions hp ..) against
-// the staged sequence sq: the chunks of the sequence from a counter, the
-// entries' forces flushed per chunk, the home particles' forces at the end.
-// SEQ: the kind of sequence (own pass: every entry an own-cell particle,
-// masked by index).
-template <int SEQ, int MODE>
-__device__ void half_batch(const SweepArgs& A, const HoodArgs& H, HalfSmem& S, const SeqInfo& sq, int hp, int nbh,
-                           float2& e, float* wv, unsigned& cnt, const ScalarRed& R) {
-  constexpr bool SCALAR = MODE == 2 || MODE >= 4;
-  const int tid = threadIdx.x, lane = tid & 31;
-  for (int t = tid; t < kHome + 4; t += kThreads) {
-    if (t < nbh) {
-      const float4 hq = A.xs[hp + t];
-      S.home[t] = make_float4(-hq.x, -hq.y, -hq.z, __int_as_float(hp + t));
-    } else {
-      S.home[t] = make_float4(kFar, -kFar, kFar, __int_as_float(0));
-    }
-  }
-  if (tid == 0) S.next = 0;
-  __syncthreads();
-  const int nch = (sq.nf + sq.nb + kChunk - 1) / kChunk;
-  for (;;) {
-    int c = 0;
-    if (lane == 0) c = atomicAdd(&S.next, 1);
-    c = __shfl_sync(0xffffffffu, c, 0);
-    if (c >= nch) break;
-    float2 jx[kEnt / 2], jy[kEnt / 2], jz[kEnt / 2];
-    const int base = c * kChunk;
-    constexpr bool MASK = SEQ == kSeqOwn;
-    if (sq.nf + sq.nb - base > 64)
-      half_chunk<MASK, SEQ, MODE, 2>(S, sq, base, nbh, A.rc2, A.irc, A.irc2, jx, jy, jz, e, cnt, R);
-    else
-      half_chunk<MASK, SEQ, MODE, 1>(S, sq, base, nbh, A.rc2, A.irc, A.irc2, jx, jy, jz, e, cnt, R);
-    if (!SCALAR) {
+// A lane's running sums over batches, in registers within one.
+struct UnitAcc {
+  float2 e;
+  float wv[6];
+  unsigned cnt;
+  unsigned long long cand;
+};
+
+// A batch (home particles [hp, hp + nbh) of the sorted arrays, at most kBatch)
+// and the entries it is swept against: positions [i0, i1) but [skip0, skip1),
+// position t at S.ent[t] (t < split) or S.ent[t + bshift]; mn of its own
+// particles at S.ent[m0 ..], home index moff on, masked by index. img0: the
+// entries from here on have an image in S.img.
+struct Unit {
+  int hp, nbh;
+  int m0, mn, moff;
+  int i0, i1, skip0, skip1, split, bshift, img0;
+};
+
+// A warp's chunk of at most kChunk listed entries against its batch: the pair
+// terms, then the entries' forces.
+template <int MODE, int SEQ>
+__device__ __forceinline__ void unit_chunk(const HalfSmem& S, const float4* home, float (*hg)[3], const SeqInfo& sq,
+                                           int nbh, UnitAcc& a, const ScalarRed& R) {
+  constexpr bool SCALAR = MODE == 2 || MODE >= 4, MASK = SEQ == kSeqOwn;
+  const HalfCtx& X = S.ctx;
+  const int lane = threadIdx.x & 31;
+  float2 jx[kEnt / 2], jy[kEnt / 2], jz[kEnt / 2];
+  if (!MASK && sq.nf > 64)
+    half_chunk<MASK, SEQ, MODE, 2>(S, home, hg, sq, 0, nbh, X.rc2, X.irc, X.irc2, jx, jy, jz, a.e, a.cnt, R);
+  else
+    half_chunk<MASK, SEQ, MODE, 1>(S, home, hg, sq, 0, nbh, X.rc2, X.irc, X.irc2, jx, jy, jz, a.e, a.cnt, R);
+  if (!SCALAR) {
 #pragma unroll
-      for (int k = 0; k < kEnt / 2; ++k) {
-        const int j0 = base + lane + 64 * k;
-        half_flush<SEQ>(H, S, sq, j0, jx[k].x, jy[k].x, jz[k].x, wv);
-        half_flush<SEQ>(H, S, sq, j0 + 32, jx[k].y, jy[k].y, jz[k].y, wv);
-      }
+    for (int k = 0; k < kEnt / 2; ++k) {
+      half_flush<SEQ>(X.hforce, X.hrow, S, sq, lane + 64 * k, jx[k].x, jy[k].x, jz[k].x, a.wv);
+      half_flush<SEQ>(X.hforce, X.hrow, S, sq, lane + 64 * k + 32, jx[k].y, jy[k].y, jz[k].y, a.wv);
     }
   }
-  __syncthreads();
-  if (!SCALAR && tid < nbh) {
-    const float gx = S.hg[tid][0], gy = S.hg[tid][1], gz = S.hg[tid][2];
-    if (gx != 0.f || gy != 0.f || gz != 0.f) atomicAdd(&H.hforce[hp + tid], make_float4(-gx, -gy, -gz, 0.f));
-    S.hg[tid][0] = S.hg[tid][1] = S.hg[tid][2] = 0.f;
-  }
-  __syncthreads();
 }
 
-// Ball of a batch of home particles (sorted positions hp .. hp + nbh): the
-// middle of their bounding box (home frame) and the squared staging radius
-// (rc + their largest distance from it + the rounding margin)^2.
-__device__ void batch_ball(const SweepArgs& A, const HoodArgs& H, HalfSmem& S, int hp, int nbh, float& bx,
-                           float& by, float& bz, float& top2) {
-  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+// One batch by one warp. Its ball (the middle of its particles' bounding box,
+// radius rc + their largest distance from it) holds its candidates: the warp
+// runs over the entries, lists those within the ball and sweeps the list
+// whenever it holds a chunk, so no barrier falls inside. Not inlined: with a
+// copy of the pair code at each call the kernel overflowed the instruction
+// cache (5.6 of 13 stalls per issue, twice the time).
+template <int MODE>
+__device__ __noinline__ void half_unit(HalfSmem& S, const Unit u, UnitAcc& acc, const ScalarRed& Rin) {
+  constexpr bool SCALAR = MODE == 2 || MODE >= 4;
+  const HalfCtx& X = S.ctx;
+  const ScalarRed R = Rin;
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const unsigned lt = (1u << lane) - 1u;
+  float4* const home = S.home + warp * (kBatch + 4);
+  float (*const hg)[3] = S.hg + warp * kBatch;
+  unsigned short* const list = S.wlist[warp];
+  UnitAcc a = acc;
+  const int nbh = u.nbh;
   float4 q = make_float4(0.f, 0.f, 0.f, 0.f);
   float v[6] = {kFar, kFar, kFar, kFar, kFar, kFar};  // min x, y, z and minus max x, y, z
-  if (tid < nbh) {
-    q = A.xs[hp + tid];
+  if (lane < nbh) {
+    q = X.xs[u.hp + lane];
     v[0] = q.x;
     v[1] = q.y;
     v[2] = q.z;
     v[3] = -q.x;
     v[4] = -q.y;
     v[5] = -q.z;
+    home[lane] = make_float4(-q.x, -q.y, -q.z, 0.f);
+  } else {
+    home[lane] = make_float4(kFar, -kFar, kFar, 0.f);
   }
 #pragma unroll
   for (int o = 16; o; o >>= 1)
 #pragma unroll
     for (int k = 0; k < 6; ++k) v[k] = fminf(v[k], __shfl_xor_sync(0xffffffffu, v[k], o));
-  if (lane < 6) S.bmin[warp][lane] = v[lane];
-  __syncthreads();
-  float m[6];
-#pragma unroll
-  for (int k = 0; k < 6; ++k) {
-    m[k] = S.bmin[0][k];
-#pragma unroll
-    for (int w = 1; w < kWarps; ++w) m[k] = fminf(m[k], S.bmin[w][k]);
-  }
-  bx = 0.5f * (m[0] - m[3]);
-  by = 0.5f * (m[1] - m[4]);
-  bz = 0.5f * (m[2] - m[5]);
+  const float bx = 0.5f * (v[0] - v[3]), by = 0.5f * (v[1] - v[4]), bz = 0.5f * (v[2] - v[5]);
   float d = 0.f;
-  if (tid < nbh) {
+  if (lane < nbh) {
     const float ex = q.x - bx, ey = q.y - by, ez = q.z - bz;
     d = sqrtf(fmaf(ex, ex, fmaf(ey, ey, ez * ez)));
   }
 #pragma unroll
   for (int o = 16; o; o >>= 1) d = fmaxf(d, __shfl_xor_sync(0xffffffffu, d, o));
-  __syncthreads();  // every warp has read S.bmin
-  if (lane == 0) S.wmax[warp] = d;
-  __syncthreads();
-  float dm = S.wmax[0];
-#pragma unroll
-  for (int w = 1; w < kWarps; ++w) dm = fmaxf(dm, S.wmax[w]);
-  const float top = H.rc + dm + H.eps;
-  top2 = top * top;
+  const float top = X.rc + d + X.eps, top2 = top * top;
+  __syncwarp();
+  SeqInfo sq;
+  sq.nb = sq.nh = 0;
+  sq.wf = u.img0;
+  sq.list = list;
+  sq.nf = u.mn;
+  sq.obase = u.m0;
+  sq.oown = u.moff;
+  if (u.mn > 0) {
+    unit_chunk<MODE, kSeqOwn>(S, home, hg, sq, nbh, a, R);
+    for (int m = 0; m < u.mn; ++m) a.cand += (unsigned long long)min(u.moff + m, nbh);
+  }
+  int n = 0;
+  for (int i = u.i0;;) {
+    for (; i < u.i1 && n < kChunk; i += 32) {
+      const int t = i + lane;
+      const int idx = t < u.split ? t : t + u.bshift;
+      bool keep = false;
+      if (t < u.i1 && (t < u.skip0 || t >= u.skip1)) {
+        const float4 p = S.ent[idx];
+        const float ex = p.x - bx, ey = p.y - by, ez = p.z - bz;
+        keep = fmaf(ex, ex, fmaf(ey, ey, ez * ez)) < top2;
+      }
+      const unsigned m = __ballot_sync(0xffffffffu, keep);
+      if (keep) list[n + __popc(m & lt)] = (unsigned short)idx;
+      n += __popc(m);
+    }
+    if (n == 0) break;
+    __syncwarp();
+    sq.nf = min(n, kChunk);
+    unit_chunk<MODE, kSeqList>(S, home, hg, sq, nbh, a, R);
+    a.cand += (unsigned long long)(nbh * sq.nf);
+    n -= sq.nf;
+    const unsigned short rest = list[kChunk + lane];
+    __syncwarp();
+    if (lane < n) list[lane] = rest;
+    __syncwarp();
+  }
+  if (!SCALAR) {  // kBatch = 32: a lane per home particle
+    const float gx = hg[lane][0], gy = hg[lane][1], gz = hg[lane][2];
+    if (lane < nbh && (gx != 0.f || gy != 0.f || gz != 0.f))
+      atomicAdd(&X.hforce[u.hp + lane], make_float4(-gx, -gy, -gz, 0.f));
+    hg[lane][0] = hg[lane][1] = hg[lane][2] = 0.f;
+  }
+  __syncwarp();
+  acc = a;
 }
 
-// A cell that does not fit the buffers: its half neighbourhood in windows,
-// each against the home particles in batches, then the pairs within the cell
-// (batch b against the particles from its first on). The batches of the
-// neighbourhood pass are the cell's particles in ranges of at most kHome,
-// split at the octant boundaries of their order (cells of kOctMin..kOctCap
-// particles are ordered by octant by the build), each with its own ball
-// (batch_ball), so the particles of a dense cell see about half the
-// candidates of the cell's ball. Returns the candidates.
+// The batches of a windowed cell against the staged window, a warp at a time
+// from a counter. A batch is at most kBatch of the cell's particles,
+// consecutive in its octant order (k_octsort), so it lies in part of one
+// octant. A cell of few batches splits the window's entries between units as
+// well. own: the window holds the cell's own particles [o0, o0 + ne) instead,
+// and a batch takes those after its own (its own ones masked by index).
 template <int MODE>
-__device__ __forceinline__ unsigned long long half_windowed(const SweepArgs& A, const HoodArgs& H, HalfSmem& S,
-                                                            int hs, int nh, int cx, int cy, int cz, float2& e,
-                                                            float* wv, unsigned& cnt, const ScalarRed& R) {
+__device__ __forceinline__ void half_units(HalfSmem& S, bool own, int hs, int wf, int wb, int o0, int ne,
+                                           const ScalarRed& R, UnitAcc& acc) {
+  const int lane = threadIdx.x & 31;
+  const int nbatch = S.nbatch;
+  const int nseg = nbatch < 2 * kWarps ? (2 * kWarps + nbatch - 1) / nbatch : 1;
+  const int seglen = ((ne + nseg - 1) / nseg + 31) & ~31;
+  for (;;) {
+    int k = 0;
+    if (lane == 0) k = atomicAdd(&S.next, 1);
+    k = __shfl_sync(0xffffffffu, k, 0);
+    if (k >= nbatch * nseg) break;
+    int bi = k / nseg;
+    Unit u;
+    u.i0 = (k - bi * nseg) * seglen;
+    u.i1 = min(ne, u.i0 + seglen);
+    int b0 = 0, b1 = 0;  // the batch's particles within the cell
+    for (int g = 0; g < 8; ++g) {
+      const int g0 = S.oct[g], len = S.oct[g + 1] - g0, ns = (len + kBatch - 1) / kBatch;
+      if (bi < ns) {
+        const int size = ((len + ns - 1) / ns + 3) & ~3;  // even parts, whole steps of four
+        b0 = g0 + bi * size;
+        b1 = min(g0 + len, b0 + size);
+        break;
+      }
+      bi -= ns;
+    }
+    if (b1 <= b0 || (own && o0 + u.i1 <= b0)) continue;
+    u.hp = hs + b0;
+    u.nbh = b1 - b0;
+    u.m0 = u.mn = u.moff = u.skip0 = u.skip1 = 0;
+    u.split = own ? kHCap : wf;
+    u.bshift = kHCap - wb - wf;
+    u.img0 = own ? kHCap : wf;
+    if (own) {  // the batch's own particles in this part of the window, then those after them
+      const int m0 = max(b0, o0 + u.i0), m1 = min(b1, o0 + u.i1);
+      u.m0 = m0 - o0;
+      u.mn = m1 - m0;
+      u.moff = m0 - b0;
+      u.i0 = max(u.i0, b1 - o0);
+    }
+    half_unit<MODE>(S, u, acc, R);
+  }
+}
+
+// A cell of at most kSmallCap particles with its half neighbourhood, by one
+// warp: the rows' segments laid end to end, shifted, tested against the cell's
+// ball and compacted into the warp's share of the buffer (every entry with
+// its image), the cell's own particles after them; then its batches. A CTA
+// per such cell spent its time at the barriers: the light cells of a 16M
+// clustered set took 11 us each.
+template <int MODE>
+__device__ __forceinline__ void half_small(const SweepArgs& A, const HoodArgs& H, HalfSmem& S, int h,
+                                           const ScalarRed& R, UnitAcc& acc) {
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const unsigned lt = (1u << lane) - 1u;
+  const int eb = warp * kSmallCap;
+  int4* const seg = S.seg + warp * kSmallSegs;
+  const int hs = A.cell_start[h], nh = A.cell_start[h + 1] - hs;
+  const int cx = h % A.nx, cy = (h / A.nx) % A.ny, cz = h / (A.nx * A.ny);
+  // lane 2r, 2r + 1: the row's segments (at most two, and at most 16 rows)
+  int len = 0;
+  int4 sg = make_int4(0, 0, 0, 0);
+  if ((lane >> 1) < S.nrows) {
+    int img = 0;
+    const RowSeg g = half_segment<0>(A, S, lane >> 1, lane & 1, cx, cy, cz, img);
+    if (g.valid) len = g.p1 - g.p0;
+    sg = make_int4(g.p0, 0, g.ebase, g.back ? img : 0);
+  }
+  float d = 0.f;
+  for (int t = lane; t < nh; t += 32) {
+    const float4 q = A.xs[hs + t];
+    d = fmaxf(d, fminf(sqrtf(fmaf(q.x, q.x, fmaf(q.y, q.y, q.z * q.z))), H.hd));
+  }
+  int inc = len;
+#pragma unroll
+  for (int o = 1; o < 32; o <<= 1) {
+    const int t = __shfl_up_sync(0xffffffffu, inc, o);
+    inc += lane >= o ? t : 0;
+  }
+  const int total = __shfl_sync(0xffffffffu, inc, 31);
+  const unsigned live = __ballot_sync(0xffffffffu, len > 0);
+  const int nseg = __popc(live);
+  __syncwarp();
+  sg.y = inc - len;
+  if (len > 0) seg[__popc(live & lt)] = sg;
+#pragma unroll
+  for (int o = 16; o; o >>= 1) d = fmaxf(d, __shfl_xor_sync(0xffffffffu, d, o));
+  __syncwarp();
+  const float top = H.rc + d + H.eps, top2 = top * top;
+  int n = 0;
+  for (int t0 = 0; t0 < total; t0 += 64) {
+    float4 v[2];
+    unsigned c[2];
+    int im[2], sb[2];
+#pragma unroll
+    for (int k = 0; k < 2; ++k) {
+      const int t = min(t0 + 32 * k + lane, total - 1);
+      int lo = 0, hi = nseg;  // the last segment starting at or before t
+      while (hi - lo > 1) {
+        const int mid = (lo + hi) >> 1;
+        if (seg[mid].y <= t) lo = mid;
+        else hi = mid;
+      }
+      const int4 g = seg[lo];
+      const int p = g.x + (t - g.y);
+      v[k] = A.xs[p];
+      v[k].w = __int_as_float(p);
+      c[k] = A.cellc[p];
+      sb[k] = g.z;
+      im[k] = g.w;
+    }
+#pragma unroll
+    for (int k = 0; k < 2; ++k) {
+      const float4 sh = S.otab[sb[k] + (int)(c[k] & 1023u)];
+      v[k].x += sh.x;
+      v[k].y += sh.y;
+      v[k].z += sh.z;
+      const bool keep = t0 + 32 * k + lane < total &&
+                        fmaf(v[k].x, v[k].x, fmaf(v[k].y, v[k].y, v[k].z * v[k].z)) < top2;
+      const unsigned m = __ballot_sync(0xffffffffu, keep);
+      if (keep) {
+        const int e = eb + n + __popc(m & lt);
+        S.ent[e] = v[k];
+        S.img[e] = (unsigned short)im[k];
+      }
+      n += __popc(m);
+    }
+  }
+  for (int t = lane; t < nh; t += 32) {
+    const float4 q = A.xs[hs + t];
+    S.ent[eb + n + t] = make_float4(q.x, q.y, q.z, __int_as_float(hs + t));
+    S.img[eb + n + t] = 0;
+  }
+  __syncwarp();
+  const int nb = (nh + kBatch - 1) / kBatch;
+  const int size = ((nh + nb - 1) / nb + 3) & ~3;
+  for (int b0 = 0; b0 < nh; b0 += size) {
+    Unit u;
+    u.hp = hs + b0;
+    u.nbh = min(size, nh - b0);
+    u.m0 = eb + n + b0;
+    u.mn = u.nbh;
+    u.moff = 0;
+    u.i0 = eb;
+    u.i1 = eb + n + nh;
+    u.skip0 = eb + n;  // the cell's particles up to the batch's own
+    u.skip1 = eb + n + b0 + u.nbh;
+    u.split = kHCap;
+    u.bshift = 0;
+    u.img0 = 0;  // every entry's image is in S.img
+    half_unit<MODE>(S, u, acc, R);
+  }
+}
+
+// A cell that does not fit the buffers: its half neighbourhood in windows of
+// kHCap particles, each swept by its batches (half_units), then the pairs
+// within the cell the same way.
+template <int MODE>
+__device__ __forceinline__ void half_windowed(const SweepArgs& A, const HoodArgs& H, HalfSmem& S, int hs, int nh,
+                                              int cx, int cy, int cz, const ScalarRed& R, UnitAcc& acc) {
   const int tid = threadIdx.x;
+  __syncthreads();
   if (threadIdx.x < 32) half_segments(A, S, cx, cy, cz);
   // octant ranges of the cell's order: S.oct[g] .. S.oct[g + 1]
   const bool octs = nh >= kOctMin && nh <= kOctCap;
   if (tid < 9) S.oct[tid] = 0;
   __syncthreads();
-  if (octs)
-    for (int t = tid; t < nh; t += kThreads) {
-      const float4 q = A.xs[hs + t];
-      atomicAdd(&S.oct[1 + ((q.x > 0.f ? 1 : 0) | (q.y > 0.f ? 2 : 0) | (q.z > 0.f ? 4 : 0))], 1);
-    }
+  // and the largest distance of the cell's particles from its centre, for
+  // the windows' staging ball
+  float d = 0.f;
+  for (int t = tid; t < nh; t += kThreads) {
+    const float4 q = A.xs[hs + t];
+    if (octs) atomicAdd(&S.oct[1 + ((q.x > 0.f ? 1 : 0) | (q.y > 0.f ? 2 : 0) | (q.z > 0.f ? 4 : 0))], 1);
+    d = fmaxf(d, fminf(sqrtf(fmaf(q.x, q.x, fmaf(q.y, q.y, q.z * q.z))), H.hd));
+  }
+#pragma unroll
+  for (int o = 16; o; o >>= 1) d = fmaxf(d, __shfl_xor_sync(0xffffffffu, d, o));
+  if ((tid & 31) == 0) S.wmax[tid >> 5] = d;
   __syncthreads();
   if (tid == 0) {
-    if (octs)
-      for (int g = 0; g < 8; ++g) S.oct[g + 1] += S.oct[g];
-    else
-      for (int g = 1; g < 9; ++g) S.oct[g] = nh;  // one group
-  }
-  __syncthreads();
-  // the window's staging ball: the cell's particles' largest distance from
-  // the cell centre
-  {
-    float d = 0.f;
-    for (int t = tid; t < nh; t += kThreads) {
-      const float4 q = A.xs[hs + t];
-      d = fmaxf(d, fminf(sqrtf(fmaf(q.x, q.x, fmaf(q.y, q.y, q.z * q.z))), H.hd));
+    int nb = 0;
+    for (int g = 0; g < 8; ++g) {
+      if (octs) S.oct[g + 1] += S.oct[g];
+      else S.oct[g + 1] = nh;  // one group
+      nb += (S.oct[g + 1] - S.oct[g] + kBatch - 1) / kBatch;
     }
-#pragma unroll
-    for (int o = 16; o; o >>= 1) d = fmaxf(d, __shfl_xor_sync(0xffffffffu, d, o));
-    if ((tid & 31) == 0) S.wmax[tid >> 5] = d;
+    S.nbatch = nb;
   }
-  __syncthreads();
   float dcell = S.wmax[0];
 #pragma unroll
   for (int w = 1; w < kWarps; ++w) dcell = fmaxf(dcell, S.wmax[w]);
   const float tcell = H.rc + dcell + H.eps;
   const int C = S.ctot;
-  unsigned long long cand = 0;
-  for (int w0 = 0; w0 < C; w0 += kHCap) {
-    if (tid == 0) {
-      S.nf = 0;
-      S.nb = 0;
-    }
+  // the neighbourhood's windows, then the cell's own
+  for (int w0 = 0; w0 < C + nh;) {
+    const bool own = w0 >= C;
+    const int o0 = own ? w0 - C : 0, no = own ? min(kHCap, nh - o0) : 0;
+    __syncthreads();  // the last window's readers are done
+    if (tid == 0) S.nf = S.nb = S.next = 0;
     __syncthreads();
-    half_stage_window(A, S, w0, min(C, w0 + kHCap), 0.f, 0.f, 0.f, tcell * tcell);
-    __syncthreads();
-    const int wf = min(S.nf, kHCap), wb = min(S.nb, kHCap - wf);
-    for (int g = 0; g < 8; ++g) {
-      const int g0 = S.oct[g], g1 = S.oct[g + 1];
-      for (int b0 = g0; b0 < g1; b0 += kHome) {
-        const int nbh = min(kHome, g1 - b0);
-        float bx, by, bz, top2;
-        batch_ball(A, H, S, hs + b0, nbh, bx, by, bz, top2);  // ends with a barrier
-        // the window's entries within the batch's ball
-        if (tid == 0) S.nl = 0;
-        __syncthreads();
-        for (int i0 = (tid >> 5) * 32; i0 < wf + wb; i0 += kThreads) {
-          const int i = i0 + (tid & 31);
-          const int idx = i < wf ? i : kHCap - wb + (i - wf);
-          bool keep = false;
-          if (i < wf + wb) {
-            const float4 q = S.ent[idx];
-            const float ex = q.x - bx, ey = q.y - by, ez = q.z - bz;
-            keep = fmaf(ex, ex, fmaf(ey, ey, ez * ez)) < top2;
-          }
-          const unsigned m = __ballot_sync(0xffffffffu, keep);
-          int at = 0;
-          if ((tid & 31) == 0 && m) at = atomicAdd(&S.nl, __popc(m));
-          at = __shfl_sync(0xffffffffu, at, 0);
-          if (keep) S.ilist[at + __popc(m & ((1u << (tid & 31)) - 1u))] = (unsigned short)idx;
-        }
-        __syncthreads();
-        SeqInfo sq;
-        sq.nf = S.nl;  // read by every thread before batch_ball's next barriers
-        sq.nb = 0;
-        sq.nh = 0;
-        sq.obase = 0;
-        sq.wf = wf;
-        half_batch<kSeqList, MODE>(A, H, S, sq, hs + b0, nbh, e, wv, cnt, R);
-        cand += (unsigned long long)nbh * (unsigned long long)sq.nf;
-      }
-    }
-  }
-  for (int b0 = 0; b0 < nh; b0 += kHome) {
-    const int nbh = min(kHome, nh - b0);
-    for (int o0 = b0; o0 < nh; o0 += kHCap) {
-      const int no = min(kHCap, nh - o0);
+    if (own) {
       for (int j = tid; j < no; j += kThreads) {
         const float4 q = A.xs[hs + o0 + j];
         S.ent[j] = make_float4(q.x, q.y, q.z, __int_as_float(hs + o0 + j));
       }
-      SeqInfo sq;
-      sq.nf = no;
-      sq.nb = 0;
-      sq.nh = 0;
-      sq.obase = o0 - b0;
-      sq.wf = 0;
-      half_batch<kSeqOwn, MODE>(A, H, S, sq, hs + b0, nbh, e, wv, cnt, R);  // its first barrier also covers the entries
-      cand += (unsigned long long)nbh * (unsigned long long)no -
-              (o0 == b0 ? (unsigned long long)nbh * (unsigned long long)(nbh + 1) / 2 : 0ull);
+    } else {
+      half_stage_window(A, S, w0, min(C, w0 + kHCap), 0.f, 0.f, 0.f, tcell * tcell);
     }
+    __syncthreads();
+    const int wf = min(S.nf, kHCap), wb = min(S.nb, kHCap - wf);
+    half_units<MODE>(S, own, hs, wf, wb, o0, own ? no : wf + wb, R, acc);
+    w0 = own ? w0 + no : min(C, w0 + kHCap);
   }
-  return cand;
 }
 
-// WIN = false: the fast-path cells (list); true: the windowed cells (dense),
-// from a counter of their own.
-template <int MODE, bool WIN>
-__global__ void __launch_bounds__(kThreads, 5) k_hood_half(const __grid_constant__ SweepArgs A,
-                                                           const __grid_constant__ HoodArgs H,
-                                                           double* __restrict__ partials) {
-  constexpr bool ENERGY = MODE != 1 && MODE != 4 && MODE != 6;  // MODE 5 sums 1/r where the energy goes
-  constexpr bool SCALAR = MODE == 2 || MODE >= 4;
-  extern __shared__ __align__(16) unsigned char smraw[];
-  HalfSmem& S = *reinterpret_cast<HalfSmem*>(smraw);
-  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  constexpr int NV = hood_nv(MODE);
-  const int ntot = WIN ? *H.ndense : H.work[6];
-  if (ntot == 0) {  // no cell of this kind
-    if (tid < NV) partials[(size_t)blockIdx.x * NV + tid] = 0.0;
-    return;
-  }
+// A warp's sums since the last call into its FP64 sums: the energy (or sum
+// 1/r) and the boundary terms.
+template <bool ENERGY>
+__device__ __forceinline__ void half_fold(HalfSmem& S, float2& e, float (&wv)[6]) {
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  float v[8] = {wv[0], wv[1], wv[2], wv[3], wv[4], wv[5], ENERGY ? e.x + e.y : 0.f, 0.f};
+  warp_reduce_multi<8>(v);  // lane l: value l >> 2
+  if ((lane & 3) == 0 && (lane >> 2) < 6) S.out[warp][lane >> 2] += -2.0 * (double)v[0];
+  if (ENERGY && lane == 24) S.out[warp][15] += (double)v[0];
+#pragma unroll
+  for (int q = 0; q < 6; ++q) wv[q] = 0.f;
+  e = f2(0.f);
+}
+
+// Shared memory of a half-shell kernel made ready: stencil table, rows,
+// context, sums.
+__device__ __forceinline__ void half_setup_smem(const SweepArgs& A, const HoodArgs& H, HalfSmem& S) {
+  const int tid = threadIdx.x;
   for (int k = tid; k < kWarps * 16; k += kThreads) (&S.out[0][0])[k] = 0.0;
   for (int k = tid; k < A.noff && k < kTab; k += kThreads) {
     const Off& o = A.off[k];
     S.otab[k] = make_float4(o.sx, o.sy, o.sz, __int_as_float(H.opk[1][k]));
   }
   for (int k = tid; k < kHome * 3; k += kThreads) (&S.hg[0][0])[k] = 0.f;
-  if (tid == 0) S.ncand = 0;
+  if (tid == 0) {
+    S.ncand = 0;
+    S.ctx.xs = A.xs;
+    S.ctx.hforce = H.hforce;
+    S.ctx.rc2 = A.rc2;
+    S.ctx.irc = A.irc;
+    S.ctx.irc2 = A.irc2;
+    S.ctx.rc = H.rc;
+    S.ctx.eps = H.eps;
+    for (int k = 0; k < 9; ++k) S.ctx.hrow[k] = H.hrow[k];
+  }
   __syncthreads();
   if (tid == 0) {
     const int ne = A.noff < kTab ? A.noff : kTab;
@@ -2071,44 +2274,72 @@ __global__ void __launch_bounds__(kThreads, 5) k_hood_half(const __grid_constant
     S.rowk[nr] = (unsigned short)(ne > 1 ? ne : 1);
     S.nrows = nr;
   }
-  // scalar modes (energy, count, sum 1/r, histogram): the cutoff, the
-  // histogram's copies after HalfSmem (as in k_hood), the lane's count
-  ScalarRed R;
-  R.rc2 = A.rc2;
-  R.irc = A.irc;
-  R.scale2 = H.hscale * H.hscale;
-  R.xlim = H.hxlim;
-  unsigned* const hist_all = reinterpret_cast<unsigned*>(smraw + sizeof(HalfSmem));
-  R.hist = hist_all + (lane & (H.hcopies - 1)) * H.hstride;
-  if (MODE == 6)
-    for (int b = tid; b < H.hcopies * H.hstride; b += kThreads) hist_all[b] = 0u;
+  __syncthreads();
+}
+
+// The CTA's partials: the FP64 sums of its warps (after a barrier).
+template <int MODE>
+__device__ __forceinline__ void half_partials(const HoodArgs& H, const HalfSmem& S, double* __restrict__ partials) {
+  constexpr bool SCALAR = MODE == 2 || MODE >= 4;
+  constexpr int NV = hood_nv(MODE);
+  const int tid = threadIdx.x;
+  if (tid == 0 && S.ncand) atomicAdd(H.cand, S.ncand);
+  if (tid < NV) {
+    int src;
+    if (SCALAR) src = 15;
+    else if (tid < kVirN3) src = tid;
+    else if (MODE == 0) src = 15;
+    else if (tid < kVirN3 + 9) src = -1;  // X: from k_half_finish
+    else src = 15;
+    double acc = 0.0;
+    if (src >= 0)
+      for (int w = 0; w < kWarps; ++w) acc += S.out[w][src];
+    partials[(size_t)blockIdx.x * NV + tid] = acc;
+  }
+}
+
+// The fast-path cells (list), a CTA per cell: energy, forces, boundary terms
+// (MODE 0, 1, 3). A cell whose kept neighbourhood overflows the buffer
+// (k_hood_list goes by the expected share of the raw one) is moved to the
+// dense list, which k_half_batch takes afterwards.
+template <int MODE>
+__global__ void __launch_bounds__(kThreads, 5) k_hood_half(const __grid_constant__ SweepArgs A,
+                                                           const __grid_constant__ HoodArgs H,
+                                                           double* __restrict__ partials) {
+  constexpr bool ENERGY = MODE != 1;
+  extern __shared__ __align__(16) unsigned char smraw[];
+  HalfSmem& S = *reinterpret_cast<HalfSmem*>(smraw);
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  constexpr int NV = hood_nv(MODE);
+  const int nlist = H.work[6];
+  if (nlist == 0) {  // no such cell
+    if (tid < NV) partials[(size_t)blockIdx.x * NV + tid] = 0.0;
+    return;
+  }
+  half_setup_smem(A, H, S);
+  const ScalarRed R{};  // not used by the force modes
   unsigned cnt = 0;
   float wv[6] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f};  // lane's sum of (T.H) (x) f over its entries across the boundary
   float2 e = f2(0.f);
-  const int* items = WIN ? H.dense : H.list;
-  int* counter = WIN ? H.work + 5 : H.work;
   int next1 = 0;
-  if (tid == 0) next1 = atomicAdd(counter, 1);
+  if (tid == 0) next1 = atomicAdd(H.work, 1);
   for (;;) {
     __syncthreads();
     if (tid == 0) {
-      S.item = next1 < ntot ? items[next1] : -1;
-      if (next1 < ntot) next1 = atomicAdd(counter, 1);
+      S.item = next1 < nlist ? H.list[next1] : -2;
+      S.kind = next1;
+      if (next1 < nlist) next1 = atomicAdd(H.work, 1);
       S.nf = 0;
       S.nb = 0;
       S.next = 0;
     }
     __syncthreads();
     const int h = S.item;
-    if (h < 0) break;
+    if (h == -2) break;
+    if (h < 0) continue;  // moved to the dense list by an earlier launch
     const int hs = A.cell_start[h];
     const int nh = A.cell_start[h + 1] - hs;
     const int cx = h % A.nx, cy = (h / A.nx) % A.ny, cz = h / (A.nx * A.ny);
-    constexpr bool win = WIN;
-    if (WIN) {
-      const unsigned long long cand = half_windowed<MODE>(A, H, S, hs, nh, cx, cy, cz, e, wv, cnt, R);
-      if (tid == 0) S.ncand += cand;
-    } else {
     float d = 0.f;
     for (int t = tid; t < kHome + 4; t += kThreads) {
       if (t < nh) {
@@ -2130,13 +2361,21 @@ __global__ void __launch_bounds__(kThreads, 5) k_hood_half(const __grid_constant
     const float top = H.rc + dmax + H.eps;
     half_stage(A, S, cx, cy, cz, top * top);
     __syncthreads();
-    const int nf = min(S.nf, kHCap), nb = min(S.nb, kHCap - nf);  // k_hood_list guarantees nf + nb <= kHCap
+    const int nf = S.nf, nb = S.nb;
+    if (nf + nb > kHCap) {  // uniform
+      if (tid == 0) {
+        H.dense[atomicAdd(H.ndense, 1)] = h;
+        H.list[S.kind] = -1;
+      }
+      continue;
+    }
     SeqInfo sq;
     sq.nf = nf;
     sq.nb = nb;
     sq.nh = nh;
-    sq.obase = 0;
+    sq.obase = sq.oown = 0;
     sq.wf = 0;
+    sq.list = nullptr;
     const int nseq = nf + nb + nh;
     const int nch = (nseq + kChunk - 1) / kChunk;
     const int cmask = (nf + nb) / kChunk;  // the first chunk holding own-cell positions
@@ -2151,47 +2390,94 @@ __global__ void __launch_bounds__(kThreads, 5) k_hood_half(const __grid_constant
       float2 jx[kEnt / 2], jy[kEnt / 2], jz[kEnt / 2];
       const int base = c * kChunk;
       const bool full = nseq - base > 64;  // else the chunk's second half is padding
-      if (c < cmask) {
-        if (full) half_chunk<false, false, MODE, 2>(S, sq, base, nh, A.rc2, A.irc, A.irc2, jx, jy, jz, e, cnt, R);
-        else half_chunk<false, false, MODE, 1>(S, sq, base, nh, A.rc2, A.irc, A.irc2, jx, jy, jz, e, cnt, R);
-      } else {
-        if (full) half_chunk<true, false, MODE, 2>(S, sq, base, nh, A.rc2, A.irc, A.irc2, jx, jy, jz, e, cnt, R);
-        else half_chunk<true, false, MODE, 1>(S, sq, base, nh, A.rc2, A.irc, A.irc2, jx, jy, jz, e, cnt, R);
-      }
-      if (!SCALAR) {
+      if (c < cmask)
+        half_chunk<false, kSeqPlain, MODE, 2>(S, S.home, S.hg, sq, base, nh, A.rc2, A.irc, A.irc2, jx, jy, jz, e, cnt, R);
+      else if (full)
+        half_chunk<true, kSeqPlain, MODE, 2>(S, S.home, S.hg, sq, base, nh, A.rc2, A.irc, A.irc2, jx, jy, jz, e, cnt, R);
+      else
+        half_chunk<true, kSeqPlain, MODE, 1>(S, S.home, S.hg, sq, base, nh, A.rc2, A.irc, A.irc2, jx, jy, jz, e, cnt, R);
 #pragma unroll
-        for (int k = 0; k < kEnt / 2; ++k) {
-          const int j0 = base + lane + 64 * k;
-          half_flush(H, S, sq, j0, jx[k].x, jy[k].x, jz[k].x, wv);
-          half_flush(H, S, sq, j0 + 32, jx[k].y, jy[k].y, jz[k].y, wv);
-        }
+      for (int k = 0; k < kEnt / 2; ++k) {
+        const int j0 = base + lane + 64 * k;
+        half_flush(H.hforce, H.hrow, S, sq, j0, jx[k].x, jy[k].x, jz[k].x, wv);
+        half_flush(H.hforce, H.hrow, S, sq, j0 + 32, jx[k].y, jy[k].y, jz[k].y, wv);
       }
     }
-    }  // fast path
-    // this cell's energy and boundary terms into the warp's FP64 sums
-    {
-      float v[8] = {wv[0], wv[1], wv[2], wv[3], wv[4], wv[5], ENERGY ? e.x + e.y : 0.f, 0.f};
-      warp_reduce_multi<8>(v);  // lane l: value l >> 2
-      if ((lane & 3) == 0 && (lane >> 2) < 6) S.out[warp][lane >> 2] += -2.0 * (double)v[0];
-      if (ENERGY && lane == 24) S.out[warp][15] += (double)v[0];
-#pragma unroll
-      for (int q = 0; q < 6; ++q) wv[q] = 0.f;
-      e = f2(0.f);
-    }
+    half_fold<ENERGY>(S, e, wv);  // this cell's energy and boundary terms
     __syncthreads();
-    // the home particles' forces: minus their sums of fsn r (the windowed
-    // path has added them per batch)
-    if (!win && !SCALAR && tid < nh) {
+    // the home particles' forces: minus their sums of fsn r
+    if (tid < nh) {
       const float gx = S.hg[tid][0], gy = S.hg[tid][1], gz = S.hg[tid][2];
       if (gx != 0.f || gy != 0.f || gz != 0.f) atomicAdd(&H.hforce[hs + tid], make_float4(-gx, -gy, -gz, 0.f));
       S.hg[tid][0] = S.hg[tid][1] = S.hg[tid][2] = 0.f;
     }
   }
-  // per-CTA partials: -2 (T.H) (x) f sums, energy (each pair-image once)
   __syncthreads();
-  if (tid == 0 && S.ncand) atomicAdd(H.cand, S.ncand);
+  half_partials<MODE>(H, S, partials);
+}
+
+// The cells swept by batches, a batch per warp: the windowed ones (dense), a
+// CTA per cell, then the small ones (the end of list, backwards), a warp per
+// cell, which fill the end of the launch. All modes; the scalar ones (2
+// energy, 4 count, 5 sum 1/r, 6 histogram, its copies after HalfSmem as in
+// k_hood) evaluate the same candidates without forces.
+template <int MODE>
+__global__ void __launch_bounds__(kThreads, 5) k_half_batch(const __grid_constant__ SweepArgs A,
+                                                            const __grid_constant__ HoodArgs H,
+                                                            double* __restrict__ partials) {
+  constexpr bool ENERGY = MODE != 1 && MODE != 4 && MODE != 6;  // MODE 5 sums 1/r where the energy goes
+  extern __shared__ __align__(16) unsigned char smraw[];
+  HalfSmem& S = *reinterpret_cast<HalfSmem*>(smraw);
+  const int tid = threadIdx.x, lane = tid & 31;
+  constexpr int NV = hood_nv(MODE);
+  const int ndense = *H.ndense, nsmall = H.work[8];
+  if (ndense + nsmall == 0) {  // no such cell
+    if (tid < NV) partials[(size_t)blockIdx.x * NV + tid] = 0.0;
+    return;
+  }
+  half_setup_smem(A, H, S);
+  ScalarRed R;
+  R.rc2 = A.rc2;
+  R.irc = A.irc;
+  R.scale2 = H.hscale * H.hscale;
+  R.xlim = H.hxlim;
+  unsigned* const hist_all = reinterpret_cast<unsigned*>(smraw + sizeof(HalfSmem));
+  R.hist = hist_all + (lane & (H.hcopies - 1)) * H.hstride;
+  if (MODE == 6)
+    for (int b = tid; b < H.hcopies * H.hstride; b += kThreads) hist_all[b] = 0u;
+  UnitAcc acc;
+  acc.e = f2(0.f);
+#pragma unroll
+  for (int q = 0; q < 6; ++q) acc.wv[q] = 0.f;
+  acc.cnt = 0;
+  acc.cand = 0;
+  int next1 = ndense;
+  if (tid == 0 && ndense) next1 = atomicAdd(H.work + 5, 1);
+  for (;;) {
+    __syncthreads();
+    if (tid == 0) {
+      S.item = next1 < ndense ? H.dense[next1] : -2;
+      if (next1 < ndense) next1 = atomicAdd(H.work + 5, 1);
+    }
+    __syncthreads();
+    const int h = S.item;
+    if (h < 0) break;
+    const int hs = A.cell_start[h];
+    half_windowed<MODE>(A, H, S, hs, A.cell_start[h + 1] - hs, h % A.nx, (h / A.nx) % A.ny, h / (A.nx * A.ny), R, acc);
+    half_fold<ENERGY>(S, acc.e, acc.wv);
+  }
+  for (;;) {
+    int k = 0;
+    if (lane == 0) k = atomicAdd(H.work + 1, 1);
+    k = __shfl_sync(0xffffffffu, k, 0);
+    if (k >= nsmall) break;
+    half_small<MODE>(A, H, S, H.list[H.ncells - 1 - k], R, acc);
+    half_fold<ENERGY>(S, acc.e, acc.wv);
+  }
+  if (lane == 0 && acc.cand) atomicAdd(&S.ncand, acc.cand);
+  __syncthreads();
   if (MODE == 4) {
-    unsigned long long c = cnt;
+    unsigned long long c = acc.cnt;
 #pragma unroll
     for (int o = 16; o; o >>= 1) c += __shfl_xor_sync(0xffffffffu, c, o);
     if (lane == 0 && c) atomicAdd(H.count, c);
@@ -2202,18 +2488,7 @@ __global__ void __launch_bounds__(kThreads, 5) k_hood_half(const __grid_constant
       for (int q = 0; q < H.hcopies; ++q) c += hist_all[q * H.hstride + b];
       if (c) atomicAdd(&H.hist[b], (unsigned long long)c);
     }
-  if (tid < NV) {
-    int src;
-    if (SCALAR) src = 15;
-    else if (tid < kVirN3) src = tid;
-    else if (MODE == 0) src = 15;
-    else if (tid < kVirN3 + 9) src = -1;  // X: from k_half_finish
-    else src = 15;
-    double acc = 0.0;
-    if (src >= 0)
-      for (int w = 0; w < kWarps; ++w) acc += S.out[w][src];
-    partials[(size_t)blockIdx.x * NV + tid] = acc;
-  }
+  half_partials<MODE>(H, S, partials);
 }
 
 // Per particle i after the half-shell sweep: its force F (from the
@@ -2388,9 +2663,11 @@ size_t half_mode_smem(int mode) {
 
 template <int M>
 cudaError_t half_setup(int bytes, int* per) {
-  cudaError_t e = cudaFuncSetAttribute(k_hood_half<M, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
-  if (e == cudaSuccess) e = cudaFuncSetAttribute(k_hood_half<M, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
-  if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(per, k_hood_half<M, false>, kThreads, bytes);
+  cudaError_t e = cudaFuncSetAttribute(k_half_batch<M>, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
+  if constexpr (M < 2 || M == 3) {
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(k_hood_half<M>, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
+  }
+  if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(per, k_half_batch<M>, kThreads, bytes);
   return e;
 }
 
@@ -2458,6 +2735,8 @@ int grid_for(K kernel, size_t smem) {
   return sms * per;
 }
 
+int list_blocks(int ncells) { return (int)(((long long)ncells * kListLanes + 255) / 256); }
+
 bool hood_half_fits(const SweepArgs& A) { return A.noff <= kTab; }
 
 // Scalar reductions over the half stencil. When the stencil fits the table,
@@ -2492,7 +2771,7 @@ int launch_hood_scalar(const SweepArgs& A, const HoodArgs& Hin, int* work, int k
   H.hcopies = kind == 2 ? hist_copies(nbins) : 1;
   H.hstride = kind == 2 ? hist_stride(nbins) : 0;
   const bool reuse = half && lists_half && *lists_half;  // the half-shell work lists of this cell list are built
-  if (cudaMemsetAsync(work, 0, (reuse ? 6 : 8) * sizeof(int), s) != cudaSuccess) return CL_ERR_CUDA;
+  if (cudaMemsetAsync(work, 0, (reuse ? 6 : kWorkWords) * sizeof(int), s) != cudaSuccess) return CL_ERR_CUDA;
   if (kind == 0 && cudaMemsetAsync(count, 0, sizeof(unsigned long long), s) != cudaSuccess) return CL_ERR_CUDA;
   if (kind == 2 && cudaMemsetAsync(hist, 0, sizeof(unsigned long long) * nbins, s) != cudaSuccess) return CL_ERR_CUDA;
   if (A.n <= 0) {
@@ -2507,10 +2786,10 @@ int launch_hood_scalar(const SweepArgs& A, const HoodArgs& Hin, int* work, int k
   if (hood_grid(mode) <= 0 || (half && half_grid(mode) <= 0)) return CL_ERR_CUDA;  // also raise the smem limits
   int nb = 0, nhb = 0;
   switch (mode) {
-    case 2: nb = grid_for(k_hood<2>, smem); nhb = grid_for(k_hood_half<2, true>, hsmem); break;
-    case 4: nb = grid_for(k_hood<4>, smem); nhb = grid_for(k_hood_half<4, true>, hsmem); break;
-    case 5: nb = grid_for(k_hood<5>, smem); nhb = grid_for(k_hood_half<5, true>, hsmem); break;
-    default: nb = grid_for(k_hood<6>, smem); nhb = grid_for(k_hood_half<6, true>, hsmem); break;
+    case 2: nb = grid_for(k_hood<2>, smem); nhb = grid_for(k_half_batch<2>, hsmem); break;
+    case 4: nb = grid_for(k_hood<4>, smem); nhb = grid_for(k_half_batch<4>, hsmem); break;
+    case 5: nb = grid_for(k_hood<5>, smem); nhb = grid_for(k_half_batch<5>, hsmem); break;
+    default: nb = grid_for(k_hood<6>, smem); nhb = grid_for(k_half_batch<6>, hsmem); break;
   }
   if (nb <= 0 || nhb <= 0) return CL_ERR_CUDA;
   nb = std::min(nb, Hin.ncells);
@@ -2518,29 +2797,29 @@ int launch_hood_scalar(const SweepArgs& A, const HoodArgs& Hin, int* work, int k
   const int nrest = half ? 0 : flagged_blocks(A.n);
   if (scalar && nb + nhb + nrest > partials_cap) return CL_ERR_INVALID_ARG;
   if (!reuse) {
-    k_hood_list<<<(H.ncells + 255) / 256, 256, 0, s>>>(A.cell_start, H.ncells, A.noff, work, H.list, H.flag, H.dense,
+    k_hood_list<<<list_blocks(H.ncells), 256, 0, s>>>(A.cell_start, H.ncells, A.noff, work, H.list, H.flag, H.dense,
                                                        H.ndense, H, half ? A.noff : 0, A.nx, A.ny, A.nz);
-    if (half && launch_octsort(H.dense, H.ndense, A.cell_start, const_cast<float4*>(A.xs), const_cast<int*>(H.slot),
-                               s) != CL_OK)
+    if (half && launch_octsort(H.dense, H.ndense, A.cell_start, A.ex, A.ey, A.ez, const_cast<float4*>(A.xs),
+                               const_cast<int*>(H.slot), s) != CL_OK)
       return CL_ERR_CUDA;
   }
   double* p2 = partials + nb;
   switch (mode) {
     case 2:
       k_hood<2><<<nb, kThreads, smem, s>>>(A, H, nullptr, nullptr, nullptr, nullptr, partials);
-      k_hood_half<2, true><<<nhb, kThreads, hsmem, s>>>(A, H, p2);
+      k_half_batch<2><<<nhb, kThreads, hsmem, s>>>(A, H, p2);
       break;
     case 4:
       k_hood<4><<<nb, kThreads, smem, s>>>(A, H, nullptr, nullptr, nullptr, nullptr, partials);
-      if (half) k_hood_half<4, true><<<nhb, kThreads, hsmem, s>>>(A, H, p2);
+      if (half) k_half_batch<4><<<nhb, kThreads, hsmem, s>>>(A, H, p2);
       break;
     case 5:
       k_hood<5><<<nb, kThreads, smem, s>>>(A, H, nullptr, nullptr, nullptr, nullptr, partials);
-      if (half) k_hood_half<5, true><<<nhb, kThreads, hsmem, s>>>(A, H, p2);
+      if (half) k_half_batch<5><<<nhb, kThreads, hsmem, s>>>(A, H, p2);
       break;
     default:
       k_hood<6><<<nb, kThreads, smem, s>>>(A, H, nullptr, nullptr, nullptr, nullptr, partials);
-      if (half) k_hood_half<6, true><<<nhb, kThreads, hsmem, s>>>(A, H, p2);
+      if (half) k_half_batch<6><<<nhb, kThreads, hsmem, s>>>(A, H, p2);
       break;
   }
   if (cudaGetLastError() != cudaSuccess) return CL_ERR_CUDA;
@@ -2598,6 +2877,24 @@ int fill_hood_args(const Geo& geo, const int* opk_full, int noff_full, const int
       H->gf[k * 3 + a] = (float)H->g[k * 3 + a];
       H->hrow[k * 3 + a] = (float)geo.h[k * 3 + a];
     }
+  // Raw half-neighbourhood size up to which a cell takes the fast path: its
+  // buffer holds kHCap kept entries, those within rc + d_max <= rc + hd of the
+  // centre, at uniform density at most the half ball's share of the half
+  // stencil. At most kCap, the buffer of the home-major scalar sweep.
+  {
+    double cell = std::fabs(geo.h[0] * (geo.h[4] * geo.h[8] - geo.h[5] * geo.h[7]) -
+                            geo.h[1] * (geo.h[3] * geo.h[8] - geo.h[5] * geo.h[6]) +
+                            geo.h[2] * (geo.h[3] * geo.h[7] - geo.h[4] * geo.h[6])) / (double)geo.ncells;
+    const double r = geo.rc + hd, half_ball = 0.5 * (4.18879020478639 * r * r * r - cell);
+    const double share = std::min(1.0, half_ball / (cell * std::max(1, noff_half - 1)));
+    H->rawcap = (int)std::min((double)kCap, kHCap / share);
+    // small cells need each row's segments in two lanes of a warp: at most 16
+    // rows, none longer than the grid (a row then has at most two segments)
+    int longest = 0;
+    for (int k = 0; k < H->nrows_half; ++k)
+      longest = std::max(longest, H->rows_half[k][1] - H->rows_half[k][0] + 1);
+    H->smallcap = H->nrows_half > 0 && H->nrows_half <= kSmallSegs / 2 && longest <= geo.n[0] ? kSmallCap : 0;
+  }
   const double eps = 1e-4 * (geo.rc + hd);
   H->rc = (float)geo.rc;
   H->hd = (float)(hd * (1.0 + 1e-6));
@@ -2626,20 +2923,19 @@ int launch_hood(const SweepArgs& A, const SweepArgs* Ahalf, const HoodArgs& Hin,
   // the half-shell work lists depend on the cell list only: built once per
   // list (lists_half says whether the buffers hold them) and reused
   const bool reuse = half && lists_half && *lists_half;
-  if (cudaMemsetAsync(work, 0, (reuse ? 6 : 8) * sizeof(int), s) != cudaSuccess) return CL_ERR_CUDA;
+  if (cudaMemsetAsync(work, 0, (reuse ? 6 : kWorkWords) * sizeof(int), s) != cudaSuccess) return CL_ERR_CUDA;
   if (!reuse) {
-    k_hood_list<<<(H.ncells + 255) / 256, 256, 0, s>>>(A.cell_start, H.ncells, A.noff, work, H.list, H.flag,
+    k_hood_list<<<list_blocks(H.ncells), 256, 0, s>>>(A.cell_start, H.ncells, A.noff, work, H.list, H.flag,
                                                        H.dense, H.ndense, H, half ? Ahalf->noff : 0, A.nx, A.ny, A.nz);
     // the windowed cells' particles in octant order (half_windowed's batches)
-    if (half && launch_octsort(H.dense, H.ndense, A.cell_start, const_cast<float4*>(A.xs), const_cast<int*>(H.slot),
-                               s) != CL_OK)
+    if (half && launch_octsort(H.dense, H.ndense, A.cell_start, A.ex, A.ey, A.ez, const_cast<float4*>(A.xs),
+                               const_cast<int*>(H.slot), s) != CL_OK)
       return CL_ERR_CUDA;
   }
   if (lists_half) *lists_half = half ? 1 : 0;
   if (half) {
-    // every non-empty cell: fast-path or windowed half-shell sweep, then the
-    // per-particle finish; partials [sweep][finish]
-    // (the windowed kernel's CTAs exit at once when no cell needs it)
+    // every non-empty cell: fast-path sweep or sweep by batches, then the
+    // per-particle finish; partials [fast][batches][finish]
     int nhb = half_grid(mode);
     const int nfin = std::min(nrest, 152 * 8);
     if (nhb <= 0) return CL_ERR_CUDA;
@@ -2650,16 +2946,16 @@ int launch_hood(const SweepArgs& A, const SweepArgs* Ahalf, const HoodArgs& Hin,
     double* pfin = pwin + (size_t)nhb * NV;
     const size_t hsmem = sizeof(HalfSmem);
     if (mode == 0) {
-      k_hood_half<0, false><<<nhb, kThreads, hsmem, s>>>(*Ahalf, H, partials);
-      k_hood_half<0, true><<<nhb, kThreads, hsmem, s>>>(*Ahalf, H, pwin);
+      k_hood_half<0><<<nhb, kThreads, hsmem, s>>>(*Ahalf, H, partials);
+      k_half_batch<0><<<nhb, kThreads, hsmem, s>>>(*Ahalf, H, pwin);
       k_half_finish<0><<<nfin, 256, 0, s>>>(*Ahalf, H, forces, grad, gE, pos, pfin);
     } else if (mode == 1) {
-      k_hood_half<1, false><<<nhb, kThreads, hsmem, s>>>(*Ahalf, H, partials);
-      k_hood_half<1, true><<<nhb, kThreads, hsmem, s>>>(*Ahalf, H, pwin);
+      k_hood_half<1><<<nhb, kThreads, hsmem, s>>>(*Ahalf, H, partials);
+      k_half_batch<1><<<nhb, kThreads, hsmem, s>>>(*Ahalf, H, pwin);
       k_half_finish<1><<<nfin, 256, 0, s>>>(*Ahalf, H, forces, grad, gE, pos, pfin);
     } else {
-      k_hood_half<3, false><<<nhb, kThreads, hsmem, s>>>(*Ahalf, H, partials);
-      k_hood_half<3, true><<<nhb, kThreads, hsmem, s>>>(*Ahalf, H, pwin);
+      k_hood_half<3><<<nhb, kThreads, hsmem, s>>>(*Ahalf, H, partials);
+      k_half_batch<3><<<nhb, kThreads, hsmem, s>>>(*Ahalf, H, pwin);
       k_half_finish<3><<<nfin, 256, 0, s>>>(*Ahalf, H, forces, grad, gE, pos, pfin);
     }
     return finish_reduction(final_mode, 3, hinv, 2 * nhb + nfin, NV, partials, sums, energy, virial, gradbox, gE, s);

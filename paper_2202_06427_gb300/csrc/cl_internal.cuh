@@ -43,11 +43,11 @@ struct DevCache {
 constexpr int kMaxOff = 768;      // stencil entries (9^3 = 729 plus margin)
 constexpr int kMaxAxis = 1023;    // cells per axis (10-bit packing)
 constexpr int kMaxBins = 4096;    // histogram bins (shared-memory histogram)
-// Cells of kOctMin to kOctCap particles are ordered by the octant of their
-// particles' local coordinates (sign of x, y, z) by the 3D half-shell sweep
-// when it builds its work lists, so that it can split their particles into
-// compact groups.
-constexpr int kOctMin = 129;
+// Windowed cells of kOctMin to kOctCap particles are ordered by the octant of
+// their particles' local coordinates (sign of x, y, z), and within it by the
+// octants of that, by the 3D half-shell sweep when it builds its work lists, so
+// that consecutive particles form compact groups.
+constexpr int kOctMin = 65;
 constexpr int kOctCap = 2048;
 
 // One neighbour-cell offset of the stencil.
@@ -150,8 +150,9 @@ int scan_tiles_for(long long ncells);
 int launch_build(const Geo& g, const BuildBufs& b, cudaStream_t s);
 // Orders the particles of the listed cells (ncells_listed of them, read on the
 // device) with kOctMin..kOctCap particles by octant; slots follow.
-int launch_octsort(const int* cells, const int* ncells_listed, const int* cell_start, float4* xs, int* slot,
-                   cudaStream_t s);
+// (hx, hy, hz: half-widths of a cell's bounding box).
+int launch_octsort(const int* cells, const int* ncells_listed, const int* cell_start, float hx, float hy, float hz,
+                   float4* xs, int* slot, cudaStream_t s);
 // Prefix sum of the per-cell counts into cell_start; meta[1], meta[2] (zeroed
 // by the caller): non-empty cells, largest count.
 int launch_scan_cells(const int* counts, long long ncells, int* tile_sum, int* meta, int* cell_start, cudaStream_t s);
@@ -189,6 +190,7 @@ int finish_reduction(int final_mode, int dim, const double* hinv, int nblocks, i
                      cudaStream_t s);
 
 // Neighbourhood sweep of the 3D shifted-force energy (cl_hood.cu).
+constexpr int kWorkWords = 16;
 struct HoodArgs {
   int opk[2][kMaxOff];  // unwrapped stencil offsets (see build_stencil): [0] full, [1] half stencil
   // rows of the half stencil (entries 1..: runs of consecutive ox with one
@@ -200,9 +202,12 @@ struct HoodArgs {
   float rc;
   float hd;           // largest distance of a cell point from the cell centre
   float eps;          // rounding margin of the staging radius
+  int rawcap;         // particles in the half neighbourhood up to which a cell takes the fast path
+  int smallcap;       // particles of a cell and its half neighbourhood up to which one warp takes it
   int ncells;
-  int* work;          // [0] work counter, [2..3] candidates, [5] the dense cells' work counter (zeroed
-                      // by the launcher); [6] list length, [7] dense cells (written by k_hood_list)
+  int* work;          // [0], [1], [5] work counters of the listed, small and dense cells, [2..3] candidates
+                      // (zeroed by the launcher); [6] list length, [7] dense cells, [8] small cells (at the end
+                      // of list, backwards; written by k_hood_list)
   int* list;          // cells the neighbourhood sweep takes (ncells capacity)
   unsigned long long* cand;  // candidate pairs evaluated (work[2..3] of the same buffer), zeroed by the launcher
   unsigned char* flag;       // per cell: 1 per-particle companion sweep, 2 dense-cell sweep
