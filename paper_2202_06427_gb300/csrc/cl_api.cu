@@ -304,6 +304,18 @@ int map_pairlist(cl_list* c, cl_result* r, cudaStream_t s) {
 
 }  // namespace
 
+namespace clk {
+void list_parts(const cl_list* cl, ListParts* p) {
+  cl_list* c = const_cast<cl_list*>(cl);
+  p->half = c->half;
+  p->full = c->full;
+  p->partials = c->partials;
+  p->sums = c->sums;
+  p->hforce = c->hforce;
+  p->rc = c->geo.rc;
+}
+}  // namespace clk
+
 extern "C" {
 
 int cl_pairlist_fits(long long npairs, long long capacity) {

@@ -295,6 +295,19 @@ long long topk_parts(long long nb, int k);
 int launch_topk_merge(const int* la, const float* ld, long long nb, int k, float* part_d, long long* part_id, int* oa,
                       int* ob, float* od, int* found, cudaStream_t s);
 
+// Mapped functions over the list (cl_pairfns.cu). The list's internals, from
+// cl_api.cu: hforce is free scratch of n float4 between sweeps, zero before
+// and after every call that uses it.
+struct ListParts {
+  const SweepArgs* half;
+  const SweepArgs* full;
+  double* partials;
+  double* sums;
+  float4* hforce;  // null in 2D
+  double rc;
+};
+void list_parts(const cl_list* cl, ListParts* p);
+
 // Neighbour list (cl_pairs.cu). count[n] (int: one particle's pairs), start[n+1]
 // (64-bit scan of count: the list may pass 2^31 pairs), tiles, meta:
 // workspace; outputs pair_i/j/d of capacity entries.

@@ -1,0 +1,73 @@
+"""The half-shell sweep's kinds of cells side by side: light cells (one warp),
+fast-path cells, cells whose kept neighbourhood overflows the fast path, cells
+of a batch's edge sizes (31-33, 64-65 particles), of more than 128 and of more
+than 2,048. Every reduction against the oracle, and again on the same list,
+whose work lists are kept (rules of parity_util)."""
+import numpy as np
+import pytest
+import torch
+
+import oracle
+from parity_util import BAND, TOL_GB, TOL_W, check_count, check_energy, check_forces, check_hist, check_matrix
+
+pytestmark = pytest.mark.gpu
+
+
+def _ball(rng, centre, radius, spacing, jitter):
+    k = int(np.ceil(radius / spacing))
+    g = np.stack(np.meshgrid(*[np.arange(-k, k + 1) * spacing] * 3, indexing="ij"), -1).reshape(-1, 3)
+    g = g[np.linalg.norm(g, axis=1) <= radius]
+    return centre + g + rng.uniform(-jitter, jitter, size=g.shape)
+
+
+def _background(rng, h, spacing, centre, clear):
+    n = max(1, int(np.abs(np.diag(h)).min() / spacing))
+    s = np.stack(np.meshgrid(*[(np.arange(n) + 0.5) / n] * 3, indexing="ij"), -1).reshape(-1, 3)
+    x = s @ h + rng.uniform(-0.2, 0.2, size=s.shape) * spacing
+    d = x - centre
+    d -= np.round(d @ np.linalg.inv(h)) @ h
+    return x[np.linalg.norm(d, axis=1) > clear]
+
+
+CASES = {
+    # light cells only: about three particles a cell, 40 in the half neighbourhood
+    "light": dict(L=24.0, tric=True, rc=3.0, lcell=1, spacing=2.1, radius=0.0, fine=1.0),
+    # a dense ball among light cells: neighbourhoods from a few to thousands, some
+    # past the fast path's buffer although their raw count is below its limit
+    "overflow": dict(L=24.0, tric=False, rc=3.0, lcell=2, spacing=1.6, radius=4.2, fine=0.42),
+    # cells of about 32 and 64 particles, windowed by their dense neighbours
+    "batches": dict(L=20.0, tric=True, rc=4.0, lcell=1, spacing=1.05, radius=4.5, fine=0.5),
+    # a cell of more than 2,048 particles
+    "huge": dict(L=16.0, tric=False, rc=4.0, lcell=1, spacing=1.5, radius=2.2, fine=0.26),
+}
+
+
+@pytest.mark.parametrize("name", sorted(CASES))
+def test_kinds_of_cells(cuda_ok, name):
+    import paper_2202_06427_gb300 as P
+    c = CASES[name]
+    rng = np.random.default_rng(len(name) + 31)
+    h = np.eye(3) * c["L"]
+    if c["tric"]:
+        h[1, 0], h[2, 0], h[2, 1] = 3.1, -2.2, 1.7
+    centre = np.array([0.375, 0.375, 0.375]) @ h  # the middle of a cell where the grid is four cells wide
+    x = _background(rng, h, c["spacing"], centre, c["radius"] + 0.6 if c["radius"] else -1.0)
+    if c["radius"]:
+        x = np.vstack([x, _ball(rng, centre, c["radius"], c["fine"], 0.15 * c["fine"])])
+    x = np.ascontiguousarray(x[rng.permutation(x.shape[0])])
+    ref = oracle.pair_map(x, h, c["rc"], band=BAND, nbins=17)
+    cl = P.cl_build(torch.from_numpy(x).cuda(), h, c["rc"], c["lcell"])
+    g = torch.tensor([0.75], dtype=torch.float64, device="cuda")
+    for _ in range(2):
+        efv = P.cl_map(cl, "energy_forces_virial")
+        check_energy(efv["energy"].item(), ref["energy"])
+        check_forces(efv["forces"].cpu().numpy(), ref["forces"])
+        check_matrix(efv["virial"].cpu().numpy(), ref["virial"], TOL_W)
+        check_energy(P.cl_map(cl, "energy")["energy"].item(), ref["energy"])
+        check_count(int(P.cl_map(cl, "count")["count"].item()), ref)
+        check_hist(P.cl_map(cl, "hist", nbins=17)["hist"].cpu().numpy(), ref)
+        gp, gb, _ = P.cl_backward(cl, g)
+        check_forces(gp.cpu().numpy(), -0.75 * ref["forces"])
+        check_matrix(gb.cpu().numpy(), 0.75 * ref["dedh"], TOL_GB)
+    occupied = P.cl_query(cl, "max_occupancy")
+    assert occupied > 2048 if name == "huge" else occupied <= 2048
