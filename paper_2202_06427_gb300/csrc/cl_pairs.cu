@@ -12,7 +12,7 @@
 //   (scan)         exclusive prefix sum of the counts in original order:
 //                  segment of i = [start[i], start[i] + count[i])
 //   k_pairs_cell<FILL>   the same staging, then the staged list's original
-//                  indices are radix-sorted, so each particle's pairs with
+//                  indices are sorted (stage_sort), so each particle's pairs with
 //                  j > i come out of a suffix of that order in ascending j and
 //                  are written in order with coalesced stores
 //   k_pairs_count / k_pairs_fill_sorted
@@ -283,40 +283,20 @@ __global__ void __launch_bounds__(32 * kFillWarps, 6) k_pairs_fill_sorted(const 
 
 // Stable LSD radix sort (8-bit digits) of the staged list's original indices,
 // the whole CTA (W warps) taking part: the slots 0..S-1 into st are sorted by
-// the key jo - kmin, read through the slot (no key array, so that four CTAs
-// fit per SM). Each warp ranks a fixed span of positions in order with
-// __match_any_sync, and the (digit, warp) offsets come from one exclusive scan
-// per pass, so equal digits keep their order. Returns the buffer that holds
-// the sorted slots.
+// the key jo - kmin (of `bits` bits), read through the slot (no key array, so
+// that five CTAs fit per SM). Each warp ranks a fixed span of positions in
+// order with __match_any_sync, and the (digit, warp) offsets come from one
+// exclusive scan per pass, so equal digits keep their order. Returns the buffer
+// that holds the sorted slots.
 template <int W>
-__device__ __forceinline__ void stage_radix(const float4* st, int S, unsigned short* s0, unsigned short* s1,
-                                            unsigned short* cnt,
-                                            int* scal, unsigned short*& slots, int& kmin) {
+__device__ __noinline__ void stage_radix(const float4* st, int S, int bits, int kmin, unsigned short* s0,
+                                         unsigned short* s1, unsigned short* cnt, int* scal,
+                                         unsigned short*& slots) {
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const unsigned lt = (1u << lane) - 1u;
-  if (threadIdx.x == 0) {
-    scal[1] = INT_MAX;
-    scal[2] = 0;
-  }
-  __syncthreads();
-  int lo = INT_MAX, hi = 0;
-  for (int i = threadIdx.x; i < S; i += blockDim.x) {
-    const int jo = __float_as_int(st[i].w);
-    lo = min(lo, jo);
-    hi = max(hi, jo);
-  }
-  lo = __reduce_min_sync(0xffffffffu, lo);
-  hi = __reduce_max_sync(0xffffffffu, hi);
-  if (lane == 0) {
-    atomicMin(scal + 1, lo);
-    atomicMax(scal + 2, hi);
-  }
-  __syncthreads();
-  kmin = scal[1];
-  const unsigned range = (unsigned)(scal[2] - kmin);
+  __syncthreads();  // every warp has read the buckets' starts
   for (int i = threadIdx.x; i < S; i += blockDim.x) s0[i] = (unsigned short)i;
   __syncthreads();
-  const int bits = range ? 32 - __clz(range) : 0;
   const int span = (((S + W - 1) / W) + 31) & ~31;
   const int b0 = min(S, warp * span), b1 = min(S, b0 + span);
   for (int sh = 0; sh < bits; sh += 8) {
@@ -375,6 +355,105 @@ __device__ __forceinline__ void stage_radix(const float4* st, int S, unsigned sh
   slots = s0;
 }
 
+constexpr int kBuckets = 1024;
+constexpr int kBucketMost = 48;  // a fuller bucket sends the cell to the radix sort
+
+// Orders the staged list's slots 0..S-1 (into st) by original index, the whole
+// CTA (W warps) taking part; scal[1], scal[2]: the smallest and largest index.
+// Returns the sorted slots (one of s0, s1) and kmin, the smallest index.
+//
+// The indices are spread over kBuckets equal parts of their range by a counting
+// sort whose slots come from shared-memory atomics, then each entry finds its
+// place within its bucket by counting the smaller ones. On an input in random
+// order a bucket holds about one entry; on one that follows space the entries
+// are runs of a few consecutive indices, a run or two to a bucket. Six barriers
+// against thirteen for the radix sort's three passes. A cell whose fullest
+// bucket passes kBucketMost (indices in a few tight clumps) takes the radix
+// sort.
+template <int W>
+__device__ __forceinline__ void stage_sort(const float4* st, int S, unsigned short* s0, unsigned short* s1, int* cnt,
+                                           int* scal, unsigned short*& slots, int& kmin) {
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  constexpr int T = 32 * W, per = kBuckets / T;
+  if (tid == 0) {
+    scal[1] = INT_MAX;
+    scal[2] = 0;
+    scal[3] = 0;
+  }
+#pragma unroll
+  for (int e = 0; e < per; ++e) cnt[tid + T * e] = 0;
+  __syncthreads();
+  int lo = INT_MAX, hi = 0;
+  for (int i = tid; i < S; i += T) {
+    const int jo = __float_as_int(st[i].w);
+    lo = min(lo, jo);
+    hi = max(hi, jo);
+  }
+  lo = __reduce_min_sync(0xffffffffu, lo);
+  hi = __reduce_max_sync(0xffffffffu, hi);
+  if (lane == 0) {
+    atomicMin(scal + 1, lo);
+    atomicMax(scal + 2, hi);
+  }
+  __syncthreads();
+  kmin = scal[1];
+  if (S == 0) {
+    slots = s0;
+    return;
+  }
+  const unsigned range = (unsigned)(scal[2] - kmin);
+  const int bits = range ? 32 - __clz(range) : 0;
+  const int sh = max(0, bits - 10);  // range >> sh < kBuckets
+  for (int i = tid; i < S; i += T)
+    s0[i] = (unsigned short)atomicAdd(&cnt[(unsigned)(__float_as_int(st[i].w) - kmin) >> sh], 1);
+  __syncthreads();
+  {  // exclusive scan of the buckets, per of them per thread
+    int v[per], loc = 0, most = 0;
+#pragma unroll
+    for (int e = 0; e < per; ++e) {
+      v[e] = cnt[tid * per + e];
+      loc += v[e];
+      most = max(most, v[e]);
+    }
+    most = __reduce_max_sync(0xffffffffu, most);
+    int inc = loc;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const int u = __shfl_up_sync(0xffffffffu, inc, o);
+      inc += lane >= o ? u : 0;
+    }
+    if (lane == 31) scal[4 + warp] = inc;
+    if (lane == 0 && most > kBucketMost) scal[3] = 1;
+    __syncthreads();
+    int off = inc - loc;
+    for (int w = 0; w < warp; ++w) off += scal[4 + w];
+#pragma unroll
+    for (int e = 0; e < per; ++e) {
+      cnt[tid * per + e] = off;
+      off += v[e];
+    }
+  }
+  __syncthreads();
+  if (scal[3]) {
+    stage_radix<W>(st, S, bits, kmin, s0, s1, reinterpret_cast<unsigned short*>(cnt), scal, slots);
+    return;
+  }
+  for (int i = tid; i < S; i += T)
+    s1[cnt[(unsigned)(__float_as_int(st[i].w) - kmin) >> sh] + s0[i]] = (unsigned short)i;
+  __syncthreads();
+  for (int p = tid; p < S; p += T) {
+    const int i = s1[p];
+    const int jo = __float_as_int(st[i].w);
+    const unsigned b = (unsigned)(jo - kmin) >> sh;
+    const int b0 = cnt[b], b1 = b + 1 < (unsigned)kBuckets ? cnt[b + 1] : S;
+    int r = b0;
+    for (int q = b0; q < b1; ++q) r += __float_as_int(st[s1[q]].w) < jo ? 1 : 0;
+    s0[r] = (unsigned short)i;
+  }
+  __syncthreads();
+  slots = s0;
+}
+
 // Squared distances of a staged entry q to two home particles (nx, ny, nz:
 // their negated coordinates), both in packed FP32: per lane the same rounding
 // as fmaf(dx, dx, fmaf(dy, dy, dz * dz)) with dx = q.x - x. The count and the
@@ -401,7 +480,7 @@ __device__ __forceinline__ float2 pair_d2(const float4& q, float2 nx, float2 ny,
 // are not staged: no pair with j > i of this cell needs them.
 // COUNT: count[a] = pairs with j > a; a cell whose list does not fit gets
 // flag 1 (else 0) and is listed in fcells. FILL: flagged cells are skipped; the staged list is ordered
-// by original index (radix sort of its indices), so a particle's pairs with
+// by original index (stage_sort), so a particle's pairs with
 // j > a come from a suffix of that order in ascending j and are written in
 // order, coalesced, as the ballot finds them.
 template <int DIM, bool FILL>
@@ -420,8 +499,8 @@ __global__ void __launch_bounds__(256, 5) k_pairs_cell(const __grid_constant__ S
   float4* st = smem;           // staged neighbourhood: (x, y, z in the cell's frame, original index)
   float4* stab = st + cap;     // stencil: (s_x, s_y, s_z, dx | dy << 10 | dz << 20)
   int* scal = reinterpret_cast<int*>(stab + A.noff);  // [0] staged count, [1..2] index range, [4..] warp sums
-  unsigned short* cnt = reinterpret_cast<unsigned short*>(scal + 16);  // FILL: radix counters and slots
-  unsigned short* rs0 = cnt + 256 * W;
+  int* cnt = scal + 16;  // FILL: bucket (or radix) counters and slots
+  unsigned short* rs0 = reinterpret_cast<unsigned short*>(cnt + kBuckets);
   unsigned short* rs1 = rs0 + cap;
   stencil_to_smem(A, stab);
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -475,7 +554,7 @@ __global__ void __launch_bounds__(256, 5) k_pairs_cell(const __grid_constant__ S
     if (S <= cap) {
       unsigned short* slots = rs0;
       int kmin = 0;
-      if (FILL) stage_radix<W>(st, S, rs0, rs1, cnt, scal, slots, kmin);
+      if (FILL) stage_sort<W>(st, S, rs0, rs1, cnt, scal, slots, kmin);
       if (!FILL) {
         // COUNT: two home particles per warp share each staged load; the
         // distance of each (particle, candidate) is computed as in the fill pass.
@@ -588,7 +667,8 @@ __global__ void __launch_bounds__(256, 5) k_pairs_cell(const __grid_constant__ S
 
 size_t pairs_cell_smem(int noff, bool fill, int cap) {
   const size_t head = (size_t)(cap + noff) * sizeof(float4) + 16 * sizeof(int);
-  return fill ? head + 256 * 8 * sizeof(unsigned short) + 2 * (size_t)cap * sizeof(unsigned short) : head;
+  static_assert(kBuckets * sizeof(int) >= 256 * 8 * sizeof(unsigned short), "the radix counters fit");
+  return fill ? head + kBuckets * sizeof(int) + 2 * (size_t)cap * sizeof(unsigned short) : head;
 }
 
 template <int DIM, bool FILL>
