@@ -285,7 +285,7 @@ int map_pairlist(cl_list* c, cl_result* r, cudaStream_t s) {
   // neighbourhood sweep, which rewrites them on every launch); pl_meta[4]: their number
   const int cap = pairs_stage_cap(c->geo, c->n, ball2);
   c->lists_half = 0;  // the pair list's passes use the list buffers
-  if ((e = clk::launch_pairs_count(*c->full, dim, ball2, cap, c->hflag, c->hlist, c->pl_meta + 4, c->pl_count, s)))
+  if ((e = clk::launch_pairs_count(*c->full, c->d_off_full, dim, ball2, cap, c->hflag, c->hlist, c->pl_meta + 4, c->pl_count, s)))
     return e;
   if ((e = clk::launch_scan64(c->pl_count, c->n, c->pl_tiles, c->pl_start, c->pl_meta, s))) return e;
   long long total = 0;
@@ -298,7 +298,7 @@ int map_pairlist(cl_list* c, cl_result* r, cudaStream_t s) {
   if ((e = cl_pairlist_fits(total, r->capacity))) return e;
   if (total == 0) return CL_OK;
   if (!r->pair_i || !r->pair_j || !r->pair_d) return CL_ERR_INVALID_ARG;
-  return clk::launch_pairs_fill(*c->full, dim, ball2, cap, c->hflag, c->hlist, c->pl_meta + 4, c->pl_count, c->pl_start,
+  return clk::launch_pairs_fill(*c->full, c->d_off_full, dim, ball2, cap, c->hflag, c->hlist, c->pl_meta + 4, c->pl_count, c->pl_start,
                                r->pair_i, r->pair_j, r->pair_d, c->pl_long, c->pl_meta + 3, s);
 }
 

@@ -316,7 +316,7 @@ constexpr int kMaxSegment = 1024;  // segments up to this length are sorted by o
 // sweep for the cells it flags (flag: ncells bytes; fcells: ncells ints, the
 // flagged cells, *nfcells of them; all written here).
 // cap: staged entries per cell (32..3072), the same for the count and fill passes.
-int launch_pairs_count(const SweepArgs& A, int dim, float ball2, int cap, unsigned char* flag, int* fcells,
+int launch_pairs_count(const SweepArgs& A, const Off* off, int dim, float ball2, int cap, unsigned char* flag, int* fcells,
                        int* nfcells, int* count, cudaStream_t s);
 // Sorts each listed segment [start[a], start[a] + count[a]), a = longs[q], q <
 // *nlong, of pj (carrying pd) by pj.
@@ -324,7 +324,7 @@ int launch_sort_long(const int* longs, const int* nlong, const int* count, const
                      cudaStream_t s);
 // Fill pass: the same two sweeps, each segment sorted by j and written.
 // longs (n ints) and nlong (1 int): workspace for segments longer than kMaxSegment.
-int launch_pairs_fill(const SweepArgs& A, int dim, float ball2, int cap, const unsigned char* flag, const int* fcells,
+int launch_pairs_fill(const SweepArgs& A, const Off* off, int dim, float ball2, int cap, const unsigned char* flag, const int* fcells,
                       const int* nfcells, const int* count, const long long* start, int* pi, int* pj, float* pd, int* longs,
                       int* nlong, cudaStream_t s);
 

@@ -15,9 +15,9 @@
 //                  indices are sorted (stage_sort), so each particle's pairs with
 //                  j > i come out of a suffix of that order in ascending j and
 //                  are written in order with coalesced stores
-//   k_pairs_count / k_pairs_fill_sorted
-//                  the listed cells' particles, one thread (count) or one warp
-//                  (fill) per particle straight from the sorted arrays; a
+//   k_pairs_count / k_pairs_fill
+//                  the listed cells' particles, one warp per particle
+//                  straight from the sorted arrays; a
 //                  segment longer than kMaxSegment is written unsorted and
 //                  listed for k_pairs_sort_long
 //   k_pairs_sort_long  one CTA per listed segment, in place in global memory
@@ -29,36 +29,99 @@
 // (rc <= w_min / 2), which the host checks before launching.
 #include <climits>
 
+#include "cl_query.cuh"
 #include "cl_sort.cuh"
-#include "cl_sweep.cuh"
 
 namespace clk {
 
 
-struct RedPairCount {
-  static constexpr bool kFull = true;
-  struct Acc { int a; int n; };
-  __device__ void init(Acc& x) const { x.n = 0; }
-  __device__ void hit(Acc& x, float, float, float, float, int j) const { x.n += (j > x.a) ? 1 : 0; }
-};
+// The particles of the listed cells (cells[0, *ncells)), a warp each: the pairs
+// with j > i by the per-point sweep of cl_query.cuh. (One thread per particle
+// for the count and a warp walking every stencil cell, with the segment
+// sorted as (key, value) pairs, for the fill: a list of 230,000 particles at
+// one cell per cutoff, whose cells all overflow, took 13.2 ms with its build
+// and histogram; now 4.5.)
+constexpr int kFillWarps = 4;
 
-// The particles of the listed cells (cells[0, *ncells)), one thread each.
-template <int DIM>
-__global__ void __launch_bounds__(256) k_pairs_count(const __grid_constant__ SweepArgs A,
-                                                     const int* __restrict__ cells, const int* __restrict__ ncells,
-                                                     int* __restrict__ count) {
+template <int G>
+__global__ void __launch_bounds__(32 * kFillWarps) k_pairs_count(const __grid_constant__ CrossArgs A,
+                                                                 const unsigned* __restrict__ cellc,
+                                                                 const int* __restrict__ cells,
+                                                                 const int* __restrict__ ncells,
+                                                                 int* __restrict__ count) {
+  extern __shared__ float4 stab[];
+  __shared__ WarpCells work[kFillWarps];
   const int m = *ncells;
+  if ((int)blockIdx.x >= m) return;
+  load_stencil<false>(A, stab, nullptr);
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   for (int q = blockIdx.x; q < m; q += gridDim.x) {
-    const int c = cells[q];
-    const int p1 = A.cell_start[c + 1];
-    for (int p = A.cell_start[c] + threadIdx.x; p < p1; p += blockDim.x) {
-      RedPairCount red;
-      RedPairCount::Acc acc;
-      red.init(acc);
-      acc.a = __float_as_int(A.xs[p].w);
-      float4 pi;
-      sweep_particle<DIM>(A, red, acc, p, pi);
-      count[acc.a] = acc.n;
+    const int c = cells[q], p1 = A.cell_start[c + 1];
+    for (int p = A.cell_start[c] + warp; p < p1; p += kFillWarps) {
+      const float4 x = A.xs[p];
+      const int i = __float_as_int(x.w);
+      const unsigned n = __reduce_add_sync(0xffffffffu, query_count<G>(A, stab, work[warp], cellc[p], x, i));
+      if (lane == 0) count[i] = (int)n;
+    }
+  }
+}
+
+// A segment of at most kMaxSegment pairs is sorted in the warp's shared memory
+// (WIDE false, fewer than 2^22 particles: by the one-word key j << 10 | slot),
+// a longer one written unsorted and listed in longs.
+template <int G, bool WIDE>
+__global__ void __launch_bounds__(32 * kFillWarps, 5) k_pairs_fill(const __grid_constant__ CrossArgs A,
+                                                                   const unsigned* __restrict__ cellc,
+                                                                   const int* __restrict__ cells,
+                                                                   const int* __restrict__ ncells,
+                                                                   const int* __restrict__ count,
+                                                                   const long long* __restrict__ start,
+                                                                   int* __restrict__ pi_out, int* __restrict__ pj_out,
+                                                                   float* __restrict__ pd_out, int* __restrict__ longs,
+                                                                   int* __restrict__ nlong) {
+  extern __shared__ float4 stab[];
+  __shared__ WarpCells work[kFillWarps];
+  const int m = *ncells;
+  if ((int)blockIdx.x >= m) return;
+  load_stencil<false>(A, stab, nullptr);
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  float* V = reinterpret_cast<float*>(stab + A.noff) + (size_t)warp * 2 * kSegPad;
+  unsigned* K = reinterpret_cast<unsigned*>(V + kSegPad);
+  for (int q = blockIdx.x; q < m; q += gridDim.x) {
+    const int c = cells[q], p1 = A.cell_start[c + 1];
+    for (int p = A.cell_start[c] + warp; p < p1; p += kFillWarps) {
+      const float4 x = A.xs[p];
+      const int i = __float_as_int(x.w), cnt = __ldg(count + i);
+      if (cnt == 0) continue;
+      const long long base = __ldg(start + i);
+      const bool big = cnt > kMaxSegment;
+      const int L = query_hits<G>(A, stab, work[warp], cellc[p], x, i, [&](int e, int j, float d2) {
+        if (e >= cnt) return;
+        if (big) {
+          pi_out[base + e] = i;
+          pj_out[base + e] = j;
+          pd_out[base + e] = d2 * rsqrt_nr(d2);
+        } else {
+          K[seg_at(e)] = WIDE ? (unsigned)j : ((unsigned)j << 10) | (unsigned)e;
+          V[seg_at(e)] = d2;
+        }
+      });
+      __syncwarp();
+      if (big) {
+        if (lane == 0) longs[atomicAdd(nlong, 1)] = i;
+        continue;
+      }
+      const int nw = min(L, cnt);
+      if (WIDE) sort_segment(reinterpret_cast<int*>(K), V, nw, lane);
+      else sort_keys(K, nw, lane);
+      for (int t = lane; t < nw; t += 32) {
+        const unsigned key = K[seg_at(t)];
+        const float d2 = V[WIDE ? seg_at(t) : seg_at((int)(key & 1023u))];
+        pi_out[base + t] = i;
+        pj_out[base + t] = WIDE ? (int)key : (int)(key >> 10);
+        pd_out[base + t] = d2 * rsqrt_nr(d2);
+      }
+      __syncwarp();
     }
   }
 }
@@ -110,17 +173,13 @@ __global__ void __launch_bounds__(1024) k_pairs_sort_long(const int* __restrict_
   }
 }
 
-// Shared pieces of the pair-list sweeps. A warp takes the stencil 32 entries
+// Shared pieces of the per-cell sweeps. A warp takes the stencil 32 entries
 // at a time, one per lane: each lane finds its neighbour cell's particle
 // range, a warp scan lays the ranges end to end, and the warp walks the
 // concatenation 32 candidates per step (a shuffle binary search finds each
-// candidate's entry), so the lanes stay busy however small the cells are. The
-// kept pairs of a particle are compacted with a ballot into the warp's
-// shared-memory segment, sorted by j in registers (bitonic) and written to
-// [start[a], start[a] + count[a]) with coalesced stores. Segments are at most
-// kMaxSegment long (the host checks the counts first).
-constexpr int kFillWarps = 4;
+// candidate's entry), so the lanes stay busy however small the cells are.
 constexpr int kStageMax = 3072;  // largest staged neighbourhood of one cell (the launch picks its capacity)
+
 // Stencil entries k0 + lane of cell (cx, cy, cz): the lane's range [j0, j0 +
 // len) of sorted particles, its shift (stencil shift + (bx, by, bz)) and, over
 // the warp, the exclusive offsets of the ranges laid end to end and their total.
@@ -186,98 +245,6 @@ __device__ __forceinline__ void stencil_to_smem(const SweepArgs& A, float4* stab
     const Off& o = A.off[k];
     stab[k] = make_float4(o.sx, o.sy, o.sz,
                           __uint_as_float((unsigned)o.dx | ((unsigned)o.dy << 10) | ((unsigned)o.dz << 20)));
-  }
-}
-
-// Sorts the warp's segment of nw kept pairs by j and writes it at base.
-__device__ __forceinline__ void segment_out(int* K, float* V, int nw, int a, long long base, int lane, int* pi_out,
-                                            int* pj_out, float* pd_out) {
-  sort_segment(K, V, nw, lane);
-  for (int i = lane; i < nw; i += 32) {
-    pi_out[base + i] = a;
-    pj_out[base + i] = K[seg_at(i)];
-    pd_out[base + i] = V[seg_at(i)];
-  }
-  __syncwarp();
-}
-
-// The listed cells' particles, one warp per particle, straight from the sorted
-// arrays: the candidate's distance is x_j + (s_o - x_i), equal in IEEE
-// arithmetic to x_j - (x_i - s_o) of k_pairs_count (same fused multiply-adds).
-template <int DIM>
-__global__ void __launch_bounds__(32 * kFillWarps, 6) k_pairs_fill_sorted(const __grid_constant__ SweepArgs A,
-                                                                          const int* __restrict__ cells,
-                                                                          const int* __restrict__ ncells,
-                                                                          const int* __restrict__ count,
-                                                                          const long long* __restrict__ start,
-                                                                          int* __restrict__ pi_out,
-                                                                          int* __restrict__ pj_out,
-                                                                          float* __restrict__ pd_out,
-                                                                          int* __restrict__ longs,
-                                                                          int* __restrict__ nlong) {
-  extern __shared__ float4 stab[];  // per entry: (s_x, s_y, s_z, dx | dy << 10 | dz << 20)
-  __shared__ int sk[kFillWarps][kSegPad];
-  __shared__ float sv[kFillWarps][kSegPad];
-  stencil_to_smem(A, stab);
-  __syncthreads();
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const unsigned lt = (1u << lane) - 1u;
-  int* K = sk[warp];
-  float* V = sv[warp];
-  const int mc = *ncells;
-  for (int q = blockIdx.x; q < mc; q += gridDim.x) {
-    const int cq = cells[q];
-    const int pend = A.cell_start[cq + 1];
-    for (int p = A.cell_start[cq] + warp; p < pend; p += kFillWarps) {
-      const float4 pi = A.xs[p];
-      const int a = __float_as_int(pi.w);
-      const unsigned cc = A.cellc[p];
-      const int cx = (int)(cc & 1023u), cy = (int)((cc >> 10) & 1023u), cz = (int)(cc >> 20);
-      const int cnt_a = __ldg(count + a);
-      const long long base = __ldg(start + a);
-      const bool big = cnt_a > kMaxSegment;  // written unsorted, sorted by k_pairs_sort_long
-      int L = 0;
-      for (int k0 = 0; k0 < A.noff; k0 += 32) {
-        const Chunk ch = chunk_ranges<DIM>(A, stab, k0, lane, cx, cy, cz, -pi.x, -pi.y, -pi.z);
-        for (int t0 = 0; t0 < ch.total; t0 += 32) {
-          const int t = t0 + lane;
-          float ax, ay, az;
-          const int j = chunk_candidate(ch, t, ax, ay, az);
-          bool keep = false;
-          int jo = 0;
-          float d2 = 0.f;
-          if (t < ch.total) {
-            const float4 q = __ldg(&A.xs[j]);
-            jo = __float_as_int(q.w);
-            const float dx = q.x + ax, dy = q.y + ay;
-            const float dz = DIM == 3 ? q.z + az : 0.f;
-            d2 = DIM == 3 ? fmaf(dx, dx, fmaf(dy, dy, dz * dz)) : fmaf(dx, dx, dy * dy);
-            keep = jo > a && d2 < A.rc2;
-          }
-          const unsigned m = __ballot_sync(0xffffffffu, keep);
-          if (keep) {
-            const int e = L + __popc(m & lt);
-            if (big) {
-              if (e < cnt_a) {
-                pi_out[base + e] = a;
-                pj_out[base + e] = jo;
-                pd_out[base + e] = d2 * rsqrt_nr(d2);
-              }
-            } else if (e < kMaxSegment) {
-              K[seg_at(e)] = jo;
-              V[seg_at(e)] = d2 * rsqrt_nr(d2);
-            }
-          }
-          L += __popc(m);
-        }
-      }
-      __syncwarp();
-      if (big) {
-        if (lane == 0) longs[atomicAdd(nlong, 1)] = a;
-      } else {
-        segment_out(K, V, min(min(L, kMaxSegment), cnt_a), a, base, lane, pi_out, pj_out, pd_out);
-      }
-    }
   }
 }
 
@@ -698,7 +665,7 @@ static int launch_cell(const SweepArgs& A, float ball2, int cap, unsigned char* 
   return cudaGetLastError() == cudaSuccess ? CL_OK : CL_ERR_CUDA;
 }
 
-int launch_pairs_count(const SweepArgs& A, int dim, float ball2, int cap, unsigned char* flag, int* fcells,
+int launch_pairs_count(const SweepArgs& A, const Off* off, int dim, float ball2, int cap, unsigned char* flag, int* fcells,
                        int* nfcells, int* count, cudaStream_t s) {
   if (A.n <= 0) return CL_OK;
   if (cudaMemsetAsync(nfcells, 0, sizeof(int), s) != cudaSuccess) return CL_ERR_CUDA;
@@ -707,8 +674,32 @@ int launch_pairs_count(const SweepArgs& A, int dim, float ball2, int cap, unsign
                          : launch_cell<2, false>(A, ball2, cap, flag, fcells, nfcells, count, nullptr, nullptr,
                                                  nullptr, nullptr, s);
   if (e) return e;
-  if (dim == 3) k_pairs_count<3><<<152 * 4, 256, 0, s>>>(A, fcells, nfcells, count);
-  else k_pairs_count<2><<<152 * 4, 256, 0, s>>>(A, fcells, nfcells, count);
+  const CrossArgs C = cross_args(A, off);
+  const size_t dyn = (size_t)C.noff * sizeof(float4);
+  switch (group_lanes(A)) {
+    case 2: k_pairs_count<2><<<152 * 8, 32 * kFillWarps, dyn, s>>>(C, A.cellc, fcells, nfcells, count); break;
+    case 4: k_pairs_count<4><<<152 * 8, 32 * kFillWarps, dyn, s>>>(C, A.cellc, fcells, nfcells, count); break;
+    default: k_pairs_count<8><<<152 * 8, 32 * kFillWarps, dyn, s>>>(C, A.cellc, fcells, nfcells, count); break;
+  }
+  return cudaGetLastError() == cudaSuccess ? CL_OK : CL_ERR_CUDA;
+}
+
+template <int G, bool WIDE>
+static int launch_fill_listed(const CrossArgs& C, const unsigned* cellc, const int* fcells, const int* nfcells,
+                              const int* count, const long long* start, int* pi, int* pj, float* pd, int* longs,
+                              int* nlong, cudaStream_t s) {
+  static DevCache ready;  // shared-memory limit raised on this device
+  const size_t seg = (size_t)kFillWarps * 2 * kSegPad * sizeof(float);
+  int dev = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess) return CL_ERR_CUDA;
+  if (!ready.get(dev)) {
+    if (cudaFuncSetAttribute(k_pairs_fill<G, WIDE>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                             (int)(seg + kMaxOff * sizeof(float4))) != cudaSuccess)
+      return CL_ERR_CUDA;
+    ready.put(dev, 1);
+  }
+  k_pairs_fill<G, WIDE><<<152 * 5, 32 * kFillWarps, seg + (size_t)C.noff * sizeof(float4), s>>>(
+      C, cellc, fcells, nfcells, count, start, pi, pj, pd, longs, nlong);
   return cudaGetLastError() == cudaSuccess ? CL_OK : CL_ERR_CUDA;
 }
 
@@ -718,7 +709,7 @@ int launch_sort_long(const int* longs, const int* nlong, const int* count, const
   return cudaGetLastError() == cudaSuccess ? CL_OK : CL_ERR_CUDA;
 }
 
-int launch_pairs_fill(const SweepArgs& A, int dim, float ball2, int cap, const unsigned char* flag, const int* fcells,
+int launch_pairs_fill(const SweepArgs& A, const Off* off, int dim, float ball2, int cap, const unsigned char* flag, const int* fcells,
                       const int* nfcells, const int* count, const long long* start, int* pi, int* pj, float* pd, int* longs,
                       int* nlong, cudaStream_t s) {
   if (A.n <= 0) return CL_OK;
@@ -727,15 +718,19 @@ int launch_pairs_fill(const SweepArgs& A, int dim, float ball2, int cap, const u
   const int e = dim == 3 ? launch_cell<3, true>(A, ball2, cap, fl, nullptr, nullptr, cn, start, pi, pj, pd, s)
                          : launch_cell<2, true>(A, ball2, cap, fl, nullptr, nullptr, cn, start, pi, pj, pd, s);
   if (e) return e;
-  const size_t dyn = (size_t)A.noff * sizeof(float4);
   if (cudaMemsetAsync(nlong, 0, sizeof(int), s) != cudaSuccess) return CL_ERR_CUDA;
-  if (dim == 3)
-    k_pairs_fill_sorted<3><<<152 * 6, 32 * kFillWarps, dyn, s>>>(A, fcells, nfcells, count, start, pi, pj, pd, longs,
-                                                                nlong);
+  const CrossArgs C = cross_args(A, off);
+  const int g = group_lanes(A);
+  int f;
+  if (A.n >= (1 << 22))
+    f = launch_fill_listed<8, true>(C, A.cellc, fcells, nfcells, count, start, pi, pj, pd, longs, nlong, s);
+  else if (g == 2)
+    f = launch_fill_listed<2, false>(C, A.cellc, fcells, nfcells, count, start, pi, pj, pd, longs, nlong, s);
+  else if (g == 4)
+    f = launch_fill_listed<4, false>(C, A.cellc, fcells, nfcells, count, start, pi, pj, pd, longs, nlong, s);
   else
-    k_pairs_fill_sorted<2><<<152 * 6, 32 * kFillWarps, dyn, s>>>(A, fcells, nfcells, count, start, pi, pj, pd, longs,
-                                                                nlong);
-  if (cudaGetLastError() != cudaSuccess) return CL_ERR_CUDA;
+    f = launch_fill_listed<8, false>(C, A.cellc, fcells, nfcells, count, start, pi, pj, pd, longs, nlong, s);
+  if (f) return f;
   return launch_sort_long(longs, nlong, count, start, pj, pd, s);
 }
 
