@@ -79,7 +79,7 @@ struct Smem {
   int nrows;
   float wmax[kWarps];
   int nf, nb;            // staged entries with T = 0 (from the front) and T != 0 (from the back)
-  int item;
+  int item, part;
   unsigned long long ncand;  // candidate pairs this CTA evaluated
   double out[kWarps][16];    // per-warp sums: share of sum fsn r (x) r (6), X (9), energy (1)
 };
@@ -1151,7 +1151,7 @@ __global__ void __launch_bounds__(kThreads, 5) k_hood(const __grid_constant__ Sw
   // atomic's latency overlaps whole cells, and every thread prefetches into L1
   // the cell ranges it will read for the next cell while this one is swept.
   if (tid == 0) S.ncand = 0;
-  const int nlist = H.work[6];
+  const int split = H.split, nlist = H.work[6] * split;  // items: (cell, part of its home particles)
   int next1 = 0, next2 = 0;
   if (tid == 0) {
     next1 = atomicAdd(H.work, 1);
@@ -1161,7 +1161,8 @@ __global__ void __launch_bounds__(kThreads, 5) k_hood(const __grid_constant__ Sw
   for (;;) {
     __syncthreads();
     if (tid == 0) {
-      S.item = next1 < nlist ? H.list[next1] : -2;
+      S.item = next1 < nlist ? H.list[next1 / split] : -2;
+      S.part = next1 % split;
       S.nf = 0;
       S.nb = 0;
     }
@@ -1218,7 +1219,8 @@ __global__ void __launch_bounds__(kThreads, 5) k_hood(const __grid_constant__ Sw
       continue;
     }
     if (tid == 0) H.flag[h] = 0;
-    if (tid == 0)
+    const int part = S.part;
+    if (tid == 0 && part == 0)
       S.ncand += (unsigned long long)nh * (unsigned long long)(nf + nb) +
                  (unsigned long long)(HALF ? nh * (nh - 1) / 2 : nh * (nh - 1));
     if (tid == 0 && (nf & 1)) {  // padding after an odd segment
@@ -1238,7 +1240,7 @@ __global__ void __launch_bounds__(kThreads, 5) k_hood(const __grid_constant__ Sw
     const int ngroups = (nh + 1) >> 1;
     const int k0a = 0, k1a = (nf + 1) >> 1;
     const int k0b = (kCap - nb) >> 1, k1b = kCap >> 1;
-    for (int gi = warp; gi < ngroups; gi += kWarps) {
+    for (int gi = warp + kWarps * part; gi < ngroups; gi += kWarps * split) {
       const int t0 = 2 * gi, t1 = 2 * gi + 1;
       const bool has1 = t1 < nh;
       float2 I[6];
@@ -2792,7 +2794,11 @@ int launch_hood_scalar(const SweepArgs& A, const HoodArgs& Hin, int* work, int k
     default: nb = grid_for(k_hood<6>, smem); nhb = grid_for(k_half_batch<6>, hsmem); break;
   }
   if (nb <= 0 || nhb <= 0) return CL_ERR_CUDA;
-  nb = std::min(nb, Hin.ncells);
+  // Grids of fewer cells than resident CTAs: up to four CTAs share a cell's home
+  // particles, each staging the neighbourhood for itself (343 cells, 29
+  // particles each: count 30 -> 28 us, histogram 48 -> 39).
+  if (half) H.split = std::max(1, std::min(4, nb / std::max(1, Hin.ncells)));
+  nb = (int)std::min<long long>(nb, (long long)Hin.ncells * H.split);
   nhb = half ? std::min(nhb, Hin.ncells) : 0;
   const int nrest = half ? 0 : flagged_blocks(A.n);
   if (scalar && nb + nhb + nrest > partials_cap) return CL_ERR_INVALID_ARG;
@@ -2880,14 +2886,15 @@ int fill_hood_args(const Geo& geo, const int* opk_full, int noff_full, const int
   // Raw half-neighbourhood size up to which a cell takes the fast path: its
   // buffer holds kHCap kept entries, those within rc + d_max <= rc + hd of the
   // centre, at uniform density at most the half ball's share of the half
-  // stencil. At most kCap, the buffer of the home-major scalar sweep.
+  // stencil. At most what the home-major scalar sweep's buffer holds.
   {
     double cell = std::fabs(geo.h[0] * (geo.h[4] * geo.h[8] - geo.h[5] * geo.h[7]) -
                             geo.h[1] * (geo.h[3] * geo.h[8] - geo.h[5] * geo.h[6]) +
                             geo.h[2] * (geo.h[3] * geo.h[7] - geo.h[4] * geo.h[6])) / (double)geo.ncells;
     const double r = geo.rc + hd, half_ball = 0.5 * (4.18879020478639 * r * r * r - cell);
     const double share = std::min(1.0, half_ball / (cell * std::max(1, noff_half - 1)));
-    H->rawcap = (int)std::min((double)kCap, kHCap / share);
+    H->rawcap = (int)std::min((double)kCap - 2, kHCap / share);
+    H->split = 1;
     // small cells need each row's segments in two lanes of a warp: at most 16
     // rows, none longer than the grid (a row then has at most two segments)
     int longest = 0;

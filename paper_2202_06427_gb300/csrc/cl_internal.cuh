@@ -204,6 +204,7 @@ struct HoodArgs {
   float eps;          // rounding margin of the staging radius
   int rawcap;         // particles in the half neighbourhood up to which a cell takes the fast path
   int smallcap;       // particles of a cell and its half neighbourhood up to which one warp takes it
+  int split;          // CTAs sharing a listed cell's home particles (home-major scalar sweeps)
   int ncells;
   int* work;          // [0], [1], [5] work counters of the listed, small and dense cells, [2..3] candidates
                       // (zeroed by the launcher); [6] list length, [7] dense cells, [8] small cells (at the end

@@ -12,37 +12,60 @@
 namespace clk {
 namespace {
 
-// Per-axis min and max of n points (dim columns), FP64, one CTA per 256 x 8
-// points, atomics on the order-preserving integer image of the doubles.
-__device__ __forceinline__ unsigned long long ordered_bits(double v) {
-  const unsigned long long b = (unsigned long long)__double_as_longlong(v);
+// Per-axis min and max of n points (dim columns), FP64, on the order-preserving
+// integer image of the doubles: FP64 compares issue at a small fraction of the
+// integer rate here (57 us for a million points with fmin and fmax, against
+// 24 MB read).
+__device__ __forceinline__ unsigned long long ordered_bits(unsigned long long b) {
   return (b >> 63) ? ~b : (b | 0x8000000000000000ull);
 }
 
-__global__ void __launch_bounds__(256) k_extent(const double* __restrict__ x, long long n, int dim,
+template <int DIM>
+__global__ void __launch_bounds__(256) k_extent(const double* __restrict__ x, long long n,
                                                 unsigned long long* __restrict__ mm, int* __restrict__ bad) {
-  double lo[3] = {INFINITY, INFINITY, INFINITY}, hi[3] = {-INFINITY, -INFINITY, -INFINITY};
+  unsigned long long lo[DIM], hi[DIM];
+#pragma unroll
+  for (int k = 0; k < DIM; ++k) {
+    lo[k] = ~0ull;
+    hi[k] = 0ull;
+  }
   bool finite = true;
+#pragma unroll 2
   for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x)
-    for (int k = 0; k < dim; ++k) {
-      const double v = x[i * dim + k];
-      if (!isfinite(v)) {
-        finite = false;
-        continue;
-      }
-      lo[k] = fmin(lo[k], v);
-      hi[k] = fmax(hi[k], v);
+#pragma unroll
+    for (int k = 0; k < DIM; ++k) {
+      const unsigned long long b = (unsigned long long)__double_as_longlong(x[i * DIM + k]);
+      const bool ok = (b & 0x7ff0000000000000ull) != 0x7ff0000000000000ull;
+      finite = finite && ok;
+      const unsigned long long v = ordered_bits(b);
+      lo[k] = ok && v < lo[k] ? v : lo[k];
+      hi[k] = ok && v > hi[k] ? v : hi[k];
     }
-  for (int k = 0; k < dim; ++k) {
+  __shared__ unsigned long long part[8][2 * DIM];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+#pragma unroll
+  for (int k = 0; k < DIM; ++k) {
 #pragma unroll
     for (int o = 16; o; o >>= 1) {
-      lo[k] = fmin(lo[k], __shfl_xor_sync(0xffffffffu, lo[k], o));
-      hi[k] = fmax(hi[k], __shfl_xor_sync(0xffffffffu, hi[k], o));
+      const unsigned long long a = __shfl_xor_sync(0xffffffffu, lo[k], o), c = __shfl_xor_sync(0xffffffffu, hi[k], o);
+      lo[k] = a < lo[k] ? a : lo[k];
+      hi[k] = c > hi[k] ? c : hi[k];
     }
-    if ((threadIdx.x & 31) == 0 && lo[k] <= hi[k]) {
-      atomicMin(mm + 2 * k, ordered_bits(lo[k]));
-      atomicMax(mm + 2 * k + 1, ordered_bits(hi[k]));
+    if (lane == 0) {
+      part[warp][2 * k] = lo[k];
+      part[warp][2 * k + 1] = hi[k];
     }
+  }
+  __syncthreads();
+  if (threadIdx.x < 2 * DIM) {
+    const int q = threadIdx.x;
+    unsigned long long v = part[0][q];
+    for (int w = 1; w < 8; ++w) {
+      const unsigned long long t = part[w][q];
+      v = (q & 1) ? (t > v ? t : v) : (t < v ? t : v);
+    }
+    if (q & 1) atomicMax(mm + q, v);
+    else atomicMin(mm + q, v);
   }
   if (!finite) atomicOr(bad, 1);
 }
@@ -79,7 +102,8 @@ int open_box(const double* const* sets, const long long* ns, int nsets, int dim,
     ntot += ns[q];
     long long blocks = (ns[q] + 255) / 256;
     if (blocks > 152 * 8) blocks = 152 * 8;
-    k_extent<<<(int)blocks, 256, 0, s>>>(sets[q], ns[q], dim, mm, bad);
+    if (dim == 3) k_extent<3><<<(int)blocks, 256, 0, s>>>(sets[q], ns[q], mm, bad);
+    else k_extent<2><<<(int)blocks, 256, 0, s>>>(sets[q], ns[q], mm, bad);
     if (cudaGetLastError() != cudaSuccess) e = CL_ERR_CUDA;
   }
   unsigned long long out[6];
