@@ -200,6 +200,11 @@ int set_geometry(cl_list* c, const cl_box* box, cudaStream_t s) {
   c->hood->slot = c->slot;
   c->half->noff = nh;
   c->full->noff = nf;
+  c->half->nrow2 = c->full->nrow2 = 0;
+  if (g.dim == 2) {
+    clk::fill_rows2(t->opk_half, nh, c->half);
+    clk::fill_rows2(t->opk_full, nf, c->full);
+  }
   c->geo = g;
   c->box = *box;
   fill_sweep_args(c, c->half);

@@ -263,6 +263,33 @@ int build_stencils(const Geo& geo, int cap, Off* half, int* opk_half, int* nhalf
   return CL_OK;
 }
 
+void fill_rows2(const int* opk, int noff, SweepArgs* A) {
+  constexpr int R = kMaxRows2 / 2;
+  int at[kMaxRows2][kMaxRows2];  // stencil entry of offset (ox, oy), or -1
+  for (auto& row : at)
+    for (int& e : row) e = -1;
+  A->nrow2 = 0;
+  for (int k = 0; k < noff; ++k) {
+    const int ox = (signed char)(opk[k] & 0xff), oy = (signed char)((opk[k] >> 8) & 0xff);
+    if (std::abs(ox) > R || std::abs(oy) > R) return;
+    at[oy + R][ox + R] = k;
+  }
+  int nr = 0, e = 0;
+  for (int y = 0; y < kMaxRows2; ++y) {
+    int a = 0, b = kMaxRows2 - 1;
+    while (a <= b && at[y][a] < 0) ++a;
+    while (b >= a && at[y][b] < 0) --b;
+    if (a > b) continue;
+    A->rows2[nr] = {(signed char)(a - R), (signed char)(b - R), (signed char)(y - R), (unsigned char)e};
+    for (int x = a; x <= b; ++x) {
+      if (at[y][x] < 0) return;  // a gap
+      A->idx2[e++] = (unsigned char)at[y][x];
+    }
+    ++nr;
+  }
+  A->nrow2 = nr;
+}
+
 int build_stencil(const Geo& geo, int half, Off* out, int cap) {
   int n = 0;
   const int e = half ? build_stencils(geo, cap, out, nullptr, &n, nullptr, nullptr, nullptr)

@@ -41,6 +41,7 @@ struct DevCache {
 };
 
 constexpr int kMaxOff = 768;      // stencil entries (9^3 = 729 plus margin)
+constexpr int kMaxRows2 = 9;      // rows of a 2D stencil, and cells of a row (reach <= 4)
 constexpr int kMaxAxis = 1023;    // cells per axis (10-bit packing)
 constexpr int kMaxBins = 4096;    // histogram bins (shared-memory histogram)
 // Windowed cells of kOctMin to kOctCap particles are ordered by the octant of
@@ -96,6 +97,16 @@ struct SweepArgs {
   // packed per-particle sweep: a neighbour cell whose box lies at least rc
   // from the particle is skipped); 0 turns the test off.
   float ex, ey, ez;
+  // 2D: the stencil as rows of cells (row_sweep): row r covers the offsets
+  // rows2[r].ox0 .. ox1 at oy, whose stencil entries are idx2[e0 ..]. nrow2 = 0
+  // when not given.
+  struct Row2 {
+    signed char ox0, ox1, oy;
+    unsigned char e0;
+  };
+  int nrow2;
+  Row2 rows2[kMaxRows2];
+  unsigned char idx2[kMaxRows2 * kMaxRows2];
   int noff;             // entries in off[]; off[0] is the own cell
   Off off[kMaxOff];
 };
@@ -108,6 +119,9 @@ int build_stencil(const Geo& geo, int half, Off* out, int cap);
 // Both at once; opk_* (optional) receive each entry's unwrapped offset packed
 // as bytes: (ox & 255) | (oy & 255) << 8 | (oz & 255) << 16.
 int build_stencils(const Geo& geo, int cap, Off* half, int* opk_half, int* nhalf, Off* full, int* opk_full, int* nfull);
+// Fills A's rows of cells from a 2D stencil of noff entries (opk as above);
+// leaves nrow2 = 0 when the entries do not form such rows.
+void fill_rows2(const int* opk, int noff, SweepArgs* A);
 // Half-widths of one cell's Cartesian bounding box (sum over the cell edge
 // vectors of |G_k,a| / 2 per axis a), each padded by 1e-3 rc.
 void cell_halfwidths(const Geo& geo, float* e);

@@ -36,14 +36,13 @@ __device__ __forceinline__ int flagged_particle(const SweepArgs& A, const unsign
   return flag[c] ? p : A.n;
 }
 
-template <int DIM>
-__global__ void __launch_bounds__(256) k_sweep_count(const __grid_constant__ SweepArgs A, unsigned long long* out,
-                                                     const unsigned char* __restrict__ flag) {
+// 2D: one thread per particle over the stencil's rows (sweep_flat).
+__global__ void __launch_bounds__(256) k_sweep_count(const __grid_constant__ SweepArgs A, unsigned long long* out) {
   RedCount red;
   RedCount::Acc acc;
   red.init(acc);
   float4 pi;
-  sweep_particle<DIM>(A, red, acc, flagged_particle(A, flag, blockIdx.x * blockDim.x + threadIdx.x), pi);
+  sweep_flat(A, red, acc, blockIdx.x * blockDim.x + threadIdx.x, pi);
   unsigned v = acc.n;
 #pragma unroll
   for (int off = 16; off; off >>= 1) v += __shfl_down_sync(0xffffffffu, v, off);
@@ -51,33 +50,30 @@ __global__ void __launch_bounds__(256) k_sweep_count(const __grid_constant__ Swe
 }
 
 // Scalar FP64 partial per CTA: sum 1/r (kind 0) or shifted-force energy (kind 1).
-template <int DIM, int KIND>
-__global__ void __launch_bounds__(256) k_sweep_scalar(const __grid_constant__ SweepArgs A, double* partials,
-                                                      const unsigned char* __restrict__ flag) {
+template <int KIND>
+__global__ void __launch_bounds__(256) k_sweep_scalar(const __grid_constant__ SweepArgs A, double* partials) {
   float4 pi;
   double v[1];
-  const int p = flagged_particle(A, flag, blockIdx.x * blockDim.x + threadIdx.x);
+  const int p = blockIdx.x * blockDim.x + threadIdx.x;
   if (KIND == 0) {
     RedSumInvR red;
     RedSumInvR::Acc acc;
     red.init(acc);
-    sweep_particle<DIM>(A, red, acc, p, pi);
+    sweep_flat(A, red, acc, p, pi);
     v[0] = (double)acc.s;
   } else {
     RedEnergy red;
     red.irc = A.irc;
     RedEnergy::Acc acc;
     red.init(acc);
-    sweep_particle<DIM>(A, red, acc, p, pi);
+    sweep_flat(A, red, acc, p, pi);
     v[0] = (double)acc.e;
   }
   block_sum_store<1>(v, partials + blockIdx.x);
 }
 
-template <int DIM>
 __global__ void __launch_bounds__(256) k_sweep_hist(const __grid_constant__ SweepArgs A, int nbins, float rmax,
-                                                    unsigned long long* __restrict__ hist,
-                                                    const unsigned char* __restrict__ flag) {
+                                                    unsigned long long* __restrict__ hist) {
   extern __shared__ unsigned sh[];
   for (int b = threadIdx.x; b < nbins; b += blockDim.x) sh[b] = 0u;
   __syncthreads();
@@ -88,7 +84,7 @@ __global__ void __launch_bounds__(256) k_sweep_hist(const __grid_constant__ Swee
   red.sh = sh;
   RedHist::Acc acc;
   float4 pi;
-  sweep_particle<DIM>(A, red, acc, flagged_particle(A, flag, blockIdx.x * blockDim.x + threadIdx.x), pi);
+  sweep_flat(A, red, acc, blockIdx.x * blockDim.x + threadIdx.x, pi);
   __syncthreads();
   for (int b = threadIdx.x; b < nbins; b += blockDim.x)
     if (sh[b]) atomicAdd(&hist[b], (unsigned long long)sh[b]);
@@ -108,7 +104,7 @@ __global__ void __launch_bounds__(256) k_sweep_force(const __grid_constant__ Swe
   red.init(acc);
   float4 pi;
   const int p = blockIdx.x * blockDim.x + threadIdx.x;
-  const bool live = sweep_particle<DIM>(A, red, acc, p, pi);
+  const bool live = sweep_flat(A, red, acc, p, pi);
   constexpr int NW = (DIM == 3) ? kVirN3 : kVirN2;
   constexpr int NV = (MODE == 0) ? 1 + NW : NW + DIM * DIM;
   double v[NV];
@@ -409,7 +405,7 @@ int launch_count(const SweepArgs& A, int dim, unsigned long long* out, cudaStrea
   if (cudaMemsetAsync(out, 0, sizeof(unsigned long long), s) != cudaSuccess) return CL_ERR_CUDA;
   if (A.n > 0) {
     if (dim == 3) k_sweep2_count<<<blocks_for(A.n), 256, 0, s>>>(A, out, nullptr);
-    else k_sweep_count<2><<<blocks_for(A.n), 256, 0, s>>>(A, out, nullptr);
+    else k_sweep_count<<<blocks_for(A.n), 256, 0, s>>>(A, out);
   }
   return cudaGetLastError() == cudaSuccess ? CL_OK : CL_ERR_CUDA;
 }
@@ -422,8 +418,8 @@ int launch_scalar(const SweepArgs& A, int dim, int kind, double* partials, doubl
       if (kind == 0) k_sweep2_suminvr<<<nb, 256, 0, s>>>(A, partials, nullptr);
       else k_sweep2_energy<<<nb, 256, 0, s>>>(A, partials);
     } else {
-      if (kind == 0) k_sweep_scalar<2, 0><<<nb, 256, 0, s>>>(A, partials, nullptr);
-      else k_sweep_scalar<2, 1><<<nb, 256, 0, s>>>(A, partials, nullptr);
+      if (kind == 0) k_sweep_scalar<0><<<nb, 256, 0, s>>>(A, partials);
+      else k_sweep_scalar<1><<<nb, 256, 0, s>>>(A, partials);
     }
   } else {
     if (cudaMemsetAsync(partials, 0, sizeof(double), s) != cudaSuccess) return CL_ERR_CUDA;
@@ -441,7 +437,7 @@ int launch_hist(const SweepArgs& A, int dim, int nbins, float rmax, unsigned lon
       k_sweep2_hist<<<blocks_for(A.n), 256, smem, s>>>(A, nbins, scale2, xlim, hist, nullptr);
     }
     else {
-      k_sweep_hist<2><<<blocks_for(A.n), 256, smem, s>>>(A, nbins, rmax, hist, nullptr);
+      k_sweep_hist<<<blocks_for(A.n), 256, smem, s>>>(A, nbins, rmax, hist);
     }
   }
   return cudaGetLastError() == cudaSuccess ? CL_OK : CL_ERR_CUDA;

@@ -181,6 +181,62 @@ __device__ __forceinline__ bool sweep_particle(const ARGS& A, const R& red, type
   return true;
 }
 
+// sweep_particle for 2D lists, row by row: the cells of a row of the stencil
+// are one contiguous range of the sorted arrays (two where it crosses the box
+// edge), so a lane runs over the row's particles in one loop and takes each
+// one's shift from its cell's column. The cells of a 2D grid hold about one
+// particle: cell by cell, a warp's 25 inner loops ran as long as their fullest
+// lane's (2.8 passes for 1.1 particles), and each cell cost its own index
+// arithmetic and two loads. sh: the CTA's table of shifts (load_rows2).
+template <class R>
+__device__ __forceinline__ bool row_sweep(const SweepArgs& A, const float2* sh, const R& red, typename R::Acc& acc,
+                                          int p, float4& pi) {
+  if (p >= A.n) return false;
+  pi = A.xs[p];
+  const unsigned cc = A.cellc[p];
+  const int cx = (int)(cc & 1023u), cy = (int)((cc >> 10) & 1023u);
+  for (int r = 0; r < A.nrow2; ++r) {
+    const SweepArgs::Row2 row = A.rows2[r];
+    int y = cy + row.oy;
+    if ((unsigned)y >= (unsigned)A.ny) y = (y % A.ny + A.ny) % A.ny;
+    bool own = !R::kFull && row.oy == 0;  // half shell: this row starts at the particle itself
+    for (int ox = row.ox0; ox <= row.ox1;) {
+      int x = cx + ox;
+      if ((unsigned)x >= (unsigned)A.nx) x = (x % A.nx + A.nx) % A.nx;
+      const int len = min(row.ox1 - ox + 1, A.nx - x);
+      const int* s = A.cell_start + x + A.nx * y;
+      const int j1 = s[len];
+      const float2* const sx = sh + ((int)row.e0 + ox - row.ox0 - x);  // shift of the cell in column c: sx[c]
+      for (int j = own ? p + 1 : s[0]; j < j1; ++j) {
+        const float4 q = __ldg(&A.xs[j]);
+        const float2 t = sx[__ldg(&A.cellc[j]) & 1023u];
+        const float dx = q.x - (pi.x - t.x), dy = q.y - (pi.y - t.y);
+        const float d2 = fmaf(dx, dx, dy * dy);
+        if (d2 < A.rc2 && (!R::kFull || j != p)) red.hit(acc, dx, dy, 0.f, d2, __float_as_int(q.w));
+      }
+      own = false;
+      ox += len;
+    }
+  }
+  return true;
+}
+
+__device__ __forceinline__ void load_rows2(const SweepArgs& A, float2* sh) {
+  if (A.nrow2 > 0 && threadIdx.x < A.rows2[A.nrow2 - 1].e0 + A.rows2[A.nrow2 - 1].ox1 - A.rows2[A.nrow2 - 1].ox0 + 1) {
+    const Off& o = A.off[A.idx2[threadIdx.x]];
+    sh[threadIdx.x] = make_float2(o.sx, o.sy);
+  }
+  __syncthreads();
+}
+
+// A 2D list by rows when they are given, else cell by cell.
+template <class R>
+__device__ __forceinline__ bool sweep_flat(const SweepArgs& A, const R& red, typename R::Acc& acc, int p, float4& pi) {
+  __shared__ float2 sh[kMaxRows2 * kMaxRows2];
+  load_rows2(A, sh);
+  return A.nrow2 > 0 ? row_sweep(A, sh, red, acc, p, pi) : sweep_particle<2>(A, red, acc, p, pi);
+}
+
 // ------------------------------------------------- packed (f32x2) sweep, 3D
 // Two neighbour candidates per iteration in packed FP32 (one instruction
 // computes both lanes of a float2): the same FMA-pipe work as the scalar loop
