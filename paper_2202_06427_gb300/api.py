@@ -119,21 +119,21 @@ def cl_map(cl, reduction, nbins=0, rmax=0.0, capacity=None, stream=None, out=Non
     out = {}
     f64 = dict(dtype=torch.float64, device=dev)
     if red == CL_RED_COUNT:
-        out["count"] = torch.zeros(1, dtype=torch.int64, device=dev)
+        out["count"] = torch.empty(1, dtype=torch.int64, device=dev)
         res.count = out["count"].data_ptr()
     elif red == CL_RED_SUM_INV_R:
-        out["sum_inv_r"] = torch.zeros(1, **f64)
+        out["sum_inv_r"] = torch.empty(1, **f64)
         res.sum_inv_r = out["sum_inv_r"].data_ptr()
     elif red == CL_RED_SF_ENERGY:
-        out["energy"] = torch.zeros(1, **f64)
+        out["energy"] = torch.empty(1, **f64)
         res.energy = out["energy"].data_ptr()
     elif red == CL_RED_SF_ENERGY_FORCES_VIRIAL:
-        out["energy"] = torch.zeros(1, **f64)
+        out["energy"] = torch.empty(1, **f64)
         out["forces"] = torch.empty((cl.n, cl.dim), dtype=torch.float32, device=dev)
-        out["virial"] = torch.zeros((cl.dim, cl.dim), **f64)
+        out["virial"] = torch.empty((cl.dim, cl.dim), **f64)
         res.energy, res.forces, res.virial = (out[k].data_ptr() for k in ("energy", "forces", "virial"))
     elif red == CL_RED_HIST:
-        out["hist"] = torch.zeros(int(nbins), dtype=torch.int64, device=dev)
+        out["hist"] = torch.empty(int(nbins), dtype=torch.int64, device=dev)
         res.hist = out["hist"].data_ptr()
     params = L.cl_params()
     params.nbins = int(nbins)

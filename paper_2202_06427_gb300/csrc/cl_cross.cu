@@ -183,19 +183,63 @@ __global__ void __launch_bounds__(32 * kFillWarps, 5) k_cross_fill(const __grid_
   }
 }
 
-// A warp's running best k of (distance, id), ascending, entry l in lane l
-// (l < k): offers the lanes' candidates (ok ones) and keeps the k smallest.
 template <class ID>
-__device__ __forceinline__ void best_offer(float& bd, ID& bi, float& kd, ID& ki, int k, bool ok, float d, ID id) {
+__device__ __forceinline__ bool nearer(float d, ID i, float e, ID j) {
+  return d < e || (d == e && i < j);
+}
+
+// One compare-exchange of a lane with its partner, `up` when it keeps the nearer.
+template <class ID>
+__device__ __forceinline__ void nearer_exchange(float& d, ID& i, int mask, bool up) {
+  const float e = __shfl_xor_sync(0xffffffffu, d, mask);
+  const ID j = __shfl_xor_sync(0xffffffffu, i, mask);
+  const bool take = nearer(e, j, d, i) == up && !(e == d && j == i);
+  d = take ? e : d;
+  i = take ? j : i;
+}
+
+// A warp's running best k of (distance, id), ascending, entry l in lane l
+// (the lanes past k hold what was pushed out): offers the lanes' candidates
+// (ok ones) and keeps the k smallest. A few candidates are inserted one by
+// one; more than kBulk, as in the first steps, when nearly every lane has one,
+// are sorted across the warp and merged with the list at once (25 against 190
+// instructions: 8 nearest and 5 closest of 60,000 queries 449 -> 418 us).
+constexpr int kBulk = 6;
+
+template <class ID>
+__device__ __forceinline__ void best_offer(float& bd, ID& bi, float& kd, ID& ki, int k, bool ok, float d, ID id,
+                                           float none_d, ID none_i) {
   const int lane = threadIdx.x & 31;
-  unsigned m = __ballot_sync(0xffffffffu, ok && (d < kd || (d == kd && id < ki)));
+  ok = ok && nearer(d, id, kd, ki);
+  unsigned m = __ballot_sync(0xffffffffu, ok);
+  if (__popc(m) > kBulk) {
+    d = ok ? d : none_d;
+    id = ok ? id : none_i;
+#pragma unroll
+    for (int size = 2; size <= 32; size <<= 1)
+#pragma unroll
+      for (int st = size >> 1; st > 0; st >>= 1)
+        nearer_exchange(d, id, st, ((lane & st) == 0) == ((lane & size) == 0 || size == 32));
+    // the 32 nearest of both lists: entry l against the other's 31 - l, a
+    // bitonic sequence, merged in five steps
+    const float rd = __shfl_sync(0xffffffffu, d, 31 - lane);
+    const ID ri = __shfl_sync(0xffffffffu, id, 31 - lane);
+    const bool take = nearer(rd, ri, bd, bi);
+    bd = take ? rd : bd;
+    bi = take ? ri : bi;
+#pragma unroll
+    for (int st = 16; st > 0; st >>= 1) nearer_exchange(bd, bi, st, (lane & st) == 0);
+    kd = __shfl_sync(0xffffffffu, bd, k - 1);
+    ki = __shfl_sync(0xffffffffu, bi, k - 1);
+    return;
+  }
   while (m) {
     const int src = __ffs(m) - 1;
     m &= m - 1;
     const float cd = __shfl_sync(0xffffffffu, d, src);
     const ID ci = __shfl_sync(0xffffffffu, id, src);
-    if (!(cd < kd || (cd == kd && ci < ki))) continue;  // uniform: a better one came in since
-    const bool before = lane < k && (bd < cd || (bd == cd && bi <= ci));
+    if (!nearer(cd, ci, kd, ki)) continue;  // uniform: a better one came in since
+    const bool before = lane < k && !nearer(cd, ci, bd, bi);
     const int at = __popc(__ballot_sync(0xffffffffu, before));
     const float ud = __shfl_up_sync(0xffffffffu, bd, 1);
     const ID ui = __shfl_up_sync(0xffffffffu, bi, 1);
@@ -251,7 +295,7 @@ __global__ void __launch_bounds__(32 * kCrossWarps) k_cross_knn(const __grid_con
             d2 = query_d2(q, s);
           }
           j += G;
-          best_offer(bd, ba, kd, ka, k, d2 < A.rc2, d2, a);
+          best_offer(bd, ba, kd, ka, k, d2 < A.rc2, d2, a, FLT_MAX, INT_MAX);
         }
       }
     }
@@ -281,7 +325,7 @@ __global__ void __launch_bounds__(32 * kTopkWarps) k_topk_part(const int* __rest
   for (long long e0 = w * share; e0 < e1; e0 += 32) {
     const long long e = e0 + lane;
     const bool ok = e < e1 && la[e] >= 0;
-    best_offer(bd, bi, kd, ki, k, ok, ok ? ld[e] : INFINITY, e);
+    best_offer(bd, bi, kd, ki, k, ok, ok ? ld[e] : INFINITY, e, INFINITY, LLONG_MAX);
   }
   if (lane < k) {
     part_d[w * k + lane] = bd;
@@ -301,7 +345,7 @@ __global__ void __launch_bounds__(1024) k_topk_last(const int* __restrict__ la, 
   for (long long e0 = warp * 32LL; e0 < m; e0 += 1024) {
     const long long e = e0 + lane;
     const long long id = e < m ? part_id[e] : LLONG_MAX;
-    best_offer(bd, bi, kd, ki, k, id != LLONG_MAX, e < m ? part_d[e] : INFINITY, id);
+    best_offer(bd, bi, kd, ki, k, id != LLONG_MAX, e < m ? part_d[e] : INFINITY, id, INFINITY, LLONG_MAX);
   }
   if (lane < k) {
     sd[warp * k + lane] = bd;
@@ -311,7 +355,8 @@ __global__ void __launch_bounds__(1024) k_topk_last(const int* __restrict__ la, 
   if (warp) return;
   bd = kd = INFINITY;
   bi = ki = LLONG_MAX;
-  for (int e = lane; e < 32 * k; e += 32) best_offer(bd, bi, kd, ki, k, sid[e] != LLONG_MAX, sd[e], sid[e]);
+  for (int e = lane; e < 32 * k; e += 32)
+    best_offer(bd, bi, kd, ki, k, sid[e] != LLONG_MAX, sd[e], sid[e], INFINITY, LLONG_MAX);
   const bool ok = lane < k && bi != LLONG_MAX;
   if (lane < k) {
     oa[lane] = ok ? la[bi] : -1;
