@@ -40,6 +40,7 @@
 // to one buffer.
 #include <algorithm>
 #include <cmath>
+#include <cstddef>
 #include <cstring>
 
 #include "cl_sweep.cuh"
@@ -1414,7 +1415,7 @@ constexpr int kBatch = 32;          // home particles of a batch, swept by one w
 static_assert(kWarps * kBatch == kHome, "the batches' force sums share the fast path's");
 // Small cells: the cell and its half neighbourhood in one warp's share of the
 // entry buffer, its row segments in the warp's share of the segment table.
-constexpr int kSmallCap = (kHCap + 32) / kWarps & ~31;
+constexpr int kSmallCap = (kHCap / kWarps) & ~31;
 constexpr int kSmallSegs = 32;
 static_assert(kWarps * kSmallCap <= kHCap && kWarps * kSmallSegs <= kTab, "the warps' shares fit");
 
@@ -1430,14 +1431,12 @@ struct HalfSmem {
   HalfCtx ctx;
   float4 ent[kHCap + 32];  // (x, y, z in the home frame, sorted position as int bits); 32 trash entries
   unsigned short img[kHCap];  // lattice image of the T != 0 entries, (tx, ty, tz) as 5-bit signed fields
-  unsigned short wlist[kWarps][kChunk + 32];  // windowed cells: a warp's staged entries within its batch's ball
   // home particles (-x, -y, -z, sorted position), padded by far entries: the
   // cell's (fast path), or kBatch + 4 per warp (windowed cells)
   float4 home[kWarps * (kBatch + 4)];
   float4 own[kHome];       // the same with (x, y, z): the own cell's entries
   float hg[kHome][3];      // per home particle: sum of fsn r over its entries
   float4 otab[kTab];       // half stencil: (shift x, y, z, unwrapped offset as int bits)
-  int4 seg[kTab];          // windowed cells: row segments (first particle, flattened start, ebase, back | image << 1)
   unsigned short rowk[kTab + 1];
   int nrows, nseg, ctot;
   int oct[9];              // windowed cells: octant ranges of the cell's particles
@@ -1447,7 +1446,17 @@ struct HalfSmem {
   int nf, nb, item, next, nl;
   unsigned long long ncand;
   double out[kWarps][16];
+  // the batches' part: k_hood_half is launched without it
+  int4 seg[kTab];          // windowed cells: row segments (first particle, flattened start, ebase, back | image << 1)
+  unsigned short wlist[kWarps][kChunk + 32];  // windowed cells: a warp's staged entries within its batch's ball
 };
+
+// Six CTAs of k_hood_half fit an SM: 80 registers, and shared memory up to the
+// batches' part (1M lattice, whole step: 1.47 ms with five at 96 registers,
+// 1.43 with six). k_half_batch spills at 80 and stays at five.
+constexpr int kHalfCtas = 6;
+constexpr size_t kHalfBytes = offsetof(HalfSmem, seg);
+static_assert(kHalfCtas * (kHalfBytes + 1024) <= 228 * 1024, "shared memory of an SM, 1 KB of it per CTA reserved");
 
 // Row segment of the half stencil (the same walk as row_segment) with the
 // segment's lattice image packed as bytes.
@@ -2305,7 +2314,7 @@ __device__ __forceinline__ void half_partials(const HoodArgs& H, const HalfSmem&
 // (k_hood_list goes by the expected share of the raw one) is moved to the
 // dense list, which k_half_batch takes afterwards.
 template <int MODE>
-__global__ void __launch_bounds__(kThreads, 5) k_hood_half(const __grid_constant__ SweepArgs A,
+__global__ void __launch_bounds__(kThreads, kHalfCtas) k_hood_half(const __grid_constant__ SweepArgs A,
                                                            const __grid_constant__ HoodArgs H,
                                                            double* __restrict__ partials) {
   constexpr bool ENERGY = MODE != 1;
@@ -2663,38 +2672,40 @@ size_t half_mode_smem(int mode) {
   return sizeof(HalfSmem) + (mode == 6 ? sizeof(unsigned) * (size_t)hist_stride(kMaxBins) : 0);
 }
 
-template <int M>
-cudaError_t half_setup(int bytes, int* per) {
-  cudaError_t e = cudaFuncSetAttribute(k_half_batch<M>, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
-  if constexpr (M < 2 || M == 3) {
-    if (e == cudaSuccess) e = cudaFuncSetAttribute(k_hood_half<M>, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
-  }
-  if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(per, k_half_batch<M>, kThreads, bytes);
-  return e;
+template <class K>
+cudaError_t half_setup(K kernel, int bytes, int* per) {
+  cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
+  return e == cudaSuccess ? cudaOccupancyMaxActiveBlocksPerMultiprocessor(per, kernel, kThreads, bytes) : e;
 }
 
-// Persistent CTAs of the half-shell sweep, per mode (0, 1, 3; scalar 2, 4,
-// 5, 6); also raises the kernels' shared-memory limit on the current device.
-int half_grid(int mode) {
-  static DevCache cached[7];
+// Persistent CTAs of k_half_batch<mode>, and with fast of k_hood_half<mode>
+// (modes 0, 1, 3); also raises the kernel's shared-memory limit on the current
+// device.
+int half_grid(int mode, bool fast = false) {
+  static DevCache cached[2][7];
   if (mode < 0 || mode > 6) return 0;
   int dev = 0, sms = 0, per = 0;
   if (cudaGetDevice(&dev) != cudaSuccess) return 0;
-  if (const int c = cached[mode].get(dev)) return c;
+  if (const int c = cached[fast][mode].get(dev)) return c;
   if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) return 0;
-  const int bytes = (int)half_mode_smem(mode);
+  const int bytes = fast ? (int)kHalfBytes : (int)half_mode_smem(mode);
   cudaError_t e;
-  switch (mode) {
-    case 0: e = half_setup<0>(bytes, &per); break;
-    case 1: e = half_setup<1>(bytes, &per); break;
-    case 3: e = half_setup<3>(bytes, &per); break;
-    case 2: e = half_setup<2>(bytes, &per); break;
-    case 4: e = half_setup<4>(bytes, &per); break;
-    case 5: e = half_setup<5>(bytes, &per); break;
-    default: e = half_setup<6>(bytes, &per); break;
+  if (fast) {
+    e = mode == 0 ? half_setup(k_hood_half<0>, bytes, &per)
+                  : (mode == 1 ? half_setup(k_hood_half<1>, bytes, &per) : half_setup(k_hood_half<3>, bytes, &per));
+  } else {
+    switch (mode) {
+      case 0: e = half_setup(k_half_batch<0>, bytes, &per); break;
+      case 1: e = half_setup(k_half_batch<1>, bytes, &per); break;
+      case 3: e = half_setup(k_half_batch<3>, bytes, &per); break;
+      case 2: e = half_setup(k_half_batch<2>, bytes, &per); break;
+      case 4: e = half_setup(k_half_batch<4>, bytes, &per); break;
+      case 5: e = half_setup(k_half_batch<5>, bytes, &per); break;
+      default: e = half_setup(k_half_batch<6>, bytes, &per); break;
+    }
   }
   if (e != cudaSuccess || per < 1) return 0;
-  cached[mode].put(dev, sms * per);
+  cached[fast][mode].put(dev, sms * per);
   return sms * per;
 }
 
@@ -2943,29 +2954,30 @@ int launch_hood(const SweepArgs& A, const SweepArgs* Ahalf, const HoodArgs& Hin,
   if (half) {
     // every non-empty cell: fast-path sweep or sweep by batches, then the
     // per-particle finish; partials [fast][batches][finish]
-    int nhb = half_grid(mode);
+    int nhf = half_grid(mode, true), nhb = half_grid(mode);
     const int nfin = std::min(nrest, 152 * 8);
-    if (nhb <= 0) return CL_ERR_CUDA;
-    if (nhb > Hin.ncells) nhb = Hin.ncells;
-    if (2 * nhb > partials_cap / NV - nfin) nhb = (int)((partials_cap / NV - nfin) / 2);
-    if (nhb < 1) return CL_ERR_INVALID_ARG;
-    double* pwin = partials + (size_t)nhb * NV;
+    if (nhf <= 0 || nhb <= 0) return CL_ERR_CUDA;
+    const int most = (int)std::min<long long>(Hin.ncells, (partials_cap / NV - nfin) / 2);
+    nhf = std::min(nhf, most);
+    nhb = std::min(nhb, most);
+    if (most < 1) return CL_ERR_INVALID_ARG;
+    double* pwin = partials + (size_t)nhf * NV;
     double* pfin = pwin + (size_t)nhb * NV;
     const size_t hsmem = sizeof(HalfSmem);
     if (mode == 0) {
-      k_hood_half<0><<<nhb, kThreads, hsmem, s>>>(*Ahalf, H, partials);
+      k_hood_half<0><<<nhf, kThreads, kHalfBytes, s>>>(*Ahalf, H, partials);
       k_half_batch<0><<<nhb, kThreads, hsmem, s>>>(*Ahalf, H, pwin);
       k_half_finish<0><<<nfin, 256, 0, s>>>(*Ahalf, H, forces, grad, gE, pos, pfin);
     } else if (mode == 1) {
-      k_hood_half<1><<<nhb, kThreads, hsmem, s>>>(*Ahalf, H, partials);
+      k_hood_half<1><<<nhf, kThreads, kHalfBytes, s>>>(*Ahalf, H, partials);
       k_half_batch<1><<<nhb, kThreads, hsmem, s>>>(*Ahalf, H, pwin);
       k_half_finish<1><<<nfin, 256, 0, s>>>(*Ahalf, H, forces, grad, gE, pos, pfin);
     } else {
-      k_hood_half<3><<<nhb, kThreads, hsmem, s>>>(*Ahalf, H, partials);
+      k_hood_half<3><<<nhf, kThreads, kHalfBytes, s>>>(*Ahalf, H, partials);
       k_half_batch<3><<<nhb, kThreads, hsmem, s>>>(*Ahalf, H, pwin);
       k_half_finish<3><<<nfin, 256, 0, s>>>(*Ahalf, H, forces, grad, gE, pos, pfin);
     }
-    return finish_reduction(final_mode, 3, hinv, 2 * nhb + nfin, NV, partials, sums, energy, virial, gradbox, gE, s);
+    return finish_reduction(final_mode, 3, hinv, nhf + nhb + nfin, NV, partials, sums, energy, virial, gradbox, gE, s);
   }
   // full-shell kernels (and the half-stencil energy, mode 2): partials
   // [neighbourhood sweep][companion][dense cells]
