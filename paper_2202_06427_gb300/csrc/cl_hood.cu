@@ -73,8 +73,6 @@ struct Smem {
   float2 zz[kCap / 2 + 16];  // (z_2k, z_2k+1)
   float4 oxy[kHome / 2]; // own cell in sorted order, same layout
   float2 ozz[kHome / 2];
-  int hid[kHome];        // original index of the home particle
-  float acc[kHome][6];   // Gn of the neighbours across the boundary (T != 0) and of the others (T = 0)
   float4 otab[kTab];     // stencil entry: (shift x, y, z, unwrapped offset as int bits)
   unsigned short rowk[kTab + 1];  // rows of the stencil: entries [rowk[r], rowk[r + 1])
   int nrows;
@@ -83,7 +81,14 @@ struct Smem {
   int item, part;
   unsigned long long ncand;  // candidate pairs this CTA evaluated
   double out[kWarps][16];    // per-warp sums: share of sum fsn r (x) r (6), X (9), energy (1)
+  // the force modes' part: the others are launched without it
+  int hid[kHome];        // original index of the home particle
+  float acc[kHome][6];   // Gn of the neighbours across the boundary (T != 0) and of the others (T = 0)
 };
+
+// Resident CTAs per SM and shared memory of k_hood<mode>.
+__host__ __device__ constexpr int hood_ctas(int mode) { return mode == 2 || mode >= 4 ? 6 : 5; }
+__host__ __device__ constexpr size_t hood_bytes(int mode) { return mode == 2 || mode >= 4 ? offsetof(Smem, hid) : sizeof(Smem); }
 
 __device__ __forceinline__ void unpack_off(int v, int& ox, int& oy, int& oz) {
   ox = (int)(signed char)(v & 0xff);
@@ -1116,7 +1121,7 @@ __global__ void __launch_bounds__(kDenseThreads, 3) k_hood_dense(const __grid_co
 // 1/r, distance histogram (half shell; the histogram in dynamic shared memory
 // after Smem).
 template <int MODE>
-__global__ void __launch_bounds__(kThreads, 5) k_hood(const __grid_constant__ SweepArgs A, const __grid_constant__ HoodArgs H,
+__global__ void __launch_bounds__(kThreads, hood_ctas(MODE)) k_hood(const __grid_constant__ SweepArgs A, const __grid_constant__ HoodArgs H,
                                                       float* __restrict__ forces, double* __restrict__ grad,
                                                       const double* __restrict__ gE, const double* __restrict__ pos,
                                                       double* __restrict__ partials) {
@@ -1140,7 +1145,7 @@ __global__ void __launch_bounds__(kThreads, 5) k_hood(const __grid_constant__ Sw
   R.rc2 = A.rc2;
   R.scale2 = H.hscale * H.hscale;
   R.xlim = H.hxlim;
-  unsigned* const hist_all = reinterpret_cast<unsigned*>(smraw + sizeof(Smem));
+  unsigned* const hist_all = reinterpret_cast<unsigned*>(smraw + hood_bytes(MODE));
   R.hist = hist_all + (lane & (H.hcopies - 1)) * H.hstride;
   if (MODE == 6)
     for (int b = tid; b < H.hcopies * H.hstride; b += kThreads) hist_all[b] = 0u;
@@ -1188,7 +1193,7 @@ __global__ void __launch_bounds__(kThreads, 5) k_hood(const __grid_constant__ Sw
     if (tid < nh) {
       const float4 hq = A.xs[hs + tid];
       d = fminf(sqrtf(fmaf(hq.x, hq.x, fmaf(hq.y, hq.y, hq.z * hq.z))), H.hd);
-      S.hid[tid] = __float_as_int(hq.w);
+      if (FORCE) S.hid[tid] = __float_as_int(hq.w);
       if (GRAD) prefetch_l1(pos + (size_t)__float_as_int(hq.w) * 3);
       oxyf[(tid >> 1) * 4 + (tid & 1)] = hq.x;
       oxyf[(tid >> 1) * 4 + 2 + (tid & 1)] = hq.y;
@@ -2628,10 +2633,11 @@ __global__ void __launch_bounds__(256) k_half_finish(const __grid_constant__ Swe
 
 // Shared memory of k_hood<mode>: Smem, and for the histogram its copies (the
 // most of the size the grid is sized for; at least one copy).
-constexpr int kHistWords = 1408;  // histogram copies fitting five CTAs per SM
+constexpr int kHistWords = 576;  // histogram copies that leave six CTAs of k_hood per SM
+static_assert(6 * (hood_bytes(6) + kHistWords * sizeof(unsigned) + 1024) <= 228 * 1024, "they do");
 static_assert(hist_stride(kMaxBins) >= kHistWords, "the largest histogram bounds every copy set");
 size_t hood_mode_smem(int mode) {
-  return sizeof(Smem) + (mode == 6 ? sizeof(unsigned) * (size_t)hist_stride(kMaxBins) : 0);
+  return hood_bytes(mode) + (mode == 6 ? sizeof(unsigned) * (size_t)hist_stride(kMaxBins) : 0);
 }
 int hist_copies(int nbins) {
   int c = 8;
@@ -2795,7 +2801,7 @@ int launch_hood_scalar(const SweepArgs& A, const HoodArgs& Hin, int* work, int k
   if (lists_half) *lists_half = half ? 1 : 0;
   // grids: the home-major kernel, and (half) the windowed kernel
   const size_t hist_bytes = kind == 2 ? sizeof(unsigned) * (size_t)H.hcopies * H.hstride : 0;
-  const size_t smem = sizeof(Smem) + hist_bytes, hsmem = sizeof(HalfSmem) + hist_bytes;
+  const size_t smem = hood_bytes(mode) + hist_bytes, hsmem = sizeof(HalfSmem) + hist_bytes;
   if (hood_grid(mode) <= 0 || (half && half_grid(mode) <= 0)) return CL_ERR_CUDA;  // also raise the smem limits
   int nb = 0, nhb = 0;
   switch (mode) {
@@ -2989,7 +2995,7 @@ int launch_hood(const SweepArgs& A, const SweepArgs* Ahalf, const HoodArgs& Hin,
   if (nb < 1) return CL_ERR_INVALID_ARG;
   double* rest = partials + (size_t)nb * NV;
   double* dpart = rest + (size_t)nrest * NV;
-  const size_t smem = sizeof(Smem);
+  const size_t smem = hood_bytes(mode);
   const size_t dsmem = dense_smem_bytes(A.noff);
   if (mode == 0) {
     k_hood<0><<<nb, kThreads, smem, s>>>(A, H, forces, grad, gE, pos, partials);
