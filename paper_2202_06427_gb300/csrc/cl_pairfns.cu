@@ -1,19 +1,16 @@
 // cl_pairfns.cu -- C entry points for the mapped functions of the paper's
 // examples (Code 5, 6, 7, 10).
 //
-// The mass-weighted sum and the velocity histogram run in 3D on sweeps of their
-// own below, one thread per cell-sorted particle like the ready-made device
-// functors of cellmap_pairfns.cuh and adding each particle's terms in the
-// functors' order, so that their FP32 sums round alike: two candidates per step
-// in packed FP32, cells beyond the cutoff skipped, the particles' masses or
-// velocities read in cell order. 2D, and the Lennard-Jones functions, run the
-// functors on the compile-time hook of cellmap_functor.cuh, as a user's own
+// In 3D the Lennard-Jones energy and forces, the mass-weighted sum and the
+// velocity histogram run on sweeps of their own below, one thread per
+// cell-sorted particle like the ready-made device functors of
+// cellmap_pairfns.cuh, and add each particle's terms in the functors' order, so
+// that their FP32 sums round alike. 2D, and the Lennard-Jones energy alone, run
+// the functors on the compile-time hook of cellmap_functor.cuh, as a user's own
 // would. (The half-shell sweep of cl_hood.cu does Lennard-Jones forces in half
-// the time, 0.74 against 1.57 ms at 500,000 particles, but its energy, summed
-// pair by pair instead of per particle from both ends, differs from the
-// functor's by 5e-9; a full-shell sweep of its own, every candidate's term in
-// packed FP32, is bound by the FMA pipe: 1.46 ms, and slower than the functor
-// at one cell per cutoff. Both were left out.)
+// the functor's time, 0.74 against 1.57 ms at 500,000 particles, but its
+// energy, summed pair by pair instead of per particle from both ends, differs
+// from the functor's by 5e-9; it was left out.)
 #include "cellmap_pairfns.cuh"
 #include "cl_sweep.cuh"
 
@@ -166,6 +163,72 @@ __global__ void k_sweep_velocity(const __grid_constant__ SweepArgs A, const floa
   }
 }
 
+// 1/v to FP32 rounding: the hardware reciprocal and one Newton-Raphson step.
+__device__ __forceinline__ float recip(float v) {
+  float w;
+  asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(w) : "f"(v));
+  return fmaf(w, fmaf(-v, w, 1.0f), w);
+}
+
+// Lennard-Jones energy and forces, full shell, one thread per sorted particle:
+// the functor's sweep and its sums term by term, without its IEEE division (a
+// warp has a pair within the cutoff at nearly every step) and without the cells
+// beyond the cutoff. Bound by issue: step of 500,000 particles, cutoff 12, two
+// cells per cutoff 1.56 -> 1.41 ms, 940,000 at one cell 3.92 -> 3.86.
+// Every candidate's term in packed FP32, masked (FMA pipe), 1.46 ms, and a warp
+// per cell over the particles of the cell's ball, 1.39 ms, were slower on cells
+// of 13 or of 170 particles.
+__global__ void __launch_bounds__(256) k_sweep_lj(const __grid_constant__ SweepArgs A, float rc2, float eps4,
+                                                  float eps24, float s2, float* __restrict__ forces,
+                                                  double* __restrict__ partials) {
+  const int p = blockIdx.x * blockDim.x + threadIdx.x;
+  float e = 0.f;
+  if (p < A.n) {
+    const float4 pi = A.xs[p];
+    const unsigned cc = A.cellc[p];
+    const int cx = (int)(cc & 1023u), cy = (int)((cc >> 10) & 1023u), cz = (int)(cc >> 20);
+    float fx = 0.f, fy = 0.f, fz = 0.f;
+    auto scan = [&](int j0, int j1, float ax, float ay, float az) {
+#pragma unroll 2
+      for (int j = j0; j < j1; ++j) {
+        const float4 q = __ldg(&A.xs[j]);
+        const float dx = q.x - ax, dy = q.y - ay, dz = q.z - az;
+        const float d2 = fmaf(dx, dx, fmaf(dy, dy, dz * dz));
+        if (d2 < rc2) {
+          const float y2 = recip(d2);
+          const float r = s2 * y2, r3 = r * r * r;
+          const float w = fmaf(r3, r3, -r3);
+          const float g = fmaf(r3, r3, w) * -eps24 * y2;
+          fx = fmaf(g, dx, fx);
+          fy = fmaf(g, dy, fy);
+          fz = fmaf(g, dz, fz);
+          e = fmaf(eps4, w, e);
+        }
+      }
+    };
+    {
+      const int c = cx + A.nx * (cy + A.ny * cz);
+      scan(A.cell_start[c], p, pi.x, pi.y, pi.z);
+      scan(p + 1, A.cell_start[c + 1], pi.x, pi.y, pi.z);
+    }
+    for (int k = 1; k < A.noff; ++k) {
+      const Off& o = A.off[k];
+      const float ax = pi.x - o.sx, ay = pi.y - o.sy, az = pi.z - o.sz;
+      const float bx = fmaxf(fabsf(ax) - A.ex, 0.f), by = fmaxf(fabsf(ay) - A.ey, 0.f),
+                  bz = fmaxf(fabsf(az) - A.ez, 0.f);
+      if (fmaf(bx, bx, fmaf(by, by, bz * bz)) >= rc2) continue;  // the whole cell is beyond the cutoff
+      const int c = stencil_cell(A, k, cx, cy, cz);
+      scan(A.cell_start[c], A.cell_start[c + 1], ax, ay, az);
+    }
+    float* f = forces + (size_t)__float_as_int(pi.w) * 3;
+    f[0] = fx;
+    f[1] = fy;
+    f[2] = fz;
+  }
+  double v[1] = {0.5 * (double)e};
+  block_sum_store<1>(v, partials + blockIdx.x);
+}
+
 // The functors' cutoff test: the FP32 cutoff squared in FP32.
 float functor_rc2(double rc) { return (float)rc * (float)rc; }
 
@@ -227,6 +290,16 @@ extern "C" int cl_map_lj(const cl_list* cl, double eps, double sigma, double* en
     f.s2 = (float)(sigma * sigma);
     f.out = energy_dev;
     return cellmap::map(cl, f, s);
+  }
+  clk::ListParts L;
+  clk::list_parts(cl, &L);
+  if (L.hforce && v.n > 0) {
+    const int blocks = (v.n + 255) / 256;
+    clk::k_sweep_lj<<<blocks, 256, 0, s>>>(*L.full, clk::functor_rc2(L.rc), (float)(4.0 * eps), (float)(24.0 * eps),
+                                           (float)(sigma * sigma), forces_dev, L.partials);
+    if (cudaGetLastError() != cudaSuccess) return CL_ERR_CUDA;
+    return clk::finish_reduction(0, 3, nullptr, blocks, 1, L.partials, L.sums, energy_dev, nullptr, nullptr, nullptr,
+                                 s);
   }
   cellmap::pairfn::LennardJonesForces f;
   f.eps4 = (float)(4.0 * eps);
