@@ -36,7 +36,7 @@ struct cl_list {
   int* work;  // work counters of the persistent neighbourhood sweeps
   float4* hforce;  // per sorted particle: forces accumulated by the half-shell sweep (kept zero between launches)
   int last_half;   // the last 3D energy/force sweep took the half-shell path
-  int lists_half;  // hlist / hdense / work[6..7] hold the half-shell work lists of the current cell list
+  int lists_half;  // hlist / hdense / work[6..8] hold the half-shell work lists of the current cell list
   unsigned long long* u64;
   // neighbour-list workspace, allocated on the first CL_RED_PAIRLIST call
   int* pl_count;
@@ -286,25 +286,26 @@ int map_pairlist(cl_list* c, cl_result* r, cudaStream_t s) {
   }
   const int dim = c->geo.dim;
   const float ball2 = pairs_ball2(c->geo);
-  // hflag / hlist: per-cell flags and the flagged cells (shared with the
-  // neighbourhood sweep, which rewrites them on every launch); pl_meta[4]: their number
+  // hflag / hlist: per-cell flags and the flagged cells, hdense: the cells'
+  // largest indices (shared with the neighbourhood sweep, which rewrites them
+  // on every launch); pl_meta[4]: the flagged cells' number, pl_meta[3]: the
+  // long segments'
   const int cap = pairs_stage_cap(c->geo, c->n, ball2);
   c->lists_half = 0;  // the pair list's passes use the list buffers
-  if ((e = clk::launch_pairs_count(*c->full, c->d_off_full, dim, ball2, cap, c->hflag, c->hlist, c->pl_meta + 4, c->pl_count, s)))
+  if ((e = clk::launch_pairs_count(*c->full, c->d_off_full, dim, ball2, cap, c->hdense, c->hflag, c->hlist,
+                                   c->pl_meta + 4, c->pl_meta + 3, c->pl_count, s)))
     return e;
   if ((e = clk::launch_scan64(c->pl_count, c->n, c->pl_tiles, c->pl_start, c->pl_meta, s))) return e;
   long long total = 0;
-  int meta[4] = {0, 0, 0, 0};
   if (cudaMemcpyAsync(&total, c->pl_start + c->n, sizeof(long long), cudaMemcpyDeviceToHost, s) != cudaSuccess ||
-      cudaMemcpyAsync(meta, c->pl_meta, sizeof(meta), cudaMemcpyDeviceToHost, s) != cudaSuccess ||
       cudaStreamSynchronize(s) != cudaSuccess)
     return CL_ERR_CUDA;
   *r->npairs = total;
   if ((e = cl_pairlist_fits(total, r->capacity))) return e;
   if (total == 0) return CL_OK;
   if (!r->pair_i || !r->pair_j || !r->pair_d) return CL_ERR_INVALID_ARG;
-  return clk::launch_pairs_fill(*c->full, c->d_off_full, dim, ball2, cap, c->hflag, c->hlist, c->pl_meta + 4, c->pl_count, c->pl_start,
-                               r->pair_i, r->pair_j, r->pair_d, c->pl_long, c->pl_meta + 3, s);
+  return clk::launch_pairs_fill(*c->full, c->d_off_full, dim, ball2, cap, c->hdense, c->hflag, c->hlist, c->pl_meta + 4,
+                               c->pl_count, c->pl_start, r->pair_i, r->pair_j, r->pair_d, c->pl_long, c->pl_meta + 3, s);
 }
 
 }  // namespace

@@ -1388,7 +1388,7 @@ __global__ void __launch_bounds__(kThreads, hood_ctas(MODE)) k_hood(const __grid
 // Each pair-image once (Sec. 2.8: "only half of the neighboring cells are
 // evaluated"): one CTA per home cell stages the particles of the half
 // stencil's cells within rc + d_max of the centre, and sweeps them
-// entry-major: a warp holds 64 staged entries (two per lane) and runs over
+// entry-major: a warp holds 128 staged entries (four per lane) and runs over
 // the home particles four at a time, so the force on each entry accumulates
 // in the lane's registers and leaves the CTA as one vector atomic per entry,
 // while the forces on the four home particles are warp-summed per step into
@@ -1406,11 +1406,11 @@ __global__ void __launch_bounds__(kThreads, hood_ctas(MODE)) k_hood(const __grid
 //
 // Cells whose particles or half neighbourhood exceed the buffers (more than
 // kHome particles, more than kHCap particles in the half stencil's cells)
-// take the windowed form of the same sweep: the half neighbourhood's row
-// segments are laid end to end and staged in windows of kHCap particles, each
-// window swept against the home particles in batches of kHome, and the pairs
-// within the cell are swept as a last window per batch (the cell's particles
-// from the batch's first on, ordered by index). Every non-empty cell is
+// take the windowed form of the same sweep (k_half_batch): the half
+// neighbourhood's row segments are laid end to end and staged in windows of
+// kHCap particles, each window swept against the home particles in batches of
+// kBatch, and the pairs within the cell are swept as a last window per batch
+// (the cell's particles from the batch's first on). Every non-empty cell is
 // swept, so the path covers the whole grid whenever both stencils fit the
 // table.
 
@@ -2671,8 +2671,7 @@ int hood_grid(int mode) {
 
 size_t hood_smem_bytes() { return sizeof(Smem); }
 
-// Persistent CTAs of the half-shell sweep, per mode (0, 1, 3).
-// Shared memory of k_hood_half<mode>: HalfSmem, and for the histogram its
+// Shared memory of k_half_batch<mode>: HalfSmem, and for the histogram its
 // largest set of copies.
 size_t half_mode_smem(int mode) {
   return sizeof(HalfSmem) + (mode == 6 ? sizeof(unsigned) * (size_t)hist_stride(kMaxBins) : 0);
@@ -2761,11 +2760,12 @@ bool hood_half_fits(const SweepArgs& A) { return A.noff <= kTab; }
 // Scalar reductions over the half stencil. When the stencil fits the table,
 // the work lists of the half-shell sweep split the cells: the fast-path cells
 // (at most kHome particles, at most kHCap in the half neighbourhood) go to the
-// home-major k_hood<mode>, the others to the windowed k_hood_half<mode, true>
-// (octant batches, index lists); otherwise k_hood<mode> takes the cells it can
-// and the per-particle sweep the rest. Measured with the half-shell kernel
-// alone for every cell: 1M lattice count 0.60 against 0.57 ms, histogram 1.05
-// against 0.93 ms (the home-major kernel is faster on small cells).
+// home-major k_hood<mode>, the others to k_half_batch<mode> (windowed cells by
+// batches of 32 home particles, small cells one per warp); otherwise
+// k_hood<mode> takes the cells it can and the per-particle sweep the rest.
+// Measured with a half-shell kernel alone for every cell: 1M lattice count
+// 0.60 against 0.57 ms, histogram 1.05 against 0.93 ms (the home-major kernel
+// is faster on cells of that size).
 int launch_hood_scalar(const SweepArgs& A, const HoodArgs& Hin, int* work, int kind, unsigned long long* count,
                        double* partials, long long partials_cap, double* sums, double* scalar_out, int nbins,
                        float rmax, unsigned long long* hist, cudaStream_t s, int* lists_half) {

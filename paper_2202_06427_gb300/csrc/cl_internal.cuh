@@ -248,7 +248,7 @@ size_t hood_smem_bytes();
 // stencil); 3: energy and the backward outputs.
 // partials_cap: doubles available in partials (sweep_partials_needed).
 // lists_half (host, may be null): 1 when the list buffers (list, dense, flag,
-// work[6..7]) hold the half-shell work lists of the current cell list; they
+// work[6..8]) hold the half-shell work lists of the current cell list; they
 // are then reused, and the flag is set after a half-shell launch and cleared
 // by any other.
 // Ahalf (modes 0, 1, 3; may be null): the half stencil, for the half-shell
@@ -331,16 +331,17 @@ constexpr int kMaxSegment = 1024;  // segments up to this length are sorted by o
 // sweep for the cells it flags (flag: ncells bytes; fcells: ncells ints, the
 // flagged cells, *nfcells of them; all written here).
 // cap: staged entries per cell (32..3072), the same for the count and fill passes.
-int launch_pairs_count(const SweepArgs& A, const Off* off, int dim, float ball2, int cap, unsigned char* flag, int* fcells,
-                       int* nfcells, int* count, cudaStream_t s);
+// last: ncells ints, written here and read by the fill pass; *nlong: cleared for it.
+int launch_pairs_count(const SweepArgs& A, const Off* off, int dim, float ball2, int cap, int* last, unsigned char* flag,
+                       int* fcells, int* nfcells, int* nlong, int* count, cudaStream_t s);
 // Sorts each listed segment [start[a], start[a] + count[a]), a = longs[q], q <
 // *nlong, of pj (carrying pd) by pj.
 int launch_sort_long(const int* longs, const int* nlong, const int* count, const long long* start, int* pj, float* pd,
                      cudaStream_t s);
 // Fill pass: the same two sweeps, each segment sorted by j and written.
 // longs (n ints) and nlong (1 int): workspace for segments longer than kMaxSegment.
-int launch_pairs_fill(const SweepArgs& A, const Off* off, int dim, float ball2, int cap, const unsigned char* flag, const int* fcells,
-                      const int* nfcells, const int* count, const long long* start, int* pi, int* pj, float* pd, int* longs,
+int launch_pairs_fill(const SweepArgs& A, const Off* off, int dim, float ball2, int cap, const int* last,
+                      const unsigned char* flag, const int* fcells, const int* nfcells, const int* count, const long long* start, int* pi, int* pj, float* pd, int* longs,
                       int* nlong, cudaStream_t s);
 
 }  // namespace clk

@@ -1,6 +1,7 @@
 // cl_pairs.cu -- the i<j neighbour list (Sec. 4.1: "the lists of pairs of
 // particles within a cutoff"), sorted by (i, j), with the FP32 distance.
 //
+//   k_cell_last    the largest original index of each cell
 //   k_pairs_cell<COUNT>  one CTA per cell stages the cell's neighbourhood
 //                  (the particles of its full stencil that lie within
 //                  rc + half a cell diagonal of its centre and whose index is
@@ -180,23 +181,24 @@ __global__ void __launch_bounds__(1024) k_pairs_sort_long(const int* __restrict_
 // candidate's entry), so the lanes stay busy however small the cells are.
 constexpr int kStageMax = 3072;  // largest staged neighbourhood of one cell (the launch picks its capacity)
 
-// Stencil entries k0 + lane of cell (cx, cy, cz): the lane's range [j0, j0 +
-// len) of sorted particles, its shift (stencil shift + (bx, by, bz)) and, over
-// the warp, the exclusive offsets of the ranges laid end to end and their total.
+// Stencil entry k (a lane's; none from A.noff on) of cell (cx, cy, cz): the
+// lane's range [j0, j0 + len) of sorted particles, its shift and, over the warp,
+// the exclusive offsets of the ranges laid end to end and their total. A cell
+// whose largest original index (last) is not above amin is left out.
 struct Chunk {
   int j0, len, excl, total;
   float sx, sy, sz;
 };
 
 template <int DIM>
-__device__ __forceinline__ Chunk chunk_ranges(const SweepArgs& A, const float4* stab, int k0, int lane, int cx,
-                                              int cy, int cz, float bx, float by, float bz, int lim = 32) {
+__device__ __forceinline__ Chunk chunk_ranges(const SweepArgs& A, const float4* stab, const int* __restrict__ last,
+                                              int amin, int k, int cx, int cy, int cz) {
+  const int lane = threadIdx.x & 31;
   Chunk ch;
   ch.j0 = 0;
   ch.len = 0;
   ch.sx = ch.sy = ch.sz = 0.f;
-  const int k = k0 + lane;
-  if (lane < lim && k < A.noff) {  // lim: the entries this warp takes (lanes 0..lim-1)
+  if (k < A.noff) {
     const float4 e = stab[k];
     const unsigned d = __float_as_uint(e.w);
     int x2 = cx + (int)(d & 1023u);
@@ -210,10 +212,10 @@ __device__ __forceinline__ Chunk chunk_ranges(const SweepArgs& A, const float4* 
     }
     const int c = x2 + A.nx * (y2 + A.ny * z2);
     ch.j0 = __ldg(A.cell_start + c);
-    ch.len = __ldg(A.cell_start + c + 1) - ch.j0;
-    ch.sx = e.x + bx;
-    ch.sy = e.y + by;
-    ch.sz = e.z + bz;
+    ch.len = __ldg(last + c) > amin ? __ldg(A.cell_start + c + 1) - ch.j0 : 0;
+    ch.sx = e.x;
+    ch.sy = e.y;
+    ch.sz = e.z;
   }
   int inc = ch.len;
 #pragma unroll
@@ -438,6 +440,29 @@ __device__ __forceinline__ float2 pair_d2(const float4& q, float2 nx, float2 ny,
   return __ffma2_rn(dx, dx, __fmul2_rn(dy, dy));
 }
 
+// Largest original index of each cell's particles (-1: none), kLastLanes lanes
+// to a cell, and the list's counters cleared. A cell's staging leaves out the
+// cells whose largest index is not above the smallest of its own: on an input
+// whose order follows space about half of the stencil (list of 2.1e8 pairs of a
+// million particles with a histogram 4.55 -> 4.28 ms; in random order no change,
+// 8 us of 4.5 ms).
+constexpr int kLastLanes = 8;
+
+__global__ void __launch_bounds__(256) k_cell_last(long long ncells, const int* __restrict__ cell_start,
+                                                   const float4* __restrict__ xs, int* __restrict__ last,
+                                                   int* __restrict__ nfcells, int* __restrict__ nlong) {
+  const long long t = blockIdx.x * (long long)blockDim.x + threadIdx.x, c = t / kLastLanes;
+  if (t == 0) *nfcells = *nlong = 0;
+  const int sub = (int)(t % kLastLanes);
+  int m = -1;
+  if (c < ncells)
+    for (int p = cell_start[c] + sub, p1 = cell_start[c + 1]; p < p1; p += kLastLanes)
+      m = max(m, __float_as_int(__ldg(&xs[p].w)));
+#pragma unroll
+  for (int o = kLastLanes / 2; o; o >>= 1) m = max(m, __shfl_xor_sync(0xffffffffu, m, o));
+  if (c < ncells && sub == 0) last[c] = m;
+}
+
 // One CTA of W warps per cell (grid-stride over the cells). The stencil
 // entries are shared among the warps 32 at a time; each warp appends the
 // particles of its entries that lie within sqrt(ball2) of the cell centre,
@@ -453,6 +478,7 @@ __device__ __forceinline__ float2 pair_d2(const float4& q, float2 nx, float2 ny,
 template <int DIM, bool FILL>
 __global__ void __launch_bounds__(256, 5) k_pairs_cell(const __grid_constant__ SweepArgs A,
                                                                                float ball2, int cap,
+                                                                               const int* __restrict__ last,
                                                                                unsigned char* __restrict__ flag,
                                                                                int* __restrict__ fcells,
                                                                                int* __restrict__ nfcells,
@@ -486,12 +512,10 @@ __global__ void __launch_bounds__(256, 5) k_pairs_cell(const __grid_constant__ S
     for (int p = h0 + lane; p < h1; p += 32) amin = min(amin, __float_as_int(__ldg(&A.xs[p].w)));
     amin = __reduce_min_sync(0xffffffffu, amin);
     __syncthreads();
-    // the stencil dealt evenly to the warps (E entries each per round, at most
-    // 32): at 32 per warp the 125 entries of a full stencil at lcell 2 would
-    // keep four of the eight warps waiting while the others stage
-    const int E = min(32, (A.noff + W - 1) / W);
-    for (int k0 = warp * E; k0 < A.noff; k0 += E * W) {
-      const Chunk ch = chunk_ranges<DIM>(A, stab, k0, lane, cx, cy, cz, 0.f, 0.f, 0.f, E);
+    // the stencil dealt to the warps entry by entry: of an input whose order
+    // follows space, the cells left out are one side of the stencil
+    for (int k0 = warp; k0 < A.noff; k0 += 32 * W) {
+      const Chunk ch = chunk_ranges<DIM>(A, stab, last, amin, k0 + W * lane, cx, cy, cz);
       for (int t0 = 0; t0 < ch.total; t0 += 32) {
         const int t = t0 + lane;
         float ax, ay, az;
@@ -639,7 +663,7 @@ size_t pairs_cell_smem(int noff, bool fill, int cap) {
 }
 
 template <int DIM, bool FILL>
-static int launch_cell(const SweepArgs& A, float ball2, int cap, unsigned char* flag, int* fcells, int* nfcells,
+static int launch_cell(const SweepArgs& A, float ball2, int cap, const int* last, unsigned char* flag, int* fcells, int* nfcells,
                        int* count, const long long* start, int* pi, int* pj, float* pd, cudaStream_t s) {
   static DevCache ready;  // shared-memory limit raised on this device
   if (cap < 32 || cap > kStageMax) return CL_ERR_INVALID_ARG;
@@ -660,18 +684,20 @@ static int launch_cell(const SweepArgs& A, float ball2, int cap, unsigned char* 
   long long blocks = (long long)sms * per;
   const long long ncells = (long long)A.nx * A.ny * A.nz;
   if (blocks > ncells) blocks = ncells;
-  k_pairs_cell<DIM, FILL><<<(int)blocks, 256, smem, s>>>(A, ball2, cap, flag, fcells, nfcells, count,
+  k_pairs_cell<DIM, FILL><<<(int)blocks, 256, smem, s>>>(A, ball2, cap, last, flag, fcells, nfcells, count,
                                                                       start, pi, pj, pd);
   return cudaGetLastError() == cudaSuccess ? CL_OK : CL_ERR_CUDA;
 }
 
-int launch_pairs_count(const SweepArgs& A, const Off* off, int dim, float ball2, int cap, unsigned char* flag, int* fcells,
-                       int* nfcells, int* count, cudaStream_t s) {
+int launch_pairs_count(const SweepArgs& A, const Off* off, int dim, float ball2, int cap, int* last, unsigned char* flag,
+                       int* fcells, int* nfcells, int* nlong, int* count, cudaStream_t s) {
   if (A.n <= 0) return CL_OK;
-  if (cudaMemsetAsync(nfcells, 0, sizeof(int), s) != cudaSuccess) return CL_ERR_CUDA;
-  const int e = dim == 3 ? launch_cell<3, false>(A, ball2, cap, flag, fcells, nfcells, count, nullptr, nullptr,
+  const long long ncells = (long long)A.nx * A.ny * A.nz;
+  k_cell_last<<<(unsigned)((ncells * kLastLanes + 255) / 256), 256, 0, s>>>(ncells, A.cell_start, A.xs, last, nfcells,
+                                                                            nlong);
+  const int e = dim == 3 ? launch_cell<3, false>(A, ball2, cap, last, flag, fcells, nfcells, count, nullptr, nullptr,
                                                  nullptr, nullptr, s)
-                         : launch_cell<2, false>(A, ball2, cap, flag, fcells, nfcells, count, nullptr, nullptr,
+                         : launch_cell<2, false>(A, ball2, cap, last, flag, fcells, nfcells, count, nullptr, nullptr,
                                                  nullptr, nullptr, s);
   if (e) return e;
   const CrossArgs C = cross_args(A, off);
@@ -709,16 +735,16 @@ int launch_sort_long(const int* longs, const int* nlong, const int* count, const
   return cudaGetLastError() == cudaSuccess ? CL_OK : CL_ERR_CUDA;
 }
 
-int launch_pairs_fill(const SweepArgs& A, const Off* off, int dim, float ball2, int cap, const unsigned char* flag, const int* fcells,
+int launch_pairs_fill(const SweepArgs& A, const Off* off, int dim, float ball2, int cap, const int* last,
+                      const unsigned char* flag, const int* fcells,
                       const int* nfcells, const int* count, const long long* start, int* pi, int* pj, float* pd, int* longs,
                       int* nlong, cudaStream_t s) {
   if (A.n <= 0) return CL_OK;
   unsigned char* fl = const_cast<unsigned char*>(flag);  // only read by the fill pass
   int* cn = const_cast<int*>(count);                     // likewise
-  const int e = dim == 3 ? launch_cell<3, true>(A, ball2, cap, fl, nullptr, nullptr, cn, start, pi, pj, pd, s)
-                         : launch_cell<2, true>(A, ball2, cap, fl, nullptr, nullptr, cn, start, pi, pj, pd, s);
+  const int e = dim == 3 ? launch_cell<3, true>(A, ball2, cap, last, fl, nullptr, nullptr, cn, start, pi, pj, pd, s)
+                         : launch_cell<2, true>(A, ball2, cap, last, fl, nullptr, nullptr, cn, start, pi, pj, pd, s);
   if (e) return e;
-  if (cudaMemsetAsync(nlong, 0, sizeof(int), s) != cudaSuccess) return CL_ERR_CUDA;
   const CrossArgs C = cross_args(A, off);
   const int g = group_lanes(A);
   int f;
