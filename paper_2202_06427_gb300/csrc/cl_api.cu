@@ -295,7 +295,7 @@ int map_pairlist(cl_list* c, cl_result* r, cudaStream_t s) {
   if ((e = clk::launch_pairs_count(*c->full, c->d_off_full, dim, ball2, cap, c->hdense, c->hflag, c->hlist,
                                    c->pl_meta + 4, c->pl_meta + 3, c->pl_count, s)))
     return e;
-  if ((e = clk::launch_scan64(c->pl_count, c->n, c->pl_tiles, c->pl_start, c->pl_meta, s))) return e;
+  if ((e = clk::launch_scan64(c->pl_count, c->n, c->pl_tiles, c->pl_start, s))) return e;
   long long total = 0;
   if (cudaMemcpyAsync(&total, c->pl_start + c->n, sizeof(long long), cudaMemcpyDeviceToHost, s) != cudaSuccess ||
       cudaStreamSynchronize(s) != cudaSuccess)
@@ -616,7 +616,7 @@ int cl_cross_pairlist(const cl_list* cc, const double* posb_dev, long long nb, l
   clk::Queries q;
   if ((e = w.open(nb, true, 0)) || (e = clk::launch_query_bin(*c->full, c->geo, posb_dev, nb, w.bin, w.err, &q, s)) ||
       (e = clk::launch_cross_count(*c->full, c->d_off_full, q, w.count, nullptr, s)) ||
-      (e = clk::launch_scan64(w.count, nb, w.tiles, w.start, w.meta, s)))
+      (e = clk::launch_scan64(w.count, nb, w.tiles, w.start, s)))
     return e;
   long long back[2] = {0, 0};  // the total and, after it, the error latch
   if (cudaMemcpyAsync(back, w.start + nb, sizeof(back), cudaMemcpyDeviceToHost, s) != cudaSuccess ||

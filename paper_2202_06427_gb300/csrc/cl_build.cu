@@ -204,6 +204,14 @@ __device__ __forceinline__ T warp_incl_scan(T v) {
   return v;
 }
 
+__device__ __forceinline__ int warp_sum(int v) { return __reduce_add_sync(0xffffffffu, v); }
+
+__device__ __forceinline__ long long warp_sum(long long v) {
+#pragma unroll
+  for (int o = 16; o; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+  return v;
+}
+
 // Exclusive scan of one value per thread across the block.
 template <class T>
 __device__ void block_excl_scan(T v, T* out_excl) {
@@ -222,7 +230,7 @@ __device__ void block_excl_scan(T v, T* out_excl) {
   __syncthreads();  // wsum is reused by the next call
 }
 
-// Per tile: sum of counts, non-empty cells, largest count. T is the offset
+// Per tile: sum of counts and, with meta, non-empty cells and largest count. T is the offset
 // type: int for cell offsets (at most n < 2^31 particles), long long for the
 // pair list, whose total may pass 2^31.
 template <class T>
@@ -256,8 +264,10 @@ __global__ void __launch_bounds__(kScanThreads) k_scan_reduce(const int* __restr
     int NE = 0, MX = 0;
     for (int w = 0; w < kScanThreads / 32; ++w) { S += ssum[w]; NE += sm[0][w]; MX = max(MX, sm[1][w]); }
     tile_sum[blockIdx.x] = S;
-    atomicAdd(&meta[1], NE);
-    atomicMax(&meta[2], MX);
+    if (meta) {
+      atomicAdd(&meta[1], NE);
+      atomicMax(&meta[2], MX);
+    }
   }
 }
 
@@ -305,19 +315,22 @@ __global__ void __launch_bounds__(kScanThreads) k_scan_final(const int* __restri
 // two kernels).
 constexpr int kScanOneTiles = 64;
 
+template <class T>
 __global__ void __launch_bounds__(1024) k_scan_one(const int* __restrict__ counts, long long ncells,
-                                                   int* __restrict__ meta, int* __restrict__ cell_start) {
+                                                   int* __restrict__ meta, T* __restrict__ cell_start) {
   constexpr int kPer = kScanTile / 1024;
-  __shared__ int part[32], wsum[32], mx[32], ne[32];
+  __shared__ T part[32], wsum[32];
+  __shared__ int mx[32], ne[32];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const long long tile0 = (long long)blockIdx.x * kScanTile;
-  int before = 0;
+  T before = 0;
   for (long long c = (long long)threadIdx.x * 4; c < tile0; c += 4096) {
     const int4 v = *reinterpret_cast<const int4*>(counts + c);
-    before += v.x + v.y + v.z + v.w;
+    before += (T)v.x + v.y + v.z + v.w;
   }
-  before = __reduce_add_sync(0xffffffffu, before);
-  int v[kPer], s = 0, big = 0, full = 0;
+  before = warp_sum(before);
+  int v[kPer], big = 0, full = 0;
+  T s = 0;
 #pragma unroll
   for (int k = 0; k < kPer; ++k) {
     const long long c = tile0 + (long long)threadIdx.x * kPer + k;
@@ -326,7 +339,7 @@ __global__ void __launch_bounds__(1024) k_scan_one(const int* __restrict__ count
     big = max(big, v[k]);
     full += v[k] > 0 ? 1 : 0;
   }
-  const int incl = warp_incl_scan(s);
+  const T incl = warp_incl_scan(s);
   big = __reduce_max_sync(0xffffffffu, big);
   full = __reduce_add_sync(0xffffffffu, full);
   if (lane == 31) wsum[warp] = incl;
@@ -336,16 +349,16 @@ __global__ void __launch_bounds__(1024) k_scan_one(const int* __restrict__ count
     ne[warp] = full;
   }
   __syncthreads();
-  const int all = __reduce_add_sync(0xffffffffu, part[lane]);
-  const int wincl = warp_incl_scan(wsum[lane]);
+  const T all = warp_sum(part[lane]);
+  const T wincl = warp_incl_scan(wsum[lane]);
   if (warp == 0) {
     const int m = __reduce_max_sync(0xffffffffu, mx[lane]), q = __reduce_add_sync(0xffffffffu, ne[lane]);
-    if (lane == 0) {
+    if (lane == 0 && meta) {
       atomicAdd(&meta[1], q);
       atomicMax(&meta[2], m);
     }
   }
-  int run = all + incl - s + (warp ? __shfl_sync(0xffffffffu, wincl, warp - 1) : 0);
+  T run = all + incl - s + (warp ? __shfl_sync(0xffffffffu, wincl, warp - 1) : 0);
 #pragma unroll
   for (int k = 0; k < kPer; ++k) {
     const long long c = tile0 + (long long)threadIdx.x * kPer + k;
@@ -478,7 +491,7 @@ int scan_tiles_for(long long ncells) { return (int)((ncells + kScanTile - 1) / k
 int launch_scan_cells(const int* counts, long long ncells, int* tile_sum, int* meta, int* cell_start, cudaStream_t s) {
   const int ntiles = scan_tiles_for(ncells);
   if (ntiles <= kScanOneTiles) {
-    k_scan_one<<<ntiles, 1024, 0, s>>>(counts, ncells, meta, cell_start);
+    k_scan_one<int><<<ntiles, 1024, 0, s>>>(counts, ncells, meta, cell_start);
     return cudaGetLastError() == cudaSuccess ? CL_OK : CL_ERR_CUDA;
   }
   k_scan_reduce<int><<<ntiles, kScanThreads, 0, s>>>(counts, ncells, tile_sum, meta);
@@ -551,11 +564,14 @@ namespace clk {
 // with the same two kernels as the cell offsets; meta receives the number of
 // non-zero counts and the largest one. The pair list's offsets and total are
 // 64-bit: a list may hold more than 2^31 pairs.
-int launch_scan64(const int* counts, long long n, long long* tile_sum, long long* start, int* meta, cudaStream_t s) {
+int launch_scan64(const int* counts, long long n, long long* tile_sum, long long* start, cudaStream_t s) {
   const int ntiles = scan_tiles_for(n);
-  if (cudaMemsetAsync(meta + 1, 0, sizeof(int) * 2, s) != cudaSuccess) return CL_ERR_CUDA;
   if (ntiles == 0) return cudaMemsetAsync(start, 0, sizeof(long long), s) == cudaSuccess ? CL_OK : CL_ERR_CUDA;
-  k_scan_reduce<long long><<<ntiles, kScanThreads, 0, s>>>(counts, n, tile_sum, meta);
+  if (ntiles <= kScanOneTiles) {
+    k_scan_one<long long><<<ntiles, 1024, 0, s>>>(counts, n, nullptr, start);
+    return cudaGetLastError() == cudaSuccess ? CL_OK : CL_ERR_CUDA;
+  }
+  k_scan_reduce<long long><<<ntiles, kScanThreads, 0, s>>>(counts, n, tile_sum, nullptr);
   k_scan_final<long long><<<ntiles, kScanThreads, 0, s>>>(counts, n, tile_sum, start);
   return cudaGetLastError() == cudaSuccess ? CL_OK : CL_ERR_CUDA;
 }

@@ -174,7 +174,7 @@ int launch_scan_cells(const int* counts, long long ncells, int* tile_sum, int* m
 // the packed cells along the sorted array.
 int launch_cell_order(int n, int nx, int ny, long long ncells, const int* slot, const float4* xl,
                       const int* cell_start, float4* xs, unsigned* cellc, cudaStream_t s);
-int launch_scan64(const int* counts, long long n, long long* tile_sum, long long* start, int* meta, cudaStream_t s);
+int launch_scan64(const int* counts, long long n, long long* tile_sum, long long* start, cudaStream_t s);
 
 // Sweeps and reductions (cl_sweep.cu).
 int sweep_partials_needed(int n);
