@@ -244,10 +244,8 @@ float pairs_ball2(const clk::Geo& g) {
   return (float)(r * r);
 }
 
-// Staged entries per cell for the pair list: the particles of the staging ball
-// at the box's mean density, with 30 % to spare, in steps of 128 (1,024 to
-// 3,072). Denser cells overflow and take the per-particle path.
-int pairs_stage_cap(const clk::Geo& g, long long n, float ball2) {
+// Particles the pair list's staging ball holds at the box's mean density.
+double pairs_expected(const clk::Geo& g, long long n, float ball2) {
   double vol = 1.0;
   if (g.dim == 3)
     vol = std::fabs(g.h[0] * (g.h[4] * g.h[8] - g.h[5] * g.h[7]) - g.h[1] * (g.h[3] * g.h[8] - g.h[5] * g.h[6]) +
@@ -256,8 +254,13 @@ int pairs_stage_cap(const clk::Geo& g, long long n, float ball2) {
     vol = std::fabs(g.h[0] * g.h[4] - g.h[1] * g.h[3]);
   const double r = std::sqrt((double)ball2);
   const double ball = g.dim == 3 ? 4.18879020478639 * r * r * r : 3.14159265358979 * r * r;
-  const double est = (vol > 0 ? (double)n / vol : 0.0) * ball * 1.3 + 64.0;
-  int cap = (int)std::ceil(est / 128.0) * 128;
+  return (vol > 0 ? (double)n / vol : 0.0) * ball;
+}
+
+// Staged entries per cell: that with 30 % to spare, in steps of 128 (1,024 to
+// 3,072). Denser cells overflow and take the per-particle path.
+int pairs_stage_cap(double expect) {
+  const int cap = (int)std::ceil((expect * 1.3 + 64.0) / 128.0) * 128;
   return std::min(3072, std::max(1024, cap));
 }
 
@@ -285,16 +288,20 @@ int map_pairlist(cl_list* c, cl_result* r, cudaStream_t s) {
     c->bytes += bytes;
   }
   const int dim = c->geo.dim;
-  const float ball2 = pairs_ball2(c->geo);
-  // hflag / hlist: per-cell flags and the flagged cells, hdense: the cells'
-  // largest indices (shared with the neighbourhood sweep, which rewrites them
-  // on every launch); pl_meta[4]: the flagged cells' number, pl_meta[3]: the
-  // long segments'
-  const int cap = pairs_stage_cap(c->geo, c->n, ball2);
+  // the cells' buffers are shared with the binning (counts) and with the
+  // neighbourhood sweep, which rewrite them on every launch
+  clk::PairLists L;
+  L.ball2 = pairs_ball2(c->geo);
+  L.expect = pairs_expected(c->geo, c->n, L.ball2);
+  L.cap = pairs_stage_cap(L.expect);
+  L.last = c->hdense;
+  L.flag = c->hflag;
+  L.fcells = c->hlist;
+  L.mid = c->counts;
+  L.ctr = c->pl_meta;
+  L.count = c->pl_count;
   c->lists_half = 0;  // the pair list's passes use the list buffers
-  if ((e = clk::launch_pairs_count(*c->full, c->d_off_full, dim, ball2, cap, c->hdense, c->hflag, c->hlist,
-                                   c->pl_meta + 4, c->pl_meta + 3, c->pl_count, s)))
-    return e;
+  if ((e = clk::launch_pairs_count(*c->full, c->d_off_full, dim, L, s))) return e;
   if ((e = clk::launch_scan64(c->pl_count, c->n, c->pl_tiles, c->pl_start, s))) return e;
   long long total = 0;
   if (cudaMemcpyAsync(&total, c->pl_start + c->n, sizeof(long long), cudaMemcpyDeviceToHost, s) != cudaSuccess ||
@@ -304,8 +311,8 @@ int map_pairlist(cl_list* c, cl_result* r, cudaStream_t s) {
   if ((e = cl_pairlist_fits(total, r->capacity))) return e;
   if (total == 0) return CL_OK;
   if (!r->pair_i || !r->pair_j || !r->pair_d) return CL_ERR_INVALID_ARG;
-  return clk::launch_pairs_fill(*c->full, c->d_off_full, dim, ball2, cap, c->hdense, c->hflag, c->hlist, c->pl_meta + 4,
-                               c->pl_count, c->pl_start, r->pair_i, r->pair_j, r->pair_d, c->pl_long, c->pl_meta + 3, s);
+  return clk::launch_pairs_fill(*c->full, c->d_off_full, dim, L, c->pl_start, r->pair_i, r->pair_j, r->pair_d, c->pl_long,
+                                s);
 }
 
 }  // namespace

@@ -327,21 +327,28 @@ void list_parts(const cl_list* cl, ListParts* p);
 // (64-bit scan of count: the list may pass 2^31 pairs), tiles, meta:
 // workspace; outputs pair_i/j/d of capacity entries.
 constexpr int kMaxSegment = 1024;  // segments up to this length are sorted by one warp in shared memory
+// Workspace and plan of the two passes, the same for both.
+struct PairLists {
+  float ball2;          // squared radius about a cell's centre that holds the cell's neighbours
+  int cap;              // staged entries per cell (32..3072)
+  double expect;        // particles expected in that ball
+  int* last;            // ncells: largest original index per cell
+  unsigned char* flag;  // ncells: 1 for the cells of fcells
+  int* fcells;          // ncells: cells whose neighbourhood passes cap
+  int* mid;             // ncells: sparse grids' cells that take the general staging
+  int* ctr;             // [0] long segments, [1] fcells, [2] mid: their numbers
+  int* count;           // n
+};
 // Count pass of the pair list: per-cell staged sweep, then the per-particle
-// sweep for the cells it flags (flag: ncells bytes; fcells: ncells ints, the
-// flagged cells, *nfcells of them; all written here).
-// cap: staged entries per cell (32..3072), the same for the count and fill passes.
-// last: ncells ints, written here and read by the fill pass; *nlong: cleared for it.
-int launch_pairs_count(const SweepArgs& A, const Off* off, int dim, float ball2, int cap, int* last, unsigned char* flag,
-                       int* fcells, int* nfcells, int* nlong, int* count, cudaStream_t s);
+// sweep for the cells it flags. Writes everything L points to.
+int launch_pairs_count(const SweepArgs& A, const Off* off, int dim, const PairLists& L, cudaStream_t s);
 // Sorts each listed segment [start[a], start[a] + count[a]), a = longs[q], q <
 // *nlong, of pj (carrying pd) by pj.
 int launch_sort_long(const int* longs, const int* nlong, const int* count, const long long* start, int* pj, float* pd,
                      cudaStream_t s);
 // Fill pass: the same two sweeps, each segment sorted by j and written.
-// longs (n ints) and nlong (1 int): workspace for segments longer than kMaxSegment.
-int launch_pairs_fill(const SweepArgs& A, const Off* off, int dim, float ball2, int cap, const int* last,
-                      const unsigned char* flag, const int* fcells, const int* nfcells, const int* count, const long long* start, int* pi, int* pj, float* pd, int* longs,
-                      int* nlong, cudaStream_t s);
+// longs (n ints): workspace for segments longer than kMaxSegment.
+int launch_pairs_fill(const SweepArgs& A, const Off* off, int dim, const PairLists& L, const long long* start, int* pi,
+                      int* pj, float* pd, int* longs, cudaStream_t s);
 
 }  // namespace clk

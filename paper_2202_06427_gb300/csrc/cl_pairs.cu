@@ -2,6 +2,8 @@
 // particles within a cutoff"), sorted by (i, j), with the FP32 distance.
 //
 //   k_cell_last    the largest original index of each cell
+//   k_pairs_sparse the two passes below with a warp per cell, on grids whose
+//                  cells have few neighbours; the cells it leaves go on to
 //   k_pairs_cell<COUNT>  one CTA per cell stages the cell's neighbourhood
 //                  (the particles of its full stencil that lie within
 //                  rc + half a cell diagonal of its centre and whose index is
@@ -28,6 +30,7 @@
 // count[i] all the same). The sweep visits the pair-images of a particle; the
 // list is only defined when each pair has at most one image within rc
 // (rc <= w_min / 2), which the host checks before launching.
+#include <algorithm>
 #include <climits>
 
 #include "cl_query.cuh"
@@ -450,9 +453,9 @@ constexpr int kLastLanes = 8;
 
 __global__ void __launch_bounds__(256) k_cell_last(long long ncells, const int* __restrict__ cell_start,
                                                    const float4* __restrict__ xs, int* __restrict__ last,
-                                                   int* __restrict__ nfcells, int* __restrict__ nlong) {
+                                                   int* __restrict__ ctr) {
   const long long t = blockIdx.x * (long long)blockDim.x + threadIdx.x, c = t / kLastLanes;
-  if (t == 0) *nfcells = *nlong = 0;
+  if (t < 3) ctr[t] = 0;
   const int sub = (int)(t % kLastLanes);
   int m = -1;
   if (c < ncells)
@@ -463,43 +466,245 @@ __global__ void __launch_bounds__(256) k_cell_last(long long ncells, const int* 
   if (c < ncells && sub == 0) last[c] = m;
 }
 
-// U steps of a warp's staging, 32 candidates of ch each from t0 on: those within
-// sqrt(ball2) of the cell's centre and of an index above amin are appended to
-// the list st (*nst of at most cap entries), shifted to the cell's frame.
-template <int DIM, int U>
-__device__ __forceinline__ void stage_steps(const SweepArgs& A, const Chunk& ch, int t0, float ball2, int amin, int cap,
-                                            float4* st, int* nst) {
-  const int lane = threadIdx.x & 31;
+// U steps of a warp's staging, 32 candidates of ch each from t0 on: the
+// particles, shifted to the cell's frame, and the lanes (m) that hold one within
+// sqrt(ball2) of the cell's centre and of an index above amin.
+template <int U>
+struct StagedSteps {
   float4 q[U];
+  unsigned m[U];
+  int total;
+};
+
+template <int DIM, int U>
+__device__ __forceinline__ StagedSteps<U> staged_steps(const SweepArgs& A, const Chunk& ch, int t0, float ball2,
+                                                       int amin) {
+  const int lane = threadIdx.x & 31;
+  StagedSteps<U> r;
   float ax[U], ay[U], az[U];
 #pragma unroll
   for (int u = 0; u < U; ++u) {
     const int t = t0 + 32 * u + lane;
     const int j = chunk_candidate(ch, t, ax[u], ay[u], az[u]);
-    q[u] = make_float4(0.f, 0.f, 0.f, __int_as_float(-1));  // beyond the end: not above amin
-    if (t < ch.total) q[u] = __ldg(&A.xs[j]);
+    r.q[u] = make_float4(0.f, 0.f, 0.f, __int_as_float(-1));  // beyond the end: not above amin
+    if (t < ch.total) r.q[u] = __ldg(&A.xs[j]);
   }
-  unsigned m[U];
-  int total = 0;
+  r.total = 0;
 #pragma unroll
   for (int u = 0; u < U; ++u) {
-    q[u].x += ax[u];
-    q[u].y += ay[u];
-    q[u].z = DIM == 3 ? q[u].z + az[u] : 0.f;
-    m[u] = __ballot_sync(0xffffffffu, fmaf(q[u].x, q[u].x, fmaf(q[u].y, q[u].y, q[u].z * q[u].z)) < ball2 &&
-                                          __float_as_int(q[u].w) > amin);
-    total += __popc(m[u]);
+    float4& q = r.q[u];
+    q.x += ax[u];
+    q.y += ay[u];
+    q.z = DIM == 3 ? q.z + az[u] : 0.f;
+    r.m[u] = __ballot_sync(0xffffffffu, fmaf(q.x, q.x, fmaf(q.y, q.y, q.z * q.z)) < ball2 && __float_as_int(q.w) > amin);
+    r.total += __popc(r.m[u]);
   }
-  int base = 0;
-  if (lane == 0 && total) base = atomicAdd(nst, total);
-  base = __shfl_sync(0xffffffffu, base, 0);
+  return r;
+}
+
+// Appends them to the list st of cap entries from entry base on.
+template <int U>
+__device__ __forceinline__ void append_steps(const StagedSteps<U>& r, int base, int cap, float4* st) {
+  const int lane = threadIdx.x & 31;
 #pragma unroll
   for (int u = 0; u < U; ++u) {
-    if (m[u] >> lane & 1u) {
-      const int e = base + __popc(m[u] & ((1u << lane) - 1u));
-      if (e < cap) st[e] = q[u];
+    if (r.m[u] >> lane & 1u) {
+      const int e = base + __popc(r.m[u] & ((1u << lane) - 1u));
+      if (e < cap) st[e] = r.q[u];
     }
-    base += __popc(m[u]);
+    base += __popc(r.m[u]);
+  }
+}
+
+template <int DIM, int U>
+__device__ __forceinline__ void stage_steps(const SweepArgs& A, const Chunk& ch, int t0, float ball2, int amin, int cap,
+                                            float4* st, int* nst) {
+  const StagedSteps<U> r = staged_steps<DIM, U>(A, ch, t0, ball2, amin);
+  int base = 0;
+  if ((threadIdx.x & 31) == 0 && r.total) base = atomicAdd(nst, r.total);
+  append_steps(r, __shfl_sync(0xffffffffu, base, 0), cap, st);
+}
+
+// Home particles p and p + 1 (the second if below h1) against the S staged
+// entries, a warp; both share each staged load. The pairs with j > i are
+// counted; the distance of each (particle, candidate) is computed as in the fill
+// pass.
+template <int DIM>
+__device__ __forceinline__ void count_two(const SweepArgs& A, int p, int h1, const float4* st, int S,
+                                          int* __restrict__ count) {
+  const int lane = threadIdx.x & 31;
+            const bool two = p + 1 < h1;
+            const float4 pa = A.xs[p];
+            const float4 pb = two ? A.xs[p + 1] : pa;
+            const int a0 = __float_as_int(pa.w), a1 = two ? __float_as_int(pb.w) : INT_MAX;
+            const float2 nx = make_float2(-pa.x, -pb.x), ny = make_float2(-pa.y, -pb.y),
+                         nz = make_float2(-pa.z, -pb.z);
+            int L0 = 0, L1 = 0;  // per lane, summed over the warp at the end
+  #pragma unroll 2
+            for (int t = lane; t < S; t += 32) {
+              const float4 q = st[t];
+              const int jo = __float_as_int(q.w);
+              float2 dx, dy, dz;
+              const float2 d2 = pair_d2<DIM>(q, nx, ny, nz, dx, dy, dz);
+              L0 += (jo > a0 && d2.x < A.rc2) ? 1 : 0;
+              L1 += (jo > a1 && d2.y < A.rc2) ? 1 : 0;
+            }
+            L0 = __reduce_add_sync(0xffffffffu, L0);
+            L1 = __reduce_add_sync(0xffffffffu, L1);
+            if (lane == 0) {
+              count[a0] = L0;
+              if (two) count[a1] = L1;
+            }
+}
+
+// The same two particles' segments of the list, from the staged entries in
+// order of their indices (at(t): entry t; kmin: the smallest index). The sweep
+// starts at the earlier of their suffixes (entries before a particle's own
+// suffix fail j > i) and each particle's kept pairs are written in order from
+// its own ballot.
+template <int DIM, class At>
+__device__ __forceinline__ void fill_two(const SweepArgs& A, int p, int h1, At at, int S, int kmin,
+                                         const int* __restrict__ count, const long long* __restrict__ start,
+                                         int* __restrict__ pi_out, int* __restrict__ pj_out,
+                                         float* __restrict__ pd_out) {
+  const int lane = threadIdx.x & 31;
+  const unsigned lt = (1u << lane) - 1u;
+            const bool two = p + 1 < h1;
+            const float4 pa = A.xs[p];
+            const float4 pb = two ? A.xs[p + 1] : pa;
+            const int a0 = __float_as_int(pa.w), a1 = two ? __float_as_int(pb.w) : INT_MAX;
+            int f0 = 0, f1 = S;  // first position (in index order) with index > a0, a1
+            {
+              const unsigned ka = a0 >= kmin ? (unsigned)(a0 - kmin) : 0u;
+              int lo = 0, hi = S;
+              while (a0 >= kmin && lo < hi) {
+                const int mid = (lo + hi) >> 1;
+                if ((unsigned)(__float_as_int(at(mid).w) - kmin) > ka) hi = mid;
+                else lo = mid + 1;
+              }
+              f0 = a0 >= kmin ? lo : 0;
+            }
+            if (two) {
+              const unsigned kb = a1 >= kmin ? (unsigned)(a1 - kmin) : 0u;
+              int lo = 0, hi = S;
+              while (a1 >= kmin && lo < hi) {
+                const int mid = (lo + hi) >> 1;
+                if ((unsigned)(__float_as_int(at(mid).w) - kmin) > kb) hi = mid;
+                else lo = mid + 1;
+              }
+              f1 = a1 >= kmin ? lo : 0;
+            }
+            const int c0 = __ldg(count + a0), c1 = two ? __ldg(count + a1) : 0;
+            const long long b0 = __ldg(start + a0), b1 = two ? __ldg(start + a1) : 0;
+            const float2 nx = make_float2(-pa.x, -pb.x), ny = make_float2(-pa.y, -pb.y),
+                         nz = make_float2(-pa.z, -pb.z);
+            int L0 = 0, L1 = 0;
+  #pragma unroll 2
+            for (int t0 = min(f0, f1); t0 < S; t0 += 32) {
+              const int t = t0 + lane;
+              bool k0 = false, k1 = false;
+              int jo = 0;
+              float d20 = 0.f, d21 = 0.f;
+              if (t < S) {
+                const float4 q = at(t);
+                jo = __float_as_int(q.w);
+                float2 dx, dy, dz;
+                const float2 d2 = pair_d2<DIM>(q, nx, ny, nz, dx, dy, dz);
+                d20 = d2.x;
+                d21 = d2.y;
+                k0 = jo > a0 && d20 < A.rc2;
+                k1 = jo > a1 && d21 < A.rc2;
+              }
+              const unsigned m0 = __ballot_sync(0xffffffffu, k0), m1 = __ballot_sync(0xffffffffu, k1);
+              if (k0) {
+                const int e = L0 + __popc(m0 & lt);
+                if (e < c0) {
+                  pi_out[b0 + e] = a0;
+                  pj_out[b0 + e] = jo;
+                  pd_out[b0 + e] = d20 * rsqrt_nr(d20);
+                }
+              }
+              if (k1) {
+                const int e = L1 + __popc(m1 & lt);
+                if (e < c1) {
+                  pi_out[b1 + e] = a1;
+                  pj_out[b1 + e] = jo;
+                  pd_out[b1 + e] = d21 * rsqrt_nr(d21);
+                }
+              }
+              L0 += __popc(m0);
+              L1 += __popc(m1);
+            }
+}
+
+// Sparse grids (at most kSparse particles expected in a staging ball): a warp
+// per cell, no barrier; the staged entries, up to kSparseCap, are ordered by
+// counting the smaller indices of each. Latency-bound: 2D lists with their
+// builds took, with a CTA of eight warps per cell of one particle, 525 us at
+// 57,000 particles and 371 at 31,000; 190 and 178 so. Cells that do not fit are
+// listed (cells) for k_pairs_cell in both passes. kSparse: the fullest list of
+// 2D grids in use holds 40 in its ball; from some hundreds on a warp's ordering
+// (S / 32 S comparisons) costs more than the CTA's buckets.
+constexpr int kSparse = 64, kSparseCap = 160, kSparseWarps = 4;
+static_assert((kMaxOff + 2 * kSparseWarps * kSparseCap) * sizeof(float4) <= 48 * 1024, "the default shared memory");
+
+template <int DIM, bool FILL>
+__global__ void __launch_bounds__(32 * kSparseWarps) k_pairs_sparse(const __grid_constant__ SweepArgs A, float ball2,
+                                                                    const int* __restrict__ last,
+                                                                    int* __restrict__ cells, int* __restrict__ nlisted,
+                                                                    int* __restrict__ count,
+                                                                    const long long* __restrict__ start,
+                                                                    int* __restrict__ pi_out, int* __restrict__ pj_out,
+                                                                    float* __restrict__ pd_out) {
+  extern __shared__ float4 smem[];
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  float4* stab = smem;
+  float4* st = stab + A.noff + warp * kSparseCap * (FILL ? 2 : 1);
+  stencil_to_smem(A, stab);
+  __syncthreads();
+  const int ncells = A.nx * A.ny * A.nz;
+  for (int c = blockIdx.x * kSparseWarps + warp; c < ncells; c += gridDim.x * kSparseWarps) {
+    const int h0 = __ldg(A.cell_start + c), h1 = __ldg(A.cell_start + c + 1);
+    if (h1 == h0) continue;
+    const int cx = c % A.nx, cy = (c / A.nx) % A.ny, cz = c / (A.nx * A.ny);
+    int amin = INT_MAX;  // as in k_pairs_cell
+    for (int p = h0 + lane; p < h1; p += 32) amin = min(amin, __float_as_int(__ldg(&A.xs[p].w)));
+    amin = __reduce_min_sync(0xffffffffu, amin);
+    __syncwarp();  // the cell before is done with
+    int S = 0;
+    for (int k0 = 0; k0 < A.noff; k0 += 32) {
+      const Chunk ch = chunk_ranges<DIM>(A, stab, last, amin, k0 + lane, cx, cy, cz);
+      for (int t0 = 0; t0 < ch.total; t0 += 32) {
+        const StagedSteps<1> q = staged_steps<DIM, 1>(A, ch, t0, ball2, amin);
+        append_steps(q, S, kSparseCap, st);
+        S += q.total;
+      }
+    }
+    __syncwarp();
+    if (S > kSparseCap) {
+      if (!FILL && lane == 0) cells[atomicAdd(nlisted, 1)] = c;
+      continue;
+    }
+    if (!FILL) {
+      for (int p = h0; p < h1; p += 2) count_two<DIM>(A, p, h1, st, S, count);
+    } else {
+      float4* so = st + kSparseCap;
+      int kmin = INT_MAX;
+      for (int e = lane; e < S; e += 32) {
+        const int v = __float_as_int(st[e].w);
+        int r = 0;
+        for (int f = 0; f < S; ++f) {
+          const int w = __float_as_int(st[f].w);
+          r += (w < v || (w == v && f < e)) ? 1 : 0;  // equal: two images, at most one within the cutoff
+        }
+        so[r] = st[e];
+        kmin = min(kmin, v);
+      }
+      kmin = __reduce_min_sync(0xffffffffu, kmin);
+      __syncwarp();
+      for (int p = h0; p < h1; p += 2)
+        fill_two<DIM>(A, p, h1, [&](int t) { return so[t]; }, S, kmin, count, start, pi_out, pj_out, pd_out);
+    }
   }
 }
 
@@ -515,9 +720,12 @@ __device__ __forceinline__ void stage_steps(const SweepArgs& A, const Chunk& ch,
 // by original index (stage_sort), so a particle's pairs with
 // j > a come from a suffix of that order in ascending j and are written in
 // order, coalesced, as the ballot finds them.
+// With cells, the *nlisted cells of that list only.
 template <int DIM, bool FILL>
-__global__ void __launch_bounds__(256, 5) k_pairs_cell(const __grid_constant__ SweepArgs A,
+__global__ void __launch_bounds__(256, FILL ? 5 : 6) k_pairs_cell(const __grid_constant__ SweepArgs A,
                                                                                float ball2, int cap,
+                                                                               const int* __restrict__ cells,
+                                                                               const int* __restrict__ nlisted,
                                                                                const int* __restrict__ last,
                                                                                unsigned char* __restrict__ flag,
                                                                                int* __restrict__ fcells,
@@ -535,11 +743,12 @@ __global__ void __launch_bounds__(256, 5) k_pairs_cell(const __grid_constant__ S
   int* cnt = scal + 16;  // FILL: bucket (or radix) counters and slots
   unsigned short* rs0 = reinterpret_cast<unsigned short*>(cnt + kBuckets);
   unsigned short* rs1 = rs0 + cap;
+  const int m = cells ? *nlisted : A.nx * A.ny * A.nz;
+  if ((int)blockIdx.x >= m) return;
   stencil_to_smem(A, stab);
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const unsigned lt = (1u << lane) - 1u;
-  const int ncells = A.nx * A.ny * A.nz;
-  for (int c = blockIdx.x; c < ncells; c += gridDim.x) {
+  for (int q = blockIdx.x; q < m; q += gridDim.x) {
+    const int c = cells ? cells[q] : q;
     const int h0 = __ldg(A.cell_start + c), h1 = __ldg(A.cell_start + c + 1);
     if (h1 == h0) continue;
     if (FILL && flag[c]) continue;
@@ -569,106 +778,11 @@ __global__ void __launch_bounds__(256, 5) k_pairs_cell(const __grid_constant__ S
       int kmin = 0;
       if (FILL) stage_sort<W>(st, S, rs0, rs1, cnt, scal, slots, kmin);
       if (!FILL) {
-        // COUNT: two home particles per warp share each staged load; the
-        // distance of each (particle, candidate) is computed as in the fill pass.
-        for (int p = h0 + 2 * warp; p < h1; p += 2 * W) {
-          const bool two = p + 1 < h1;
-          const float4 pa = A.xs[p];
-          const float4 pb = two ? A.xs[p + 1] : pa;
-          const int a0 = __float_as_int(pa.w), a1 = two ? __float_as_int(pb.w) : INT_MAX;
-          const float2 nx = make_float2(-pa.x, -pb.x), ny = make_float2(-pa.y, -pb.y),
-                       nz = make_float2(-pa.z, -pb.z);
-          int L0 = 0, L1 = 0;  // per lane, summed over the warp at the end
-#pragma unroll 2
-          for (int t = lane; t < S; t += 32) {
-            const float4 q = st[t];
-            const int jo = __float_as_int(q.w);
-            float2 dx, dy, dz;
-            const float2 d2 = pair_d2<DIM>(q, nx, ny, nz, dx, dy, dz);
-            L0 += (jo > a0 && d2.x < A.rc2) ? 1 : 0;
-            L1 += (jo > a1 && d2.y < A.rc2) ? 1 : 0;
-          }
-          L0 = __reduce_add_sync(0xffffffffu, L0);
-          L1 = __reduce_add_sync(0xffffffffu, L1);
-          if (lane == 0) {
-            count[a0] = L0;
-            if (two) count[a1] = L1;
-          }
-        }
+        for (int p = h0 + 2 * warp; p < h1; p += 2 * W) count_two<DIM>(A, p, h1, st, S, count);
       }
-      if (FILL) {
-        // FILL: two home particles per warp; the sweep starts at the earlier of
-        // their suffixes (entries before a particle's own suffix fail j > i) and
-        // each particle's kept pairs are written in order from its own ballot.
-        for (int p = h0 + 2 * warp; p < h1; p += 2 * W) {
-          const bool two = p + 1 < h1;
-          const float4 pa = A.xs[p];
-          const float4 pb = two ? A.xs[p + 1] : pa;
-          const int a0 = __float_as_int(pa.w), a1 = two ? __float_as_int(pb.w) : INT_MAX;
-          int f0 = 0, f1 = S;  // first position (in index order) with index > a0, a1
-          {
-            const unsigned ka = a0 >= kmin ? (unsigned)(a0 - kmin) : 0u;
-            int lo = 0, hi = S;
-            while (a0 >= kmin && lo < hi) {
-              const int mid = (lo + hi) >> 1;
-              if ((unsigned)(__float_as_int(st[slots[mid]].w) - kmin) > ka) hi = mid;
-              else lo = mid + 1;
-            }
-            f0 = a0 >= kmin ? lo : 0;
-          }
-          if (two) {
-            const unsigned kb = a1 >= kmin ? (unsigned)(a1 - kmin) : 0u;
-            int lo = 0, hi = S;
-            while (a1 >= kmin && lo < hi) {
-              const int mid = (lo + hi) >> 1;
-              if ((unsigned)(__float_as_int(st[slots[mid]].w) - kmin) > kb) hi = mid;
-              else lo = mid + 1;
-            }
-            f1 = a1 >= kmin ? lo : 0;
-          }
-          const int c0 = __ldg(count + a0), c1 = two ? __ldg(count + a1) : 0;
-          const long long b0 = __ldg(start + a0), b1 = two ? __ldg(start + a1) : 0;
-          const float2 nx = make_float2(-pa.x, -pb.x), ny = make_float2(-pa.y, -pb.y),
-                       nz = make_float2(-pa.z, -pb.z);
-          int L0 = 0, L1 = 0;
-#pragma unroll 2
-          for (int t0 = min(f0, f1); t0 < S; t0 += 32) {
-            const int t = t0 + lane;
-            bool k0 = false, k1 = false;
-            int jo = 0;
-            float d20 = 0.f, d21 = 0.f;
-            if (t < S) {
-              const float4 q = st[(int)slots[t]];
-              jo = __float_as_int(q.w);
-              float2 dx, dy, dz;
-              const float2 d2 = pair_d2<DIM>(q, nx, ny, nz, dx, dy, dz);
-              d20 = d2.x;
-              d21 = d2.y;
-              k0 = jo > a0 && d20 < A.rc2;
-              k1 = jo > a1 && d21 < A.rc2;
-            }
-            const unsigned m0 = __ballot_sync(0xffffffffu, k0), m1 = __ballot_sync(0xffffffffu, k1);
-            if (k0) {
-              const int e = L0 + __popc(m0 & lt);
-              if (e < c0) {
-                pi_out[b0 + e] = a0;
-                pj_out[b0 + e] = jo;
-                pd_out[b0 + e] = d20 * rsqrt_nr(d20);
-              }
-            }
-            if (k1) {
-              const int e = L1 + __popc(m1 & lt);
-              if (e < c1) {
-                pi_out[b1 + e] = a1;
-                pj_out[b1 + e] = jo;
-                pd_out[b1 + e] = d21 * rsqrt_nr(d21);
-              }
-            }
-            L0 += __popc(m0);
-            L1 += __popc(m1);
-          }
-        }
-      }
+      if (FILL)
+        for (int p = h0 + 2 * warp; p < h1; p += 2 * W)
+          fill_two<DIM>(A, p, h1, [&](int t) { return st[(int)slots[t]]; }, S, kmin, count, start, pi_out, pj_out, pd_out);
     }
     if (!FILL && threadIdx.x == 0) {
       flag[c] = S > cap ? 1 : 0;
@@ -684,11 +798,13 @@ size_t pairs_cell_smem(int noff, bool fill, int cap) {
   return fill ? head + kBuckets * sizeof(int) + 2 * (size_t)cap * sizeof(unsigned short) : head;
 }
 
+// The staged passes: k_pairs_sparse for sparse grids and k_pairs_cell for the
+// cells it lists, k_pairs_cell alone otherwise.
 template <int DIM, bool FILL>
-static int launch_cell(const SweepArgs& A, float ball2, int cap, const int* last, unsigned char* flag, int* fcells, int* nfcells,
-                       int* count, const long long* start, int* pi, int* pj, float* pd, cudaStream_t s) {
+static int launch_cell(const SweepArgs& A, const PairLists& L, const long long* start, int* pi, int* pj, float* pd,
+                       cudaStream_t s) {
   static DevCache ready;  // shared-memory limit raised on this device
-  if (cap < 32 || cap > kStageMax) return CL_ERR_INVALID_ARG;
+  if (L.cap < 32 || L.cap > kStageMax) return CL_ERR_INVALID_ARG;
   int dev = 0, sms = 0, per = 0;
   if (cudaGetDevice(&dev) != cudaSuccess) return CL_ERR_CUDA;
   if (!ready.get(dev)) {
@@ -697,7 +813,7 @@ static int launch_cell(const SweepArgs& A, float ball2, int cap, const int* last
       return CL_ERR_CUDA;
     ready.put(dev, 1);
   }
-  const size_t smem = pairs_cell_smem(A.noff, FILL, cap);
+  const size_t smem = pairs_cell_smem(A.noff, FILL, L.cap);
   if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess ||
       cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, k_pairs_cell<DIM, FILL>, 256, smem) !=
           cudaSuccess ||
@@ -706,28 +822,32 @@ static int launch_cell(const SweepArgs& A, float ball2, int cap, const int* last
   long long blocks = (long long)sms * per;
   const long long ncells = (long long)A.nx * A.ny * A.nz;
   if (blocks > ncells) blocks = ncells;
-  k_pairs_cell<DIM, FILL><<<(int)blocks, 256, smem, s>>>(A, ball2, cap, last, flag, fcells, nfcells, count,
-                                                                      start, pi, pj, pd);
+  const bool sparse = L.expect <= kSparse;
+  if (sparse) {
+    const size_t sm = sizeof(float4) * (size_t)(A.noff + kSparseWarps * kSparseCap * (FILL ? 2 : 1));
+    const long long sb = std::min<long long>((ncells + kSparseWarps - 1) / kSparseWarps, (long long)sms * 64);
+    k_pairs_sparse<DIM, FILL><<<(int)sb, 32 * kSparseWarps, sm, s>>>(A, L.ball2, L.last, L.mid, L.ctr + 2, L.count,
+                                                                    start, pi, pj, pd);
+  }
+  k_pairs_cell<DIM, FILL><<<(int)blocks, 256, smem, s>>>(A, L.ball2, L.cap, sparse ? L.mid : nullptr, L.ctr + 2, L.last,
+                                                        L.flag, L.fcells, L.ctr + 1, L.count, start, pi, pj, pd);
   return cudaGetLastError() == cudaSuccess ? CL_OK : CL_ERR_CUDA;
 }
 
-int launch_pairs_count(const SweepArgs& A, const Off* off, int dim, float ball2, int cap, int* last, unsigned char* flag,
-                       int* fcells, int* nfcells, int* nlong, int* count, cudaStream_t s) {
+int launch_pairs_count(const SweepArgs& A, const Off* off, int dim, const PairLists& L, cudaStream_t s) {
   if (A.n <= 0) return CL_OK;
   const long long ncells = (long long)A.nx * A.ny * A.nz;
-  k_cell_last<<<(unsigned)((ncells * kLastLanes + 255) / 256), 256, 0, s>>>(ncells, A.cell_start, A.xs, last, nfcells,
-                                                                            nlong);
-  const int e = dim == 3 ? launch_cell<3, false>(A, ball2, cap, last, flag, fcells, nfcells, count, nullptr, nullptr,
-                                                 nullptr, nullptr, s)
-                         : launch_cell<2, false>(A, ball2, cap, last, flag, fcells, nfcells, count, nullptr, nullptr,
-                                                 nullptr, nullptr, s);
+  k_cell_last<<<(unsigned)((ncells * kLastLanes + 255) / 256), 256, 0, s>>>(ncells, A.cell_start, A.xs, L.last, L.ctr);
+  const int e = dim == 3 ? launch_cell<3, false>(A, L, nullptr, nullptr, nullptr, nullptr, s)
+                         : launch_cell<2, false>(A, L, nullptr, nullptr, nullptr, nullptr, s);
   if (e) return e;
   const CrossArgs C = cross_args(A, off);
   const size_t dyn = (size_t)C.noff * sizeof(float4);
+  const int* nf = L.ctr + 1;
   switch (group_lanes(A)) {
-    case 2: k_pairs_count<2><<<152 * 8, 32 * kFillWarps, dyn, s>>>(C, A.cellc, fcells, nfcells, count); break;
-    case 4: k_pairs_count<4><<<152 * 8, 32 * kFillWarps, dyn, s>>>(C, A.cellc, fcells, nfcells, count); break;
-    default: k_pairs_count<8><<<152 * 8, 32 * kFillWarps, dyn, s>>>(C, A.cellc, fcells, nfcells, count); break;
+    case 2: k_pairs_count<2><<<152 * 8, 32 * kFillWarps, dyn, s>>>(C, A.cellc, L.fcells, nf, L.count); break;
+    case 4: k_pairs_count<4><<<152 * 8, 32 * kFillWarps, dyn, s>>>(C, A.cellc, L.fcells, nf, L.count); break;
+    default: k_pairs_count<8><<<152 * 8, 32 * kFillWarps, dyn, s>>>(C, A.cellc, L.fcells, nf, L.count); break;
   }
   return cudaGetLastError() == cudaSuccess ? CL_OK : CL_ERR_CUDA;
 }
@@ -757,29 +877,26 @@ int launch_sort_long(const int* longs, const int* nlong, const int* count, const
   return cudaGetLastError() == cudaSuccess ? CL_OK : CL_ERR_CUDA;
 }
 
-int launch_pairs_fill(const SweepArgs& A, const Off* off, int dim, float ball2, int cap, const int* last,
-                      const unsigned char* flag, const int* fcells,
-                      const int* nfcells, const int* count, const long long* start, int* pi, int* pj, float* pd, int* longs,
-                      int* nlong, cudaStream_t s) {
+int launch_pairs_fill(const SweepArgs& A, const Off* off, int dim, const PairLists& L, const long long* start, int* pi,
+                      int* pj, float* pd, int* longs, cudaStream_t s) {
   if (A.n <= 0) return CL_OK;
-  unsigned char* fl = const_cast<unsigned char*>(flag);  // only read by the fill pass
-  int* cn = const_cast<int*>(count);                     // likewise
-  const int e = dim == 3 ? launch_cell<3, true>(A, ball2, cap, last, fl, nullptr, nullptr, cn, start, pi, pj, pd, s)
-                         : launch_cell<2, true>(A, ball2, cap, last, fl, nullptr, nullptr, cn, start, pi, pj, pd, s);
+  const int e = dim == 3 ? launch_cell<3, true>(A, L, start, pi, pj, pd, s)
+                         : launch_cell<2, true>(A, L, start, pi, pj, pd, s);
   if (e) return e;
   const CrossArgs C = cross_args(A, off);
   const int g = group_lanes(A);
+  int *nf = L.ctr + 1, *nlong = L.ctr;
   int f;
   if (A.n >= (1 << 22))
-    f = launch_fill_listed<8, true>(C, A.cellc, fcells, nfcells, count, start, pi, pj, pd, longs, nlong, s);
+    f = launch_fill_listed<8, true>(C, A.cellc, L.fcells, nf, L.count, start, pi, pj, pd, longs, nlong, s);
   else if (g == 2)
-    f = launch_fill_listed<2, false>(C, A.cellc, fcells, nfcells, count, start, pi, pj, pd, longs, nlong, s);
+    f = launch_fill_listed<2, false>(C, A.cellc, L.fcells, nf, L.count, start, pi, pj, pd, longs, nlong, s);
   else if (g == 4)
-    f = launch_fill_listed<4, false>(C, A.cellc, fcells, nfcells, count, start, pi, pj, pd, longs, nlong, s);
+    f = launch_fill_listed<4, false>(C, A.cellc, L.fcells, nf, L.count, start, pi, pj, pd, longs, nlong, s);
   else
-    f = launch_fill_listed<8, false>(C, A.cellc, fcells, nfcells, count, start, pi, pj, pd, longs, nlong, s);
+    f = launch_fill_listed<8, false>(C, A.cellc, L.fcells, nf, L.count, start, pi, pj, pd, longs, nlong, s);
   if (f) return f;
-  return launch_sort_long(longs, nlong, count, start, pj, pd, s);
+  return launch_sort_long(longs, nlong, L.count, start, pj, pd, s);
 }
 
 }  // namespace clk
