@@ -742,8 +742,10 @@ __device__ __forceinline__ int run_count(const int* __restrict__ cell_start, int
 // every non-empty cell is listed: on list when it holds at most kHome
 // particles and its half stencil's cells at most H.rawcap, on dense (the
 // windowed cells) otherwise. kListLanes lanes share a cell's rows: one thread
-// per cell took 13 us on a grid of 343 cells and 18 on one of 42,875.
-constexpr int kListLanes = 8;
+// per cell took 13 us on a grid of 343 cells and 18 on one of 42,875 (now 11;
+// bound by the latency of the row bounds). Listed by warps instead of blocks,
+// the lists' three counters took 15 us there, 104 at 421,875 cells (now 32).
+constexpr int kListLanes = 8;  // 32 cells to a block of 256
 __global__ void __launch_bounds__(256) k_hood_list(const int* __restrict__ cell_start, int ncells, int noff,
                                                    int* __restrict__ work, int* __restrict__ list,
                                                    unsigned char* __restrict__ flag, int* __restrict__ dense,
@@ -752,7 +754,6 @@ __global__ void __launch_bounds__(256) k_hood_list(const int* __restrict__ cell_
   const int half = H.half;
   const int* opk_half = H.opk[1];
   const int h = (blockIdx.x * blockDim.x + threadIdx.x) / kListLanes, sub = threadIdx.x % kListLanes;
-  const unsigned lt = (1u << (threadIdx.x & 31)) - 1u;
   bool take = false, big = false;
   int cnt = 0;
   if (h < ncells) {
@@ -789,30 +790,33 @@ __global__ void __launch_bounds__(256) k_hood_list(const int* __restrict__ cell_
     take = false;
     big = half != 0;
   }
-  take = take && sub == 0;
-  big = big && sub == 0;
-  // small cells go to the end of list
-  const bool small = take && half && h < ncells && cnt + (cell_start[h + 1] - cell_start[h]) <= H.smallcap;
-  const unsigned ms = __ballot_sync(0xffffffffu, small);
-  int sbase = 0;
-  if ((threadIdx.x & 31) == 0 && ms) sbase = atomicAdd(work + 8, __popc(ms));
-  sbase = __shfl_sync(0xffffffffu, sbase, 0);
-  if (small) {
-    list[ncells - 1 - (sbase + __popc(ms & lt))] = h;
-    flag[h] = 0;
-    take = false;
+  // the block's cells listed by its first warp, a cell per lane: one atomic per
+  // block and list
+  __shared__ unsigned char kind[32];  // 0 empty, 1 listed, 2 dense, 3 small, 4 left to the companion
+  if (sub == 0) {
+    const int nh = h < ncells ? cell_start[h + 1] - cell_start[h] : 0;
+    const bool small = take && half && cnt + nh <= H.smallcap;
+    kind[threadIdx.x / kListLanes] = nh == 0 ? 0 : (small ? 3 : (take ? 1 : (big ? 2 : 4)));
   }
-  if (h < ncells && sub == 0 && !small) flag[h] = take || cell_start[h + 1] == cell_start[h] ? 0 : (big ? 2 : 1);
-  const unsigned m = __ballot_sync(0xffffffffu, take), mb = __ballot_sync(0xffffffffu, big);
-  int base = 0, bbase = 0;
-  if ((threadIdx.x & 31) == 0) {
+  __syncthreads();
+  if (threadIdx.x >= 32) return;
+  const int lane = threadIdx.x, c = blockIdx.x * 32 + lane, k = kind[lane];
+  if (c < ncells) flag[c] = k == 2 ? 2 : (k == 4 ? 1 : 0);
+  const unsigned lt = (1u << lane) - 1u;
+  const unsigned m = __ballot_sync(0xffffffffu, k == 1), mb = __ballot_sync(0xffffffffu, k == 2),
+                 ms = __ballot_sync(0xffffffffu, k == 3);
+  int base = 0, bbase = 0, sbase = 0;
+  if (lane == 0) {
     if (m) base = atomicAdd(work + 6, __popc(m));
     if (mb) bbase = atomicAdd(ndense, __popc(mb));
+    if (ms) sbase = atomicAdd(work + 8, __popc(ms));
   }
   base = __shfl_sync(0xffffffffu, base, 0);
   bbase = __shfl_sync(0xffffffffu, bbase, 0);
-  if (take) list[base + __popc(m & lt)] = h;
-  if (big) dense[bbase + __popc(mb & lt)] = h;
+  sbase = __shfl_sync(0xffffffffu, sbase, 0);
+  if (k == 1) list[base + __popc(m & lt)] = c;
+  if (k == 2) dense[bbase + __popc(mb & lt)] = c;
+  if (k == 3) list[ncells - 1 - (sbase + __popc(ms & lt))] = c;  // small cells go to the end of list
 }
 
 // Per-CTA partials from the per-thread outputs (layout of the other sweeps).

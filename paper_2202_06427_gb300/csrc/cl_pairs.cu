@@ -642,9 +642,8 @@ __device__ __forceinline__ void fill_two(const SweepArgs& A, int p, int h1, At a
 // counting the smaller indices of each. Latency-bound: 2D lists with their
 // builds took, with a CTA of eight warps per cell of one particle, 525 us at
 // 57,000 particles and 371 at 31,000; 190 and 178 so. Cells that do not fit are
-// listed (cells) for k_pairs_cell in both passes. kSparse: the fullest list of
-// 2D grids in use holds 40 in its ball; from some hundreds on a warp's ordering
-// (S / 32 S comparisons) costs more than the CTA's buckets.
+// listed (cells) for k_pairs_cell in both passes. kSparse: those two lists expect
+// 25 in a ball, 2D lists at other cell sizes up to 40; denser grids keep the CTA.
 constexpr int kSparse = 64, kSparseCap = 160, kSparseWarps = 4;
 static_assert((kMaxOff + 2 * kSparseWarps * kSparseCap) * sizeof(float4) <= 48 * 1024, "the default shared memory");
 
