@@ -64,18 +64,19 @@ FLOP_PER_HIT_HALF = 22
 # original index (4 B); the per-cell counts and offsets add 8 B per cell.
 BIN_BYTES_PER_PARTICLE = 44
 BIN_BYTES_PER_CELL = 8
-# DRAM bytes per launch of the dominant kernel (k_hood_half<3, 0> on the 1M
+# DRAM bytes per launch of the dominant kernel (k_hood_half<3> on the 1M
 # lattice) from one ncu capture of its current version (dram__bytes_read.sum +
-# dram__bytes_write.sum = 36.40 + 0.00 MB), or None when the kernel has changed
+# dram__bytes_write.sum = 36.40 + 0.16 MB), or None when the kernel has changed
 # since the counters were taken.
-SWEEP_DRAM_BYTES = 36_400_384
+SWEEP_DRAM_BYTES = 36_554_496
 FP32_LANES_PER_SM = 128
-# kernels of one headline step: bin, 2 scan, scatter, packed cells (binning);
-# cell list, octant order of the windowed cells, half-shell sweep of the
-# fast-path cells, of the windowed cells (both exit at once when there are
-# none), per-particle finish, final reduction (cl_energy_grad); 2 scale
-# (chain rule for positions and box)
-STEP_LAUNCHES = 13
+# kernels of one headline step: bin, scan, scatter (binning); cell list, order
+# of the windowed cells, half-shell sweep of the fast-path cells, of the
+# windowed and small cells (the last two exit at once when there are none),
+# per-particle finish, final reduction (cl_energy_grad); 2 scale (chain rule for
+# positions and box). The clustered set's grid of 421,875 cells takes a second
+# scan kernel, and its 16M particles' packed cells a kernel of their own.
+STEP_LAUNCHES = {"w1_lattice_1m": 11, "w4_clustered_16m": 13}
 
 
 def parse():
@@ -445,7 +446,7 @@ def pairlist_leg(dev, steps, warmup, pool=None):
                         "kernel_ms": lms, "bytes_per_launch": nbytes,
                         "bytes_basis": "12 B per pair written + 16 B per particle read per pass", "peak_basis": basis},
            "binning": binning_record(n, P.cl_query(cl, "ncells"), bms, peaks, basis),
-           "gpu_launches_per_step": 15}
+           "gpu_launches_per_step": 12}
     if pool is not None:
         pool.load(w["x"])
         ref = pool.run(h, rc, nbins=nbins, forces=False)
@@ -625,7 +626,7 @@ def run_ours(args, rank, world, local):
                        "step": "binning + fused energy/forces/box-gradient sweep (forward) + chain rule (backward)",
                        "l2": "flushed between steps by a 256 MB write outside the timed events",
                        "parallelism": "replicas" if world > 1 else "single GPU"},
-            "gpu_launches": STEP_LAUNCHES * args.steps,
+            "gpu_launches": STEP_LAUNCHES[workload] * args.steps,
             "clocks": clocks, "roofline": roofline,
             "binning": binning_record(n, ncells, bms, peaks, basis),
             "sweep_pairs_per_s": pairs / (kms / 1e3)}
