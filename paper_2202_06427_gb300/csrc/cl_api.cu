@@ -554,7 +554,7 @@ struct QueryWs {
     const long long nc = c->geo.ncells;
     v.take(&bin.q, n);
     v.take(&bin.cell, n);
-    if (clk::queries_sorted(nb, nc)) {
+    if (clk::queries_sorted(c->n, nb, nc)) {
       v.take(&bin.raw, n);
       v.take(&bin.slot, n);
       v.take(&bin.counts, (size_t)nc);

@@ -14,7 +14,8 @@
 //                  cell's range: the per-cell contiguous copy of Sec. 2.6
 //                  ("vector of lists ... an immutable copy of the particle
 //                  coordinates and index", Sec. 2.8).
-//   k_cellc        the packed cell of every sorted particle, cell by cell.
+//   k_cellc        the packed cell of every sorted particle, cell by cell, where
+//                  k_scatter does not write it (launch_cell_order).
 //   k_octsort      (launched by the 3D half-shell sweep on its windowed cells)
 //                  cells of kOctMin..kOctCap particles ordered by the octant
 //                  of their local coordinates (slots updated to match).

@@ -291,7 +291,7 @@ struct QueryBufs {
   int* tiles;       // scan_tiles_for(ncells), sorted only
   int* meta;        // 4, sorted only
 };
-bool queries_sorted(long long nb, long long ncells);
+bool queries_sorted(long long n, long long nb, long long ncells);
 int launch_query_bin(const SweepArgs& A, const Geo& g, const double* posb, long long nb, const QueryBufs& b, int* err,
                      Queries* out, cudaStream_t s);
 // The sweeps (off: the full stencil in device memory). Count: per query (count

@@ -18,18 +18,20 @@ def _dev(x):
     return torch.from_numpy(np.ascontiguousarray(x)).cuda()
 
 
-@pytest.mark.parametrize("dim,tric,nb", [(3, False, 2048), (3, True, 2049), (2, True, 5003)])
-def test_query_order(cuda_ok, dim, tric, nb):
-    """From 2,048 queries on they are taken in the order of their cells: the
-    same lists, bit for bit, as in calls of at most 2,047."""
+@pytest.mark.parametrize("dim,L,nb", [(3, 40.0, 16400), (2, 200.0, 10400)])
+def test_query_order(cuda_ok, dim, L, nb):
+    """About a set that passes the L2, many queries are taken in the order of
+    their cells: the same lists, bit for bit, as in calls of at most 2,047."""
     import paper_2202_06427_gb300 as P
-    rng = np.random.default_rng(31 + nb)
-    L = 20.0 if dim == 3 else 60.0
+    g = torch.Generator(device="cuda").manual_seed(31 + nb)
+    n = (6 << 20) + 11
     h = np.eye(dim) * L
-    if tric:
-        h[1, 0] = 0.2 * L
-    cl = P.cl_build(_dev(rng.uniform(-1, 2, size=(4000, dim)) @ h), h, 2.5, 2)
-    y = _dev(rng.uniform(-1, 2, size=(nb, dim)) @ h)
+    h[1, 0] = 0.2 * L
+    ht = torch.from_numpy(h).cuda()
+    x = (3 * torch.rand((n, dim), generator=g, device="cuda", dtype=torch.float64) - 1) @ ht
+    y = (3 * torch.rand((nb, dim), generator=g, device="cuda", dtype=torch.float64) - 1) @ ht
+    cl = P.cl_build(x, h, 1.0, 1)
+    assert 4 * nb >= P.cl_query(cl, "ncells")
     parts = [(s, y[s:s + 1999].contiguous()) for s in range(0, nb, 1999)]
     whole, lists = P.cl_cross_pairlist(cl, y), [P.cl_cross_pairlist(cl, p) for _, p in parts]
     assert P.cl_cross_count(cl, y) == sum(P.cl_cross_count(cl, p) for _, p in parts) == whole["a"].numel()
