@@ -257,6 +257,14 @@ double pairs_expected(const clk::Geo& g, long long n, float ball2) {
   return (vol > 0 ? (double)n / vol : 0.0) * ball;
 }
 
+// The stencil holds a cell twice: it reaches m_k cells each way along an axis of
+// fewer than 2 m_k + 1 (the reach of build_stencils).
+bool stencil_wraps(const clk::Geo& g) {
+  for (int k = 0; k < g.dim; ++k)
+    if (g.n[k] < 2 * (int)std::ceil(g.rc * g.n[k] / g.w[k]) + 1) return true;
+  return false;
+}
+
 // Staged entries per cell: that with 30 % to spare, in steps of 128 (1,024 to
 // 3,072). Denser cells overflow and take the per-particle path.
 int pairs_stage_cap(double expect) {
@@ -294,6 +302,7 @@ int map_pairlist(cl_list* c, cl_result* r, cudaStream_t s) {
   L.ball2 = pairs_ball2(c->geo);
   L.expect = pairs_expected(c->geo, c->n, L.ball2);
   L.cap = pairs_stage_cap(L.expect);
+  L.images = stencil_wraps(c->geo);
   L.last = c->hdense;
   L.flag = c->hflag;
   L.fcells = c->hlist;

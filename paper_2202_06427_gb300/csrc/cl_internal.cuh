@@ -332,6 +332,7 @@ struct PairLists {
   float ball2;          // squared radius about a cell's centre that holds the cell's neighbours
   int cap;              // staged entries per cell (32..3072)
   double expect;        // particles expected in that ball
+  bool images;          // the stencil reaches some cell twice: two images of a particle may be staged
   int* last;            // ncells: largest original index per cell
   unsigned char* flag;  // ncells: 1 for the cells of fcells
   int* fcells;          // ncells: cells whose neighbourhood passes cap

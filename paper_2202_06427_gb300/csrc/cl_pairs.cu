@@ -342,7 +342,12 @@ constexpr int kBucketMost = 48;  // a fuller bucket sends the cell to the radix 
 // against thirteen for the radix sort's three passes. A cell whose fullest
 // bucket passes kBucketMost (indices in a few tight clumps) takes the radix
 // sort.
-template <int W>
+//
+// IMAGES: two images of a particle may be staged (PairLists), one at most within
+// the cutoff. Each needs a place of its own, so an entry also counts the equal
+// ones before it: a variant of its own, because doing so always took a list of
+// 2.1e8 pairs with a histogram from 4.12 to 4.22 ms (a branch on it 4.16).
+template <int W, bool IMAGES>
 __device__ __forceinline__ void stage_sort(const float4* st, int S, unsigned short* s0, unsigned short* s1, int* cnt,
                                            int* scal, unsigned short*& slots, int& kmin) {
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
@@ -419,7 +424,7 @@ __device__ __forceinline__ void stage_sort(const float4* st, int S, unsigned sho
     const unsigned b = (unsigned)(jo - kmin) >> sh;
     const int b0 = cnt[b], b1 = b + 1 < (unsigned)kBuckets ? cnt[b + 1] : S;
     int r = b0;
-    for (int q = b0; q < b1; ++q) r += __float_as_int(st[s1[q]].w) < jo ? 1 : 0;
+    for (int q = b0; q < b1; ++q) r += __float_as_int(st[s1[q]].w) < jo + (IMAGES && q < p ? 1 : 0) ? 1 : 0;
     s0[r] = (unsigned short)i;
   }
   __syncthreads();
@@ -719,8 +724,8 @@ __global__ void __launch_bounds__(32 * kSparseWarps) k_pairs_sparse(const __grid
 // by original index (stage_sort), so a particle's pairs with
 // j > a come from a suffix of that order in ascending j and are written in
 // order, coalesced, as the ballot finds them.
-// With cells, the *nlisted cells of that list only.
-template <int DIM, bool FILL>
+// With cells, the *nlisted cells of that list only. IMAGES: see stage_sort.
+template <int DIM, bool FILL, bool IMAGES>
 __global__ void __launch_bounds__(256, FILL ? 5 : 6) k_pairs_cell(const __grid_constant__ SweepArgs A,
                                                                                float ball2, int cap,
                                                                                const int* __restrict__ cells,
@@ -775,7 +780,7 @@ __global__ void __launch_bounds__(256, FILL ? 5 : 6) k_pairs_cell(const __grid_c
     if (S <= cap) {
       unsigned short* slots = rs0;
       int kmin = 0;
-      if (FILL) stage_sort<W>(st, S, rs0, rs1, cnt, scal, slots, kmin);
+      if (FILL) stage_sort<W, IMAGES>(st, S, rs0, rs1, cnt, scal, slots, kmin);
       if (!FILL) {
         for (int p = h0 + 2 * warp; p < h1; p += 2 * W) count_two<DIM>(A, p, h1, st, S, count);
       }
@@ -799,7 +804,7 @@ size_t pairs_cell_smem(int noff, bool fill, int cap) {
 
 // The staged passes: k_pairs_sparse for sparse grids and k_pairs_cell for the
 // cells it lists, k_pairs_cell alone otherwise.
-template <int DIM, bool FILL>
+template <int DIM, bool FILL, bool IMAGES>
 static int launch_cell(const SweepArgs& A, const PairLists& L, const long long* start, int* pi, int* pj, float* pd,
                        cudaStream_t s) {
   static DevCache ready;  // shared-memory limit raised on this device
@@ -807,14 +812,14 @@ static int launch_cell(const SweepArgs& A, const PairLists& L, const long long* 
   int dev = 0, sms = 0, per = 0;
   if (cudaGetDevice(&dev) != cudaSuccess) return CL_ERR_CUDA;
   if (!ready.get(dev)) {
-    if (cudaFuncSetAttribute(k_pairs_cell<DIM, FILL>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+    if (cudaFuncSetAttribute(k_pairs_cell<DIM, FILL, IMAGES>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                              (int)pairs_cell_smem(kMaxOff, FILL, kStageMax)) != cudaSuccess)
       return CL_ERR_CUDA;
     ready.put(dev, 1);
   }
   const size_t smem = pairs_cell_smem(A.noff, FILL, L.cap);
   if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess ||
-      cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, k_pairs_cell<DIM, FILL>, 256, smem) !=
+      cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, k_pairs_cell<DIM, FILL, IMAGES>, 256, smem) !=
           cudaSuccess ||
       per < 1)
     return CL_ERR_CUDA;
@@ -828,8 +833,9 @@ static int launch_cell(const SweepArgs& A, const PairLists& L, const long long* 
     k_pairs_sparse<DIM, FILL><<<(int)sb, 32 * kSparseWarps, sm, s>>>(A, L.ball2, L.last, L.mid, L.ctr + 2, L.count,
                                                                     start, pi, pj, pd);
   }
-  k_pairs_cell<DIM, FILL><<<(int)blocks, 256, smem, s>>>(A, L.ball2, L.cap, sparse ? L.mid : nullptr, L.ctr + 2, L.last,
-                                                        L.flag, L.fcells, L.ctr + 1, L.count, start, pi, pj, pd);
+  k_pairs_cell<DIM, FILL, IMAGES><<<(int)blocks, 256, smem, s>>>(A, L.ball2, L.cap, sparse ? L.mid : nullptr,
+                                                                L.ctr + 2, L.last, L.flag, L.fcells, L.ctr + 1,
+                                                                L.count, start, pi, pj, pd);
   return cudaGetLastError() == cudaSuccess ? CL_OK : CL_ERR_CUDA;
 }
 
@@ -837,8 +843,8 @@ int launch_pairs_count(const SweepArgs& A, const Off* off, int dim, const PairLi
   if (A.n <= 0) return CL_OK;
   const long long ncells = (long long)A.nx * A.ny * A.nz;
   k_cell_last<<<(unsigned)((ncells * kLastLanes + 255) / 256), 256, 0, s>>>(ncells, A.cell_start, A.xs, L.last, L.ctr);
-  const int e = dim == 3 ? launch_cell<3, false>(A, L, nullptr, nullptr, nullptr, nullptr, s)
-                         : launch_cell<2, false>(A, L, nullptr, nullptr, nullptr, nullptr, s);
+  const int e = dim == 3 ? launch_cell<3, false, false>(A, L, nullptr, nullptr, nullptr, nullptr, s)
+                         : launch_cell<2, false, false>(A, L, nullptr, nullptr, nullptr, nullptr, s);
   if (e) return e;
   const CrossArgs C = cross_args(A, off);
   const size_t dyn = (size_t)C.noff * sizeof(float4);
@@ -879,8 +885,13 @@ int launch_sort_long(const int* longs, const int* nlong, const int* count, const
 int launch_pairs_fill(const SweepArgs& A, const Off* off, int dim, const PairLists& L, const long long* start, int* pi,
                       int* pj, float* pd, int* longs, cudaStream_t s) {
   if (A.n <= 0) return CL_OK;
-  const int e = dim == 3 ? launch_cell<3, true>(A, L, start, pi, pj, pd, s)
-                         : launch_cell<2, true>(A, L, start, pi, pj, pd, s);
+  int e;
+  if (dim == 3)
+    e = L.images ? launch_cell<3, true, true>(A, L, start, pi, pj, pd, s)
+                 : launch_cell<3, true, false>(A, L, start, pi, pj, pd, s);
+  else
+    e = L.images ? launch_cell<2, true, true>(A, L, start, pi, pj, pd, s)
+                 : launch_cell<2, true, false>(A, L, start, pi, pj, pd, s);
   if (e) return e;
   const CrossArgs C = cross_args(A, off);
   const int g = group_lanes(A);
