@@ -2013,6 +2013,7 @@ __device__ __noinline__ void half_unit(HalfSmem& S, const Unit u, UnitAcc& acc, 
     __syncwarp();
   }
   if (!SCALAR) {  // kBatch = 32: a lane per home particle
+    __syncwarp();  // the sums' last additions: after the own part alone nothing else orders them
     const float gx = hg[lane][0], gy = hg[lane][1], gz = hg[lane][2];
     if (lane < nbh && (gx != 0.f || gy != 0.f || gz != 0.f))
       atomicAdd(&X.hforce[u.hp + lane], make_float4(-gx, -gy, -gz, 0.f));

@@ -71,3 +71,34 @@ def test_kinds_of_cells(cuda_ok, name):
         check_matrix(gb.cpu().numpy(), 0.75 * ref["dedh"], TOL_GB)
     occupied = P.cl_query(cl, "max_occupancy")
     assert occupied > 2048 if name == "huge" else occupied <= 2048
+
+
+@pytest.mark.parametrize("lcell", [1, 2])
+def test_clumps_beyond_each_others_cutoff(cuda_ok, lcell):
+    """Clumps of 2 to 300 particles farther apart than the cutoff: a batch's own
+    particles are all it is swept against (nothing listed), in the cells of one
+    warp and, last batch by last batch, in the windowed ones."""
+    import paper_2202_06427_gb300 as P
+    rng = np.random.default_rng(8 + lcell)
+    L, rc = 36.0, 3.0
+    h = np.eye(3) * L
+    h[2, 1] = 2.0
+    sizes = [2, 3, 4, 5, 8, 31, 32, 33, 63, 64, 65, 128, 129, 160, 257, 300]
+    sites = np.stack(np.meshgrid(*[np.arange(6)] * 3, indexing="ij"), -1).reshape(-1, 3) / 6 + 0.5 / 12
+    x = []
+    for k, s in enumerate(sites):
+        g = np.stack(np.meshgrid(*[np.arange(-3, 4) * 0.2] * 3, indexing="ij"), -1).reshape(-1, 3)
+        g = g[rng.permutation(len(g))[:sizes[k % len(sizes)]]]
+        x.append(s @ h + g + rng.uniform(-0.05, 0.05, size=g.shape))
+    x = np.vstack(x)
+    x = np.ascontiguousarray(x[rng.permutation(len(x))])
+    ref = oracle.pair_map(x, h, rc, band=BAND, nbins=17)
+    cl = P.cl_build(torch.from_numpy(x).cuda(), h, rc, lcell)
+    g = torch.tensor([0.75], dtype=torch.float64, device="cuda")
+    for _ in range(2):
+        efv = P.cl_map(cl, "energy_forces_virial")
+        check_energy(efv["energy"].item(), ref["energy"])
+        check_forces(efv["forces"].cpu().numpy(), ref["forces"])
+        check_matrix(efv["virial"].cpu().numpy(), ref["virial"], TOL_W)
+        gp, _, _ = P.cl_backward(cl, g)  # (no pair crosses the boundary: dE/dH is zero)
+        check_forces(gp.cpu().numpy(), -0.75 * ref["forces"])
