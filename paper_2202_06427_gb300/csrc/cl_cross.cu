@@ -367,25 +367,37 @@ __global__ void __launch_bounds__(1024) k_topk_last(const int* __restrict__ la, 
   if (lane == 0) *found = __popc(have);
 }
 
+// CTAs of one wave of the kernel for nb queries. The kernel's shared-memory limit
+// is raised once per device, to what its largest stencil takes: a limit set to
+// each call's own size could be lowered by another thread's smaller grid between
+// this call's set and its launch, which then failed. ready: the kernel's own.
 template <class K>
-int cross_grid(K kernel, int warps, size_t smem, long long nb) {
+int cross_grid(K kernel, DevCache& ready, int warps, size_t most, size_t smem, long long nb) {
   int dev = 0, sms = 0, per = 0;
   if (cudaGetDevice(&dev) != cudaSuccess ||
       cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
     return 0;
-  if (smem > 32 * 1024 &&
-      cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess)
-    return 0;
+  if (!ready.get(dev)) {
+    if (cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)most) != cudaSuccess) return 0;
+    ready.put(dev, 1);
+  }
   if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, kernel, 32 * warps, smem) != cudaSuccess || per < 1)
     return 0;
   const long long want = (nb + warps - 1) / warps;
   return (int)(want < (long long)sms * per ? want : (long long)sms * per);
 }
 
+constexpr size_t count_smem(int noff) { return (size_t)noff * sizeof(float4); }
+constexpr size_t fill_smem(int noff) {
+  return (size_t)noff * sizeof(float4) + (size_t)kFillWarps * 2 * kSegPad * sizeof(float);
+}
+constexpr size_t knn_smem(int noff) { return (size_t)noff * (sizeof(float4) + sizeof(float)); }
+
 template <int G>
 int run_count(const CrossArgs& C, const Queries& Q, int* count, unsigned long long* total, cudaStream_t s) {
-  const size_t smem = (size_t)C.noff * sizeof(float4);
-  const int grid = cross_grid(k_cross_count<G>, kCrossWarps, smem, Q.nb);
+  static DevCache ready;
+  const size_t smem = count_smem(C.noff);
+  const int grid = cross_grid(k_cross_count<G>, ready, kCrossWarps, count_smem(kMaxOff), smem, Q.nb);
   if (grid < 1) return CL_ERR_CUDA;
   k_cross_count<G><<<grid, 32 * kCrossWarps, smem, s>>>(C, Q, count, total);
   return cudaGetLastError() == cudaSuccess ? CL_OK : CL_ERR_CUDA;
@@ -394,8 +406,9 @@ int run_count(const CrossArgs& C, const Queries& Q, int* count, unsigned long lo
 template <int G, bool WIDE>
 int run_fill(const CrossArgs& C, const Queries& Q, const int* count, const long long* start, int* pa, int* pb,
              float* pd, int* longs, int* nlong, cudaStream_t s) {
-  const size_t smem = (size_t)C.noff * sizeof(float4) + (size_t)kFillWarps * 2 * kSegPad * sizeof(float);
-  const int grid = cross_grid(k_cross_fill<G, WIDE>, kFillWarps, smem, Q.nb);
+  static DevCache ready;
+  const size_t smem = fill_smem(C.noff);
+  const int grid = cross_grid(k_cross_fill<G, WIDE>, ready, kFillWarps, fill_smem(kMaxOff), smem, Q.nb);
   if (grid < 1) return CL_ERR_CUDA;
   k_cross_fill<G, WIDE><<<grid, 32 * kFillWarps, smem, s>>>(C, Q, count, start, pa, pb, pd, longs, nlong);
   return cudaGetLastError() == cudaSuccess ? CL_OK : CL_ERR_CUDA;
@@ -403,8 +416,9 @@ int run_fill(const CrossArgs& C, const Queries& Q, const int* count, const long 
 
 template <int G>
 int run_knn(const CrossArgs& C, const Queries& Q, int k, int* out_a, float* out_d, cudaStream_t s) {
-  const size_t smem = (size_t)C.noff * (sizeof(float4) + sizeof(float));
-  const int grid = cross_grid(k_cross_knn<G>, kCrossWarps, smem, Q.nb);
+  static DevCache ready;
+  const size_t smem = knn_smem(C.noff);
+  const int grid = cross_grid(k_cross_knn<G>, ready, kCrossWarps, knn_smem(kMaxOff), smem, Q.nb);
   if (grid < 1) return CL_ERR_CUDA;
   k_cross_knn<G><<<grid, 32 * kCrossWarps, smem, s>>>(C, Q, k, out_a, out_d);
   return cudaGetLastError() == cudaSuccess ? CL_OK : CL_ERR_CUDA;
