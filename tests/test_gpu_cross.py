@@ -163,3 +163,30 @@ def test_cross_errors(cuda_ok):
     assert e.value.code == -3
     empty = P.cl_cross_topk(cl, torch.zeros((0, 3), dtype=torch.float64, device="cuda"), 5)
     assert empty["n"] == 0
+
+
+@pytest.mark.parametrize("dim,tric", [(2, True), (3, True), (3, False)])
+@pytest.mark.parametrize("lcell", [1, 2, 3])
+def test_nearest_ties_at_zero(cuda_ok, dim, tric, lcell):
+    """Queries on points of A that stand three times in it, as different images,
+    many on cell boundaries, where rounding puts images into different cells:
+    distances of 0 tie, the smaller index goes first, and the k nearest are the
+    first k of the 8 nearest."""
+    import paper_2202_06427_gb300 as P
+    rng = np.random.default_rng(11 * dim + lcell)
+    h = np.eye(dim) * 20.0
+    if tric:
+        h[np.tril_indices(dim, -1)] = [3.7] if dim == 2 else [3.7, -2.3, 1.9]
+    rc, m = 2.0, 6000
+    n = np.array(P.cl_box_info(h, rc, lcell)["grid"])
+    s = rng.uniform(size=(m, dim))
+    s = np.where(rng.random((m, dim)) < 0.7, np.round(s * n) / n, s)
+    x = s @ h
+    xa = np.vstack([(s + rng.integers(-3, 4, size=s.shape)) @ h, x + rng.integers(-3, 4, size=s.shape) @ h, x])
+    cl = P.cl_build(torch.from_numpy(xa).cuda(), h, rc, lcell)
+    y = torch.from_numpy(x).cuda()
+    a8, d8 = P.cl_cross_knn(cl, y, 8)
+    assert int((d8[:, 0] == 0).sum()) > m // 2
+    for k in (1, 2, 3):
+        a, d = P.cl_cross_knn(cl, y, k)
+        assert torch.equal(a, a8[:, :k]) and torch.equal(d, d8[:, :k])
