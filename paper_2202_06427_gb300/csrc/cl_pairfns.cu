@@ -229,6 +229,14 @@ __global__ void __launch_bounds__(256) k_sweep_lj(const __grid_constant__ SweepA
   block_sum_store<1>(v, partials + blockIdx.x);
 }
 
+// After a sweep that used the list's force buffer as scratch: the buffer cleared
+// for the next force sweep, also when the launches report an error (an earlier
+// error of the calling thread is enough for that), and their status.
+int scratch_done(float4* hforce, int n, cudaStream_t s) {
+  const bool ok = cudaGetLastError() == cudaSuccess;
+  return cudaMemsetAsync(hforce, 0, sizeof(float4) * (size_t)n, s) == cudaSuccess && ok ? CL_OK : CL_ERR_CUDA;
+}
+
 // The functors' cutoff test: the FP32 cutoff squared in FP32.
 float functor_rc2(double rc) { return (float)rc * (float)rc; }
 
@@ -266,8 +274,7 @@ extern "C" int cl_map_mass(const cl_list* cl, const float* mass_dev, double* out
     const int blocks = (v.n + 255) / 256;
     clk::k_sorted_mass<<<blocks, 256, 0, s>>>(L.half->xs, v.n, mass_dev, L.hforce);
     clk::k_sweep_mass<<<blocks, 256, 0, s>>>(*L.half, L.hforce, clk::functor_rc2(L.rc), L.partials);
-    if (cudaGetLastError() != cudaSuccess) return CL_ERR_CUDA;
-    if (cudaMemsetAsync(L.hforce, 0, sizeof(float4) * (size_t)v.n, s) != cudaSuccess) return CL_ERR_CUDA;
+    if ((e = clk::scratch_done(L.hforce, v.n, s))) return e;
     return clk::finish_reduction(0, 3, nullptr, blocks, 1, L.partials, L.sums, out_dev, nullptr, nullptr, nullptr, s);
   }
   cellmap::pairfn::MassPotential f;
@@ -333,8 +340,7 @@ extern "C" int cl_map_velocity_hist(const cl_list* cl, const float* vel_dev, dou
     clk::k_sorted_velocity<<<(v.n + 255) / 256, 256, 0, s>>>(L.half->xs, v.n, vel_dev, L.hforce);
     clk::k_sweep_velocity<<<(v.n + T - 1) / T, T, sizeof(float2) * nbins * T, s>>>(
         *L.half, L.hforce, clk::functor_rc2(L.rc), (float)(1.0 / binstep), nbins, counts_dev, vsum_dev);
-    if (cudaGetLastError() != cudaSuccess) return CL_ERR_CUDA;
-    return cudaMemsetAsync(L.hforce, 0, sizeof(float4) * (size_t)v.n, s) == cudaSuccess ? CL_OK : CL_ERR_CUDA;
+    return clk::scratch_done(L.hforce, v.n, s);
   }
   if (nbins <= 16) return velocity_hist_nb<16>(cl, vel_dev, v.dim, binstep, nbins, counts_dev, vsum_dev, s);
   return velocity_hist_nb<CL_VHIST_MAX_BINS>(cl, vel_dev, v.dim, binstep, nbins, counts_dev, vsum_dev, s);

@@ -95,3 +95,32 @@ def test_pair_functions_reject_bad_arguments(cuda_ok):
         P.cl_map_velocity_hist(cl, torch.zeros((4, 3), device="cuda"), 0.5, 0)
     with pytest.raises(CellMapError):
         P.cl_map_velocity_hist(cl, torch.zeros((4, 3), device="cuda"), 0.5, 65)
+
+
+@pytest.mark.parametrize("call", ["mass", "velocity"])
+def test_failed_call_leaves_the_list_usable(cuda_ok, call):
+    """A call that reports an error (here one that the calling thread had left
+    pending) leaves nothing in the list's buffers: the forces are as before."""
+    import ctypes
+    import paper_2202_06427_gb300 as P
+    from paper_2202_06427_gb300 import _lib
+    lib = _lib.lib()
+    n = 4000
+    x = torch.from_numpy(np.random.default_rng(3).uniform(0, 20, size=(n, 3))).cuda()
+    cl = P.cl_build(x, np.eye(3) * 20.0, 3.0, 1)
+    want = P.cl_map(cl, "energy_forces_virial")["forces"]
+    v = torch.ones((n, 3), dtype=torch.float32, device="cuda")
+    out = torch.zeros(32, dtype=torch.float64, device="cuda")
+    torch.cuda.synchronize()
+    ptr = lambda t: ctypes.c_void_p(t.data_ptr())
+    stream = ctypes.c_void_p(torch.cuda.current_stream().cuda_stream)
+    runtime = ctypes.CDLL("libcudart.so.13")
+    assert runtime.cudaSetDevice(9999) != 0  # refused on the host; stays pending
+    if call == "mass":
+        code = lib.cl_map_mass(cl.handle, ptr(v), ptr(out), stream)
+    else:
+        code = lib.cl_map_velocity_hist(cl.handle, ptr(v), 0.3, 10, ptr(out), ptr(out[16:]), stream)
+    assert code == -8 and runtime.cudaGetLastError() == 0
+    got = P.cl_map(cl, "energy_forces_virial")["forces"]
+    # the sums of a particle's forces come in another order from call to call
+    assert torch.allclose(got, want, rtol=0, atol=1e-5 * want.abs().max().item())
