@@ -119,6 +119,7 @@ int alloc_cells(cl_list* c, long long ncells, cudaStream_t s) {
     c->bytes -= carve_cells(&old, nullptr, c->ncells_alloc);
     cudaDeviceSynchronize();
     clk::mem_free(c->cell_block, s);
+    clk::mem_settle(s);
   }
   c->cell_block = block;
   c->counts = p.counts;
@@ -548,10 +549,15 @@ struct QueryWs {
   long long* part_id = nullptr;
 
   QueryWs(cl_list* list, cudaStream_t stream) : c(list), s(stream) {}
-  ~QueryWs() { clk::mem_free(base, s); }
+  ~QueryWs() {
+    clk::mem_free(base, s);
+    if (bytes > clk::kPoolKeep) clk::mem_settle(s);
+  }
   // list: the arrays of the cross list; k > 0: those of the global k closest.
   int open(long long nb, bool list, int k) {
-    if (int e = clk::mem_alloc(&base, carve(nullptr, nb, list, k), s)) return e;
+    const size_t need = carve(nullptr, nb, list, k);
+    if (int e = clk::mem_alloc(&base, need, s)) return e;
+    bytes = need;
     carve((char*)base, nb, list, k);
     return cudaMemsetAsync(err, 0, sizeof(long long), s) == cudaSuccess ? CL_OK : CL_ERR_CUDA;
   }
@@ -591,6 +597,7 @@ struct QueryWs {
   cl_list* c;
   cudaStream_t s;
   void* base = nullptr;
+  size_t bytes = 0;
 };
 
 int read_err(const int* err_dev, cudaStream_t s) {
@@ -770,8 +777,9 @@ void cl_free(cl_list* c) {
   int dev = -1;
   const bool other = cudaGetDevice(&dev) == cudaSuccess && dev != c->device;
   if (other) cudaSetDevice(c->device);
-  cudaDeviceSynchronize();
+  cudaDeviceSynchronize();  // what earlier calls freed beyond kPoolKeep goes back here
   free_all(c);
+  if (c->bytes > clk::kPoolKeep / 16) clk::mem_settle(nullptr);
   if (other) cudaSetDevice(dev);
   delete c;
 }

@@ -134,6 +134,10 @@ namespace clk {
 // that keeps at most kPoolKeep bytes of freed memory for later calls.
 int mem_alloc(void** p, size_t bytes, cudaStream_t s);
 void mem_free(void* p, cudaStream_t s);
+constexpr unsigned long long kPoolKeep = 256ull << 20;
+// After frees on s: freed memory beyond kPoolKeep goes back to the device now.
+// Waits for s when the pool holds more than that.
+void mem_settle(cudaStream_t s);
 // Pieces of one block, 256-byte aligned: with base null only their total is
 // counted.
 struct Carver {

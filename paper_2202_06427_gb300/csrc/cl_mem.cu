@@ -3,7 +3,8 @@
 // both). A list's arrays are two blocks of it and the two-set calls' workspace
 // one, where each array was a cudaMalloc of its own (about twenty per list,
 // 0.5 ms of host time per build and free at 200,000 particles). Freed memory
-// beyond kPoolKeep goes back to the device at the next synchronisation.
+// beyond kPoolKeep goes back to the device: by the pool itself at the next
+// synchronisation, and by mem_settle before a call that freed a lot returns.
 #include <mutex>
 
 #include "cl_internal.cuh"
@@ -11,8 +12,6 @@
 namespace clk {
 
 namespace {
-
-constexpr unsigned long long kPoolKeep = 256ull << 20;
 
 std::mutex pool_mu;
 cudaMemPool_t pools[kCacheDevices];
@@ -55,6 +54,16 @@ int mem_alloc(void** p, size_t bytes, cudaStream_t s) {
 
 void mem_free(void* p, cudaStream_t s) {
   if (p) cudaFreeAsync(p, s);
+}
+
+void mem_settle(cudaStream_t s) {
+  cudaMemPool_t pool;
+  unsigned long long held = 0, used = 0;
+  if (device_pool(&pool) || cudaMemPoolGetAttribute(pool, cudaMemPoolAttrReservedMemCurrent, &held) != cudaSuccess ||
+      held <= kPoolKeep || cudaStreamSynchronize(s) != cudaSuccess ||
+      cudaMemPoolGetAttribute(pool, cudaMemPoolAttrUsedMemCurrent, &used) != cudaSuccess)
+    return;
+  cudaMemPoolTrimTo(pool, (size_t)(used + kPoolKeep));
 }
 
 }  // namespace clk

@@ -1,0 +1,43 @@
+"""The library's device memory: what is given back, and when."""
+import numpy as np
+import pytest
+import torch
+
+pytestmark = pytest.mark.gpu
+
+KEPT = 256 << 20  # freed memory that the library keeps for later calls
+MARGIN = 64 << 20  # the driver maps memory in pieces of up to 32 MB; kernels loaded meanwhile
+
+
+def _free_bytes():
+    torch.cuda.synchronize()
+    return torch.cuda.mem_get_info()[0]
+
+
+def test_freed_lists_go_back_to_the_device(cuda_ok):
+    """cl_free returns a large list's memory, beyond what is kept, at once."""
+    import paper_2202_06427_gb300 as P
+    n = 16_000_000
+    h = np.eye(3) * 1000.0
+    x = torch.rand((n, 3), dtype=torch.float64, device="cuda") * 1000
+    P.cl_free(P.cl_build(x[:1000].contiguous(), h, 100.0, 1))  # the pool and the kernels exist
+    before = _free_bytes()
+    cl = P.cl_build(x, h, 12.0, 1)
+    assert P.cl_query(cl, "bytes") > KEPT + 2 * MARGIN
+    P.cl_free(cl)
+    left = before - torch.cuda.mem_get_info()[0]  # no synchronisation in between
+    assert left <= KEPT + MARGIN
+
+
+def test_two_set_workspace_goes_back_to_the_device(cuda_ok):
+    """So does a two-set call its workspace (here 32 closest of 4M queries' lists)."""
+    import paper_2202_06427_gb300 as P
+    h = np.eye(3) * 1000.0
+    x = torch.rand((10000, 3), dtype=torch.float64, device="cuda") * 1000
+    y = torch.rand((4_000_000, 3), dtype=torch.float64, device="cuda") * 1000
+    cl = P.cl_build(x, h, 12.0, 1)
+    P.cl_cross_topk(cl, y[:100].contiguous(), 32)
+    before = _free_bytes()
+    P.cl_cross_topk(cl, y, 32)
+    left = before - torch.cuda.mem_get_info()[0]
+    assert left <= KEPT + MARGIN
