@@ -119,8 +119,8 @@ int cl_build(const double* pos_dev, long long n, const cl_box* box, void* stream
 
 /* Rebuild the cell list for new positions of the same n particles (Sec. 4.2:
  * the lists are updated between steps), reusing the workspace. box may be
- * NULL (unchanged) or a box; one that needs more cells than any before it
- * reallocates.
+ * NULL (unchanged) or a box; one that needs more cells than the list has room
+ * for, or fewer than a quarter of them (above 2^20), reallocates.
  * Same errors as cl_build. */
 int cl_update(cl_list* cl, const double* pos_dev, const cl_box* box, void* stream);
 

@@ -104,16 +104,10 @@ void free_all(cl_list* c) {
   delete c->hood;
 }
 
-// Room for ncells cells. A larger grid than before gets a new block first, so
-// that a failure leaves the list as it was; the old one may still be in use on
-// another stream, so it is given back after a device synchronisation.
-int alloc_cells(cl_list* c, long long ncells, cudaStream_t s) {
-  Cells p;
-  const size_t bytes = carve_cells(&p, nullptr, ncells);
-  void* block = nullptr;
-  int e = clk::mem_alloc(&block, bytes, s);
-  if (e) return e;
-  carve_cells(&p, (char*)block, ncells);
+// Makes block (of carve_cells' size for ncells cells) the list's per-cell arrays.
+// The old block may still be in use on another stream, so it is given back after
+// a device synchronisation.
+void adopt_cells(cl_list* c, void* block, long long ncells, cudaStream_t s) {
   if (c->cell_block) {
     Cells old;
     c->bytes -= carve_cells(&old, nullptr, c->ncells_alloc);
@@ -121,6 +115,8 @@ int alloc_cells(cl_list* c, long long ncells, cudaStream_t s) {
     clk::mem_free(c->cell_block, s);
     clk::mem_settle(s);
   }
+  Cells p;
+  c->bytes += carve_cells(&p, (char*)block, ncells);
   c->cell_block = block;
   c->counts = p.counts;
   c->cell_start = p.cell_start;
@@ -129,8 +125,6 @@ int alloc_cells(cl_list* c, long long ncells, cudaStream_t s) {
   c->hdense = p.hdense;
   c->hflag = p.hflag;
   c->ncells_alloc = ncells;
-  c->bytes += bytes;
-  return CL_OK;
 }
 
 // Partials (doubles) available to the neighbourhood sweep and its per-particle companion.
@@ -184,10 +178,24 @@ int set_geometry(cl_list* c, const cl_box* box, cudaStream_t s) {
   int nh = 0, nf = 0;
   if ((e = clk::build_stencils(g, clk::kMaxOff, t->off, t->opk_half, &nh, t->off + clk::kMaxOff, t->opk_full, &nf)))
     return e;
-  if (g.ncells > c->ncells_alloc && (e = alloc_cells(c, g.ncells, s))) return e;
+  // A larger grid than the block has room for needs a new one. One of less than a
+  // quarter of a large block (2^20 cells: 18 MB) gives the surplus back, if it
+  // can: the old block serves as well. The list is unchanged until nothing can
+  // fail.
+  void* block = nullptr;
+  const bool grows = g.ncells > c->ncells_alloc;
+  if (grows || (c->ncells_alloc > (1 << 20) && g.ncells < c->ncells_alloc / 4)) {
+    Cells p;
+    e = clk::mem_alloc(&block, carve_cells(&p, nullptr, g.ncells), s);
+    if (e && grows) return e;
+  }
   std::memmove(t->off + nh, t->off + clk::kMaxOff, sizeof(clk::Off) * nf);  // one after the other: one copy
-  if (cudaMemcpyAsync(c->d_off_half, t->off, sizeof(clk::Off) * (nh + nf), cudaMemcpyHostToDevice, s) != cudaSuccess)
-    return CL_ERR_CUDA;  // pageable source: staged before the call returns
+  // pageable source: staged before the call returns
+  if (cudaMemcpyAsync(c->d_off_half, t->off, sizeof(clk::Off) * (nh + nf), cudaMemcpyHostToDevice, s) != cudaSuccess) {
+    clk::mem_free(block, s);
+    return CL_ERR_CUDA;
+  }
+  if (block) adopt_cells(c, block, g.ncells, s);
   c->d_off_full = c->d_off_half + nh;
   std::memcpy(c->half->off, t->off, sizeof(clk::Off) * nh);
   std::memcpy(c->full->off, t->off + nh, sizeof(clk::Off) * nf);

@@ -41,3 +41,23 @@ def test_two_set_workspace_goes_back_to_the_device(cuda_ok):
     P.cl_cross_topk(cl, y, 32)
     left = before - torch.cuda.mem_get_info()[0]
     assert left <= KEPT + MARGIN
+
+
+def test_smaller_grid_gives_its_cells_back(cuda_ok):
+    """A list updated to a grid of far fewer cells holds their memory no longer,
+    and grows again; the pairs are those of a list built for the grid."""
+    import paper_2202_06427_gb300 as P
+    h = np.eye(3) * 1000.0
+    x = torch.rand((20000, 3), dtype=torch.float64, device="cuda") * 1000
+    cl = P.cl_build(x, h, 40.0, 2)
+    small, want = P.cl_query(cl, "bytes"), P.cl_map(cl, "count")["count"].item()
+    P.cl_update(cl, x, cutoff=3.0, lcell=1)
+    large, fine = P.cl_query(cl, "bytes"), P.cl_map(cl, "count")["count"].item()
+    assert large > small + (500 << 20)
+    before = torch.cuda.mem_get_info()[0]
+    P.cl_update(cl, x, cutoff=40.0, lcell=2)
+    assert P.cl_query(cl, "bytes") == small
+    assert torch.cuda.mem_get_info()[0] - before > large - small - KEPT - MARGIN
+    assert P.cl_map(cl, "count")["count"].item() == want
+    P.cl_update(cl, x, cutoff=3.0, lcell=1)
+    assert P.cl_query(cl, "bytes") == large and P.cl_map(cl, "count")["count"].item() == fine
