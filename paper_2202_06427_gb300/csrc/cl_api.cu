@@ -111,8 +111,8 @@ void adopt_cells(cl_list* c, void* block, long long ncells, cudaStream_t s) {
   if (c->cell_block) {
     Cells old;
     c->bytes -= carve_cells(&old, nullptr, c->ncells_alloc);
-    cudaDeviceSynchronize();
-    clk::mem_free(c->cell_block, s);
+    if (!clk::capturing(s)) cudaDeviceSynchronize();
+    clk::mem_free(c->cell_block, s);  // (under capture cudaFree, which waits itself)
     clk::mem_settle(s);
   }
   Cells p;
@@ -190,8 +190,11 @@ int set_geometry(cl_list* c, const cl_box* box, cudaStream_t s) {
     if (e && grows) return e;
   }
   std::memmove(t->off + nh, t->off + clk::kMaxOff, sizeof(clk::Off) * nf);  // one after the other: one copy
-  // pageable source: staged before the call returns
-  if (cudaMemcpyAsync(c->d_off_half, t->off, sizeof(clk::Off) * (nh + nf), cudaMemcpyHostToDevice, s) != cudaSuccess) {
+  // pageable source: staged before the call returns, where a captured copy would
+  // read it when the graph runs
+  const size_t bytes = sizeof(clk::Off) * (nh + nf);
+  if ((clk::capturing(s) ? cudaMemcpy(c->d_off_half, t->off, bytes, cudaMemcpyHostToDevice)
+                         : cudaMemcpyAsync(c->d_off_half, t->off, bytes, cudaMemcpyHostToDevice, s)) != cudaSuccess) {
     clk::mem_free(block, s);
     return CL_ERR_CUDA;
   }
@@ -425,7 +428,7 @@ int cl_build(const double* pos_dev, long long n, const cl_box* box, void* stream
   if (!e) e = set_geometry(c, box, s);
   if (!e) e = run_build(c, s);
   if (e) {
-    cudaStreamSynchronize(s);
+    if (!clk::capturing(s)) cudaStreamSynchronize(s);
     free_all(c);
     delete c;
     return e;

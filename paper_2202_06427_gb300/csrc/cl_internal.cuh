@@ -132,6 +132,7 @@ namespace clk {
 
 // Stream-ordered device memory of the library (cl_mem.cu): a pool per device
 // that keeps at most kPoolKeep bytes of freed memory for later calls.
+bool capturing(cudaStream_t s);  // work on s is being recorded into a graph
 int mem_alloc(void** p, size_t bytes, cudaStream_t s);
 void mem_free(void* p, cudaStream_t s);
 constexpr unsigned long long kPoolKeep = 256ull << 20;

@@ -40,11 +40,25 @@ int device_pool(cudaMemPool_t* out) {
 
 }  // namespace
 
+bool capturing(cudaStream_t s) {
+  cudaStreamCaptureStatus st = cudaStreamCaptureStatusNone;
+  if (cudaStreamIsCapturing(s, &st) == cudaSuccess) return st != cudaStreamCaptureStatusNone;
+  cudaGetLastError();  // the legacy stream, and another one is being captured
+  return true;
+}
+
+// While a stream is captured, an allocation on it would become a node of the
+// graph: memory that does not exist until the graph runs. The calls then allocate
+// and free for themselves, which most capture modes refuse.
 int mem_alloc(void** p, size_t bytes, cudaStream_t s) {
   *p = nullptr;
   cudaMemPool_t pool;
-  int e = device_pool(&pool);
-  if (!e && cudaMallocFromPoolAsync(p, bytes ? bytes : 1, pool, s) != cudaSuccess) e = CL_ERR_OOM;
+  int e = CL_OK;
+  if (capturing(s)) {
+    if (cudaMalloc(p, bytes ? bytes : 1) != cudaSuccess) e = CL_ERR_OOM;
+  } else if (!(e = device_pool(&pool)) && cudaMallocFromPoolAsync(p, bytes ? bytes : 1, pool, s) != cudaSuccess) {
+    e = CL_ERR_OOM;
+  }
   if (e) {
     cudaGetLastError();
     *p = nullptr;
@@ -53,13 +67,15 @@ int mem_alloc(void** p, size_t bytes, cudaStream_t s) {
 }
 
 void mem_free(void* p, cudaStream_t s) {
-  if (p) cudaFreeAsync(p, s);
+  if (!p) return;
+  if (capturing(s)) cudaFree(p);
+  else cudaFreeAsync(p, s);
 }
 
 void mem_settle(cudaStream_t s) {
   cudaMemPool_t pool;
   unsigned long long held = 0, used = 0;
-  if (device_pool(&pool) || cudaMemPoolGetAttribute(pool, cudaMemPoolAttrReservedMemCurrent, &held) != cudaSuccess ||
+  if (capturing(s) || device_pool(&pool) || cudaMemPoolGetAttribute(pool, cudaMemPoolAttrReservedMemCurrent, &held) != cudaSuccess ||
       held <= kPoolKeep || cudaStreamSynchronize(s) != cudaSuccess ||
       cudaMemPoolGetAttribute(pool, cudaMemPoolAttrUsedMemCurrent, &used) != cudaSuccess)
     return;
