@@ -275,9 +275,7 @@ __global__ void __launch_bounds__(32 * kCrossWarps) k_cross_knn(const __grid_con
     float bd = FLT_MAX, kd = FLT_MAX;
     int ba = INT_MAX, ka = INT_MAX;
     for (int k0 = 0; k0 < A.noff; k0 += 32) {
-      // a cell at a box distance of 0 stays in when the k-th distance is 0: a
-      // smaller index may tie there (beyond 0 the boxes' padding excludes a tie)
-      const int nk = query_cells(A, stab, W, k0, lane, cc, p, fminf(A.rc2, fmaxf(kd, FLT_MIN)));
+      const int nk = query_cells(A, stab, W, k0, lane, cc, p, fminf(A.rc2, kd));
       for (int i0 = 0; i0 < nk; i0 += 32 / G) {
         const int i = i0 + lane / G;
         float4 s = make_float4(0.f, 0.f, 0.f, 0.f);
@@ -286,7 +284,7 @@ __global__ void __launch_bounds__(32 * kCrossWarps) k_cross_knn(const __grid_con
           s = W.s[i];
           const int2 r = W.j[i];
           j = r.x + lane % G;
-          j1 = s.w < fmaxf(kd, FLT_MIN) ? r.y : 0;
+          j1 = s.w < kd ? r.y : 0;
         }
         while (__any_sync(0xffffffffu, j < j1)) {
           int a = 0;

@@ -57,7 +57,10 @@ __device__ __forceinline__ void load_stencil(const CrossArgs& A, float4* stab, f
 
 // Entries k0 + lane of the stencil about the query's cell: the non-empty cells
 // within sqrt(lim) of the query (all of them without culling) go to W; returns
-// their number.
+// their number. The squared box distance is taken FLT_MIN low, which changes it at
+// 0 only: such a cell stays in when lim is 0, the k-th distance of a query on k
+// points of the set, as a smaller index may tie there (beyond 0 the boxes'
+// padding excludes a tie).
 __device__ __forceinline__ int query_cells(const CrossArgs& A, const float4* stab, WarpCells& W, int k0, int lane,
                                            unsigned cc, const float4& p, float lim) {
   const int k = k0 + lane;
@@ -69,8 +72,8 @@ __device__ __forceinline__ int query_cells(const CrossArgs& A, const float4* sta
     const unsigned d = __float_as_uint(e.w);
     const float bx = fmaxf(fabsf(p.x - e.x) - A.ex, 0.f), by = fmaxf(fabsf(p.y - e.y) - A.ey, 0.f),
                 bz = fmaxf(fabsf(p.z - e.z) - A.ez, 0.f);
-    e.w = fmaf(bx, bx, fmaf(by, by, bz * bz));
-    if (!A.cull) e.w = 0.f;
+    e.w = fmaf(bx, bx, fmaf(by, by, fmaf(bz, bz, -FLT_MIN)));
+    if (!A.cull) e.w = -FLT_MIN;
     if (e.w < lim) {
       int x2 = (int)(cc & 1023u) + (int)(d & 1023u);
       x2 -= (x2 >= A.nx) ? A.nx : 0;
