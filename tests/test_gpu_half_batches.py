@@ -3,6 +3,8 @@ fast-path cells, cells whose kept neighbourhood overflows the fast path, cells
 of a batch's edge sizes (31-33, 64-65 particles), of more than 128 and of more
 than 2,048. Every reduction against the oracle, and again on the same list,
 whose work lists are kept (rules of parity_util)."""
+import itertools
+
 import numpy as np
 import pytest
 import torch
@@ -102,3 +104,71 @@ def test_clumps_beyond_each_others_cutoff(cuda_ok, lcell):
         check_matrix(efv["virial"].cpu().numpy(), ref["virial"], TOL_W)
         gp, _, _ = P.cl_backward(cl, g)  # (no pair crosses the boundary: dE/dH is zero)
         check_forces(gp.cpu().numpy(), -0.75 * ref["forces"])
+
+
+def _handed_over(x, h, rc, lcell):
+    """Cells of at most 128 particles that the sweep lists for the fast path (the
+    particles of the half neighbourhood, raw, within the share of the cells that
+    lies in the staging ball) although those kept pass its buffer of 1,536."""
+    hinv = np.linalg.inv(h)
+    n = np.floor(lcell / np.linalg.norm(hinv, axis=0) / rc).astype(int)
+    s = x @ hinv
+    s -= np.floor(s)
+    c = np.minimum((s * n).astype(int), n - 1)
+    G = h / n[:, None]
+    local = (s * n - c - 0.5) @ G
+    assert np.allclose(h, np.diag(np.diag(h)))
+    far = lambda o: sum((max(abs(v) - 1, 0) * G[k, k]) ** 2 for k, v in enumerate(o))
+    off = [o for o in itertools.product(range(-lcell - 1, lcell + 2), repeat=3) if o[::-1] > (0, 0, 0) and far(o) < rc * rc]
+    hd = 0.5 * np.linalg.norm(np.diag(G))
+    cell = np.prod(np.diag(G))
+    share = min(1.0, 0.5 * (4 / 3 * np.pi * (rc + hd) ** 3 - cell) / (cell * len(off)))
+    cells = {}
+    for i, k in enumerate(map(tuple, c)):
+        cells.setdefault(k, []).append(i)
+    found = 0
+    for k, own in cells.items():
+        near = [(j, o) for o in off for j in cells.get(tuple((np.array(k) + o) % n), [])]
+        if len(own) > 128 or not 1536 < len(near) <= 1536 / share:
+            continue
+        j, o = np.array([v[0] for v in near]), np.array([v[1] for v in near])
+        top = rc + np.linalg.norm(local[own], axis=1).max()
+        found += np.linalg.norm(local[j] + o @ G, axis=1).__lt__(top).sum() > 1536
+    return found
+
+
+def test_cells_handed_over_by_the_sweep(cuda_ok):
+    """Cells that the fast path finds too full while it stages them, and moves to
+    the batches' list, which later calls on the same list take over: every
+    reduction, the moving sweep first and last."""
+    import paper_2202_06427_gb300 as P
+    rng = np.random.default_rng(29)
+    L, rc, lcell = 24.0, 6.0, 2
+    h = np.eye(3) * L
+    centre = np.array([10.5, 10.5, 10.5])  # the middle of a cell
+    x = np.vstack([_background(rng, h, 1.2, centre, 1.6), _ball(rng, centre, 1.3, 0.215, 0.03)])
+    x = np.ascontiguousarray(x[rng.permutation(x.shape[0])])
+    assert len(x) >= 16 * 8 ** 3  # count and histogram staged as well
+    assert _handed_over(x, h, rc, lcell) > 0
+    ref = oracle.pair_map(x, h, rc, band=BAND, nbins=17)
+    g = torch.tensor([0.75], dtype=torch.float64, device="cuda")
+
+    def forces(cl):
+        efv = P.cl_map(cl, "energy_forces_virial")
+        check_energy(efv["energy"].item(), ref["energy"])
+        check_forces(efv["forces"].cpu().numpy(), ref["forces"])
+        check_matrix(efv["virial"].cpu().numpy(), ref["virial"], TOL_W)
+        gp, gb, _ = P.cl_backward(cl, g)
+        check_forces(gp.cpu().numpy(), -0.75 * ref["forces"])
+        check_matrix(gb.cpu().numpy(), 0.75 * ref["dedh"], TOL_GB)
+
+    def scalars(cl):
+        check_energy(P.cl_map(cl, "energy")["energy"].item(), ref["energy"])
+        check_count(int(P.cl_map(cl, "count")["count"].item()), ref)
+        check_hist(P.cl_map(cl, "hist", nbins=17)["hist"].cpu().numpy(), ref)
+
+    xd = torch.from_numpy(x).cuda()
+    for order in ((forces, scalars, forces), (scalars, forces, scalars)):
+        cl = P.cl_build(xd, h, rc, lcell)
+        for part in order:
+            part(cl)
