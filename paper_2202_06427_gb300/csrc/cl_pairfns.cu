@@ -163,13 +163,6 @@ __global__ void k_sweep_velocity(const __grid_constant__ SweepArgs A, const floa
   }
 }
 
-// 1/v to FP32 rounding: the hardware reciprocal and one Newton-Raphson step.
-__device__ __forceinline__ float recip(float v) {
-  float w;
-  asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(w) : "f"(v));
-  return fmaf(w, fmaf(-v, w, 1.0f), w);
-}
-
 // Lennard-Jones energy and forces, full shell, one thread per sorted particle:
 // the functor's sweep and its sums term by term, without its IEEE division (a
 // warp has a pair within the cutoff at nearly every step) and without the cells

@@ -17,6 +17,15 @@ __device__ __forceinline__ float rsqrt_nr(float d2) {
   return fmaf(0.5f * y, e, y);
 }
 
+// 1/v from the hardware reciprocal and one Newton-Raphson step, w1 = w0 + w0 (1 -
+// v w0): within 2^-24 (1 + 2^-10) of it relative for v in [2^-126, 2^126], where
+// the IEEE division is within 2^-24.
+__device__ __forceinline__ float recip(float v) {
+  float w;
+  asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(w) : "f"(v));
+  return fmaf(w, fmaf(-v, w, 1.0f), w);
+}
+
 // ---------------------------------------------------------------- reductions
 // Each reduction: per-thread accumulator, hit() for a pair within the cutoff
 // (displacement r = x_j - x_i under the image of the offset), and an

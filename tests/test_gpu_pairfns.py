@@ -124,3 +124,44 @@ def test_failed_call_leaves_the_list_usable(cuda_ok, call):
     got = P.cl_map(cl, "energy_forces_virial")["forces"]
     # the sums of a particle's forces come in another order from call to call
     assert torch.allclose(got, want, rtol=0, atol=1e-5 * want.abs().max().item())
+
+
+@pytest.mark.parametrize("nbins", [1, 16, 17, 32, 33, 64])
+def test_velocity_histogram_bins(cuda_ok, nbins):
+    """The numbers of bins at which the sweep's blocks change their size."""
+    import paper_2202_06427_gb300 as P
+    x, h, rc = _set(3, True, 3.0, 640 + nbins)
+    v = np.random.default_rng(7).normal(size=x.shape).astype(np.float32)
+    binstep = rc / nbins
+    ref = oracle.velocity_hist(x, h, rc, v.astype(np.float64), binstep, nbins, band=BAND)
+    cl = P.cl_build(torch.from_numpy(x).cuda(), h, rc, 2)
+    counts, vsum = P.cl_map_velocity_hist(cl, torch.from_numpy(v).cuda(), binstep, nbins)
+    c = counts.cpu().numpy()
+    bc, bv = ref["band_counts"], ref["band_vsum"]
+    near_c = bc + np.roll(bc, 1) + np.roll(bc, -1)
+    near_v = bv + np.roll(bv, 1) + np.roll(bv, -1)
+    assert np.all(c >= ref["counts"]) and np.all(c <= ref["counts"] + near_c), (c, ref["counts"])
+    dv = vsum.cpu().numpy() - ref["vsum"]
+    assert np.all(dv >= -1e-5 * ref["vsum"] - 1e-9) and np.all(dv <= 1e-5 * ref["vsum"] + near_v + 1e-9)
+
+
+def test_reciprocal_of_the_lennard_jones_sweep(cuda_ok, tmp_path):
+    """Every float of a few binades, the ends of its range among them. Newton's
+    step on an estimate w0 of relative error e0 <= 2^-23 leaves e0^2 and the
+    rounding of 1 - v w0 (2^-24 e0), below 2^-45 together; the last fma rounds
+    with 2^-24."""
+    import ctypes
+    import os
+    import subprocess
+    from paper_2202_06427_gb300 import build
+    root = build.ROOT
+    out = str(tmp_path / "librecip.so")
+    subprocess.run([build._nvcc()] + build.ARCH + build.FLAGS + ["-shared", "-cudart", "shared",
+                   os.path.join(root, "tests", "recip_probe.cu"), "-o", out], check=True)
+    lib = ctypes.CDLL(out)
+    worst = torch.zeros(1, dtype=torch.int64, device="cuda")
+    torch.cuda.synchronize()
+    for exponent in (-126, -20, -1, 0, 1, 7, 30, 125):
+        first = (exponent + 127) << 23
+        assert lib.recip_error(ctypes.c_uint(first), ctypes.c_uint(1 << 23), ctypes.c_void_p(worst.data_ptr())) == 0
+    assert 0 < worst.cpu().view(torch.float64).item() <= 2.0 ** -24 * (1 + 2.0 ** -10)
