@@ -140,6 +140,15 @@ bool scalar_staged(const cl_list* c) {
   return c->geo.dim == 3 && c->n > 0 && (double)c->n >= kStagedMinOccupancy * (double)c->geo.ncells;
 }
 
+// 2D sweeps go by rows of cells (row_sweep) up to this mean occupancy, above it
+// cell by cell: rows keep a warp's lanes together where cells hold a few
+// particles, but read each candidate's cell as well. Rows against cells, count
+// and forces at two cells per cutoff: 400,000 particles 0.93 and 0.85 at one per
+// cell, 0.95 and 0.92 at 4, 1.09 and 1.04 at 8, 1.52 and 1.32 at 32; 4M 0.81 and
+// 0.80 at 4, 0.97 and 0.95 at 8; 20,000, whose sweep ends with its slowest warps,
+// 0.98 and 0.97 at one, 1.07 and 1.09 at 4, 1.58 and 1.60 at 32.
+double rows_max_occupancy(long long n) { return n >= 152 * 2048 ? 8.0 : 3.0; }
+
 void fill_sweep_args(cl_list* c, clk::SweepArgs* A) {
   A->xs = c->xs;
   A->cellc = c->cellc;
@@ -213,7 +222,7 @@ int set_geometry(cl_list* c, const cl_box* box, cudaStream_t s) {
   c->half->noff = nh;
   c->full->noff = nf;
   c->half->nrow2 = c->full->nrow2 = 0;
-  if (g.dim == 2) {
+  if (g.dim == 2 && (double)c->n < rows_max_occupancy(c->n) * (double)g.ncells) {
     clk::fill_rows2(t->opk_half, nh, c->half);
     clk::fill_rows2(t->opk_full, nf, c->full);
   }

@@ -132,3 +132,29 @@ def test_rows_of_small_2d_grids(cuda_ok, ratio, lcell, tric):
     out = P.cl_map(cl, "energy_forces_virial")
     check_energy(out["energy"].item(), ref["energy"])
     check_forces(out["forces"].cpu().numpy(), ref["forces"])
+
+
+@pytest.mark.parametrize("occupancy", [1.5, 2.9, 3.1, 20.0])
+@pytest.mark.parametrize("ratio,lcell,tric", [(1.2, 1, False), (1.9, 1, True), (2.4, 2, True), (3.1, 1, True),
+                                              (9.3, 3, False), (6.1, 4, True)])
+def test_2d_rows_and_cells(cuda_ok, ratio, lcell, tric, occupancy):
+    """Both sides of the mean occupancy up to which 2D sweeps go by rows, on grids
+    down to one cell per axis."""
+    import paper_2202_06427_gb300 as P
+    rc = 4.0
+    h = np.eye(2) * (ratio * rc)
+    if tric:
+        h[1, 0] = 0.15 * ratio * rc
+        h *= ratio * rc / oracle.geom_info(h, rc)["w"].min()
+    cells = int(np.prod(P.cl_box_info(h, rc, lcell)["grid"]))
+    n = max(2, int(occupancy * cells))
+    side = int(np.ceil(np.sqrt(n)))
+    x = synth.jittered_fractional(h, side, n, 0.3, 17)
+    cl = P.cl_build(_dev(x), h, rc, lcell)
+    ref = oracle.pair_map(x, h, rc, band=BAND, nbins=50)
+    check_count(P.cl_map(cl, "count")["count"].item(), ref)
+    check_hist(P.cl_map(cl, "hist", nbins=50)["hist"].cpu().numpy(), ref)
+    if n >= 16:  # the relative rules are for sums over many pairs, not for two near the cutoff
+        out = P.cl_map(cl, "energy_forces_virial")
+        check_energy(out["energy"].item(), ref["energy"])
+        check_forces(out["forces"].cpu().numpy(), ref["forces"])
