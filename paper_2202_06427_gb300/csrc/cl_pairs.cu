@@ -649,6 +649,11 @@ __device__ __forceinline__ void fill_two(const SweepArgs& A, int p, int h1, At a
 // 57,000 particles and 371 at 31,000; 190 and 178 so. Cells that do not fit are
 // listed (cells) for k_pairs_cell in both passes. kSparse: those two lists expect
 // 25 in a ball, 2D lists at other cell sizes up to 40; denser grids keep the CTA.
+// So do large stencils about few particles, where the list takes as long as one
+// warp needs for its cell's entries: 3D at 0.1 per cell, 613 entries, 646 us by
+// warps and 275 by CTAs for 5,000 particles, 716 and 634 for 20,000, 875 and 1,067
+// for 40,000; 311 entries 318 and 224 for 5,000, 340 and 306 for 10,000, 385 and
+// 487 for 20,000; 125 entries 117 and 121 for 2,000.
 constexpr int kSparse = 64, kSparseCap = 160, kSparseWarps = 4;
 static_assert((kMaxOff + 2 * kSparseWarps * kSparseCap) * sizeof(float4) <= 48 * 1024, "the default shared memory");
 
@@ -802,6 +807,11 @@ size_t pairs_cell_smem(int noff, bool fill, int cap) {
   return fill ? head + kBuckets * sizeof(int) + 2 * (size_t)cap * sizeof(unsigned short) : head;
 }
 
+// The grids of k_pairs_sparse (measured at kSparse).
+static bool by_warps(const SweepArgs& A, const PairLists& L) {
+  return L.expect <= kSparse && (A.noff <= 160 || A.n >= 40 * A.noff);
+}
+
 // The staged passes: k_pairs_sparse for sparse grids and k_pairs_cell for the
 // cells it lists, k_pairs_cell alone otherwise.
 template <int DIM, bool FILL, bool IMAGES>
@@ -826,7 +836,7 @@ static int launch_cell(const SweepArgs& A, const PairLists& L, const long long* 
   long long blocks = (long long)sms * per;
   const long long ncells = (long long)A.nx * A.ny * A.nz;
   if (blocks > ncells) blocks = ncells;
-  const bool sparse = L.expect <= kSparse;
+  const bool sparse = by_warps(A, L);
   if (sparse) {
     const size_t sm = sizeof(float4) * (size_t)(A.noff + kSparseWarps * kSparseCap * (FILL ? 2 : 1));
     const long long sb = std::min<long long>((ncells + kSparseWarps - 1) / kSparseWarps, (long long)sms * 64);

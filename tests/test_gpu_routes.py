@@ -158,3 +158,16 @@ def test_2d_rows_and_cells(cuda_ok, ratio, lcell, tric, occupancy):
         out = P.cl_map(cl, "energy_forces_virial")
         check_energy(out["energy"].item(), ref["energy"])
         check_forces(out["forces"].cpu().numpy(), ref["forces"])
+
+
+@pytest.mark.parametrize("lcell,extra", [(3, -1), (3, 0), (4, -1), (4, 0)])
+def test_pairlist_large_stencils(cuda_ok, lcell, extra):
+    """Sparse grids of 300 and 600 stencil entries: a CTA per cell below 40
+    particles per entry, a warp per cell from there on."""
+    import paper_2202_06427_gb300 as P
+    rc, L = 2.0, 60.0
+    h = np.eye(3) * L
+    h[1, 0], h[2, 1] = 4.0, -6.0
+    n = 40 * P.cl_box_info(h, rc, lcell)["stencil_full"] + extra
+    x = synth.jittered_fractional(h, int(np.ceil(n ** (1 / 3))), n, 0.5, 71)
+    _check_against_oracle(P, x, h, rc, lcell)
