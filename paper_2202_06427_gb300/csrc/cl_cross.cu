@@ -212,6 +212,24 @@ __device__ __forceinline__ void best_offer(float& bd, ID& bi, float& kd, ID& ki,
   const int lane = threadIdx.x & 31;
   ok = ok && nearer(d, id, kd, ki);
   unsigned m = __ballot_sync(0xffffffffu, ok);
+  // The nearest alone: two warp minima. Sorting and merging lost to the one thread
+  // per query that came before (100,000 queries in 2D, 28 candidates each, against a
+  // million particles: 79 us then, 131 so, 84 now).
+  if (k == 1 && __popc(m) > 1) {
+    d = ok ? d : none_d;
+    id = ok ? id : none_i;
+    if (sizeof(ID) == 4) {  // squared distances are not negative: their bits order like them
+      const unsigned b = __reduce_min_sync(0xffffffffu, __float_as_uint(d));
+      id = __reduce_min_sync(0xffffffffu, __float_as_uint(d) == b ? (int)id : INT_MAX);
+      d = __uint_as_float(b);
+    } else {
+#pragma unroll
+      for (int st = 16; st > 0; st >>= 1) nearer_exchange(d, id, st, true);
+    }
+    kd = bd = d;
+    ki = bi = id;
+    return;
+  }
   if (__popc(m) > kBulk) {
     d = ok ? d : none_d;
     id = ok ? id : none_i;

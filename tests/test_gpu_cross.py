@@ -190,3 +190,19 @@ def test_nearest_ties_at_zero(cuda_ok, dim, tric, lcell):
     for k in (1, 2, 3):
         a, d = P.cl_cross_knn(cl, y, k)
         assert torch.equal(a, a8[:, :k]) and torch.equal(d, d8[:, :k])
+
+
+@pytest.mark.parametrize("dim,n", [(2, 300), (2, 30000), (3, 1000), (3, 40000)])
+def test_nearest_one(cuda_ok, dim, n):
+    """k = 1, whose candidates are not sorted: the first of longer lists."""
+    import paper_2202_06427_gb300 as P
+    xa, yb, h = _sets(dim, True, 12.0, n, 3000, 77 + n)
+    xa[n // 2:] = xa[:n - n // 2]  # every point twice: distances tie
+    cl = P.cl_build(torch.from_numpy(xa).cuda(), h, 1.5, 1)
+    y = torch.from_numpy(yb).cuda()
+    a1, d1 = P.cl_cross_knn(cl, y, 1)
+    a9, d9 = P.cl_cross_knn(cl, y, 9)
+    assert torch.equal(a1, a9[:, :1]) and torch.equal(d1, d9[:, :1])
+    top1, top9 = P.cl_cross_topk(cl, y, 1), P.cl_cross_topk(cl, y, 9)
+    for key in ("a", "b", "d"):
+        assert torch.equal(top1[key], top9[key][:1])
