@@ -230,6 +230,15 @@ int scratch_done(float4* hforce, int n, cudaStream_t s) {
   return cudaMemsetAsync(hforce, 0, sizeof(float4) * (size_t)n, s) == cudaSuccess && ok ? CL_OK : CL_ERR_CUDA;
 }
 
+// Candidates per particle at the mean occupancy.
+double candidates(const SweepArgs& A) { return (double)A.n * A.noff / ((double)A.nx * A.ny * A.nz); }
+
+// Fewer, and the mass sum is the functor's: gathering the attributes, clearing the
+// scratch and the final sum are launches of their own. Functor against sweep, 20,000
+// particles: 41 and 57 us at 3 candidates, 49 and 56 at 14, 56 and 59 at 42; 300,000:
+// 94 and 115 at 13, 131 and 142 at 63, 292 and 250 at 160.
+constexpr double kMassMinCandidates = 80.0;
+
 // The functors' cutoff test: the FP32 cutoff squared in FP32.
 float functor_rc2(double rc) { return (float)rc * (float)rc; }
 
@@ -263,7 +272,7 @@ extern "C" int cl_map_mass(const cl_list* cl, const float* mass_dev, double* out
   if (cudaMemsetAsync(out_dev, 0, sizeof(double), s) != cudaSuccess) return CL_ERR_CUDA;
   clk::ListParts L;
   clk::list_parts(cl, &L);
-  if (L.hforce && v.n > 0) {
+  if (L.hforce && v.n > 0 && clk::candidates(*L.half) >= clk::kMassMinCandidates) {
     const int blocks = (v.n + 255) / 256;
     clk::k_sorted_mass<<<blocks, 256, 0, s>>>(L.half->xs, v.n, mass_dev, L.hforce);
     clk::k_sweep_mass<<<blocks, 256, 0, s>>>(*L.half, L.hforce, clk::functor_rc2(L.rc), L.partials);

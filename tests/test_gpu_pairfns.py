@@ -165,3 +165,20 @@ def test_reciprocal_of_the_lennard_jones_sweep(cuda_ok, tmp_path):
         first = (exponent + 127) << 23
         assert lib.recip_error(ctypes.c_uint(first), ctypes.c_uint(1 << 23), ctypes.c_void_p(worst.data_ptr())) == 0
     assert 0 < worst.cpu().view(torch.float64).item() <= 2.0 ** -24 * (1 + 2.0 ** -10)
+
+
+@pytest.mark.parametrize("candidates", [79.5, 80.5])
+@pytest.mark.parametrize("lcell", [1, 2])
+def test_mass_potential_of_sparse_lists(cuda_ok, lcell, candidates):
+    """Both sides of the 80 candidates per particle from which on the sum is the
+    sweep's and not the functor's."""
+    import paper_2202_06427_gb300 as P
+    h = np.array([[26.0, 0, 0], [3.0, 25.0, 0], [-2.0, 4.0, 27.0]])
+    rc = 2.5
+    info = P.cl_box_info(h, rc, lcell)
+    n = int(candidates * np.prod(info["grid"]) / info["stencil_half"])
+    x = synth.jittered_fractional(h, int(np.ceil(n ** (1 / 3))), n, 0.4, 81)
+    m = np.random.default_rng(9).uniform(0.5, 2.0, size=n).astype(np.float32)
+    ref = oracle.mass_potential(x, h, rc, m.astype(np.float64), band=BAND)
+    got = P.cl_map_mass(P.cl_build(torch.from_numpy(x).cuda(), h, rc, lcell), torch.from_numpy(m).cuda()).item()
+    assert abs(got - ref["value"]) <= 1e-5 * abs(ref["value"]) + ref["band"]
