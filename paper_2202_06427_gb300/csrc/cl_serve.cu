@@ -2,8 +2,8 @@
 //
 // Device side: one persistent sweep kernel per batch. Its CTAs take work
 // items from a device counter; item k of the batch is tile (k - base_r) of
-// the request r whose item range holds k (a tile = kServeThreads cell-sorted particles
-// of one request). Each request carries its own geometry, stencil, cell list
+// the request r whose item range holds k (a tile = kServeThreads or kServeWide
+// cell-sorted particles of one request). Each request carries its own geometry, stencil, cell list
 // and outputs in a descriptor, so requests of different sizes, boxes,
 // dimensions and tasks share one launch. A finalize kernel (one CTA per
 // request) sums the per-tile FP64 partials in a fixed order.
@@ -52,13 +52,19 @@ struct ReqDesc {
 // take (24 warps per SM), 1.79 to 1.90 at 256 and 64, 2.03 with 64 threads.
 constexpr int kServeThreads = 128;
 constexpr int kServeCtas = 8;
+// A batch of no more than one wide tile per SM takes those (128 registers): its time
+// is that of a tile, whose warps' loads bring the cells of each other's neighbours
+// into L1. One 3D forces request alone: 20,000 particles 499 us in tiles of 128
+// (also at 80 registers, without spills), 366 in wide ones; 1,000 particles 334
+// and 292.
+constexpr int kServeWide = 256;
 
 // One tile of a request: one thread per cell-sorted particle over the
 // stencil, the packed (f32x2) sweep in 3D as in the library's per-particle
 // kernels, the scalar one in 2D.
 template <int DIM>
 __device__ void serve_tile(const ReqDesc& R, int blk, unsigned* shist) {
-  const int p = blk * kServeThreads + threadIdx.x;
+  const int p = blk * (int)blockDim.x + threadIdx.x;
   float4 pi;
   if (R.task == CL_TASK_ENERGY) {
     double v[1];
@@ -140,8 +146,9 @@ __device__ void serve_tile(const ReqDesc& R, int blk, unsigned* shist) {
   }
 }
 
-__global__ void __launch_bounds__(kServeThreads, kServeCtas) k_serve_sweep(const ReqDesc* __restrict__ reqs, int nreq,
-                                                                int nitems, int* __restrict__ counter) {
+template <int T, int CTAS>
+__global__ void __launch_bounds__(T, CTAS) k_serve_sweep(const ReqDesc* __restrict__ reqs, int nreq, int nitems,
+                                                         int* __restrict__ counter) {
   extern __shared__ unsigned shist[];
   __shared__ int s_item;
   for (;;) {
@@ -442,9 +449,13 @@ void cl_server::launch_batch(Batch& b) {
   // The requests' tiles are taken in order, so the costliest tiles go first:
   // the batch then ends on cheap tiles instead of waiting for a few long ones.
   std::stable_sort(b.reqs.begin(), b.reqs.end(), [](const Req* x, const Req* y) { return x->tile_cost > y->tile_cost; });
+  long long wide = 0;
+  for (const Req* q : b.reqs) wide += (q->r.n + clk::kServeWide - 1) / clk::kServeWide;
+  const int tile = wide <= sm_count ? clk::kServeWide : clk::kServeThreads;
   for (size_t k = 0; k < b.reqs.size(); ++k) {
     Req* q = b.reqs[k];
     q->t[2] = tl;
+    q->nitems = (int)((q->r.n + tile - 1) / tile);
     clk::ReqDesc& D = b.h_desc[k];
     std::memset(&D, 0, sizeof(D));
     D.dim = q->geo.dim;
@@ -487,9 +498,14 @@ void cl_server::launch_batch(Batch& b) {
   ok(cudaMemcpyAsync(b.d_desc, b.h_desc, sizeof(clk::ReqDesc) * nreq, cudaMemcpyHostToDevice, b.stream));
   ok(cudaMemsetAsync(b.d_counter, 0, sizeof(int), b.stream));
   if (items > 0 && !b.err) {
-    int grid = std::min(items, sm_count * ctas_per_sm);
-    clk::k_serve_sweep<<<grid, clk::kServeThreads, sizeof(unsigned) * maxbins, b.stream>>>(b.d_desc, nreq, items,
-                                                                                       b.d_counter);
+    const size_t smem = sizeof(unsigned) * maxbins;
+    if (tile == clk::kServeWide)
+      clk::k_serve_sweep<clk::kServeWide, 2><<<items, clk::kServeWide, smem, b.stream>>>(b.d_desc, nreq, items,
+                                                                                        b.d_counter);
+    else
+      clk::k_serve_sweep<clk::kServeThreads, clk::kServeCtas>
+          <<<std::min(items, sm_count * ctas_per_sm), clk::kServeThreads, smem, b.stream>>>(b.d_desc, nreq, items,
+                                                                                         b.d_counter);
     ok(cudaGetLastError());
   }
   if (!b.err) {
@@ -598,7 +614,7 @@ int cl_serve_create(long long arena_bytes, int max_inflight, int device, cl_serv
   if (!e) {
     s->sm_count = prop.multiProcessorCount;
     int per = 0;
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, clk::k_serve_sweep, clk::kServeThreads,
+    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, clk::k_serve_sweep<clk::kServeThreads, clk::kServeCtas>, clk::kServeThreads,
                                                       sizeof(unsigned) * clk::kMaxBins) != cudaSuccess)
       e = CL_ERR_CUDA;
     s->ctas_per_sm = std::max(per, 1);
@@ -642,7 +658,8 @@ int cl_serve_submit(cl_server* s, const cl_request* req, long long* ticket) {
     int noff = clk::build_stencil(q->geo, req->task == CL_TASK_FORCES ? 0 : 1, q->off.data(), clk::kMaxOff);
     if (noff < 0) e = noff;
     else q->off.resize(noff);
-    // pair terms per particle: candidates, and about twice the work for forces
+    // what orders a batch's requests: candidates per particle (the full stencil's for
+    // forces), half as much again where a pair takes forces or a bin
     q->tile_cost = (double)q->off.size() * (double)req->n / (double)q->geo.ncells *
                    (req->task == CL_TASK_ENERGY ? 1.0 : 1.5);
   }

@@ -176,3 +176,33 @@ def test_whole_served_stream_matches_oracle(cuda_ok):
         if spec["task"] == "forces":
             check_forces(r.forces.numpy(), ref["forces"])
             check_matrix(r.virial.numpy(), ref["virial"], TOL_W)
+
+
+@pytest.mark.parametrize("dim", [2, 3])
+@pytest.mark.parametrize("n", [127, 128, 129, 255, 256, 257, 700])
+def test_small_requests_alone(cuda_ok, dim, n):
+    """Requests of a tile or two, alone (wide tiles) and among enough others that
+    the batch takes the narrow ones."""
+    S = _S()
+    h = np.eye(dim) * (12.0 if dim == 3 else 30.0)
+    h[1, 0] = 1.5
+    x = synth.jittered_fractional(h, int(np.ceil(n ** (1 / dim))), n, 0.3, 9100 + n)
+    ref = oracle.pair_map(x, h, 3.0, band=BAND, nbins=20)
+    fill = synth.jittered_fractional(h, 40 if dim == 3 else 220, 45_000, 0.3, 5)
+    srv = S.Server(arena_bytes=1 << 30, max_inflight=16)
+    try:
+        for others in (0, 2):
+            reqs = [S.Request(x, h, 3.0, task, lcell=2, nbins=20) for task in ("energy", "forces", "hist")]
+            rest = [S.Request(fill, h, 1.0, "energy", lcell=1) for _ in range(others)]
+            for r in rest + reqs:
+                srv.submit(r)
+            for r in rest + reqs:
+                assert srv.wait(r.ticket, 120.0) == 0
+            e, f, q = reqs
+            check_energy(e.energy.item(), ref["energy"])
+            check_energy(f.energy.item(), ref["energy"])
+            check_forces(f.forces.numpy(), ref["forces"])
+            check_matrix(f.virial.numpy(), ref["virial"], TOL_W)
+            check_hist(q.hist.numpy(), ref)
+    finally:
+        srv.close()
