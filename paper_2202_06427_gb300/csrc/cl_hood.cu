@@ -2026,15 +2026,17 @@ __device__ __noinline__ void half_unit(HalfSmem& S, const Unit u, UnitAcc& acc, 
 // The batches of a windowed cell against the staged window, a warp at a time
 // from a counter. A batch is at most kBatch of the cell's particles,
 // consecutive in its octant order (k_octsort), so it lies in part of one
-// octant. A cell of few batches splits the window's entries between units as
-// well. own: the window holds the cell's own particles [o0, o0 + ne) instead,
+// octant. A cell of fewer batches than warps splits the window's entries between
+// units as well, to one unit per warp (to two, cells of two batches spent more on
+// listing entries and on short last chunks: 2M particles at 40 per cell, two cells
+// per cutoff, count 2.90 -> 2.68 ms, forces 5.49 -> 5.04). own: the window holds the cell's own particles [o0, o0 + ne) instead,
 // and a batch takes those after its own (its own ones masked by index).
 template <int MODE>
 __device__ __forceinline__ void half_units(HalfSmem& S, bool own, int hs, int wf, int wb, int o0, int ne,
                                            const ScalarRed& R, UnitAcc& acc) {
   const int lane = threadIdx.x & 31;
   const int nbatch = S.nbatch;
-  const int nseg = nbatch < 2 * kWarps ? (2 * kWarps + nbatch - 1) / nbatch : 1;
+  const int nseg = nbatch < kWarps ? (kWarps + nbatch - 1) / nbatch : 1;
   const int seglen = ((ne + nseg - 1) / nseg + 31) & ~31;
   for (;;) {
     int k = 0;
