@@ -232,8 +232,9 @@ int cl_cross_topk(const cl_list* cl, const double* posb_dev, long long nb, int k
 int cl_box_nonperiodic(const double* pos_dev, long long n, const double* pos2_dev, long long n2, int dim,
                        double cutoff, int lcell, void* stream, cl_box* box_out);
 
-/* Mapped functions of the paper's examples, built on the compile-time functor
- * hook (cellmap_pairfns.cuh) with one thread per cell-sorted particle. All
+/* Mapped functions of the paper's examples, one thread per cell-sorted particle:
+ * in 3D sweeps of the library's own, in 2D, for the Lennard-Jones energy alone and
+ * for the mass sum of sparse lists the ready-made functors of cellmap_pairfns.cuh. All
  * arrays are DEVICE arrays in original particle order; scalar and histogram
  * outputs are zeroed and then accumulated, FP64. Asynchronous on `stream`.
  *

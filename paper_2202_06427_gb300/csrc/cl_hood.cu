@@ -1409,8 +1409,9 @@ __global__ void __launch_bounds__(kThreads, hood_ctas(MODE)) k_hood(const __grid
 // the other sweeps (minus the sum over ordered pairs) this is -2 times it.
 //
 // Cells whose particles or half neighbourhood exceed the buffers (more than
-// kHome particles, more than kHCap particles in the half stencil's cells)
-// take the windowed form of the same sweep (k_half_batch): the half
+// kHome particles; a half neighbourhood of more than rawcap particles, so that
+// more than kHCap are expected within its ball, or one that holds more all the
+// same) take the windowed form of the same sweep (k_half_batch): the half
 // neighbourhood's row segments are laid end to end and staged in windows of
 // kHCap particles, each window swept against the home particles in batches of
 // kBatch, and the pairs within the cell are swept as a last window per batch
@@ -2024,13 +2025,16 @@ __device__ __noinline__ void half_unit(HalfSmem& S, const Unit u, UnitAcc& acc, 
 }
 
 // The batches of a windowed cell against the staged window, a warp at a time
-// from a counter. A batch is at most kBatch of the cell's particles,
-// consecutive in its octant order (k_octsort), so it lies in part of one
-// octant. A cell of fewer batches than warps splits the window's entries between
+// from a counter. A batch is at most kBatch consecutive particles of the cell,
+// within one of the ranges S.oct: in a cell that k_octsort has ordered part of an
+// octant, so that the batch's ball is small; in one that overflowed the fast path
+// after the ordering (65 to kHome particles) any of the cell's, with a ball of about
+// the cell's. A cell of fewer batches than warps splits the window's entries between
 // units as well, to one unit per warp (to two, cells of two batches spent more on
 // listing entries and on short last chunks: 2M particles at 40 per cell, two cells
-// per cutoff, count 2.90 -> 2.68 ms, forces 5.49 -> 5.04). own: the window holds the cell's own particles [o0, o0 + ne) instead,
-// and a batch takes those after its own (its own ones masked by index).
+// per cutoff, count 2.90 -> 2.68 ms, forces 5.49 -> 5.04). own: the window holds the
+// cell's own particles [o0, o0 + ne) instead, and a batch takes those after its own
+// (its own ones masked by index).
 template <int MODE>
 __device__ __forceinline__ void half_units(HalfSmem& S, bool own, int hs, int wf, int wb, int o0, int ne,
                                            const ScalarRed& R, UnitAcc& acc) {
@@ -2766,7 +2770,7 @@ bool hood_half_fits(const SweepArgs& A) { return A.noff <= kTab; }
 
 // Scalar reductions over the half stencil. When the stencil fits the table,
 // the work lists of the half-shell sweep split the cells: the fast-path cells
-// (at most kHome particles, at most kHCap in the half neighbourhood) go to the
+// (at most kHome particles, at most rawcap in the half neighbourhood) go to the
 // home-major k_hood<mode>, the others to k_half_batch<mode> (windowed cells by
 // batches of 32 home particles, small cells one per warp); otherwise
 // k_hood<mode> takes the cells it can and the per-particle sweep the rest.

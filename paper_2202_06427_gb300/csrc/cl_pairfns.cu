@@ -5,9 +5,9 @@
 // velocity histogram run on sweeps of their own below, one thread per
 // cell-sorted particle like the ready-made device functors of
 // cellmap_pairfns.cuh, and add each particle's terms in the functors' order, so
-// that their FP32 sums round alike. 2D, and the Lennard-Jones energy alone, run
-// the functors on the compile-time hook of cellmap_functor.cuh, as a user's own
-// would. (The half-shell sweep of cl_hood.cu does Lennard-Jones forces in half
+// that their FP32 sums round alike. 2D, the Lennard-Jones energy alone and the mass
+// sum of sparse lists run the functors on the compile-time hook of
+// cellmap_functor.cuh, as a user's own would. (The half-shell sweep of cl_hood.cu does Lennard-Jones forces in half
 // the functor's time, 0.74 against 1.57 ms at 500,000 particles, but its
 // energy, summed pair by pair instead of per particle from both ends, differs
 // from the functor's by 5e-9; it was left out.)

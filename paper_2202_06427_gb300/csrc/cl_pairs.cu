@@ -538,28 +538,28 @@ template <int DIM>
 __device__ __forceinline__ void count_two(const SweepArgs& A, int p, int h1, const float4* st, int S,
                                           int* __restrict__ count) {
   const int lane = threadIdx.x & 31;
-            const bool two = p + 1 < h1;
-            const float4 pa = A.xs[p];
-            const float4 pb = two ? A.xs[p + 1] : pa;
-            const int a0 = __float_as_int(pa.w), a1 = two ? __float_as_int(pb.w) : INT_MAX;
-            const float2 nx = make_float2(-pa.x, -pb.x), ny = make_float2(-pa.y, -pb.y),
-                         nz = make_float2(-pa.z, -pb.z);
-            int L0 = 0, L1 = 0;  // per lane, summed over the warp at the end
-  #pragma unroll 2
-            for (int t = lane; t < S; t += 32) {
-              const float4 q = st[t];
-              const int jo = __float_as_int(q.w);
-              float2 dx, dy, dz;
-              const float2 d2 = pair_d2<DIM>(q, nx, ny, nz, dx, dy, dz);
-              L0 += (jo > a0 && d2.x < A.rc2) ? 1 : 0;
-              L1 += (jo > a1 && d2.y < A.rc2) ? 1 : 0;
-            }
-            L0 = __reduce_add_sync(0xffffffffu, L0);
-            L1 = __reduce_add_sync(0xffffffffu, L1);
-            if (lane == 0) {
-              count[a0] = L0;
-              if (two) count[a1] = L1;
-            }
+  const bool two = p + 1 < h1;
+  const float4 pa = A.xs[p];
+  const float4 pb = two ? A.xs[p + 1] : pa;
+  const int a0 = __float_as_int(pa.w), a1 = two ? __float_as_int(pb.w) : INT_MAX;
+  const float2 nx = make_float2(-pa.x, -pb.x), ny = make_float2(-pa.y, -pb.y),
+               nz = make_float2(-pa.z, -pb.z);
+  int L0 = 0, L1 = 0;  // per lane, summed over the warp at the end
+#pragma unroll 2
+  for (int t = lane; t < S; t += 32) {
+    const float4 q = st[t];
+    const int jo = __float_as_int(q.w);
+    float2 dx, dy, dz;
+    const float2 d2 = pair_d2<DIM>(q, nx, ny, nz, dx, dy, dz);
+    L0 += (jo > a0 && d2.x < A.rc2) ? 1 : 0;
+    L1 += (jo > a1 && d2.y < A.rc2) ? 1 : 0;
+  }
+  L0 = __reduce_add_sync(0xffffffffu, L0);
+  L1 = __reduce_add_sync(0xffffffffu, L1);
+  if (lane == 0) {
+    count[a0] = L0;
+    if (two) count[a1] = L1;
+  }
 }
 
 // The same two particles' segments of the list, from the staged entries in
@@ -574,72 +574,72 @@ __device__ __forceinline__ void fill_two(const SweepArgs& A, int p, int h1, At a
                                          float* __restrict__ pd_out) {
   const int lane = threadIdx.x & 31;
   const unsigned lt = (1u << lane) - 1u;
-            const bool two = p + 1 < h1;
-            const float4 pa = A.xs[p];
-            const float4 pb = two ? A.xs[p + 1] : pa;
-            const int a0 = __float_as_int(pa.w), a1 = two ? __float_as_int(pb.w) : INT_MAX;
-            int f0 = 0, f1 = S;  // first position (in index order) with index > a0, a1
-            {
-              const unsigned ka = a0 >= kmin ? (unsigned)(a0 - kmin) : 0u;
-              int lo = 0, hi = S;
-              while (a0 >= kmin && lo < hi) {
-                const int mid = (lo + hi) >> 1;
-                if ((unsigned)(__float_as_int(at(mid).w) - kmin) > ka) hi = mid;
-                else lo = mid + 1;
-              }
-              f0 = a0 >= kmin ? lo : 0;
-            }
-            if (two) {
-              const unsigned kb = a1 >= kmin ? (unsigned)(a1 - kmin) : 0u;
-              int lo = 0, hi = S;
-              while (a1 >= kmin && lo < hi) {
-                const int mid = (lo + hi) >> 1;
-                if ((unsigned)(__float_as_int(at(mid).w) - kmin) > kb) hi = mid;
-                else lo = mid + 1;
-              }
-              f1 = a1 >= kmin ? lo : 0;
-            }
-            const int c0 = __ldg(count + a0), c1 = two ? __ldg(count + a1) : 0;
-            const long long b0 = __ldg(start + a0), b1 = two ? __ldg(start + a1) : 0;
-            const float2 nx = make_float2(-pa.x, -pb.x), ny = make_float2(-pa.y, -pb.y),
-                         nz = make_float2(-pa.z, -pb.z);
-            int L0 = 0, L1 = 0;
-  #pragma unroll 2
-            for (int t0 = min(f0, f1); t0 < S; t0 += 32) {
-              const int t = t0 + lane;
-              bool k0 = false, k1 = false;
-              int jo = 0;
-              float d20 = 0.f, d21 = 0.f;
-              if (t < S) {
-                const float4 q = at(t);
-                jo = __float_as_int(q.w);
-                float2 dx, dy, dz;
-                const float2 d2 = pair_d2<DIM>(q, nx, ny, nz, dx, dy, dz);
-                d20 = d2.x;
-                d21 = d2.y;
-                k0 = jo > a0 && d20 < A.rc2;
-                k1 = jo > a1 && d21 < A.rc2;
-              }
-              const unsigned m0 = __ballot_sync(0xffffffffu, k0), m1 = __ballot_sync(0xffffffffu, k1);
-              if (k0) {
-                const int e = L0 + __popc(m0 & lt);
-                if (e < c0) {
-                  pi_out[b0 + e] = a0;
-                  pj_out[b0 + e] = jo;
-                  pd_out[b0 + e] = d20 * rsqrt_nr(d20);
-                }
-              }
-              if (k1) {
-                const int e = L1 + __popc(m1 & lt);
-                if (e < c1) {
-                  pi_out[b1 + e] = a1;
-                  pj_out[b1 + e] = jo;
-                  pd_out[b1 + e] = d21 * rsqrt_nr(d21);
-                }
-              }
-              L0 += __popc(m0);
-              L1 += __popc(m1);
-            }
+  const bool two = p + 1 < h1;
+  const float4 pa = A.xs[p];
+  const float4 pb = two ? A.xs[p + 1] : pa;
+  const int a0 = __float_as_int(pa.w), a1 = two ? __float_as_int(pb.w) : INT_MAX;
+  int f0 = 0, f1 = S;  // first position (in index order) with index > a0, a1
+  {
+    const unsigned ka = a0 >= kmin ? (unsigned)(a0 - kmin) : 0u;
+    int lo = 0, hi = S;
+    while (a0 >= kmin && lo < hi) {
+      const int mid = (lo + hi) >> 1;
+      if ((unsigned)(__float_as_int(at(mid).w) - kmin) > ka) hi = mid;
+      else lo = mid + 1;
+    }
+    f0 = a0 >= kmin ? lo : 0;
+  }
+  if (two) {
+    const unsigned kb = a1 >= kmin ? (unsigned)(a1 - kmin) : 0u;
+    int lo = 0, hi = S;
+    while (a1 >= kmin && lo < hi) {
+      const int mid = (lo + hi) >> 1;
+      if ((unsigned)(__float_as_int(at(mid).w) - kmin) > kb) hi = mid;
+      else lo = mid + 1;
+    }
+    f1 = a1 >= kmin ? lo : 0;
+  }
+  const int c0 = __ldg(count + a0), c1 = two ? __ldg(count + a1) : 0;
+  const long long b0 = __ldg(start + a0), b1 = two ? __ldg(start + a1) : 0;
+  const float2 nx = make_float2(-pa.x, -pb.x), ny = make_float2(-pa.y, -pb.y),
+               nz = make_float2(-pa.z, -pb.z);
+  int L0 = 0, L1 = 0;
+#pragma unroll 2
+  for (int t0 = min(f0, f1); t0 < S; t0 += 32) {
+    const int t = t0 + lane;
+    bool k0 = false, k1 = false;
+    int jo = 0;
+    float d20 = 0.f, d21 = 0.f;
+    if (t < S) {
+      const float4 q = at(t);
+      jo = __float_as_int(q.w);
+      float2 dx, dy, dz;
+      const float2 d2 = pair_d2<DIM>(q, nx, ny, nz, dx, dy, dz);
+      d20 = d2.x;
+      d21 = d2.y;
+      k0 = jo > a0 && d20 < A.rc2;
+      k1 = jo > a1 && d21 < A.rc2;
+    }
+    const unsigned m0 = __ballot_sync(0xffffffffu, k0), m1 = __ballot_sync(0xffffffffu, k1);
+    if (k0) {
+      const int e = L0 + __popc(m0 & lt);
+      if (e < c0) {
+        pi_out[b0 + e] = a0;
+        pj_out[b0 + e] = jo;
+        pd_out[b0 + e] = d20 * rsqrt_nr(d20);
+      }
+    }
+    if (k1) {
+      const int e = L1 + __popc(m1 & lt);
+      if (e < c1) {
+        pi_out[b1 + e] = a1;
+        pj_out[b1 + e] = jo;
+        pd_out[b1 + e] = d21 * rsqrt_nr(d21);
+      }
+    }
+    L0 += __popc(m0);
+    L1 += __popc(m1);
+  }
 }
 
 // Sparse grids (at most kSparse particles expected in a staging ball): a warp
