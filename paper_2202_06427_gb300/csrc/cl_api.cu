@@ -36,7 +36,7 @@ struct cl_list {
   int* work;  // work counters of the persistent neighbourhood sweeps
   float4* hforce;  // per sorted particle: forces accumulated by the half-shell sweep (kept zero between launches)
   int last_half;   // the last 3D energy/force sweep took the half-shell path
-  int lists_half;  // hlist / hdense / work[6..8] hold the half-shell work lists of the current cell list
+  int lists_half;  // hlist / hdense / work[6..9] hold the half-shell work lists of the current cell list
   unsigned long long* u64;
   // neighbour-list workspace, allocated on the first CL_RED_PAIRLIST call
   int* pl_count;

@@ -56,6 +56,7 @@ constexpr int kMinHome = 8;            // fewer home particles: the per-particle
 constexpr int kCap = 2560;             // staged neighbour entries (even)
 constexpr int kTab = 1 + kWarps * 32;  // stencil entries the fast path takes (32 per warp)
 constexpr int kHCap = 1536;            // staged entries of the half-shell path
+constexpr int kBatch = 32;             // home particles of a batch of the half-shell path, swept by one warp
 // Padding entries sit at (kFar, kFar, kFar) and a missing second home particle
 // of a group at -kFar: far from everything and from each other (the stand-ins
 // of non-finite inputs lie within [1e15, 2e15) per axis), with squared
@@ -740,11 +741,15 @@ __device__ __forceinline__ int run_count(const int* __restrict__ cell_start, int
 // A cell whose staged neighbourhood overflows is moved to the dense list by
 // the sweep itself. With half != 0 (the half-shell sweep takes the launch)
 // every non-empty cell is listed: on list when it holds at most kHome
-// particles and its half stencil's cells at most H.rawcap, on dense (the
-// windowed cells) otherwise. kListLanes lanes share a cell's rows: one thread
-// per cell took 13 us on a grid of 343 cells and 18 on one of 42,875 (now 11;
-// bound by the latency of the row bounds). Listed by warps instead of blocks,
-// the lists' three counters took 15 us there, 104 at 421,875 cells (now 32).
+// particles and its half stencil's cells at most H.rawcap, else on dense: from
+// its end backwards (work[9] of them) the cells of kBatch + 1 to kOctMin - 1
+// particles in a neighbourhood of less than twice their density, which the whole
+// CTA sweeps (half_whole_cells; beside denser cells batches gain by their smaller
+// balls: 16M clustered 18.28 ms so, 18.41 with all cells of that size), the others
+// from its start. kListLanes lanes share a cell's rows: one thread per cell took 13
+// us on a grid of 343 cells and 18 on one of 42,875 (now 11; bound by the latency of
+// the row bounds). Listed by warps instead of blocks, the lists' three counters took
+// 15 us there, 104 at 421,875 cells (now 32).
 constexpr int kListLanes = 8;  // 32 cells to a block of 256
 __global__ void __launch_bounds__(256) k_hood_list(const int* __restrict__ cell_start, int ncells, int noff,
                                                    int* __restrict__ work, int* __restrict__ list,
@@ -792,11 +797,12 @@ __global__ void __launch_bounds__(256) k_hood_list(const int* __restrict__ cell_
   }
   // the block's cells listed by its first warp, a cell per lane: one atomic per
   // block and list
-  __shared__ unsigned char kind[32];  // 0 empty, 1 listed, 2 dense, 3 small, 4 left to the companion
+  __shared__ unsigned char kind[32];  // 0 empty, 1 listed, 2 dense, 3 small, 4 left to the companion, 5 whole
   if (sub == 0) {
     const int nh = h < ncells ? cell_start[h + 1] - cell_start[h] : 0;
     const bool small = take && half && cnt + nh <= H.smallcap;
-    kind[threadIdx.x / kListLanes] = nh == 0 ? 0 : (small ? 3 : (take ? 1 : (big ? 2 : 4)));
+    const bool whole = half && nh > kBatch && nh < kOctMin && cnt < 2 * noff_half * nh;
+    kind[threadIdx.x / kListLanes] = nh == 0 ? 0 : (small ? 3 : (take ? 1 : (big ? (whole ? 5 : 2) : 4)));
   }
   __syncthreads();
   if (threadIdx.x >= 32) return;
@@ -804,18 +810,21 @@ __global__ void __launch_bounds__(256) k_hood_list(const int* __restrict__ cell_
   if (c < ncells) flag[c] = k == 2 ? 2 : (k == 4 ? 1 : 0);
   const unsigned lt = (1u << lane) - 1u;
   const unsigned m = __ballot_sync(0xffffffffu, k == 1), mb = __ballot_sync(0xffffffffu, k == 2),
-                 ms = __ballot_sync(0xffffffffu, k == 3);
-  int base = 0, bbase = 0, sbase = 0;
+                 ms = __ballot_sync(0xffffffffu, k == 3), mw = __ballot_sync(0xffffffffu, k == 5);
+  int base = 0, bbase = 0, sbase = 0, wbase = 0;
   if (lane == 0) {
     if (m) base = atomicAdd(work + 6, __popc(m));
     if (mb) bbase = atomicAdd(ndense, __popc(mb));
     if (ms) sbase = atomicAdd(work + 8, __popc(ms));
+    if (mw) wbase = atomicAdd(work + 9, __popc(mw));
   }
   base = __shfl_sync(0xffffffffu, base, 0);
   bbase = __shfl_sync(0xffffffffu, bbase, 0);
   sbase = __shfl_sync(0xffffffffu, sbase, 0);
+  wbase = __shfl_sync(0xffffffffu, wbase, 0);
   if (k == 1) list[base + __popc(m & lt)] = c;
   if (k == 2) dense[bbase + __popc(mb & lt)] = c;
+  if (k == 5) dense[ncells - 1 - (wbase + __popc(mw & lt))] = c;
   if (k == 3) list[ncells - 1 - (sbase + __popc(ms & lt))] = c;  // small cells go to the end of list
 }
 
@@ -1415,13 +1424,12 @@ __global__ void __launch_bounds__(kThreads, hood_ctas(MODE)) k_hood(const __grid
 // neighbourhood's row segments are laid end to end and staged in windows of
 // kHCap particles, each window swept against the home particles in batches of
 // kBatch, and the pairs within the cell are swept as a last window per batch
-// (the cell's particles from the batch's first on). Every non-empty cell is
-// swept, so the path covers the whole grid whenever both stencils fit the
-// table.
+// (the cell's particles from the batch's first on), or against all of them at once
+// (half_whole_cells). Every non-empty cell is swept, so the path covers the whole
+// grid whenever both stencils fit the table.
 
 constexpr int kEnt = 4;             // staged entries per lane in a chunk of the half-shell sweep
 constexpr int kChunk = 32 * kEnt;   // entries per chunk
-constexpr int kBatch = 32;          // home particles of a batch, swept by one warp
 static_assert(kWarps * kBatch == kHome, "the batches' force sums share the fast path's");
 // Small cells: the cell and its half neighbourhood in one warp's share of the
 // entry buffer, its row segments in the warp's share of the segment table.
@@ -2026,15 +2034,14 @@ __device__ __noinline__ void half_unit(HalfSmem& S, const Unit u, UnitAcc& acc, 
 
 // The batches of a windowed cell against the staged window, a warp at a time
 // from a counter. A batch is at most kBatch consecutive particles of the cell,
-// within one of the ranges S.oct: in a cell that k_octsort has ordered part of an
-// octant, so that the batch's ball is small; in one that overflowed the fast path
-// after the ordering (65 to kHome particles) any of the cell's, with a ball of about
-// the cell's. A cell of fewer batches than warps splits the window's entries between
-// units as well, to one unit per warp (to two, cells of two batches spent more on
-// listing entries and on short last chunks: 2M particles at 40 per cell, two cells
-// per cutoff, count 2.90 -> 2.68 ms, forces 5.49 -> 5.04). own: the window holds the
-// cell's own particles [o0, o0 + ne) instead, and a batch takes those after its own
-// (its own ones masked by index).
+// within one of the ranges S.oct: part of an octant in a cell that k_octsort has
+// ordered, so that the batch's ball is small, any of the cell's in others. A cell of
+// fewer batches than warps splits the window's entries between units as well, to one
+// unit per warp (to two, cells of two batches spent more on listing entries and on
+// short last chunks: 2M particles at 40 per cell, two cells per cutoff, by batches,
+// count 2.90 -> 2.68 ms, forces 5.49 -> 5.04). own: the window holds the cell's own
+// particles [o0, o0 + ne) instead, and a batch takes those after its own (its own
+// ones masked by index).
 template <int MODE>
 __device__ __forceinline__ void half_units(HalfSmem& S, bool own, int hs, int wf, int wb, int o0, int ne,
                                            const ScalarRed& R, UnitAcc& acc) {
@@ -2328,7 +2335,7 @@ __device__ __forceinline__ void half_partials(const HoodArgs& H, const HalfSmem&
 // The fast-path cells (list), a CTA per cell: energy, forces, boundary terms
 // (MODE 0, 1, 3). A cell whose kept neighbourhood overflows the buffer
 // (k_hood_list goes by the expected share of the raw one) is moved to the
-// dense list, which k_half_batch takes afterwards.
+// dense list's end, which k_half_batch takes afterwards.
 template <int MODE>
 __global__ void __launch_bounds__(kThreads, kHalfCtas) k_hood_half(const __grid_constant__ SweepArgs A,
                                                            const __grid_constant__ HoodArgs H,
@@ -2391,7 +2398,7 @@ __global__ void __launch_bounds__(kThreads, kHalfCtas) k_hood_half(const __grid_
     const int nf = S.nf, nb = S.nb;
     if (nf + nb > kHCap) {  // uniform
       if (tid == 0) {
-        H.dense[atomicAdd(H.ndense, 1)] = h;
+        H.dense[H.ncells - 1 - atomicAdd(H.work + 9, 1)] = h;
         H.list[S.kind] = -1;
       }
       continue;
@@ -2443,9 +2450,114 @@ __global__ void __launch_bounds__(kThreads, kHalfCtas) k_hood_half(const __grid_
   half_partials<MODE>(H, S, partials);
 }
 
-// The cells swept by batches, a batch per warp: the windowed ones (dense), a
-// CTA per cell, then the small ones (the end of list, backwards), a warp per
-// cell, which fill the end of the launch. All modes; the scalar ones (2
+// The end of dense, backwards: cells of at most kHome particles in no order
+// (k_hood_list; those that overflowed the fast path), a CTA per cell. Their batches'
+// balls would be about the cell's own, so that the batches' lists leave out few
+// entries and every batch adds its own force to each; here a window's chunks, from
+// a counter, are swept against all home particles (S.home), and after the last
+// window the cell's own (S.own), as on the fast path. 2M particles, two cells per
+// cutoff, against batches: 40 per cell count 2.68 -> 1.91 ms, forces 5.00 -> 4.00; 33
+// per cell 2.63 -> 2.05 and 4.85 -> 4.14; 64 per cell 3.52 -> 3.34 and 6.68 -> 6.56.
+// After the batches instead of among them: the two kinds of code side by side on an SM
+// do not fit the instruction cache (forces at 33 per cell 5.8 ms with the kinds mixed,
+// at 64 7.6). As a function of its own (not inlined) it cost the batches registers
+// (16M clustered 18.37 -> 18.52 ms; inlined 18.27).
+template <int MODE>
+__device__ __forceinline__ void half_whole_cells(const SweepArgs& A, const HoodArgs& H, HalfSmem& S, UnitAcc& acc,
+                                                 const ScalarRed& Rin) {
+  constexpr bool SCALAR = MODE == 2 || MODE >= 4, ENERGY = MODE != 1 && MODE != 4 && MODE != 6;
+  const HalfCtx& X = S.ctx;
+  const ScalarRed R = Rin;
+  const int tid = threadIdx.x, lane = tid & 31;
+  UnitAcc a = acc;
+  const int nwhole = H.work[9];
+  int next1 = nwhole;
+  if (tid == 0) next1 = atomicAdd(H.work + 4, 1);
+  for (;;) {
+    __syncthreads();
+    if (tid == 0) {
+      S.item = next1 < nwhole ? H.dense[H.ncells - 1 - next1] : -2;
+      if (next1 < nwhole) next1 = atomicAdd(H.work + 4, 1);
+    }
+    __syncthreads();
+    const int h = S.item;
+    if (h < 0) break;
+    const int hs = A.cell_start[h], nh = A.cell_start[h + 1] - hs;
+    if (tid < 32) half_segments(A, S, h % A.nx, (h / A.nx) % A.ny, h / (A.nx * A.ny));
+    float d = 0.f;
+    for (int t = tid; t < nh + 4; t += kThreads) {
+      float4 q = make_float4(-kFar, kFar, -kFar, 0.f);  // padding: far from every entry
+      if (t < nh) {
+        q = A.xs[hs + t];
+        d = fmaxf(d, fminf(sqrtf(fmaf(q.x, q.x, fmaf(q.y, q.y, q.z * q.z))), H.hd));
+        S.own[t] = make_float4(q.x, q.y, q.z, __int_as_float(hs + t));
+      }
+      S.home[t] = make_float4(-q.x, -q.y, -q.z, 0.f);
+    }
+#pragma unroll
+    for (int o = 16; o; o >>= 1) d = fmaxf(d, __shfl_xor_sync(0xffffffffu, d, o));
+    if (lane == 0) S.wmax[tid >> 5] = d;
+    __syncthreads();
+#pragma unroll
+    for (int w = 0; w < kWarps; ++w) d = fmaxf(d, S.wmax[w]);
+    const float top = H.rc + d + H.eps;
+    const int C = S.ctot;
+    for (int w0 = 0;;) {
+      __syncthreads();  // the last window's readers are done
+      if (tid == 0) S.nf = S.nb = S.next = 0;
+      __syncthreads();
+      const int w1 = min(C, w0 + kHCap);
+      half_stage_window(A, S, w0, w1, 0.f, 0.f, 0.f, top * top);
+      __syncthreads();
+      SeqInfo sq;
+      sq.nf = S.nf;
+      sq.nb = S.nb;
+      sq.nh = w1 == C ? nh : 0;
+      sq.obase = sq.oown = 0;
+      sq.wf = 0;
+      sq.list = nullptr;
+      const int ne = sq.nf + sq.nb, nch = (ne + sq.nh + kChunk - 1) / kChunk;
+      for (;;) {
+        int c = 0;
+        if (lane == 0) c = atomicAdd(&S.next, 1);
+        c = __shfl_sync(0xffffffffu, c, 0);
+        if (c >= nch) break;
+        const int base = c * kChunk;
+        float2 jx[kEnt / 2], jy[kEnt / 2], jz[kEnt / 2];
+        if (sq.nh == 0 || base + kChunk <= ne)
+          half_chunk<false, kSeqPlain, MODE, 2>(S, S.home, S.hg, sq, base, nh, X.rc2, X.irc, X.irc2, jx, jy, jz, a.e, a.cnt, R);
+        else
+          half_chunk<true, kSeqPlain, MODE, 2>(S, S.home, S.hg, sq, base, nh, X.rc2, X.irc, X.irc2, jx, jy, jz, a.e, a.cnt, R);
+        if (!SCALAR) {
+#pragma unroll
+          for (int k = 0; k < kEnt / 2; ++k) {
+            half_flush(X.hforce, X.hrow, S, sq, base + lane + 64 * k, jx[k].x, jy[k].x, jz[k].x, a.wv);
+            half_flush(X.hforce, X.hrow, S, sq, base + lane + 64 * k + 32, jx[k].y, jy[k].y, jz[k].y, a.wv);
+          }
+        }
+        a.cand += (unsigned long long)(nh * max(0, min(kChunk, ne - base)));
+        if (c == nch - 1 && sq.nh) a.cand += (unsigned long long)(nh * (nh - 1) / 2);
+      }
+      if (w1 == C) break;
+      w0 = w1;
+    }
+    half_fold<ENERGY>(S, a.e, a.wv);
+    if (!SCALAR) {
+      __syncthreads();
+      if (tid < nh) {
+        const float gx = S.hg[tid][0], gy = S.hg[tid][1], gz = S.hg[tid][2];
+        if (gx != 0.f || gy != 0.f || gz != 0.f) atomicAdd(&X.hforce[hs + tid], make_float4(-gx, -gy, -gz, 0.f));
+        S.hg[tid][0] = S.hg[tid][1] = S.hg[tid][2] = 0.f;
+      }
+    }
+  }
+  __syncthreads();  // the small cells' warps write what other warps have read and cleared
+  acc = a;
+}
+
+// The other cells: the windowed ones, a CTA per cell, by batches (the start of
+// dense) and then as a whole (its end), and the small ones (the end of list,
+// backwards), a warp per cell, which fill the end of the launch. All modes; the scalar ones (2
 // energy, 4 count, 5 sum 1/r, 6 histogram, its copies after HalfSmem as in
 // k_hood) evaluate the same candidates without forces.
 template <int MODE>
@@ -2457,8 +2569,8 @@ __global__ void __launch_bounds__(kThreads, 5) k_half_batch(const __grid_constan
   HalfSmem& S = *reinterpret_cast<HalfSmem*>(smraw);
   const int tid = threadIdx.x, lane = tid & 31;
   constexpr int NV = hood_nv(MODE);
-  const int ndense = *H.ndense, nsmall = H.work[8];
-  if (ndense + nsmall == 0) {  // no such cell
+  const int ndense = *H.ndense;
+  if (ndense + H.work[8] + H.work[9] == 0) {  // no such cell
     if (tid < NV) partials[(size_t)blockIdx.x * NV + tid] = 0.0;
     return;
   }
@@ -2493,6 +2605,8 @@ __global__ void __launch_bounds__(kThreads, 5) k_half_batch(const __grid_constan
     half_windowed<MODE>(A, H, S, hs, A.cell_start[h + 1] - hs, h % A.nx, (h / A.nx) % A.ny, h / (A.nx * A.ny), R, acc);
     half_fold<ENERGY>(S, acc.e, acc.wv);
   }
+  if (H.work[9]) half_whole_cells<MODE>(A, H, S, acc, R);
+  const int nsmall = H.work[8];
   for (;;) {
     int k = 0;
     if (lane == 0) k = atomicAdd(H.work + 1, 1);

@@ -225,9 +225,9 @@ struct HoodArgs {
   int smallcap;       // particles of a cell and its half neighbourhood up to which one warp takes it
   int split;          // CTAs sharing a listed cell's home particles (home-major scalar sweeps)
   int ncells;
-  int* work;          // [0], [1], [5] work counters of the listed, small and dense cells, [2..3] candidates
+  int* work;          // [0], [1], [4], [5] work counters of the listed, small, whole and dense cells, [2..3] candidates
                       // (zeroed by the launcher); [6] list length, [7] dense cells, [8] small cells (at the end
-                      // of list, backwards; written by k_hood_list)
+                      // of list, backwards), [9] whole cells (at the end of dense, backwards; written by k_hood_list)
   int* list;          // cells the neighbourhood sweep takes (ncells capacity)
   unsigned long long* cand;  // candidate pairs evaluated (work[2..3] of the same buffer), zeroed by the launcher
   unsigned char* flag;       // per cell: 1 per-particle companion sweep, 2 dense-cell sweep
@@ -253,7 +253,7 @@ size_t hood_smem_bytes();
 // stencil); 3: energy and the backward outputs.
 // partials_cap: doubles available in partials (sweep_partials_needed).
 // lists_half (host, may be null): 1 when the list buffers (list, dense, flag,
-// work[6..8]) hold the half-shell work lists of the current cell list; they
+// work[6..9]) hold the half-shell work lists of the current cell list; they
 // are then reused, and the flag is set after a half-shell launch and cleared
 // by any other.
 // Ahalf (modes 0, 1, 3; may be null): the half stencil, for the half-shell

@@ -75,6 +75,37 @@ def test_kinds_of_cells(cuda_ok, name):
     assert occupied > 2048 if name == "huge" else occupied <= 2048
 
 
+@pytest.mark.parametrize("side", [19, 20, 22, 24])
+@pytest.mark.parametrize("tric", [False, True])
+def test_windowed_cells_in_no_order(cuda_ok, side, tric):
+    """Uniform sets of 32 to 64 particles a cell on average, whose half
+    neighbourhoods take two windows: the edges of the batches (32) and of the
+    ordered cells (65), with and without a boundary in the stencil."""
+    import paper_2202_06427_gb300 as P
+    rng = np.random.default_rng(side)
+    L, rc, lcell = 12.0, 4.0, 2
+    h = np.eye(3) * L
+    if tric:
+        h[1, 0], h[2, 0], h[2, 1] = 1.1, -0.8, 0.7
+    x = _background(rng, h, L / (side + 0.5), np.zeros(3), -1.0)
+    assert len(x) == side ** 3
+    x = np.ascontiguousarray(x[rng.permutation(len(x))])
+    ref = oracle.pair_map(x, h, rc, band=BAND, nbins=17)
+    cl = P.cl_build(torch.from_numpy(x).cuda(), h, rc, lcell)
+    g = torch.tensor([0.75], dtype=torch.float64, device="cuda")
+    for _ in range(2):
+        efv = P.cl_map(cl, "energy_forces_virial")
+        check_energy(efv["energy"].item(), ref["energy"])
+        check_forces(efv["forces"].cpu().numpy(), ref["forces"])
+        check_matrix(efv["virial"].cpu().numpy(), ref["virial"], TOL_W)
+        check_energy(P.cl_map(cl, "energy")["energy"].item(), ref["energy"])
+        check_count(int(P.cl_map(cl, "count")["count"].item()), ref)
+        check_hist(P.cl_map(cl, "hist", nbins=17)["hist"].cpu().numpy(), ref)
+        gp, gb, _ = P.cl_backward(cl, g)
+        check_forces(gp.cpu().numpy(), -0.75 * ref["forces"])
+        check_matrix(gb.cpu().numpy(), 0.75 * ref["dedh"], TOL_GB)
+
+
 @pytest.mark.parametrize("lcell", [1, 2])
 def test_clumps_beyond_each_others_cutoff(cuda_ok, lcell):
     """Clumps of 2 to 300 particles farther apart than the cutoff: a batch's own
