@@ -47,9 +47,11 @@ struct ReqDesc {
   double* virial;
 };
 
-// Tiles of 128 particles, eight CTAs to an SM (64 registers): 32 mixed requests
-// 1.85 ms, against 2.19 with 256 threads at the 80 registers the compiler would
-// take (24 warps per SM), 1.79 to 1.90 at 256 and 64, 2.03 with 64 threads.
+// Tiles of 128 particles, eight CTAs to an SM (64 registers). 32 mixed requests in
+// one session 1.85 ms, 2.19 with 256 threads at the 80 registers the compiler would
+// take (24 warps per SM), 1.79 to 1.90 at 256 and 64, 2.03 with 64 threads; over
+// sessions 1.83 to 1.90 (spread of one 8 %), and with other positions of the same
+// requests about 1 % below 256 threads.
 constexpr int kServeThreads = 128;
 constexpr int kServeCtas = 8;
 // A batch of no more than one wide tile per SM takes those (128 registers): its time
