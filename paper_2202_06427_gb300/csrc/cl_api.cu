@@ -37,6 +37,8 @@ struct cl_list {
   float4* hforce;  // per sorted particle: forces accumulated by the half-shell sweep (kept zero between launches)
   int last_half;   // the last 3D energy/force sweep took the half-shell path
   int lists_half;  // hlist / hdense / work[6..9] hold the half-shell work lists of the current cell list
+  int replayed;    // a graph may bin into this list: its cell contents change without a call (kept_lists)
+  int lists_none;
   unsigned long long* u64;
   // neighbour-list workspace, allocated on the first CL_RED_PAIRLIST call
   int* pl_count;
@@ -239,6 +241,7 @@ int run_build(cl_list* c, cudaStream_t s) {
   b.n = c->n;
   b.slot = c->slot;
   c->lists_half = 0;  // new cell contents: the sweeps' work lists are rebuilt
+  if (clk::capturing(s)) c->replayed = 1;
   b.xl = c->xl;
   b.counts = c->counts;
   b.cell_start = c->cell_start;
@@ -247,6 +250,16 @@ int run_build(cl_list* c, cudaStream_t s) {
   b.xs = c->xs;
   b.cellc = c->cellc;
   return clk::launch_build(c->geo, b, s);
+}
+
+// The flag that tells a sweep whether the work lists are there. A captured sweep
+// makes its own, for the cell contents it is replayed on, and lists of contents that
+// a graph may replace are made at every sweep: the sweeps' buffers are sized by the
+// lists, which must be those of the cells they meet.
+int* kept_lists(cl_list* c, cudaStream_t s) {
+  if (!c->replayed && !clk::capturing(s)) return &c->lists_half;
+  c->lists_none = 0;
+  return &c->lists_none;
 }
 
 // Squared radius about a cell's centre that holds every particle within rc of
@@ -468,29 +481,29 @@ int cl_map(const cl_list* cc, cl_reduction red, const cl_params* params, cl_resu
       if (!r->count) return CL_ERR_INVALID_ARG;
       if (scalar_staged(c))
         return clk::launch_hood_scalar(*c->half, *c->hood, c->work, 0, r->count, c->partials, hood_cap(c), c->sums,
-                                       nullptr, 0, 0.f, nullptr, s, &c->lists_half);
+                                       nullptr, 0, 0.f, nullptr, s, kept_lists(c, s));
       return clk::launch_count(*c->half, dim, r->count, s);
     case CL_RED_SUM_INV_R:
       if (!r->sum_inv_r) return CL_ERR_INVALID_ARG;
       if (scalar_staged(c))
         return clk::launch_hood_scalar(*c->half, *c->hood, c->work, 1, nullptr, c->partials, hood_cap(c), c->sums,
-                                       r->sum_inv_r, 0, 0.f, nullptr, s, &c->lists_half);
+                                       r->sum_inv_r, 0, 0.f, nullptr, s, kept_lists(c, s));
       return clk::launch_scalar(*c->half, dim, 0, c->partials, c->sums, r->sum_inv_r, s);
     case CL_RED_SF_ENERGY:
       if (!r->energy) return CL_ERR_INVALID_ARG;
       if (dim == 3 && c->n > 0 && clk::hood_half_fits(*c->half))
         return clk::launch_hood_scalar(*c->half, *c->hood, c->work, 3, nullptr, c->partials, hood_cap(c), c->sums,
-                                       r->energy, 0, 0.f, nullptr, s, &c->lists_half);
+                                       r->energy, 0, 0.f, nullptr, s, kept_lists(c, s));
       if (dim == 3 && c->n > 0)
         return clk::launch_hood(*c->half, nullptr, *c->hood, c->work, 2, c->geo.hinv, nullptr, nullptr, nullptr, nullptr,
-                                c->partials, hood_cap(c), c->sums, r->energy, nullptr, nullptr, s, &c->lists_half);
+                                c->partials, hood_cap(c), c->sums, r->energy, nullptr, nullptr, s, kept_lists(c, s));
       return clk::launch_scalar(*c->half, dim, 1, c->partials, c->sums, r->energy, s);
     case CL_RED_SF_ENERGY_FORCES_VIRIAL:
       if (!r->forces && c->n > 0) return CL_ERR_INVALID_ARG;
       if (dim == 3 && c->n > 0) {
         c->last_half = clk::half_path_applies(*c->full, c->half, *c->hood, 0) ? 1 : 0;
         return clk::launch_hood(*c->full, c->half, *c->hood, c->work, 0, c->geo.hinv, r->forces, nullptr, nullptr, nullptr,
-                                c->partials, hood_cap(c), c->sums, r->energy, r->virial, nullptr, s, &c->lists_half);
+                                c->partials, hood_cap(c), c->sums, r->energy, r->virial, nullptr, s, kept_lists(c, s));
       }
       return clk::launch_force(*c->full, dim, 0, c->geo.hinv, r->forces, nullptr, nullptr, nullptr, c->partials,
                                c->sums, r->energy, r->virial, nullptr, s);
@@ -499,7 +512,7 @@ int cl_map(const cl_list* cc, cl_reduction red, const cl_params* params, cl_resu
       double rmax = params->rmax > 0 ? params->rmax : c->geo.rc;
       if (scalar_staged(c))
         return clk::launch_hood_scalar(*c->half, *c->hood, c->work, 2, nullptr, c->partials, hood_cap(c), c->sums,
-                                       nullptr, params->nbins, (float)rmax, r->hist, s, &c->lists_half);
+                                       nullptr, params->nbins, (float)rmax, r->hist, s, kept_lists(c, s));
       return clk::launch_hist(*c->half, dim, params->nbins, (float)rmax, r->hist, s);
     }
     case CL_RED_PAIRLIST:
@@ -513,14 +526,15 @@ int cl_backward(const cl_list* cc, const double* grad_energy_dev, double* grad_p
                 double* virial_dev, void* stream) {
   if (!cc || !grad_energy_dev || (cc->n > 0 && !grad_pos_dev)) return CL_ERR_INVALID_ARG;
   cl_list* c = const_cast<cl_list*>(cc);
+  cudaStream_t s = (cudaStream_t)stream;
   if (c->geo.dim == 3 && c->n > 0) {
     c->last_half = clk::half_path_applies(*c->full, c->half, *c->hood, 1) ? 1 : 0;
     return clk::launch_hood(*c->full, c->half, *c->hood, c->work, 1, c->geo.hinv, nullptr, grad_pos_dev, grad_energy_dev,
                             c->pos, c->partials, hood_cap(c), c->sums, nullptr, virial_dev, grad_box_dev,
-                            (cudaStream_t)stream, &c->lists_half);
+                            s, kept_lists(c, s));
   }
   return clk::launch_force(*c->full, c->geo.dim, 1, c->geo.hinv, nullptr, grad_pos_dev, grad_energy_dev, c->pos,
-                           c->partials, c->sums, nullptr, virial_dev, grad_box_dev, (cudaStream_t)stream);
+                           c->partials, c->sums, nullptr, virial_dev, grad_box_dev, s);
 }
 
 int cl_energy_grad(const cl_list* cc, const double* scale_dev, double* energy_dev, double* grad_pos_dev,
@@ -532,7 +546,7 @@ int cl_energy_grad(const cl_list* cc, const double* scale_dev, double* energy_de
     c->last_half = clk::half_path_applies(*c->full, c->half, *c->hood, 3) ? 1 : 0;
     return clk::launch_hood(*c->full, c->half, *c->hood, c->work, 3, c->geo.hinv, nullptr, grad_pos_dev, scale_dev, c->pos,
                             c->partials, hood_cap(c), c->sums, energy_dev, virial_dev, grad_box_dev, s,
-                            &c->lists_half);
+                            kept_lists(c, s));
   }
   // 2D (and the empty list): the energy sweep, then the backward sweep
   int e = clk::launch_scalar(*c->half, c->geo.dim, 1, c->partials, c->sums, energy_dev, s);

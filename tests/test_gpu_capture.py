@@ -92,3 +92,64 @@ def test_build_in_a_relaxed_capture(cuda_ok):
     P.cl_free(cl)
     del graph
     assert _count(P, P.cl_build(x, H, RC, 2)) == want[0]
+
+
+def _sweeps(P, cl):
+    efv = P.cl_map(cl, "energy_forces_virial")
+    return P.cl_map(cl, "energy")["energy"], efv["energy"], efv["forces"], P.cl_map(cl, "count")["count"]
+
+
+def _same(got, want):
+    for a, b in zip(got[:2], want[:2]):
+        assert a.item() == pytest.approx(b.item(), rel=1e-6)
+    assert (got[2] - want[2]).abs().max() <= 1e-5 * want[2].abs().max()
+    assert got[3].item() == want[3].item()
+
+
+def _sets():
+    """One particle a cell or so, and the same number in an eighth of the box, on a
+    jittered grid: cells of other sizes take other routes through the sweeps."""
+    rng = np.random.default_rng(5)
+    g = np.stack(np.meshgrid(*[np.arange(18)] * 3, indexing="ij"), -1).reshape(-1, 3)[:N]
+    return [torch.from_numpy((g + 0.5 + rng.uniform(-0.2, 0.2, size=g.shape)) * s).cuda() for s in (20 / 18, 10 / 18)]
+
+
+def test_sweeps_between_replays_of_an_update(cuda_ok):
+    """A replayed update changes the cells without a call: the sweeps' work lists
+    of the cells before must not be used."""
+    import paper_2202_06427_gb300 as P
+    sets = _sets()
+    want = [_sweeps(P, P.cl_build(x, H, RC, 2)) for x in sets]
+    held = sets[0].clone()
+    cl = P.cl_build(held, H, RC, 2)
+    torch.cuda.synchronize()
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.stream(torch.cuda.Stream()):
+        graph.capture_begin()
+        P.cl_update(cl, held)
+        graph.capture_end()
+    for k in (0, 1, 0, 1):
+        held.copy_(sets[k])
+        graph.replay()
+        _same(_sweeps(P, cl), want[k])
+
+
+def test_replayed_sweeps_after_an_update(cuda_ok):
+    """Sweeps captured on a list whose work lists were there, replayed after an
+    update of the list."""
+    import paper_2202_06427_gb300 as P
+    sets = _sets()
+    want = [_sweeps(P, P.cl_build(x, H, RC, 2)) for x in sets]
+    cl = P.cl_build(sets[0], H, RC, 2)
+    _sweeps(P, cl)
+    torch.cuda.synchronize()
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.stream(torch.cuda.Stream()):
+        graph.capture_begin()
+        got = _sweeps(P, cl)
+        graph.capture_end()
+    for k in (1, 0, 1):
+        P.cl_update(cl, sets[k])
+        graph.replay()
+        _same(got, want[k])
+        _same(_sweeps(P, cl), want[k])
