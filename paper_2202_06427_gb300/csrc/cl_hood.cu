@@ -749,7 +749,7 @@ __device__ __forceinline__ int run_count(const int* __restrict__ cell_start, int
 // from its start. kListLanes lanes share a cell's rows: one thread per cell took 13
 // us on a grid of 343 cells and 18 on one of 42,875 (now 11; bound by the latency of
 // the row bounds). Listed by warps instead of blocks, the lists' three counters took
-// 15 us there, 104 at 421,875 cells (now 32).
+// 15 us there, 104 at 421,875 cells (now, with a fourth, 38).
 constexpr int kListLanes = 8;  // 32 cells to a block of 256
 __global__ void __launch_bounds__(256) k_hood_list(const int* __restrict__ cell_start, int ncells, int noff,
                                                    int* __restrict__ work, int* __restrict__ list,
